@@ -229,7 +229,9 @@ typedef struct fit_batch_opts {
     int history;          /* L-BFGS pairs kept, 1..32 (default 32; the two-loop recursion runs
                              on one warp, a lane per pair)                                   */
     double f_noise_rel;   /* relative noise allowance of -2lnL in the line search (1e-6)     */
-    int threads;          /* threads per block, multiple of 32 in [64, 128]; 0 = default 128 */
+    int threads;          /* threads per block, multiple of 32 in [64, 128]; 0 = chosen by the
+                             library from the models' sizes (128, 256 or 512) when blocks_per_sm
+                             and placement are 0 too, else 128                              */
     int blocks_per_sm;    /* resident blocks per SM (an upper bound): 5 or more selects the
                              96-register build of the kernel, 1-4 the 128-register one;
                              0 = automatic                                                  */

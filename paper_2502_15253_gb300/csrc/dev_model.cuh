@@ -52,13 +52,37 @@ struct DevDataset {
     const int *sp_param;     // [n_sp] parameter index
     const int *sp_ptr;       // [n_sp + 1] CSR offsets into sp_k
     const int *sp_k;         // true bins of each shape parameter
+    int sp_lanes;            // lanes that share one shape parameter's sum (a power of two <= 32)
     float w[FIT_MAX_CORES];  // core flux shares
     float kl_hi[FIT_MAX_CORES], kl_lo[FIT_MAX_CORES];  // K L_dc / pi as a float pair (half-turns)
+};
+
+// One tile of a triangular matrix-vector product: out rows row0..row0+31 of a block (clipped to it),
+// summed over `cols` <= kTriCols columns from col0.
+constexpr int kTriCols = 64;
+struct TriTile {
+    int mat;                 // offset of the block's matrix (rows of n floats, column-major over the
+                             // tile's lanes: element (out r, in c) at mat + c * n + r)
+    int n;                   // block size
+    int row0, col0, cols;
+    int in0;                 // first input index when the block's parameters are consecutive, else -1
+    int idx;                 // offset of the block's parameter indices (DevModel::blk_idx)
+    int out;                 // concatenated row of the block's row 0
+    int seg;                 // partial-sum slot
+};
+
+// Bin j of background q (dataset d, row of the data vector of that dataset) scaled by a shape parameter
+struct BkgShapeRef {
+    int d, q, j;
+    float tmpl;
 };
 
 struct DevModel {
     int P, N_t, C, n_ds, n_data, osc_mode, n_blocks, n_bkg;
     float e_lo, de, inv_de;
+    float e_first, e_last;   // e_edge[0], e_edge[N_t]
+    int shared_roles;        // 1: some parameter has two roles (say, a shape of two datasets, or a
+                             // rate that is also a norm): its gradient additions need ordering
     int n_osc;               // survival parameters of osc_mode: 4, or 6 (FIT_OSC_STERILE4)
     int remap_mode;          // FIT_REMAP_OVERLAP or FIT_REMAP_SPLINE
     int osc_idx[kMaxOsc];
@@ -81,14 +105,28 @@ struct DevModel {
     const int *blk_size;     // [n_blocks]
     const int *blk_idx_off;  // [n_blocks]
     const int *blk_idx;      // concatenated parameter indices
-    const int *blk_first;    // [n_blocks] first index when a block's indices are consecutive, else -1
     const int64_t *blk_mat_off;  // [n_blocks] offset of the block's m x m matrices
     const float *blk_L;      // lower Cholesky factor of V (row-major, dense)
     const float *blk_W;      // L^-1 (row-major, dense lower triangle)
     const double *blk_L64;   // L in double (final theta of a fit)
     const float *asimov;     // [n_data] expectation at theta0
     const int *slot_ds;      // [n_data] dataset of each data bin
-    int ws_eval_floats;      // per-block workspace of one evaluation
+    int ws_eval_floats;      // workspace of one dataset of one evaluation (a multiple of 4)
+    int ws_group;            // datasets evaluated together (their workspaces are held at once)
+    // matrix-vector products with the triangular prior blocks as tiles of 32 rows x kTriCols
+    // columns (see tri_apply): tri_lo for L z / W d, tri_up for L^T g / W^T z
+    const TriTile *tri_lo, *tri_up;
+    int n_tri_lo, n_tri_up, tri_segs, tri_rows;   // tiles, column segments, rows of all blocks
+    const int *tri_param;    // [tri_rows] parameter of each concatenated row
+    const int *tri_seg;      // [tri_rows] its segments: lower 0..(x & 255) - 1, upper
+                             // (x >> 8 & 255)..(x >> 16) - 1
+    int ws_floats;           // per-block workspace of one evaluation: ws_group datasets, or the
+                             // tri_segs x tri_rows partial sums if larger
+    // background-shape parameters and the (background, bin) pairs each one scales, by dataset
+    const int *bs_param;     // [n_bs]
+    const int *bs_ptr;       // [n_bs + 1]
+    const BkgShapeRef *bs_ref;
+    int n_bs;
     int max_reco;
     int ldt;                 // row stride of the dense response (N_t rounded up to 4)
     // Fisher preconditioner (nullptr until built): z = T w, T = I + Q diag(c) Q^T; pre_Q holds
@@ -100,60 +138,46 @@ struct DevModel {
 // ------------------------------------------------------------------------------------
 // Reductions: FP32 within a warp, FP64 across warps.
 // ------------------------------------------------------------------------------------
-template <int N>
-__device__ __forceinline__ void warp_sum(float (&v)[N]) {
+// Sum of one value per thread over the block, on every thread: FP32 within a warp, then one
+// warp adds the warps' totals in double (a double addition occupies the SM's FP64 pipe for 16
+// cycles per warp, so only one warp does it). red: kMaxWarps + 1 doubles of shared scratch,
+// reusable by the next call without another barrier. Contains two __syncthreads.
+__device__ __forceinline__ double block_sum(float v, double *red) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    if (lane == 0) red[warp] = (double)v;
+    __syncthreads();
+    if (warp == 0) {
+        double t = lane < nw ? red[lane] : 0.0;
 #pragma unroll
-        for (int i = 0; i < N; ++i) v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
+        for (int o = kMaxWarps / 2; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        if (lane == 0) red[kMaxWarps] = t;
     }
+    __syncthreads();
+    return red[kMaxWarps];
 }
 
-// Sums N per-thread values over the block. red: shared scratch of kMaxWarps * N doubles
-// (+ N result slots). Every thread returns the N totals. Contains two __syncthreads.
+// Warp totals of N (a power of two <= 32) per-lane values with N - 1 + log2(32 / N) shuffles
+// instead of 5 N: each step exchanges half of the values with the partner lane and keeps the
+// sums of the other half. Lane l returns the total of value l >> (5 - log2 N), every lane of
+// the group the same; the additions are those of warp_sum's tree.
 template <int N>
-__device__ __forceinline__ void block_sum(float (&v)[N], double *red, double (&out)[N]) {
-    warp_sum<N>(v);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    if (lane == 0) {
+__device__ __forceinline__ float warp_sum_split(float (&v)[N]) {
+    const int lane = threadIdx.x & 31;
+    int o = 16;
 #pragma unroll
-        for (int i = 0; i < N; ++i) red[warp * N + i] = (double)v[i];
+    for (int n = N; n > 1; n >>= 1, o >>= 1) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int i = 0; i < n / 2; ++i) {
+            const float give = up ? v[i] : v[i + n / 2], keep = up ? v[i + n / 2] : v[i];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+        }
     }
-    __syncthreads();
-    if (threadIdx.x < N) {
-        double s = 0.0;
-        for (int w = 0; w < nw; ++w) s += red[w * N + threadIdx.x];
-        red[kMaxWarps * N + threadIdx.x] = s;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < N; ++i) out[i] = red[kMaxWarps * N + i];
-    __syncthreads();
-}
-
-// Same with double per-thread inputs (used where a thread already sums many terms).
-template <int N>
-__device__ __forceinline__ void block_sum_d(double (&v)[N], double *red, double (&out)[N]) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-#pragma unroll
-        for (int i = 0; i < N; ++i) v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
-    }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    if (lane == 0) {
-#pragma unroll
-        for (int i = 0; i < N; ++i) red[warp * N + i] = v[i];
-    }
-    __syncthreads();
-    if (threadIdx.x < N) {
-        double s = 0.0;
-        for (int w = 0; w < nw; ++w) s += red[w * N + threadIdx.x];
-        red[kMaxWarps * N + threadIdx.x] = s;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < N; ++i) out[i] = red[kMaxWarps * N + i];
-    __syncthreads();
+    float t = v[0];
+    for (; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    return t;
 }
 
 // ------------------------------------------------------------------------------------
@@ -448,33 +472,10 @@ __device__ __forceinline__ float deviance(float n, float mu) {
     return 2.f * mu * h;
 }
 
-// ------------------------------------------------------------------------------------
-// Per-dataset workspace (floats), all of length N_t unless noted:
-//   u, v(->gv), ts = t s, ptot, dp0..dp3 (dp0 is reused for the shape gradient),
-//   pcw[C] = w_c P_c per core, f0[max_reco], gmu[max_reco]
-// ------------------------------------------------------------------------------------
-struct EvalWs {
-    float *u, *v, *ts, *ptot, *dp, *pcw, *f0, *gmu;
+// Parameter access: pv = value, pd = value - theta0, pl = the rounding residual of pv (see PP).
+struct ParVecs {
+    const float *pv, *pd, *pl;
 };
-
-__host__ __device__ inline int eval_ws_floats(int N_t, int C, int max_reco, int n_osc) {
-    return (4 + n_osc + C) * N_t + 2 * max_reco;
-}
-
-__device__ __forceinline__ EvalWs carve_eval_ws(float *base, int N_t, int C, int max_reco, int n_osc) {
-    EvalWs w;
-    w.u = base;
-    w.v = w.u + N_t;
-    w.ts = w.v + N_t;
-    w.ptot = w.ts + N_t;
-    w.dp = w.ptot + N_t;          // n_osc * N_t
-    w.pcw = w.dp + n_osc * N_t;   // C * N_t
-    w.f0 = w.pcw + C * N_t;       // max_reco
-    w.gmu = w.f0 + max_reco;      // max_reco
-    return w;
-}
-
-// Parameter access: pv = value, pd = value - theta0 (kept separately for precision).
 __device__ __forceinline__ float pval(const float *pv, int idx, float dflt) {
     return idx >= 0 ? pv[idx] : dflt;
 }
@@ -492,6 +493,15 @@ __device__ __forceinline__ PP ppair(const DevModel &m, const float *pv, const fl
     if (p < 0) return PP{dflt, 0.f};
     const float h = pv[p];
     return PP{h, ((m.theta0_f[p] - h) + pd[p]) + m.theta0_lo[p]};
+}
+
+// the residual l of parameter p, for a vector of them
+__device__ __forceinline__ float presid(const DevModel &m, float h, float delta, int p) {
+    return ((m.theta0_f[p] - h) + delta) + m.theta0_lo[p];
+}
+
+__device__ __forceinline__ PP ppair(const ParVecs &q, int p, float dflt) {
+    return p < 0 ? PP{dflt, 0.f} : PP{q.pv[p], q.pl[p]};
 }
 
 __device__ __forceinline__ float pmul(PP a, float x) { return fmaf(x, a.l, x * a.h); }
@@ -655,440 +665,713 @@ __device__ __forceinline__ EMap make_emap(const DevModel &m, const DevDataset &d
 }
 
 // ------------------------------------------------------------------------------------
-// Block-level evaluation of one dataset, in stages that the fit kernels call either in one
-// sequence (eval_dataset) or split over two launches (forward + likelihood, then adjoint).
+// Block-level evaluation of one parameter vector.
+//
+// What bounds it: a few hundred kFLOP per vector in a dozen dependent stages over a few hundred
+// to a few thousand bins, so with one block per vector the time is the chain of barriers,
+// reductions and load latencies, not arithmetic or bandwidth. So every stage runs over all
+// datasets of the vector together (a "group": the datasets whose workspaces are held at once,
+// DevModel::ws_group), with one barrier per stage for the group instead of one per dataset and
+// stage, and the warps that one dataset leaves over start on the next (each dataset's bins
+// begin at the warp where the previous dataset's ended).
 // ------------------------------------------------------------------------------------
-// Per-dataset constants of one evaluation: survival parameters and coefficients,
-// normalisation, efficiency, energy map.
-template <int NOSC>
-struct DsCtxT {
-    typename OscTraits<NOSC>::Coef kc;
-    float eta[NOSC], eta_lo[NOSC];
-    PP nrm, eff;
-    EMap em;
+// Per-dataset workspace (floats), arrays of length N_t unless noted:
+//   u, v (-> gv), ts = t s, ptot, dp[n_osc] (dp[0] is reused for the shape gradient),
+//   pcw[C] = w_c P_c per core, f0[max_reco], gmu[max_reco]
+struct DsWs {
+    float *u, *v, *ts, *ptot, *dp, *pcw, *f0, *gmu;
 };
-using DsCtx = DsCtxT<4>;
 
-// Fills c; false (and status |= kStEscale) when the energy map is not increasing with slope in
-// (1/4, 4) on the grid. Contains a barrier.
+__host__ __device__ inline int eval_ws_floats(int N_t, int C, int max_reco, int n_osc) {
+    return ((4 + n_osc + C) * N_t + 2 * max_reco + 3) & ~3;
+}
+
+__device__ __forceinline__ DsWs carve_ds_ws(float *base, int N_t, int C, int max_reco, int n_osc) {
+    DsWs w;
+    w.u = base;
+    w.v = w.u + N_t;
+    w.ts = w.v + N_t;
+    w.ptot = w.ts + N_t;
+    w.dp = w.ptot + N_t;          // n_osc * N_t
+    w.pcw = w.dp + n_osc * N_t;   // C * N_t
+    w.f0 = w.pcw + C * N_t;       // max_reco
+    w.gmu = w.f0 + max_reco;      // max_reco
+    return w;
+}
+
+// Shared state of one evaluation (one per block).
+struct EvalShared {
+    typename OscTraits<6>::Coef kc;         // sin^2 coefficients (the first three for 4 parameters)
+    float eta[kMaxOsc], eta_lo[kMaxOsc];
+    PP nrm[FIT_MAX_DATASETS], eff[FIT_MAX_DATASETS];
+    EMap em[FIT_MAX_DATASETS];
+    PP power[FIT_MAX_CORES], rate[FIT_MAX_BACKGROUNDS];
+    int dl[FIT_MAX_DATASETS];               // datasets of the current group
+    int n;                                  // their number
+    int bad;                                // 1: the dataset after them has an invalid energy map
+    int status;                             // kSt* bits
+    double nll;                             // sum over the datasets so far
+    // warp totals: likelihood sums [dataset][warp][8], then energy-map sums [dataset][warp][4] and
+    // survival / power sums [warp][32] (the two uses are barriers apart)
+    float part[FIT_MAX_DATASETS * kMaxWarps * 8];
+};
+
+// Logical thread index of this thread in a stage whose datasets take `per` warps each: dataset
+// number i starts at the warp where dataset i - 1 ended.
+__device__ __forceinline__ int rot_tid(int i, int per) {
+    const int nw = blockDim.x >> 5;
+    int w = (int)(threadIdx.x >> 5) - (i * per) % nw;
+    if (w < 0) w += nw;
+    return w * 32 + (int)(threadIdx.x & 31);
+}
+
+// Group setup: the datasets `first`, ... of the mask, at most m.ws_group of them (E.dl, E.n),
+// survival parameters and coefficients, normalisations, efficiencies, energy maps, powers,
+// rates. A dataset whose energy map is not increasing with slope in (1/4, 4) on the grid ends
+// the list (E.bad). Returns the dataset after the group. Starts and ends with a barrier.
 template <int NOSC>
-static __device__ bool ds_setup(const DevModel &m, int d, const float *pv, const float *pd, DsCtxT<NOSC> &c,
-                                int *status) {
-    const DevDataset &ds = m.ds[d];
-    const int N_t = m.N_t;
-    const int tid = threadIdx.x;
-    // Survival parameters: mass splittings as theta0_f + (theta0_lo + delta) inside the
-    // phase.
-    float *eta = c.eta, *eta_lo = c.eta_lo;
+static __device__ int eval_setup(const DevModel &m, EvalShared &E, const ParVecs &q, uint32_t mask, int first,
+                                 int group) {
+    __syncthreads();
+    const int tid = threadIdx.x, lane = tid & 31;
+    int next = first;
+    {   // every thread walks the mask (at most 8 datasets)
+        int n = 0;
+        bool bad = false;
+        while (next < m.n_ds && n < group) {
+            const int d = next++;
+            if (!((mask >> d) & 1u)) continue;
+            const DevDataset &ds = m.ds[d];
+            const EMap em = make_emap(m, ds, q.pv, q.pd);
+            const float s0 = em.slope(m.e_first), s1 = em.slope(m.e_last);
+            if (!(s0 > 0.25f && s0 < 4.f && s1 > 0.25f && s1 < 4.f)) {
+                bad = true;
+                break;
+            }
+            if (tid == 32 + n) {
+                E.dl[n] = d;
+                E.em[n] = em;
+                E.nrm[n] = ppair(q, ds.norm_idx, 1.f);
+                E.eff[n] = ppair(q, ds.eff_idx, 1.f);
+            }
+            ++n;
+        }
+        if (tid == 0) {
+            E.n = n;
+            E.bad = bad;
+        }
+    }
+    const int warp = tid >> 5;
+    if (warp == 0) {
+        // survival parameters: mass splittings as theta0_f + (theta0_lo + delta) inside the phase
+        if (lane < NOSC) {
+            const int p = m.osc_idx[lane];
+            float h, l;
+            if (osc_is_dm(m.osc_mode, lane)) {
+                h = p >= 0 ? m.theta0_f[p] : m.osc_val[lane];
+                l = p >= 0 ? m.theta0_lo[p] + q.pd[p] : m.osc_val_lo[lane];
+            } else {
+                h = p >= 0 ? q.pv[p] : m.osc_val[lane];
+                l = 0.f;
+            }
+            E.eta[lane] = h;
+            E.eta_lo[lane] = l;
+        }
+        // the sin^2 coefficients from float pairs of the exact parameter values
+        F2 e[NOSC];
 #pragma unroll
-    for (int i = 0; i < NOSC; ++i) {
-        const int p = m.osc_idx[i];
-        if (osc_is_dm(m.osc_mode, i)) {
-            eta[i] = p >= 0 ? m.theta0_f[p] : m.osc_val[i];
-            eta_lo[i] = p >= 0 ? m.theta0_lo[p] + pd[p] : m.osc_val_lo[i];
-        } else {
-            eta[i] = p >= 0 ? pv[p] : m.osc_val[i];
-            eta_lo[i] = 0.f;
+        for (int i = 0; i < NOSC; ++i) {
+            const int p = m.osc_idx[i];
+            e[i] = p >= 0 ? f2_norm(q.pv[p], q.pl[p]) : F2{m.osc_val[i], m.osc_val_lo[i]};
         }
-    }
-    // the sin^2 coefficients from float pairs of the exact parameter values (every thread
-    // forms the same values; no barrier)
-    F2 e[NOSC];
+        const auto k = OscTraits<NOSC>::coef(m.osc_mode, e);
+        if (lane == 0) {
 #pragma unroll
-    for (int i = 0; i < NOSC; ++i) {
-        const int p = m.osc_idx[i];
-        if (p >= 0) {
-            const float h = pv[p];
-            e[i] = f2_norm(h, ((m.theta0_f[p] - h) + pd[p]) + m.theta0_lo[p]);
-        } else {
-            e[i] = F2{m.osc_val[i], m.osc_val_lo[i]};
+            for (int i = 0; i < (int)(sizeof(k.hi) / sizeof(float)); ++i) {
+                E.kc.hi[i] = k.hi[i];
+                E.kc.lo[i] = k.lo[i];
+            }
         }
+    } else if (warp == 1) {
+        if (lane >= 16 && lane - 16 < m.C) E.power[lane - 16] = ppair(q, m.core_power_idx[lane - 16], 1.f);
     }
-    c.kc = OscTraits<NOSC>::coef(m.osc_mode, e);
-    c.nrm = ppair(m, pv, pd, ds.norm_idx, 1.f);
-    c.eff = ppair(m, pv, pd, ds.eff_idx, 1.f);
-    c.em = make_emap(m, ds, pv, pd);
-    const EMap &em = c.em;
-
-    // the map must be increasing with slope in (1/4, 4) everywhere on the grid
-    {
-        const float s0 = em.slope(m.e_edge[0]), s1 = em.slope(m.e_edge[N_t]);
-        if (!(s0 > 0.25f && s0 < 4.f && s1 > 0.25f && s1 < 4.f)) {
-            if (tid == 0) atomicOr(status, kStEscale);
-            return false;
-        }
-    }
-
-    return true;
+    if (warp == (int)(blockDim.x >> 5) - 1 && lane < m.n_bkg) E.rate[lane] = ppair(q, m.bkg[lane].rate_idx, 1.f);
+    __syncthreads();
+    return next;
 }
 
 // Stage A: u_k (and with DERIV the per-bin partials the adjoint needs). Ends with a barrier.
-template <bool DERIV, int NOSC>
-static __device__ void ds_signal(const DevModel &m, int d, const float *pv, const float *pd,
-                                 const DsCtxT<NOSC> &c, EvalWs ws) {
-    const DevDataset &ds = m.ds[d];
-    const int N_t = m.N_t, C = m.C;
-    const int tid = threadIdx.x, nth = blockDim.x;
-    // ---- stage A: signal on the true grid (Eq. 1/2 x shares x reweights) -----------------
-    for (int k = tid; k < N_t; k += nth) {
-        const float ih = m.inv_e_hi[k], il = m.inv_e_lo[k];
-        float pt = 0.f, dpt[NOSC];
+template <bool DERIV, int NOSC, int MODE>
+static __device__ __forceinline__ void st_signal_mode(const DevModel &m, const EvalShared &E, const ParVecs &q,
+                                                      float *wsb) {
+    const int N_t = m.N_t, C = m.C, nth = blockDim.x;
+    typename OscTraits<NOSC>::Coef kc;
 #pragma unroll
-        for (int i = 0; i < NOSC; ++i) dpt[i] = 0.f;
-        for (int cc = 0; cc < C; ++cc) {
-            const float w = ds.w[cc];
-            if (w == 0.f) {
-                if (DERIV) ws.pcw[cc * N_t + k] = 0.f;
-                continue;
+    for (int i = 0; i < (int)(sizeof(kc.hi) / sizeof(float)); ++i) {
+        kc.hi[i] = E.kc.hi[i];
+        kc.lo[i] = E.kc.lo[i];
+    }
+    float eta[NOSC], eta_lo[NOSC];
+#pragma unroll
+    for (int i = 0; i < NOSC; ++i) {
+        eta[i] = E.eta[i];
+        eta_lo[i] = E.eta_lo[i];
+    }
+    for (int i = 0; i < E.n; ++i) {
+        const DevDataset &ds = m.ds[E.dl[i]];
+        const DsWs ws = carve_ds_ws(wsb + (int64_t)i * m.ws_eval_floats, N_t, C, m.max_reco, m.n_osc);
+        const PP nrm = E.nrm[i];
+        for (int k = rot_tid(i, (N_t + 31) >> 5); k < N_t; k += nth) {
+            const float ih = m.inv_e_hi[k], il = m.inv_e_lo[k];
+            const int sp = ds.shape_idx[k];
+            const float tk = ds.t[k];
+            float pt = 0.f, dpt[NOSC];
+#pragma unroll
+            for (int j = 0; j < NOSC; ++j) dpt[j] = 0.f;
+            for (int c = 0; c < C; ++c) {
+                const float w = ds.w[c];
+                if (w == 0.f) {
+                    if (DERIV) ws.pcw[c * N_t + k] = 0.f;
+                    continue;
+                }
+                const float ch = ds.kl_hi[c] * ih;
+                const float cl = fmaf(ds.kl_hi[c], ih, -ch) + ds.kl_hi[c] * il + ds.kl_lo[c] * ih;
+                float dP[NOSC];
+                const float P = OscTraits<NOSC>::survival(MODE, eta, eta_lo, kc, ch, cl, dP);
+                const PP pw = E.power[c];
+                const float wP = w * P;
+                if (DERIV) ws.pcw[c * N_t + k] = wP;
+                pt += pmul(pw, wP);
+                if (DERIV) {
+#pragma unroll
+                    for (int j = 0; j < NOSC; ++j) dpt[j] = fmaf(pw.h * w, dP[j], dpt[j]);
+                }
             }
-            const float ch = ds.kl_hi[cc] * ih;
-            const float cl = fmaf(ds.kl_hi[cc], ih, -ch) + ds.kl_hi[cc] * il + ds.kl_lo[cc] * ih;
-            float dP[NOSC];
-            const float P = OscTraits<NOSC>::survival(m.osc_mode, c.eta, c.eta_lo, c.kc, ch, cl, dP);
-            const PP pw = ppair(m, pv, pd, m.core_power_idx[cc], 1.f);
-            const float wP = w * P;
-            if (DERIV) ws.pcw[cc * N_t + k] = wP;
-            pt += pmul(pw, wP);
+            const float ts = pmul(ppair(q, sp, 1.f), tk);
+            if (DERIV) {
+                ws.ts[k] = ts;
+                ws.ptot[k] = pt;
 #pragma unroll
-            for (int i = 0; i < NOSC; ++i) if (DERIV) dpt[i] = fmaf(pw.h * w, dP[i], dpt[i]);
+                for (int j = 0; j < NOSC; ++j) ws.dp[j * N_t + k] = dpt[j];
+            }
+            ws.u[k] = pmul(nrm, ts * pt);
         }
-        const float ts = pmul(ppair(m, pv, pd, ds.shape_idx[k], 1.f), ds.t[k]);
-        if (DERIV) {
-            ws.ts[k] = ts;
-            ws.ptot[k] = pt;
-        }
-#pragma unroll
-        for (int i = 0; i < NOSC; ++i)
-            if (DERIV) ws.dp[i * N_t + k] = dpt[i];
-        ws.u[k] = pmul(c.nrm, ts * pt);
     }
     __syncthreads();
-
 }
 
-// Stage B: v = M(a) u. Ends with a barrier.
-// SPL: compiled with the area-conserving spline option (the general kernel builds)
-template <bool SPL, class Ctx>
-static __device__ void ds_remap(const DevModel &m, int d, const Ctx &c, EvalWs ws) {
-    (void)d;   // the energy map is in c
-    const int N_t = m.N_t;
-    const int tid = threadIdx.x, nth = blockDim.x;
-    const EMap &em = c.em;
-    if (SPL && m.remap_mode == FIT_REMAP_SPLINE) {
-        for (int t = tid; t < N_t; t += nth) ws.v[t] = spline_target(ws.u, m.e_edge, em, t, N_t);
-        __syncthreads();
-        return;
+// GEN: the general build (any formula); else Eq. 1 or the three-flavour formula.
+template <bool DERIV, bool GEN>
+static __device__ __forceinline__ void st_signal(const DevModel &m, const EvalShared &E, const ParVecs &q, float *wsb) {
+    if (GEN && m.osc_mode == FIT_OSC_STERILE4)
+        st_signal_mode<DERIV, 6, FIT_OSC_STERILE4>(m, E, q, wsb);
+    else if (m.osc_mode == FIT_OSC_EQ1)
+        st_signal_mode<DERIV, 4, FIT_OSC_EQ1>(m, E, q, wsb);
+    else
+        st_signal_mode<DERIV, 4, FIT_OSC_VACUUM3>(m, E, q, wsb);
+}
+
+// Corrected content of target bin t under the overlap rule. Source bin k covers [Y_k, Y_k+1] in
+// grid units, Y_k = k + D(e_k); target t gathers the sources whose mapped interval overlaps
+// [t, t+1]; overlaps are computed relative to the target (k - t is an exact small integer),
+// which keeps them accurate in FP32.
+__device__ __forceinline__ float overlap_target(const float *u, const float *e_edge, const EMap &em, int t, int N_t) {
+    // first source whose mapped upper edge lies above t: start from the fixed point
+    // k ~ t - D(k) and step until the bracket is right
+    int k = t - (int)floorf(em.disp(e_edge[t]));
+    k = min(max(k, 0), N_t - 1);
+    k = t - (int)floorf(em.disp(e_edge[k]));
+    k = min(max(k - 1, 0), N_t - 1);
+    while (k > 0 && (float)(k - t) + em.disp(e_edge[k]) > 0.f) --k;
+    float acc = 0.f;
+    float dlo = em.disp(e_edge[k]);
+    for (int it = 0; it < 64 && k < N_t; ++it, ++k) {
+        const float dhi = em.disp(e_edge[k + 1]);
+        const float ylo = (float)(k - t) + dlo;      // mapped edges relative to target t
+        const float yhi = (float)(k + 1 - t) + dhi;
+        if (ylo >= 1.f) break;
+        const float ov = fminf(yhi, 1.f) - fmaxf(ylo, 0.f);
+        if (ov > 0.f) acc = fmaf(u[k], ov / (1.f + (dhi - dlo)), acc);
+        dlo = dhi;
     }
-    // ---- stage B: energy correction, gather per target bin ------------------------------
-    // Source bin k covers [Y_k, Y_k+1] in grid units, Y_k = k + D(e_k). Target m gathers the
-    // sources whose mapped interval overlaps [m, m+1]; overlaps are computed relative to the
-    // target (k - m is an exact small integer), which keeps them accurate in FP32.
-    for (int t = tid; t < N_t; t += nth) {
-        // first source whose mapped upper edge lies above t: start from the fixed point
-        // k ~ t - D(k) and step until the bracket is right
-        int k = t - (int)floorf(em.disp(m.e_edge[t]));
-        k = min(max(k, 0), N_t - 1);
-        k = t - (int)floorf(em.disp(m.e_edge[k]));
-        k = min(max(k - 1, 0), N_t - 1);
-        while (k > 0 && (float)(k - t) + em.disp(m.e_edge[k]) > 0.f) --k;
-        float acc = 0.f;
-        float dlo = em.disp(m.e_edge[k]);
-        for (int it = 0; it < 64 && k < N_t; ++it, ++k) {
-            const float dhi = em.disp(m.e_edge[k + 1]);
-            const float ylo = (float)(k - t) + dlo;      // mapped edges relative to target t
-            const float yhi = (float)(k + 1 - t) + dhi;
-            if (ylo >= 1.f) break;
-            const float ov = fminf(yhi, 1.f) - fmaxf(ylo, 0.f);
-            if (ov > 0.f) acc = fmaf(ws.u[k], ov / (1.f + (dhi - dlo)), acc);
-            dlo = dhi;
-        }
-        ws.v[t] = acc;
+    return acc;
+}
+
+// Stage B: v = M(a) u. Ends with a barrier. GEN: compiled with the spline option.
+template <bool GEN>
+static __device__ __forceinline__ void st_remap(const DevModel &m, const EvalShared &E, float *wsb) {
+    const int N_t = m.N_t, nth = blockDim.x;
+    const bool spline = GEN && m.remap_mode == FIT_REMAP_SPLINE;
+    for (int i = 0; i < E.n; ++i) {
+        const DsWs ws = carve_ds_ws(wsb + (int64_t)i * m.ws_eval_floats, N_t, m.C, m.max_reco, m.n_osc);
+        const EMap em = E.em[i];
+        for (int t = rot_tid(i, (N_t + 31) >> 5); t < N_t; t += nth)
+            ws.v[t] = spline ? spline_target(ws.u, m.e_edge, em, t, N_t) : overlap_target(ws.u, m.e_edge, em, t, N_t);
     }
     __syncthreads();
-
 }
 
-// Stage C: fold into reco bins, ws.f0 = R v (before the efficiency). Ends with a barrier.
-static __device__ void ds_fold(const DevModel &m, int d, EvalWs ws) {
-    const DevDataset &ds = m.ds[d];
-    const DevDetector &dt = m.det[ds.det];
-    const int nr = ds.n_reco;
-    const int tid = threadIdx.x, nth = blockDim.x;
-    const int lane = tid & 31, warp = tid >> 5, nw = nth >> 5;
-    // ---- stage C: fold into reco bins (banded rows, warp per row) ------------------------
-    // Each warp takes four rows at a time and two strides of each, so eight independent
-    // load/FMA chains per lane are in flight.
-    for (int j0 = warp; j0 < nr; j0 += 4 * nw) {
-        int lo[4], len[4];
-        const float *rr[4];
-        int lmax = 0;
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int j = j0 + u * nw;
-            const bool on = j < nr;
-            lo[u] = on ? dt.row_lo[j] : 0;
-            len[u] = on ? dt.row_len[j] : 0;
-            rr[u] = dt.rrow + (on ? dt.row_off[j] : 0);
-            lmax = max(lmax, len[u]);
-        }
-        float s[4][2] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
-        for (int b = lane; b < lmax; b += 64) {
+// Stage C: fold into reco bins, f0 = R v (before the efficiency), banded rows. Each warp takes
+// four rows at a time and two strides of each, so eight independent load/FMA chains per lane
+// are in flight. Ends with a barrier.
+static __device__ __forceinline__ void st_fold(const DevModel &m, const EvalShared &E, float *wsb) {
+    const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    for (int i = 0; i < E.n; ++i) {
+        const DevDataset &ds = m.ds[E.dl[i]];
+        const DevDetector &dt = m.det[ds.det];
+        const DsWs ws = carve_ds_ws(wsb + (int64_t)i * m.ws_eval_floats, m.N_t, m.C, m.max_reco, m.n_osc);
+        const int nr = ds.n_reco;
+        for (int j0 = rot_tid(i, nr) >> 5; j0 < nr; j0 += 4 * nw) {
+            int lo[4], len[4];
+            const float *rr[4];
+            int lmax = 0;
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                if (b < len[u]) s[u][0] = fmaf(rr[u][b], ws.v[lo[u] + b], s[u][0]);
-                if (b + 32 < len[u]) s[u][1] = fmaf(rr[u][b + 32], ws.v[lo[u] + b + 32], s[u][1]);
+                const int j = j0 + u * nw;
+                const bool on = j < nr;
+                lo[u] = on ? dt.row_lo[j] : 0;
+                len[u] = on ? dt.row_len[j] : 0;
+                rr[u] = dt.rrow + (on ? dt.row_off[j] : 0);
+                lmax = max(lmax, len[u]);
             }
-        }
-        float t[4];
+            float s[4][2] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
+            for (int b = lane; b < lmax; b += 64) {
 #pragma unroll
-        for (int u = 0; u < 4; ++u) t[u] = s[u][0] + s[u][1];
+                for (int u = 0; u < 4; ++u) {
+                    if (b < len[u]) s[u][0] = fmaf(rr[u][b], ws.v[lo[u] + b], s[u][0]);
+                    if (b + 32 < len[u]) s[u][1] = fmaf(rr[u][b + 32], ws.v[lo[u] + b + 32], s[u][1]);
+                }
+            }
+            float t[4];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-#pragma unroll
-            for (int u = 0; u < 4; ++u) t[u] += __shfl_xor_sync(0xffffffffu, t[u], o);
-        }
-        if (lane == 0) {
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-                if (j0 + u * nw < nr) ws.f0[j0 + u * nw] = t[u];
+            for (int u = 0; u < 4; ++u) t[u] = s[u][0] + s[u][1];
+            const float tot = warp_sum_split<4>(t);
+            const int j = j0 + (lane >> 3) * nw;
+            if ((lane & 7) == 0 && j < nr) ws.f0[j] = tot;
         }
     }
     __syncthreads();
 }
 
-// Stage C2: backgrounds, deviance, dD/dmu (ws.gmu) and the background-shape gradient from the
-// folded spectrum ws.f0; returns the dataset's -2lnL (all threads). The efficiency and rate
-// gradients are added when grad != nullptr, data != nullptr and no status bit is set.
-template <class Ctx>
-static __device__ double ds_lik(const DevModel &m, int d, const float *pv, const float *pd, const Ctx &c,
-                                const float *data, EvalWs ws, float *grad, double *red, int *status,
-                                float *mu_out) {
-    const DevDataset &ds = m.ds[d];
-    const int nr = ds.n_reco;
-    const int tid = threadIdx.x, nth = blockDim.x;
-    // ---- stage C2: backgrounds, deviance, dD/dmu ----------------------------------------
-    const int nb = ds.bkg_end - ds.bkg_begin;
-    float part[2 + kMaxBkgDs];
-    // part[0] = deviance, part[1] = d/d eff, part[2+b] = d/d rate_b
+// Expected counts of one bin: efficiency x fold + backgrounds; tm / sh receive the templates and
+// 1 + delta of the dataset's backgrounds (the loads of all of them in flight together).
+__device__ __forceinline__ float bin_mu(const DevModel &m, const EvalShared &E, int i, const DevDataset &ds,
+                                        const ParVecs &q, float f0, int j, int nb, float (&tm)[kMaxBkgDs],
+                                        float (&sh)[kMaxBkgDs]) {
+    int si[kMaxBkgDs];
 #pragma unroll
-    for (int i = 0; i < 2 + kMaxBkgDs; ++i) part[i] = 0.f;
-    for (int j = tid; j < nr; j += nth) {
-        float mu = pmul(c.eff, ws.f0[j]);
-#pragma unroll
-        for (int b = 0; b < kMaxBkgDs; ++b) {
-            if (b >= nb) break;
-            const DevBkg &bk = m.bkg[ds.bkg_begin + b];
-            const float tm = bk.tmpl[j];
-            const float shaped = bk.shape_idx[j] >= 0 ? fmaf(tm, pv[bk.shape_idx[j]], tm) : tm;
-            mu += pmul(ppair(m, pv, pd, bk.rate_idx, 1.f), shaped);
-        }
-        if (mu_out) mu_out[j] = mu;
-        if (data == nullptr) continue;
-        const float n = data[ds.data_off + j];
-        if (!(mu > 0.f)) {
-            atomicOr(status, kStMuNonpos);
-            continue;
-        }
-        part[0] += deviance(n, mu);
-        const float g = 2.f * (mu - n) / mu;
-        ws.gmu[j] = g;
-        if (grad) {
-            part[1] = fmaf(g, ws.f0[j], part[1]);
-#pragma unroll
-            for (int b = 0; b < kMaxBkgDs; ++b) {
-                if (b >= nb) break;
-                const DevBkg &bk = m.bkg[ds.bkg_begin + b];
-                const int si = bk.shape_idx[j];
-                const float sh = 1.f + (si >= 0 ? pv[si] : 0.f);
-                part[2 + b] = fmaf(g * bk.tmpl[j], sh, part[2 + b]);
-                if (si >= 0) atomicAdd(&grad[si], g * pval(pv, bk.rate_idx, 1.f) * bk.tmpl[j]);
-            }
-        }
+    for (int b = 0; b < kMaxBkgDs; ++b) {
+        const DevBkg &bk = m.bkg[ds.bkg_begin + min(b, max(nb - 1, 0))];
+        tm[b] = b < nb ? bk.tmpl[j] : 0.f;
+        si[b] = b < nb ? bk.shape_idx[j] : -1;
     }
-    double tot[2 + kMaxBkgDs];
-    block_sum<2 + kMaxBkgDs>(part, red, tot);
-    const double nll_d = tot[0];
-    if (data == nullptr || grad == nullptr || (*(volatile int *)status) != 0) return nll_d;
-    if (tid == 0) {
-        if (ds.eff_idx >= 0) grad[ds.eff_idx] += (float)tot[1];
+    float mu = pmul(E.eff[i], f0);
 #pragma unroll
-        for (int b = 0; b < kMaxBkgDs; ++b) {
-            if (b >= nb) break;
-            const int ri = m.bkg[ds.bkg_begin + b].rate_idx;
-            if (ri >= 0) grad[ri] += (float)tot[2 + b];
-        }
+    for (int b = 0; b < kMaxBkgDs; ++b) {
+        if (b >= nb) break;
+        const float del = si[b] >= 0 ? q.pv[si[b]] : 0.f;
+        sh[b] = 1.f + del;
+        mu += pmul(E.rate[ds.bkg_begin + b], fmaf(tm[b], del, tm[b]));
     }
-
-    return nll_d;
+    return mu;
 }
 
-// Stages C and C2 in one sequence.
-template <class Ctx>
-static __device__ double ds_fold_lik(const DevModel &m, int d, const float *pv, const float *pd, const Ctx &c,
-                                     const float *data, EvalWs ws, float *grad, double *red, int *status,
-                                     float *mu_out) {
-    ds_fold(m, d, ws);
-    return ds_lik(m, d, pv, pd, c, data, ws, grad, red, status, mu_out);
-}
-
-// Stage D: adjoint of the fold, ws.v <- gv = eff R^T gmu (column bands). Ends with a barrier.
-template <int NOSC>
-static __device__ void ds_adjoint_fold(const DevModel &m, int d, const DsCtxT<NOSC> &c, EvalWs ws) {
-    const DevDataset &ds = m.ds[d];
-    const DevDetector &dt = m.det[ds.det];
-    const int N_t = m.N_t, nr = ds.n_reco;
-    const int tid = threadIdx.x, nth = blockDim.x;
-    // ---- stage D: adjoint of the fold, gv = eff R^T gmu (column bands) --------------------
-    float *gv = ws.v;   // v is dead after the fold
-    // rcol is exactly 0 past each column's band, so the loop runs the widest band of the
-    // warp's 32 adjacent columns (nearly their own widths: the resolution changes slowly with
-    // energy) with the row index clamped (no early exit) and four partial sums
-    for (int k = tid; k < N_t; k += nth) {
-        const int lo = dt.col_lo[k], jmax = nr - 1;
-        const int cw = __reduce_max_sync(__activemask(), dt.col_len[k]);
-        const float *rc = dt.rcol + k;
-        float s[4] = {0.f, 0.f, 0.f, 0.f};
-        int b = 0;
-        for (; b + 7 < cw; b += 8) {   // eight loads in flight
-#pragma unroll
-            for (int q = 0; q < 8; ++q)
-                s[q & 3] = fmaf(rc[(int64_t)(b + q) * N_t], ws.gmu[min(lo + b + q, jmax)], s[q & 3]);
+// Expected counts of the group's datasets into mu (the whole data vector). Ends with a barrier.
+static __device__ __forceinline__ void st_mu(const DevModel &m, const EvalShared &E, const ParVecs &q, float *wsb,
+                                             float *mu) {
+    const int nth = blockDim.x;
+    for (int i = 0; i < E.n; ++i) {
+        const DevDataset &ds = m.ds[E.dl[i]];
+        const DsWs ws = carve_ds_ws(wsb + (int64_t)i * m.ws_eval_floats, m.N_t, m.C, m.max_reco, m.n_osc);
+        for (int j = rot_tid(i, (ds.n_reco + 31) >> 5); j < ds.n_reco; j += nth) {
+            float tm[kMaxBkgDs], sh[kMaxBkgDs];
+            mu[ds.data_off + j] = bin_mu(m, E, i, ds, q, ws.f0[j], j, ds.bkg_end - ds.bkg_begin, tm, sh);
         }
-        for (; b < cw; ++b) s[0] = fmaf(rc[(int64_t)b * N_t], ws.gmu[min(lo + b, jmax)], s[0]);
-        gv[k] = pmul(c.eff, (s[0] + s[1]) + (s[2] + s[3]));
     }
     __syncthreads();
 }
 
-// Stages E and F: adjoint of the energy map and of the signal from gv (in ws.v); adds the
-// gradient contributions to grad. Needs ws.u/ts/ptot/dp/pcw (ds_signal<true>).
-template <int NC, int NOSC, bool SPL>
-static __device__ void ds_adjoint_ef(const DevModel &m, int d, const float *pv, const float *pd,
-                                     const DsCtxT<NOSC> &c, EvalWs ws, float *grad, double *red) {
-    const DevDataset &ds = m.ds[d];
-    const int N_t = m.N_t, C = m.C;
-    const int tid = threadIdx.x, nth = blockDim.x;
-    const EMap &em = c.em;
-    const float *gv = ws.v;
-    (void)pv;
-    (void)pd;
-    // ---- stage E: adjoint of the energy map and of the signal ---------------------------
-    // per source k: gu = sum_t F_kt gv_t; A0 = (gu - gv(floor Y_k)) / w, A1 = (gv(floor Y_k+1) - gu) / w
-    constexpr int kN = 3 + NOSC, kP = 4 + NOSC;   // index of d/d norm, first d/d power
-    float ep[kP + NC];
-    // ep[0..2] d/da, ep[3..3+NOSC) d/d eta, ep[kN] d/d norm, ep[kP+c] d/d power_c (NC >= C)
+// Stage C2: backgrounds, deviance, dD/dmu (gmu) from the folded spectra f0, and the warp totals
+// of the deviance and of the efficiency and rate gradients (E.part). Bins with mu <= 0 raise
+// kStMuNonpos. Ends with a barrier; lik_finish adds the totals up.
+template <bool GRAD>
+static __device__ __forceinline__ void st_lik(const DevModel &m, EvalShared &E, const ParVecs &q, const float *data,
+                                              float *wsb) {
+    const int nth = blockDim.x, lane = threadIdx.x & 31;
+    for (int i = 0; i < E.n; ++i) {
+        const DevDataset &ds = m.ds[E.dl[i]];
+        const DsWs ws = carve_ds_ws(wsb + (int64_t)i * m.ws_eval_floats, m.N_t, m.C, m.max_reco, m.n_osc);
+        const int nr = ds.n_reco, nb = ds.bkg_end - ds.bkg_begin;
+        const int t0 = rot_tid(i, (nr + 31) >> 5);
+        if ((t0 & ~31) >= nr) continue;      // this warp has no bin of this dataset
+        float part[8];   // deviance, d/d eff, d/d rate_b
 #pragma unroll
-    for (int i = 0; i < kP + NC; ++i) ep[i] = 0.f;
-    const bool spline = SPL && m.remap_mode == FIT_REMAP_SPLINE;
-    for (int k = tid; k < N_t; k += nth) {
-        float gu = 0.f;
-        if (spline) {
-            gu = spline_adjoint_source(gv, m.e_edge, em, k, N_t);
-            spline_adjoint_edge(ws.u, gv, m.e_edge, em, k, N_t, ep);
-            if (k == N_t - 1) spline_adjoint_edge(ws.u, gv, m.e_edge, em, N_t, N_t, ep);
-        } else {
-        const float e0 = m.e_edge[k], e1 = m.e_edge[k + 1];
-        const float d0 = em.disp(e0), d1 = em.disp(e1);
-        const float w = 1.f + (d1 - d0), iw = 1.f / w;
-        const int f0i = (int)floorf(d0), f1i = (int)floorf(d1);
-        const int t0 = k + f0i, t1 = k + 1 + f1i;
-        for (int t = max(t0, 0); t <= min(t1, N_t - 1); ++t) {
-            const float ylo = (float)(k - t) + d0, yhi = (float)(k + 1 - t) + d1;
-            const float ov = fminf(yhi, 1.f) - fmaxf(ylo, 0.f);
-            if (ov > 0.f) gu = fmaf(ov * iw, gv[t], gu);
+        for (int b = 0; b < 8; ++b) part[b] = 0.f;
+        for (int j = t0; j < nr; j += nth) {
+            const float n = data[ds.data_off + j], f0 = ws.f0[j];
+            float tm[kMaxBkgDs], sh[kMaxBkgDs];
+            const float mu = bin_mu(m, E, i, ds, q, f0, j, nb, tm, sh);
+            if (!(mu > 0.f)) {
+                atomicOr(&E.status, kStMuNonpos);
+                continue;
+            }
+            part[0] += deviance(n, mu);
+            const float g = 2.f * (mu - n) / mu;
+            ws.gmu[j] = g;
+            if (GRAD) {
+                part[1] = fmaf(g, f0, part[1]);
+#pragma unroll
+                for (int b = 0; b < kMaxBkgDs; ++b) {
+                    if (b >= nb) break;
+                    part[2 + b] = fmaf(g * tm[b], sh[b], part[2 + b]);
+                }
+            }
         }
-        const float g0 = (t0 >= 0 && t0 < N_t) ? gv[t0] : 0.f;
-        const float g1 = (t1 >= 0 && t1 < N_t) ? gv[t1] : 0.f;
-        const float uk = ws.u[k] * iw;
-        const float A0 = uk * (gu - g0), A1 = uk * (g1 - gu);
-        ep[0] += (A0 + A1) * em.inv_de;
-        ep[1] += (A0 * e0 + A1 * e1) * em.inv_de;
-        ep[2] += (A0 * e0 * e0 + A1 * e1 * e1) * em.inv_de;
+        __syncwarp();
+        const float tot = warp_sum_split<8>(part);
+        if ((lane & 3) == 0) E.part[(i * kMaxWarps + (t0 >> 5)) * 8 + (lane >> 2)] = tot;
+    }
+    __syncthreads();
+}
+
+// One warp (`warp_id`): the likelihood sums of the group in double, added to E.nll, and the
+// efficiency and rate gradients to grad.
+template <bool GRAD>
+static __device__ __forceinline__ void lik_finish(const DevModel &m, EvalShared &E, float *grad, int warp_id) {
+    if ((int)(threadIdx.x >> 5) != warp_id) return;
+    const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    double nll = E.nll;
+    for (int i = 0; i < E.n; ++i) {
+        const DevDataset &ds = m.ds[E.dl[i]];
+        const int used = min(nw, (ds.n_reco + 31) >> 5);
+        // lane = value (low three bits) x quarter of the warps
+        const float *p = E.part + (int64_t)i * kMaxWarps * 8 + (lane & 7);
+        double s = 0.0;
+        for (int w = lane >> 3; w < used; w += 4) s += (double)p[w * 8];
+        s += __shfl_xor_sync(0xffffffffu, s, 8);
+        s += __shfl_xor_sync(0xffffffffu, s, 16);
+        nll += __shfl_sync(0xffffffffu, s, 0);
+        if (GRAD) {
+            const int nb = ds.bkg_end - ds.bkg_begin;
+            const int p2 = lane == 1 ? ds.eff_idx : (lane >= 2 && lane - 2 < nb) ? m.bkg[ds.bkg_begin + lane - 2].rate_idx : -1;
+            if (lane >= 1 && lane < 8 && p2 >= 0) atomicAdd(&grad[p2], (float)s);
+            __syncwarp();
         }
-        const float ts = ws.ts[k], pt = ws.ptot[k];
-        const float gb = pmul(c.nrm, gu * ts);    // d nll / d(ptot)
-#pragma unroll
-        for (int i = 0; i < NOSC; ++i) ep[3 + i] = fmaf(gb, ws.dp[i * N_t + k], ep[3 + i]);
-        ep[kN] = fmaf(gu * ts, pt, ep[kN]);
-#pragma unroll
-        for (int cc = 0; cc < NC; ++cc)
-            if (cc < C) ep[kP + cc] = fmaf(gb, ws.pcw[cc * N_t + k], ep[kP + cc]);
-        ws.dp[k] = pmul(c.nrm, gu * ds.t[k] * pt);    // d nll / d s for this bin (dp0 reused)
     }
-    double etot[kP + NC];
-    block_sum<kP + NC>(ep, red, etot);
-    if (tid == 0) {
-        for (int i = 0; i < 3; ++i)
-            if (ds.esc_idx[i] >= 0) grad[ds.esc_idx[i]] += (float)etot[i];
-        for (int i = 0; i < NOSC; ++i)
-            if (m.osc_idx[i] >= 0) grad[m.osc_idx[i]] += (float)etot[3 + i];
-        if (ds.norm_idx >= 0) grad[ds.norm_idx] += (float)etot[kN];
-#pragma unroll
-        for (int cc = 0; cc < NC; ++cc)
-            if (cc < C && m.core_power_idx[cc] >= 0) grad[m.core_power_idx[cc]] += (float)etot[kP + cc];
-    }
-    // ---- stage F: shape reweights (one thread per distinct parameter, CSR over bins) -----
-    for (int i = tid; i < ds.n_sp; i += nth) {
+    if (lane == 0) E.nll = nll;
+}
+
+// Background-shape gradient: a thread per shape parameter sums its (background, bin) pairs of
+// the group's datasets in a fixed order (several datasets may share a shape).
+static __device__ __forceinline__ void st_bkg_shape(const DevModel &m, const EvalShared &E, float *wsb, float *grad) {
+    for (int p = threadIdx.x; p < m.n_bs; p += blockDim.x) {
         float s = 0.f;
-        for (int q = ds.sp_ptr[i]; q < ds.sp_ptr[i + 1]; ++q) s += ws.dp[ds.sp_k[q]];
-        grad[ds.sp_param[i]] += s;
+        for (int r = m.bs_ptr[p]; r < m.bs_ptr[p + 1]; ++r) {
+            const BkgShapeRef ref = m.bs_ref[r];
+            for (int i = 0; i < E.n; ++i) {
+                if (E.dl[i] != ref.d) continue;
+                const DsWs ws = carve_ds_ws(wsb + (int64_t)i * m.ws_eval_floats, m.N_t, m.C, m.max_reco, m.n_osc);
+                s += ws.gmu[ref.j] * E.rate[ref.q].h * ref.tmpl;
+            }
+        }
+        grad[m.bs_param[p]] += s;
+    }
+}
+
+// Stage D: adjoint of the fold, v <- gv = eff R^T gmu (column bands). rcol is exactly 0 past each
+// column's band, so the loop runs the widest band of the warp's 32 adjacent columns (nearly
+// their own widths: the resolution changes slowly with energy) with the row index clamped (no
+// early exit) and four partial sums. No barrier.
+static __device__ __forceinline__ void st_adjoint_fold(const DevModel &m, const EvalShared &E, float *wsb) {
+    const int N_t = m.N_t, nth = blockDim.x;
+    for (int i = 0; i < E.n; ++i) {
+        const DevDataset &ds = m.ds[E.dl[i]];
+        const DevDetector &dt = m.det[ds.det];
+        const DsWs ws = carve_ds_ws(wsb + (int64_t)i * m.ws_eval_floats, N_t, m.C, m.max_reco, m.n_osc);
+        const int jmax = ds.n_reco - 1;
+        const PP eff = E.eff[i];
+        float *gv = ws.v;   // v is dead after the fold
+        for (int k = rot_tid(i, (N_t + 31) >> 5); k < N_t; k += nth) {
+            const int lo = dt.col_lo[k];
+            const int cw = __reduce_max_sync(__activemask(), dt.col_len[k]);
+            const float *rc = dt.rcol + k;
+            float s[4] = {0.f, 0.f, 0.f, 0.f};
+            int b = 0;
+            for (; b + 7 < cw; b += 8) {   // eight loads in flight
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+                    s[u & 3] = fmaf(rc[(int64_t)(b + u) * N_t], ws.gmu[min(lo + b + u, jmax)], s[u & 3]);
+            }
+            for (; b < cw; ++b) s[0] = fmaf(rc[(int64_t)b * N_t], ws.gmu[min(lo + b, jmax)], s[0]);
+            gv[k] = pmul(eff, (s[0] + s[1]) + (s[2] + s[3]));
+        }
+    }
+}
+
+// Stage E: adjoint of the energy map and of the signal from gv (in v); leaves d(-2lnL)/ds of each
+// bin in dp[0] and the warp totals of the energy-map, normalisation, survival and power
+// gradients in E.part. Needs u/ts/ptot/dp/pcw (st_signal<true>). Ends with a barrier.
+template <int NC, int NOSC, bool GEN>
+static __device__ __forceinline__ void st_adjoint_rest_n(const DevModel &m, EvalShared &E, float *wsb) {
+    const int N_t = m.N_t, C = m.C, nth = blockDim.x;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const bool spline = GEN && m.remap_mode == FIT_REMAP_SPLINE;
+    float eo[NOSC], ec[NC];   // d/d eta, d/d power_c (NC >= C), over all datasets of the group
+#pragma unroll
+    for (int j = 0; j < NOSC; ++j) eo[j] = 0.f;
+#pragma unroll
+    for (int c = 0; c < NC; ++c) ec[c] = 0.f;
+    for (int i = 0; i < E.n; ++i) {
+        const DevDataset &ds = m.ds[E.dl[i]];
+        const DsWs ws = carve_ds_ws(wsb + (int64_t)i * m.ws_eval_floats, N_t, C, m.max_reco, m.n_osc);
+        const EMap em = E.em[i];
+        const PP nrm = E.nrm[i];
+        const float *gv = ws.v;
+        float ep[4] = {0.f, 0.f, 0.f, 0.f};   // d/da0, d/da1, d/da2, d/d norm
+        for (int k = rot_tid(i, (N_t + 31) >> 5); k < N_t; k += nth) {
+            float gu = 0.f;
+            if (spline) {
+                gu = spline_adjoint_source(gv, m.e_edge, em, k, N_t);
+                spline_adjoint_edge(ws.u, gv, m.e_edge, em, k, N_t, ep);
+                if (k == N_t - 1) spline_adjoint_edge(ws.u, gv, m.e_edge, em, N_t, N_t, ep);
+            } else {
+                // per source k: gu = sum_t F_kt gv_t; A0 = (gu - gv(floor Y_k)) / w,
+                // A1 = (gv(floor Y_k+1) - gu) / w
+                const float e0 = m.e_edge[k], e1 = m.e_edge[k + 1];
+                const float d0 = em.disp(e0), d1 = em.disp(e1);
+                const float w = 1.f + (d1 - d0), iw = 1.f / w;
+                const int f0i = (int)floorf(d0), f1i = (int)floorf(d1);
+                const int t0 = k + f0i, t1 = k + 1 + f1i;
+                for (int t = max(t0, 0); t <= min(t1, N_t - 1); ++t) {
+                    const float ylo = (float)(k - t) + d0, yhi = (float)(k + 1 - t) + d1;
+                    const float ov = fminf(yhi, 1.f) - fmaxf(ylo, 0.f);
+                    if (ov > 0.f) gu = fmaf(ov * iw, gv[t], gu);
+                }
+                const float g0 = (t0 >= 0 && t0 < N_t) ? gv[t0] : 0.f;
+                const float g1 = (t1 >= 0 && t1 < N_t) ? gv[t1] : 0.f;
+                const float uk = ws.u[k] * iw;
+                const float A0 = uk * (gu - g0), A1 = uk * (g1 - gu);
+                ep[0] += (A0 + A1) * em.inv_de;
+                ep[1] += (A0 * e0 + A1 * e1) * em.inv_de;
+                ep[2] += (A0 * e0 * e0 + A1 * e1 * e1) * em.inv_de;
+            }
+            const float ts = ws.ts[k], pt = ws.ptot[k];
+            const float gb = pmul(nrm, gu * ts);    // d nll / d(ptot)
+#pragma unroll
+            for (int j = 0; j < NOSC; ++j) eo[j] = fmaf(gb, ws.dp[j * N_t + k], eo[j]);
+            ep[3] = fmaf(gu * ts, pt, ep[3]);
+#pragma unroll
+            for (int c = 0; c < NC; ++c)
+                if (c < C) ec[c] = fmaf(gb, ws.pcw[c * N_t + k], ec[c]);
+            ws.dp[k] = pmul(nrm, gu * ds.t[k] * pt);    // d nll / d s for this bin (dp[0] reused)
+        }
+        __syncwarp();
+        const float tot = warp_sum_split<4>(ep);
+        if ((lane & 7) == 0) E.part[(i * kMaxWarps + warp) * 4 + (lane >> 3)] = tot;
+    }
+    float *pw = E.part + FIT_MAX_DATASETS * kMaxWarps * 4 + warp * 32;
+    float v[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) v[j] = j < NOSC ? eo[j] : (j - NOSC < NC ? ec[j - NOSC < NC ? j - NOSC : 0] : 0.f);
+    const float t8 = warp_sum_split<8>(v);
+    if ((lane & 3) == 0) pw[lane >> 2] = t8;
+    if constexpr (NC > 8 - NOSC) {   // the cores past the first 8 - NOSC
+        constexpr int c0 = 8 - NOSC;
+        float w[16];
+#pragma unroll
+        for (int c = 0; c < 16; ++c) w[c] = c0 + c < NC ? ec[c0 + c < NC ? c0 + c : 0] : 0.f;
+        const float t16 = warp_sum_split<16>(w);
+        if ((lane & 1) == 0) pw[8 + (lane >> 1)] = t16;
     }
     __syncthreads();
 }
 
-// Stages E-F with the per-core sums sized for the model's core count.
-template <bool SPL, int NOSC>
-static __device__ void ds_adjoint_rest(const DevModel &m, int d, const float *pv, const float *pd,
-                                       const DsCtxT<NOSC> &c, EvalWs ws, float *grad, double *red) {
-    if (m.C <= 2)
-        ds_adjoint_ef<2, NOSC, SPL>(m, d, pv, pd, c, ws, grad, red);
-    else
-        ds_adjoint_ef<FIT_MAX_CORES, NOSC, SPL>(m, d, pv, pd, c, ws, grad, red);
-}
-
-// Stages D-F: adjoint of the fold, of the energy map and of the signal; adds the gradient
-// contributions to grad. Needs ws.u/ts/ptot/dp/pcw (ds_signal<true>) and ws.gmu.
-template <bool SPL, int NOSC>
-static __device__ void ds_adjoint(const DevModel &m, int d, const float *pv, const float *pd,
-                                  const DsCtxT<NOSC> &c, EvalWs ws, float *grad, double *red) {
-    ds_adjoint_fold(m, d, c, ws);
-    ds_adjoint_rest<SPL>(m, d, pv, pd, c, ws, grad, red);
-}
-
-// One dataset in one sequence: adds its Poisson -2lnL and (if grad != nullptr) its gradient
-// contributions (theta space, P floats). Returns the dataset's -2lnL (all threads); *status |=
-// kSt* bits on failure.
-
-template <int NOSC, bool SPL>
-static __device__ double eval_dataset_n(const DevModel &m, int d, const float *pv, const float *pd,
-                                        const float *data, EvalWs ws, float *grad, double *red,
-                                        int *status, float *mu_out) {
-    DsCtxT<NOSC> c;
-    if (!ds_setup(m, d, pv, pd, c, status)) return 0.0;
-    if (grad != nullptr && data != nullptr)
-        ds_signal<true>(m, d, pv, pd, c, ws);
-    else
-        ds_signal<false>(m, d, pv, pd, c, ws);
-    ds_remap<SPL>(m, d, c, ws);
-    const double nll_d = ds_fold_lik(m, d, pv, pd, c, data, ws, grad, red, status, mu_out);
-    if (data == nullptr || grad == nullptr || (*(volatile int *)status) != 0) return nll_d;
-    ds_adjoint<SPL>(m, d, pv, pd, c, ws, grad, red);
-    return nll_d;
-}
-
-// One dataset's -2lnL (and gradient). NOSC = 4 (the basic build): models of Eq. 1 or the
-// three-flavour formula with the overlap-length energy correction; NOSC = 6 (the general
-// build): any model (the 3+1 formula, the spline energy correction).
-template <int NOSC = 4>
-static __device__ double eval_dataset(const DevModel &m, int d, const float *pv, const float *pd,
-                                      const float *data, EvalWs ws, float *grad, double *red,
-                                      int *status, float *mu_out) {
-    if constexpr (NOSC == 6) {
-        if (m.osc_mode == FIT_OSC_STERILE4)
-            return eval_dataset_n<6, true>(m, d, pv, pd, data, ws, grad, red, status, mu_out);
-        return eval_dataset_n<4, true>(m, d, pv, pd, data, ws, grad, red, status, mu_out);
+// Stage F, after st_adjoint_rest: the totals of stage E in double into grad (the last warp), and the
+// shape reweights: the bins of each distinct shape parameter (CSR) summed by sp_lanes lanes.
+// Ends with a barrier.
+template <int NOSC>
+static __device__ __forceinline__ void st_adjoint_finish(const DevModel &m, EvalShared &E, float *wsb, float *grad) {
+    const int tid = threadIdx.x, lane = tid & 31, nw = blockDim.x >> 5, nth = blockDim.x;
+    if ((tid >> 5) == nw - 1) {
+        // energy maps and normalisations: lane = value (low two bits) x eighth of the warps
+        for (int i = 0; i < E.n; ++i) {
+            const DevDataset &ds = m.ds[E.dl[i]];
+            const float *p = E.part + (int64_t)i * kMaxWarps * 4 + (lane & 3);
+            double s = 0.0;
+            for (int w = lane >> 2; w < nw; w += 8) s += (double)p[w * 4];
+#pragma unroll
+            for (int o = 4; o < 32; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            const int p2 = lane < 3 ? ds.esc_idx[lane] : lane == 3 ? ds.norm_idx : -1;
+            if (p2 >= 0) atomicAdd(&grad[p2], (float)s);
+            __syncwarp();
+        }
+        // survival parameters and core powers: a lane per value
+        if (lane < NOSC + m.C) {
+            const float *p = E.part + FIT_MAX_DATASETS * kMaxWarps * 4 + lane;
+            double s0 = 0.0, s1 = 0.0;
+            for (int w = 0; w < nw; w += 2) {
+                s0 += (double)p[w * 32];
+                if (w + 1 < nw) s1 += (double)p[(w + 1) * 32];
+            }
+            const int p2 = lane < NOSC ? m.osc_idx[lane] : m.core_power_idx[lane - NOSC];
+            if (p2 >= 0) atomicAdd(&grad[p2], (float)(s0 + s1));
+        }
+        __syncwarp();
     }
-    return eval_dataset_n<4, false>(m, d, pv, pd, data, ws, grad, red, status, mu_out);
+    if (m.shared_roles) __syncthreads();
+    for (int i = 0; i < E.n; ++i) {
+        const DevDataset &ds = m.ds[E.dl[i]];
+        const float *gs = carve_ds_ws(wsb + (int64_t)i * m.ws_eval_floats, m.N_t, m.C, m.max_reco, m.n_osc).dp;
+        const int L = ds.sp_lanes, per = nth / L;   // lanes per parameter, parameters per pass
+        const int work = ds.n_sp * L;
+        for (int q0 = rot_tid(i, (work + 31) >> 5); q0 < ((work + 31) & ~31); q0 += per * L) {
+            const int p = q0 / L, sub = q0 & (L - 1);
+            float s = 0.f;
+            if (p < ds.n_sp)
+                for (int r = ds.sp_ptr[p] + sub; r < ds.sp_ptr[p + 1]; r += L) s += gs[ds.sp_k[r]];
+            for (int o = L >> 1; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if (p < ds.n_sp && sub == 0) grad[ds.sp_param[p]] += s;
+        }
+        if (m.shared_roles) __syncthreads();
+    }
+    __syncthreads();
+}
+
+template <bool GEN>
+static __device__ __forceinline__ void st_adjoint_rest(const DevModel &m, EvalShared &E, float *wsb, float *grad) {
+    if (GEN && m.osc_mode == FIT_OSC_STERILE4) {
+        if (m.C <= 2)
+            st_adjoint_rest_n<2, 6, GEN>(m, E, wsb);
+        else
+            st_adjoint_rest_n<FIT_MAX_CORES, 6, GEN>(m, E, wsb);
+        st_adjoint_finish<6>(m, E, wsb, grad);
+    } else {
+        if (m.C <= 2)
+            st_adjoint_rest_n<2, 4, GEN>(m, E, wsb);
+        else
+            st_adjoint_rest_n<FIT_MAX_CORES, 4, GEN>(m, E, wsb);
+        st_adjoint_finish<4>(m, E, wsb, grad);
+    }
+}
+
+template <bool GEN>
+static __device__ __forceinline__ int eval_setup_any(const DevModel &m, EvalShared &E, const ParVecs &q, uint32_t mask,
+                                                     int first, int group) {
+    if (GEN && m.osc_mode == FIT_OSC_STERILE4) return eval_setup<6>(m, E, q, mask, first, group);
+    return eval_setup<4>(m, E, q, mask, first, group);
+}
+
+// The Poisson -2lnL of the datasets in `mask` and (grad != nullptr) its theta gradient added to
+// grad. wsb: ws_group dataset workspaces. Returns the -2lnL on every thread; E.status (cleared
+// here) holds kSt* bits on failure. Starts and ends with a barrier.
+template <bool GEN>
+static __device__ double eval_datasets(const DevModel &m, EvalShared &E, const ParVecs &q, uint32_t mask,
+                                       const float *data, float *wsb, float *grad) {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        E.status = 0;
+        E.nll = 0.0;
+    }
+    for (int first = 0; first < m.n_ds;) {
+        first = eval_setup_any<GEN>(m, E, q, mask, first, m.ws_group);
+        if (E.n > 0) {
+            if (grad != nullptr)
+                st_signal<true, GEN>(m, E, q, wsb);
+            else
+                st_signal<false, GEN>(m, E, q, wsb);
+            st_remap<GEN>(m, E, wsb);
+            st_fold(m, E, wsb);
+            if (grad != nullptr)
+                st_lik<true>(m, E, q, data, wsb);
+            else
+                st_lik<false>(m, E, q, data, wsb);
+        }
+        if (E.status || E.bad) {   // block-uniform after the barriers
+            __syncthreads();
+            if (threadIdx.x == 0 && !E.status) E.status = kStEscale;
+            __syncthreads();
+            return INFINITY;
+        }
+        if (E.n == 0) continue;
+        if (grad != nullptr) {
+            lik_finish<true>(m, E, grad, 0);
+            if (m.shared_roles) __syncthreads();
+            st_bkg_shape(m, E, wsb, grad);
+            st_adjoint_fold(m, E, wsb);
+            __syncthreads();
+            st_adjoint_rest<GEN>(m, E, wsb, grad);
+        } else {
+            lik_finish<false>(m, E, nullptr, 0);
+        }
+    }
+    __syncthreads();
+    return E.nll;
+}
+
+// Expected counts of every dataset into mu (n_data floats). E.status as eval_datasets; datasets
+// before an invalid energy map are written. Starts and ends with a barrier.
+template <bool GEN>
+static __device__ void expected_datasets(const DevModel &m, EvalShared &E, const ParVecs &q, float *wsb, float *mu) {
+    __syncthreads();
+    if (threadIdx.x == 0) E.status = 0;
+    for (int first = 0; first < m.n_ds;) {
+        first = eval_setup_any<GEN>(m, E, q, 0xffffffffu, first, m.ws_group);
+        if (E.n > 0) {
+            st_signal<false, GEN>(m, E, q, wsb);
+            st_remap<GEN>(m, E, wsb);
+            st_fold(m, E, wsb);
+            st_mu(m, E, q, wsb, mu);
+        }
+        if (E.bad) {
+            __syncthreads();
+            if (threadIdx.x == 0) E.status = kStEscale;
+            __syncthreads();
+            return;
+        }
+    }
+    __syncthreads();
+}
+
+// ------------------------------------------------------------------------------------
+// Triangular matrix-vector products of the prior blocks: out_r = sum_c M(r, c) x_c over the rows
+// of all blocks together, as tiles of 32 rows x kTriCols columns (a warp per tile, a lane per
+// row: every column is one coalesced load and one broadcast of x, sixteen in flight). A tile
+// leaves its partial sum at part[seg * tri_rows + row]; after a barrier tri_sum adds a row's
+// segments in order. x: by parameter index.
+static __device__ __forceinline__ void tri_apply(const DevModel &m, const TriTile *tiles, int n_tiles, const float *M,
+                                                 const float *x, float *part) {
+    const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    for (int t = threadIdx.x >> 5; t < n_tiles; t += nw) {
+        const TriTile T = tiles[t];
+        const int r = min(T.row0 + lane, T.n - 1), cols = T.cols;
+        const float *col = M + T.mat + (int64_t)T.col0 * T.n + r;
+        float s[4] = {0.f, 0.f, 0.f, 0.f};
+        int c = 0;
+        if (T.in0 >= 0) {
+            const float *xb = x + T.in0 + T.col0;
+            for (; c + 15 < cols; c += 16) {
+#pragma unroll
+                for (int u = 0; u < 16; ++u) s[u & 3] = fmaf(col[(int64_t)(c + u) * T.n], xb[c + u], s[u & 3]);
+            }
+            for (; c < cols; ++c) s[0] = fmaf(col[(int64_t)c * T.n], xb[c], s[0]);
+        } else {
+            const int *idx = m.blk_idx + T.idx + T.col0;
+            for (; c + 7 < cols; c += 8) {
+#pragma unroll
+                for (int u = 0; u < 8; ++u) s[u & 3] = fmaf(col[(int64_t)(c + u) * T.n], x[idx[c + u]], s[u & 3]);
+            }
+            for (; c < cols; ++c) s[0] = fmaf(col[(int64_t)c * T.n], x[idx[c]], s[0]);
+        }
+        if (T.row0 + lane < T.n) part[T.seg * m.tri_rows + T.out + T.row0 + lane] = (s[0] + s[1]) + (s[2] + s[3]);
+    }
+}
+
+__device__ __forceinline__ float tri_sum(const DevModel &m, const float *part, int row, bool upper) {
+    const int x = m.tri_seg[row];
+    const int s0 = upper ? (x >> 8) & 255 : 0, s1 = upper ? x >> 16 : x & 255;
+    float t = part[s0 * m.tri_rows + row];
+    for (int q = s0 + 1; q < s1; ++q) t += part[q * m.tri_rows + row];
+    return t;
 }
 
 }  // namespace fitcore

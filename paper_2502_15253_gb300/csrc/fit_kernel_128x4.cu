@@ -1,0 +1,8 @@
+// The persistent fit kernel for blocks of up to 128 threads, 4 resident per SM (see fit_dev.cuh).
+#include "fit_dev.cuh"
+
+namespace fitcore {
+
+const void *fit_kernel_128x4(bool general, bool pre) { return fit_kernel_of<128, 4>(general, pre); }
+
+}  // namespace fitcore

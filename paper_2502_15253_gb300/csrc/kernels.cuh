@@ -39,9 +39,21 @@ struct FitArgs {
     int pre_per_model;           // of the dataset subsets the instances fit
 };
 
-__global__ void eval_kernel(const DevModel *gm, int B, const double *theta, const float *data,
-                            const uint32_t *masks, double *nll_out, float *grad_out,
-                            float *mu_out, int *status_out, float *ws_global, int ws_in_smem);
+// Batched expectation (mu != nullptr) or -2lnL and gradient; a block per parameter vector at a time
+struct EvalArgs {
+    const DevModel *model;       // device
+    int B;
+    const double *theta;         // device [B x P]
+    const float *data;           // device [B x n_data] or nullptr (Asimov data)
+    const uint32_t *masks;       // device [B] or nullptr
+    double *nll;
+    float *grad;                 // or nullptr
+    float *mu;
+    int *status;                 // or nullptr
+    float *ws_global;            // workspace slices of m.ws_floats per block, unless ws_in_smem
+    int ws_in_smem;
+};
+const void *eval_kernel_func(int threads, bool general);   // host entry address
 // Lockstep engine: the instances of one model advance together, one evaluation per round;
 // a round is three launches (forward + likelihood per (instance, dataset), adjoint per
 // (instance, dataset), minimiser step per instance). Group-local index g addresses the state
@@ -58,7 +70,7 @@ struct LsArgs {
     double *best;
     fit_result *results;
     FitState *state;             // [n]
-    float *vec;                  // [n x vec_stride]: 12 working P-vectors, then the history
+    float *vec;                  // [n x vec_stride]: 15 working P-vectors, then the history
     int64_t vec_stride;
     float *gsl;                  // [n x n_ds x P] gradient contributions per dataset
     double *nll_ds;              // [n x n_ds]
@@ -98,11 +110,16 @@ __global__ void ls_forward_kernel6(LsArgs A);   // models with the 3+1 formula
 __global__ void ls_adjoint_kernel6(LsArgs A);
 __global__ void ls_step_kernel(LsArgs A);
 size_t ls_state_bytes();
-size_t ls_step_smem_bytes();
+size_t ls_step_smem_bytes(const DevModel &hm);
 size_t ls_eval_smem_bytes(int P, int ws_floats);
 
-// the persistent fit kernel compiled for 4 or 5 resident blocks per SM (host entry address)
-const void *fit_kernel_func(int variant, int n_osc, bool pre);
+// the persistent fit kernel (host entry address): blocks of up to 128 threads compiled for 4 or 5
+// resident blocks per SM (variant), of 256 threads (2 per SM) or of 512 (1 per SM)
+const void *fit_kernel_func(int threads, int variant, bool general, bool pre);
+const void *fit_kernel_128x4(bool general, bool pre);
+const void *fit_kernel_128x5(bool general, bool pre);
+const void *fit_kernel_256(bool general, bool pre);
+const void *fit_kernel_512(bool general, bool pre);
 
 size_t eval_smem_bytes(const DevModel &hm, bool ws_in_smem);
 
@@ -143,8 +160,19 @@ size_t fit_smem_bytes(int floats);
 // 16-byte boundary and the history can be read as float4.
 __host__ __device__ inline int fit_vec_pitch(int P) { return (P + 3) & ~3; }
 constexpr int kMaxPreRank = 32;   // eigen-directions of the Fisher preconditioner
-__host__ __device__ inline int fit_vec_floats(int P, int hist) { return (14 + 2 * hist) * fit_vec_pitch(P); }
+__host__ __device__ inline int fit_vec_floats(int P, int hist) { return (15 + 2 * hist) * fit_vec_pitch(P); }
 __host__ __device__ inline int fit_hist_floats(int P, int hist) { return 2 * hist * fit_vec_pitch(P); }
-__host__ __device__ inline int fit_work_floats(int P) { return 14 * fit_vec_pitch(P); }
+__host__ __device__ inline int fit_work_floats(int P) { return 15 * fit_vec_pitch(P); }
+
+// Threads per block for a model: one wide block per vector or fit leaves the fewest dependent
+// steps, but each thread then holds fewer bins and every barrier spans more warps, so the block
+// grows with the true bins evaluated together. Measured (us, batched -2lnL with gradient, 128 /
+// 256 / 512 threads): 200 bins x 4096 vectors 116 / 182 / 338; 1200 bins x 4096 550 / 504 / 720;
+// 2000 bins x 2048 3636 / 2124 / 1407. A property of the model alone: the result of a vector or
+// a fit does not depend on the batch around it.
+inline int model_threads(const DevModel &h) {
+    const int bins = h.N_t * h.ws_group;
+    return bins <= 512 ? 128 : bins <= 1600 ? 256 : 512;
+}
 
 }  // namespace fitcore

@@ -32,7 +32,8 @@ extern "C" int fit_model_eval_noalloc(fit_model *model, int B, const double *the
 // The model's device layout lives in capi.cu; it hands the pieces needed here through this hook.
 int fitcore_model_device(fit_model *model, const fitcore::DevModel **dev, const fitcore::DevModel **host,
                          int *device);
-int fitcore_raise_eval_smem(size_t bytes);
+int fitcore_raise_eval_smem(const void *func, size_t bytes);
+const void *fitcore_eval_func(const fitcore::DevModel &h, int *threads);
 void fitcore_count_launch();
 
 // Host-side decision on where the call's memory lives (no CUDA call): the model must be on the
@@ -58,7 +59,7 @@ extern "C" int fit_model_eval_noalloc(fit_model *model, int B, const double *the
     const fitcore::DevModel *dev = nullptr, *h = nullptr;
     int model_device = -1;
     fitcore_model_device(model, &dev, &h, &model_device);
-    const size_t per_block = (size_t)h->ws_eval_floats;
+    const size_t per_block = (size_t)h->ws_floats;
     if (per_block > kScratchFloats)
         return fitcore_noalloc_fail(FIT_ERR_INVALID_ARG,
                                     "fit_model_eval_noalloc: the model needs " + std::to_string(per_block * 4) +
@@ -112,15 +113,16 @@ extern "C" int fit_model_eval_noalloc(fit_model *model, int B, const double *the
         cudaGetLastError();
         return fitcore_noalloc_fail(FIT_ERR_CUDA, "fit_model_eval_noalloc: device attribute");
     }
-    const int threads = 256;
+    int threads = 0;
+    const void *func = fitcore_eval_func(*h, &threads);   // the build fit_model_eval uses: the same results
     const size_t smem = fitcore::eval_smem_bytes(*h, false);
     // (raised only: the attribute is shared with fit_model_eval's launches in other threads)
-    if (fitcore_raise_eval_smem(smem) != FIT_OK) {
+    if (fitcore_raise_eval_smem(func, smem) != FIT_OK) {
         cudaGetLastError();
         return fitcore_noalloc_fail(FIT_ERR_CUDA, "fit_model_eval_noalloc: cudaFuncSetAttribute");
     }
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fitcore::eval_kernel, threads, smem) != cudaSuccess ||
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, func, threads, smem) != cudaSuccess ||
         per_sm < 1) {
         cudaGetLastError();
         return fitcore_noalloc_fail(FIT_ERR_CUDA, "fit_model_eval_noalloc: occupancy");
@@ -128,10 +130,10 @@ extern "C" int fit_model_eval_noalloc(fit_model *model, int B, const double *the
     // one workspace slice per block: the grid never exceeds what the scratch holds
     const int slices = (int)(kScratchFloats / per_block);
     const int grid = std::max(1, std::min(std::min(B, per_sm * sms), slices));
-    fitcore::eval_kernel<<<grid, threads, smem, (cudaStream_t)stream>>>(
-        dev, B, theta, data, masks, nll_out, grad_out, nullptr, status_out, scratch, 0);
+    fitcore::EvalArgs a{dev, B, theta, data, masks, nll_out, grad_out, nullptr, status_out, scratch, 0};
+    void *args[] = {&a};
+    const cudaError_t e = cudaLaunchKernel(func, dim3(grid), dim3(threads), args, smem, (cudaStream_t)stream);
     fitcore_count_launch();
-    cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess)
         return fitcore_noalloc_fail(FIT_ERR_CUDA, std::string("fit_model_eval_noalloc: launch: ") + cudaGetErrorString(e));
     return FIT_OK;

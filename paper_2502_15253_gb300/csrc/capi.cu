@@ -625,6 +625,40 @@ int fit_model_create(const fit_model_desc *d, fit_model **out) {
             for (int k = 0; k < Nt; ++k) mark(d->ds_shape_idx[(size_t)q * Nt + k]);
         }
         h.shared_roles = shared ? 1 : 0;
+        // totals that share a parameter are added in order by one thread (the dup masks)
+        vector<int> uses(P, 0);
+        auto count = [&](int p) {
+            if (p >= 0) uses[p]++;
+        };
+        auto twice = [&](int p) { return p >= 0 && uses[p] > 1; };
+        for (int q = 0; q < h.n_ds; ++q) count(h.ds[q].eff_idx);
+        for (int q = 0; q < h.n_bkg; ++q) count(h.bkg[q].rate_idx);
+        for (int q = 0; q < h.n_ds; ++q) {
+            fitcore::DevDataset &D = h.ds[q];
+            D.lik_dup = twice(D.eff_idx) ? 2 : 0;
+            for (int b = D.bkg_begin; b < D.bkg_end; ++b)
+                if (twice(h.bkg[b].rate_idx)) D.lik_dup |= 4 << (b - D.bkg_begin);
+        }
+        std::fill(uses.begin(), uses.end(), 0);
+        for (int q = 0; q < h.n_ds; ++q) {
+            for (int i = 0; i < 3; ++i) count(h.ds[q].esc_idx[i]);
+            count(h.ds[q].norm_idx);
+        }
+        for (int i = 0; i < n_osc; ++i) count(h.osc_idx[i]);
+        for (int i = 0; i < C; ++i) count(h.core_power_idx[i]);
+        h.osc_dup = 0;
+        for (int i = 0; i < n_osc; ++i)
+            if (twice(h.osc_idx[i])) h.osc_dup |= 1 << i;
+        for (int i = 0; i < C; ++i)
+            if (twice(h.core_power_idx[i])) h.osc_dup |= 1 << (n_osc + i);
+        h.any_map_dup = h.osc_dup != 0;
+        for (int q = 0; q < h.n_ds; ++q) {
+            fitcore::DevDataset &D = h.ds[q];
+            D.map_dup = twice(D.norm_idx) ? 8 : 0;
+            for (int i = 0; i < 3; ++i)
+                if (twice(D.esc_idx[i])) D.map_dup |= 1 << i;
+            if (D.map_dup) h.any_map_dup = 1;
+        }
     }
     // ---- parameters, priors, transformation layer ----------------------------------------
     {
@@ -688,6 +722,11 @@ int fit_model_create(const fit_model_desc *d, fit_model **out) {
         for (int i = 0; i < P; ++i) {
             th0f[i] = (float)th0[i];
             th0lo[i] = (float)(th0[i] - (double)th0f[i]);
+            for (int k = 0; k < n_osc; ++k)
+                if (h.osc_idx[k] == i) {
+                    h.osc_th_f[k] = th0f[i];
+                    h.osc_th_lo[k] = th0lo[i];
+                }
             if (in_block[i]) continue;
             const double ps = d->prior_sigma[i], sc = d->scale[i];
             if (ps < 0.0 || !std::isfinite(ps)) {

@@ -52,6 +52,8 @@ struct DevDataset {
     const int *sp_param;     // [n_sp] parameter index
     const int *sp_ptr;       // [n_sp + 1] CSR offsets into sp_k
     const int *sp_k;         // true bins of each shape parameter
+    int lik_dup, map_dup;    // gradient totals whose parameter receives another total too: bits of
+                             // (deviance, efficiency, rates) and of (a0, a1, a2, norm)
     int sp_lanes;            // lanes that share one shape parameter's sum (a power of two <= 32)
     float w[FIT_MAX_CORES];  // core flux shares
     float kl_hi[FIT_MAX_CORES], kl_lo[FIT_MAX_CORES];  // K L_dc / pi as a float pair (half-turns)
@@ -89,6 +91,9 @@ struct DevModel {
     float osc_val[kMaxOsc];
     float osc_val_lo[kMaxOsc];   // low parts of the constant survival parameters
     double osc_val_d[kMaxOsc];   // the constant survival parameters in double
+    float osc_th_f[kMaxOsc], osc_th_lo[kMaxOsc];   // theta0 of the fitted ones as a float pair
+    int osc_dup;             // as DevDataset::map_dup: bits of the survival parameters, then the powers
+    int any_map_dup;         // 1: osc_dup or some dataset's map_dup is not 0
     int core_power_idx[FIT_MAX_CORES];
     const float *e_edge;     // [N_t + 1]
     const float *inv_e_hi;   // [N_t] 1 / E_k (true-bin centre) as a float pair
@@ -711,6 +716,8 @@ struct EvalShared {
     int bad;                                // 1: the dataset after them has an invalid energy map
     int status;                             // kSt* bits
     double nll;                             // sum over the datasets so far
+    double nll_ds[FIT_MAX_DATASETS];        // the group's datasets
+    float dup[FIT_MAX_DATASETS * 8 + 32];   // totals of parameters that receive several (in order)
     // warp totals: likelihood sums [dataset][warp][8], then energy-map sums [dataset][warp][4] and
     // survival / power sums [warp][32] (the two uses are barriers apart)
     float part[FIT_MAX_DATASETS * kMaxWarps * 8];
@@ -768,8 +775,8 @@ static __device__ int eval_setup(const DevModel &m, EvalShared &E, const ParVecs
             const int p = m.osc_idx[lane];
             float h, l;
             if (osc_is_dm(m.osc_mode, lane)) {
-                h = p >= 0 ? m.theta0_f[p] : m.osc_val[lane];
-                l = p >= 0 ? m.theta0_lo[p] + q.pd[p] : m.osc_val_lo[lane];
+                h = p >= 0 ? m.osc_th_f[lane] : m.osc_val[lane];
+                l = p >= 0 ? m.osc_th_lo[lane] + q.pd[p] : m.osc_val_lo[lane];
             } else {
                 h = p >= 0 ? q.pv[p] : m.osc_val[lane];
                 l = 0.f;
@@ -1034,31 +1041,59 @@ static __device__ __forceinline__ void st_lik(const DevModel &m, EvalShared &E, 
     __syncthreads();
 }
 
-// One warp (`warp_id`): the likelihood sums of the group in double, added to E.nll, and the
-// efficiency and rate gradients to grad.
+// Total over n <= kMaxWarps warps of the floats p[0], p[stride], ..., in double, by four
+// neighbouring lanes (sub = lane & 3); on each of them. A double addition has a latency of 66
+// cycles here, so four lanes halve the chain of a lane per total (which measured 5 000 cycles
+// over three datasets, one warp working through them), and all totals of a stage run at once
+// on as many warps as they need.
+__device__ __forceinline__ double quad_total(const float *p, int stride, int n, int sub) {
+    double s = 0.0;
+    for (int w = sub; w < n; w += 4) s += (double)p[w * stride];
+    s += __shfl_xor_sync(0xffffffffu, s, 1);
+    s += __shfl_xor_sync(0xffffffffu, s, 2);
+    return s;
+}
+
+// After st_lik: the group's likelihood sums in double (E.nll_ds), and with GRAD the efficiency and
+// rate gradients into grad; totals whose parameter receives several are left in E.dup for
+// lik_dups, a barrier later.
 template <bool GRAD>
-static __device__ __forceinline__ void lik_finish(const DevModel &m, EvalShared &E, float *grad, int warp_id) {
-    if ((int)(threadIdx.x >> 5) != warp_id) return;
-    const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    double nll = E.nll;
-    for (int i = 0; i < E.n; ++i) {
+static __device__ __forceinline__ void lik_finish(const DevModel &m, EvalShared &E, float *grad) {
+    const int nw = blockDim.x >> 5, sub = threadIdx.x & 3;
+    for (int v0 = 0; v0 < 8 * E.n; v0 += blockDim.x >> 2) {
+        const int v = v0 + (int)(threadIdx.x >> 2), i = v >> 3, q = v & 7;
+        if ((v & ~7) >= 8 * E.n) break;   // uniform over the warp
         const DevDataset &ds = m.ds[E.dl[i]];
-        const int used = min(nw, (ds.n_reco + 31) >> 5);
-        // lane = value (low three bits) x quarter of the warps
-        const float *p = E.part + (int64_t)i * kMaxWarps * 8 + (lane & 7);
-        double s = 0.0;
-        for (int w = lane >> 3; w < used; w += 4) s += (double)p[w * 8];
-        s += __shfl_xor_sync(0xffffffffu, s, 8);
-        s += __shfl_xor_sync(0xffffffffu, s, 16);
-        nll += __shfl_sync(0xffffffffu, s, 0);
-        if (GRAD) {
-            const int nb = ds.bkg_end - ds.bkg_begin;
-            const int p2 = lane == 1 ? ds.eff_idx : (lane >= 2 && lane - 2 < nb) ? m.bkg[ds.bkg_begin + lane - 2].rate_idx : -1;
-            if (lane >= 1 && lane < 8 && p2 >= 0) atomicAdd(&grad[p2], (float)s);
-            __syncwarp();
+        const double s = quad_total(E.part + (int64_t)i * kMaxWarps * 8 + q, 8, min(nw, (ds.n_reco + 31) >> 5), sub);
+        if (sub != 0) continue;
+        if (q == 0) E.nll_ds[i] = s;
+        if (GRAD && q >= 1) {
+            const int p = q == 1 ? ds.eff_idx : q - 2 < ds.bkg_end - ds.bkg_begin ? m.bkg[ds.bkg_begin + q - 2].rate_idx : -1;
+            if (p >= 0) {
+                if ((ds.lik_dup >> q) & 1)
+                    E.dup[v] = (float)s;
+                else
+                    grad[p] += (float)s;
+            }
         }
     }
-    if (lane == 0) E.nll = nll;
+}
+
+// One thread, a barrier after lik_finish: the sum of the group's -2lnL and (grad) the totals left
+// in E.dup, in order.
+static __device__ __forceinline__ void lik_dups(const DevModel &m, EvalShared &E, float *grad) {
+    double nll = E.nll;
+    for (int i = 0; i < E.n; ++i) nll += E.nll_ds[i];
+    E.nll = nll;
+    if (grad == nullptr) return;
+    for (int i = 0; i < E.n; ++i) {
+        const DevDataset &ds = m.ds[E.dl[i]];
+        for (int left = ds.lik_dup; left; left &= left - 1) {
+            const int q = __ffs(left) - 1;
+            const int p = q == 1 ? ds.eff_idx : m.bkg[ds.bkg_begin + q - 2].rate_idx;
+            grad[p] += E.dup[i * 8 + q];
+        }
+    }
 }
 
 // Background-shape gradient: a thread per shape parameter sums its (background, bin) pairs of
@@ -1186,37 +1221,45 @@ static __device__ __forceinline__ void st_adjoint_rest_n(const DevModel &m, Eval
     __syncthreads();
 }
 
-// Stage F, after st_adjoint_rest: the totals of stage E in double into grad (the last warp), and the
-// shape reweights: the bins of each distinct shape parameter (CSR) summed by sp_lanes lanes.
-// Ends with a barrier.
+// Stage F, after stage E: its totals in double into grad, and the shape reweights: the bins of
+// each distinct shape parameter (CSR) summed by sp_lanes lanes. Ends with a barrier.
 template <int NOSC>
 static __device__ __forceinline__ void st_adjoint_finish(const DevModel &m, EvalShared &E, float *wsb, float *grad) {
-    const int tid = threadIdx.x, lane = tid & 31, nw = blockDim.x >> 5, nth = blockDim.x;
-    if ((tid >> 5) == nw - 1) {
-        // energy maps and normalisations: lane = value (low two bits) x eighth of the warps
-        for (int i = 0; i < E.n; ++i) {
-            const DevDataset &ds = m.ds[E.dl[i]];
-            const float *p = E.part + (int64_t)i * kMaxWarps * 4 + (lane & 3);
-            double s = 0.0;
-            for (int w = lane >> 2; w < nw; w += 8) s += (double)p[w * 4];
-#pragma unroll
-            for (int o = 4; o < 32; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-            const int p2 = lane < 3 ? ds.esc_idx[lane] : lane == 3 ? ds.norm_idx : -1;
-            if (p2 >= 0) atomicAdd(&grad[p2], (float)s);
-            __syncwarp();
+    const int tid = threadIdx.x, nw = blockDim.x >> 5, nth = blockDim.x;
+    {
+        // totals: four per dataset, then the survival parameters and powers; four lanes each,
+        // from the last warp down (the shapes below start at the first)
+        const int nmap = 4 * E.n, nv = nmap + NOSC + m.C, sub = tid & 3;
+        for (int v0 = 0; v0 < nv; v0 += nth >> 2) {
+            const int v = v0 + ((nth - 1 - tid) >> 2);
+            if (v0 + (((nth - 1 - (tid | 31))) >> 2) >= nv) break;   // uniform over the warp
+            const bool map = v < nmap;
+            const int i = v >> 2, q = map ? (v & 3) : v - nmap;
+            const float *p = map ? E.part + (int64_t)i * kMaxWarps * 4 + q
+                                 : E.part + FIT_MAX_DATASETS * kMaxWarps * 4 + min(q, 31);
+            const double s = quad_total(p, map ? 4 : 32, v < nv ? nw : 0, sub);
+            if (sub != 0 || v >= nv) continue;
+            const DevDataset &ds = m.ds[E.dl[map ? i : 0]];
+            const int pi = map ? (q < 3 ? ds.esc_idx[q] : ds.norm_idx) : q < NOSC ? m.osc_idx[q] : m.core_power_idx[q - NOSC];
+            const int dup = map ? ds.map_dup : m.osc_dup;
+            if (pi < 0) continue;
+            if ((dup >> q) & 1)
+                E.dup[v] = (float)s;
+            else
+                grad[pi] += (float)s;
         }
-        // survival parameters and core powers: a lane per value
-        if (lane < NOSC + m.C) {
-            const float *p = E.part + FIT_MAX_DATASETS * kMaxWarps * 4 + lane;
-            double s0 = 0.0, s1 = 0.0;
-            for (int w = 0; w < nw; w += 2) {
-                s0 += (double)p[w * 32];
-                if (w + 1 < nw) s1 += (double)p[(w + 1) * 32];
+    }
+    if (m.any_map_dup) {
+        __syncthreads();
+        if (tid == 0) {
+            for (int v = 0; v < 4 * E.n + NOSC + m.C; ++v) {
+                const bool map = v < 4 * E.n;
+                const int q = map ? (v & 3) : v - 4 * E.n;
+                const DevDataset &ds = m.ds[E.dl[map ? v >> 2 : 0]];
+                const int pi = map ? (q < 3 ? ds.esc_idx[q] : ds.norm_idx) : q < NOSC ? m.osc_idx[q] : m.core_power_idx[q - NOSC];
+                if (pi >= 0 && (((map ? ds.map_dup : m.osc_dup) >> q) & 1)) grad[pi] += E.dup[v];
             }
-            const int p2 = lane < NOSC ? m.osc_idx[lane] : m.core_power_idx[lane - NOSC];
-            if (p2 >= 0) atomicAdd(&grad[p2], (float)(s0 + s1));
         }
-        __syncwarp();
     }
     if (m.shared_roles) __syncthreads();
     for (int i = 0; i < E.n; ++i) {
@@ -1294,14 +1337,18 @@ static __device__ double eval_datasets(const DevModel &m, EvalShared &E, const P
         }
         if (E.n == 0) continue;
         if (grad != nullptr) {
-            lik_finish<true>(m, E, grad, 0);
+            lik_finish<true>(m, E, grad);
             if (m.shared_roles) __syncthreads();
             st_bkg_shape(m, E, wsb, grad);
             st_adjoint_fold(m, E, wsb);
             __syncthreads();
+            if (threadIdx.x == 0) lik_dups(m, E, grad);
+            if (m.shared_roles) __syncthreads();
             st_adjoint_rest<GEN>(m, E, wsb, grad);
         } else {
-            lik_finish<false>(m, E, nullptr, 0);
+            lik_finish<false>(m, E, nullptr);
+            __syncthreads();
+            if (threadIdx.x == 0) lik_dups(m, E, nullptr);
         }
     }
     __syncthreads();

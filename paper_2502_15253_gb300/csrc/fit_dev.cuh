@@ -38,7 +38,8 @@ constexpr int kPhStart = 0, kPhTrial = 1, kPhDone = 2;
 struct FitState {
     // L-BFGS history in scalars: SY[i][j] = s_i.y_j (needed for i older than j and i = j),
     // YY[i][j] = y_i.y_j (symmetric), rho_i = 1 / s_i.y_i, by history slot
-    double SY[kMaxHist][kMaxHist], YY[kMaxHist][kMaxHist];
+    // (rows padded by one double: a lane per row otherwise meets one bank)
+    double SY[kMaxHist][kMaxHist + 1], YY[kMaxHist][kMaxHist + 1];
     double rho[kMaxHist];
     double gamma;
     double f, edm;
@@ -168,71 +169,95 @@ __device__ __forceinline__ void reset_history(FitState &st) {
     st.gamma = 1.0;
 }
 
-// Warp 0: folds the pending curvature pair (slot S.head, if `pending`) into the scalar
+// num / den in double from the FP32 reciprocal, two Newton steps and one correction of the quotient
+// by its residual (within an ulp): the library's double division takes 1467 cycles here, this
+// about 450. Operands outside FP32's normal range take the division.
+static __device__ double quick_div(double num, double den) {
+    const float d = (float)den;
+    if (!(fabsf(d) > 1e-30f && fabsf(d) < 1e30f)) return num / den;
+    double r = (double)__frcp_rn(d);
+    r = fma(r, fma(-den, r, 1.0), r);
+    r = fma(r, fma(-den, r, 1.0), r);
+    const double q = num * r;
+    return fma(r, fma(-den, q, num), q);
+}
+
+// One warp: folds the pending curvature pair (slot S.st.head, if `pending`) into the scalar
 // history and runs the L-BFGS two-loop recursion on scalars. Every inner product the
 // recursion needs is one of s_i.g, y_i.g, s_i.y_j (i older than j) or y_i.y_j, so the
 // direction is d = -(cg g + sum_j cs_j s_j + sum_j cy_j y_j) with coefficients from the
-// recurrence, and g^T H g (returned, on every lane) follows from the same scalars. Lane k holds chronological history
-// position k; both triangular recurrences run column by column (one shuffle per step).
+// recurrence, and g^T H g (returned, on every lane) follows from the same scalars. Lane k holds
+// chronological history position k; both triangular recurrences run column by column.
+//
+// What bounds it: the chain of double operations, 66 cycles each, one column after another. So
+// the columns' matrix entries are scaled by rho off the chain (a column costs one broadcast and
+// one fma), the products with YY ride along, slots advance without a modulo, and the pending
+// pair's rows are written by a lane per slot. On the three-dataset model (nine pairs on
+// average) a step's direction took 38 700 cycles before.
 static __device__ double lbfgs_scalars(FitSmem &S, int hist_max, bool pending) {
     const int lane = threadIdx.x & 31;
     const double *dt = S.dots;
-    if (pending && lane == 0) {
-        const int c = S.st.head;
+    FitState &st = S.st;
+    if (pending) {
+        const int c = st.head, occ = st.occ;
         const double sy = dt[c], yy = dt[kMaxHist + c];
         if (sy > 1e-10 * yy && yy > 0.0) {
-            for (int j = 0; j < hist_max; ++j)
-                if (((S.st.occ >> j) & 1) && j != c) {
-                    S.st.SY[j][c] = dt[j];
-                    S.st.YY[j][c] = S.st.YY[c][j] = dt[kMaxHist + j];
-                }
-            S.st.SY[c][c] = sy;
-            S.st.YY[c][c] = yy;
-            S.st.rho[c] = 1.0 / sy;
-            S.st.occ |= 1u << c;
-            S.st.head = (c + 1) % hist_max;
-            S.st.hn = min(S.st.hn + 1, hist_max);
-            S.st.gamma = sy / yy;
-        } else if ((S.st.occ >> c) & 1) {
+            const double q = quick_div(lane == 1 ? sy : 1.0, lane == 1 ? yy : sy);   // 1/s.y, s.y/y.y
+            __syncwarp();
+            if (lane < hist_max && ((occ >> lane) & 1) && lane != c) {
+                st.SY[lane][c] = dt[lane];
+                st.YY[lane][c] = st.YY[c][lane] = dt[kMaxHist + lane];
+            }
+            if (lane == 0) {
+                st.SY[c][c] = sy;
+                st.YY[c][c] = yy;
+                st.rho[c] = q;
+                st.occ = occ | (1 << c);
+                st.head = c + 1 == hist_max ? 0 : c + 1;
+                st.hn = min(st.hn + 1, hist_max);
+            }
+            if (lane == 1) st.gamma = q;
+        } else if ((occ >> c) & 1) {
             // rejected pair written over the oldest one: that pair is gone as well
-            S.st.occ &= ~(1u << c);
-            S.st.hn -= 1;
+            __syncwarp();
+            if (lane == 0) {
+                st.occ = occ & ~(1 << c);
+                st.hn -= 1;
+            }
         }
     }
     __syncwarp();
-    const int hn = S.st.hn, oldest = (S.st.head - hn + hist_max) % hist_max;
-    const double gam = S.st.gamma, gg = dt[kNDots - 1];
+    const int hn = st.hn;
+    const int oldest = st.head >= hn ? st.head - hn : st.head - hn + hist_max;
+    const double gam = st.gamma, gg = dt[kNDots - 1];
     const bool live = lane < hn;
-    const int sl = live ? (oldest + lane) % hist_max : 0;    // this lane's history slot
+    auto slot_of = [&](int k) { return oldest + k >= hist_max ? oldest + k - hist_max : oldest + k; };
+    const int sl = live ? slot_of(lane) : 0;    // this lane's history slot
     const double sg = live ? dt[2 * kMaxHist + sl] : 0.0, yg = live ? dt[3 * kMaxHist + sl] : 0.0;
-    const double rho = live ? S.st.rho[sl] : 0.0;
-    // alpha_k = rho_k (s_k.g - sum_{l > k} alpha_l s_k.y_l), newest first
-    double acc = sg, alpha = 0.0;
+    const double rho = live ? st.rho[sl] : 0.0;
+    // alpha_k = rho_k (s_k.g - sum_{l > k} alpha_l s_k.y_l), newest first; u_k = sum_l alpha_l y_k.y_l
+    double a = rho * sg, alpha = 0.0, u = 0.0;
     for (int l = hn - 1; l >= 0; --l) {
-        const double al = __shfl_sync(0xffffffffu, rho * acc, l);
+        const int sll = slot_of(l);
+        const double rs = lane < l ? rho * st.SY[sl][sll] : 0.0, yy = live ? st.YY[sl][sll] : 0.0;
+        const double al = __shfl_sync(0xffffffffu, a, l);
         if (lane == l) alpha = al;
-        const int sll = (oldest + l) % hist_max;
-        if (lane < l) acc -= al * S.st.SY[sl][sll];
-    }
-    // u_k = sum_l alpha_l y_k.y_l
-    double u = 0.0;
-    for (int l = 0; l < hn; ++l) {
-        const double al = __shfl_sync(0xffffffffu, alpha, l);
-        if (live) u += al * S.st.YY[sl][(oldest + l) % hist_max];
+        a = fma(-al, rs, a);
+        u = fma(al, yy, u);
     }
     // beta_k = rho_k (gam (y_k.g - u_k) + sum_{l < k} (alpha_l - beta_l) s_l.y_k), oldest first
-    double acc2 = gam * (yg - u), beta = 0.0;
+    double b = rho * (gam * (yg - u)), beta = 0.0;
     for (int l = 0; l < hn; ++l) {
-        const double bl = __shfl_sync(0xffffffffu, rho * acc2, l);
-        const double cl = __shfl_sync(0xffffffffu, alpha, l) - bl;
+        const double rs = live && lane > l ? rho * st.SY[slot_of(l)][sl] : 0.0;
+        const double al = __shfl_sync(0xffffffffu, alpha, l), bl = __shfl_sync(0xffffffffu, b, l);
         if (lane == l) beta = bl;
-        if (live && lane > l) acc2 += cl * S.st.SY[(oldest + l) % hist_max][sl];
+        b = fma(al - bl, rs, b);
     }
     const double cs = alpha - beta, cy = -gam * alpha;
     double part = live ? cs * sg + cy * yg : 0.0;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-    double ghg = gam * gg + part;
+    const double ghg = gam * gg + part;
     if (live) {
         S.cs[lane] = (float)cs;
         S.cy[lane] = (float)cy;
@@ -243,7 +268,7 @@ static __device__ double lbfgs_scalars(FitSmem &S, int hist_max, bool pending) {
     if (lane == 0) {
         S.n_dir = ok ? hn : 0;
         S.cg = ok ? (float)gam : 1.f;
-        if (!ok) reset_history(S.st);
+        if (!ok) reset_history(st);
     }
     __syncwarp();
     return ok ? ghg : gg;
@@ -322,34 +347,49 @@ static __device__ void pre_apply(const DevModel &m, const float *coef, const flo
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int nfull = P >> 2;
     const float4 *x4 = reinterpret_cast<const float4 *>(x);
-    for (int k = warp; k < r; k += nw) {
-        const float *q = m.pre_Q + (int64_t)k * Pp;
-        const float4 *q4 = reinterpret_cast<const float4 *>(q);
-        float acc = 0.f;
+    // four rows per warp and pass, so that their loads are in flight together
+    for (int k0 = warp; k0 < r; k0 += 4 * nw) {
+        const float4 *q4[4];
+#pragma unroll
+        for (int u4 = 0; u4 < 4; ++u4) q4[u4] = reinterpret_cast<const float4 *>(m.pre_Q + (int64_t)min(k0 + u4 * nw, r - 1) * Pp);
+        float acc[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 2
         for (int c = lane; c < nfull; c += 32) {
-            float4 a = __ldg(q4 + c);
-            const float4 b = x4[c];
+            float4 b = x4[c];
             if (fixed) {
                 const uint8_t *f = fixed + 4 * c;
-                if (f[0]) a.x = 0.f;
-                if (f[1]) a.y = 0.f;
-                if (f[2]) a.z = 0.f;
-                if (f[3]) a.w = 0.f;
+                if (f[0]) b.x = 0.f;
+                if (f[1]) b.y = 0.f;
+                if (f[2]) b.z = 0.f;
+                if (f[3]) b.w = 0.f;
             }
-            acc = fmaf(a.x, b.x, fmaf(a.y, b.y, fmaf(a.z, b.z, fmaf(a.w, b.w, acc))));
-        }
-        if (lane < (P & 3) && !(fixed && fixed[4 * nfull + lane]))
-            acc = fmaf(__ldg(q + 4 * nfull + lane), x[4 * nfull + lane], acc);
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-        if (lane == 0) u[k] = __ldg(coef + k) * acc;
+            for (int u4 = 0; u4 < 4; ++u4) {
+                const float4 a = __ldg(q4[u4] + c);
+                acc[u4] = fmaf(a.x, b.x, fmaf(a.y, b.y, fmaf(a.z, b.z, fmaf(a.w, b.w, acc[u4]))));
+            }
+        }
+        if (lane < (P & 3) && !(fixed && fixed[4 * nfull + lane])) {
+            const float b = x[4 * nfull + lane];
+#pragma unroll
+            for (int u4 = 0; u4 < 4; ++u4)
+                acc[u4] = fmaf(__ldg(reinterpret_cast<const float *>(q4[u4]) + 4 * nfull + lane), b, acc[u4]);
+        }
+        const float t = warp_sum_split<4>(acc);
+        const int k = k0 + (lane >> 3) * nw;
+        if ((lane & 7) == 0 && k < r) u[k] = __ldg(coef + k) * t;
     }
     __syncthreads();
     for (int i = threadIdx.x; i < P; i += blockDim.x) {
         float acc = x[i];
         if (!(fixed && fixed[i])) {
-#pragma unroll 8
-            for (int k = 0; k < r; ++k) acc = fmaf(__ldg(m.pre_Q + (int64_t)k * Pp + i), u[k], acc);
+            for (int k0 = 0; k0 < r; k0 += 16) {   // sixteen rows' loads in flight
+                float q[16];
+#pragma unroll
+                for (int k = 0; k < 16; ++k) q[k] = __ldg(m.pre_Q + (int64_t)min(k0 + k, r - 1) * Pp + i);
+#pragma unroll
+                for (int k = 0; k < 16; ++k) acc = fmaf(q[k], k0 + k < r ? u[k0 + k] : 0.f, acc);
+            }
         }
         y[i] = acc;
     }

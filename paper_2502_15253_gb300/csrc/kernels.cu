@@ -236,7 +236,9 @@ __device__ __forceinline__ void ls_forward_body(LsArgs A) {
             st_fold(m, S.E, wsb);
             st_lik<true>(m, S.E, q, A.data + in.data_off, wsb);
             if (!S.E.status) {
-                lik_finish<true>(m, S.E, A.gsl + gd * P, 0);
+                lik_finish<true>(m, S.E, A.gsl + gd * P);
+                __syncthreads();
+                if (threadIdx.x == 0) lik_dups(m, S.E, A.gsl + gd * P);
                 if (m.shared_roles) __syncthreads();
                 st_bkg_shape(m, S.E, wsb, A.gsl + gd * P);
             }
@@ -375,7 +377,9 @@ __device__ __forceinline__ void ls_tc_lik_body(LsArgs A) {
         if (S.E.n) {
             st_lik<true>(m, S.E, q, A.data + in.data_off, wsb);
             if (!S.E.status) {
-                lik_finish<true>(m, S.E, A.gsl + gd * P, 0);
+                lik_finish<true>(m, S.E, A.gsl + gd * P);
+                __syncthreads();
+                if (threadIdx.x == 0) lik_dups(m, S.E, A.gsl + gd * P);
                 if (m.shared_roles) __syncthreads();
                 st_bkg_shape(m, S.E, wsb, A.gsl + gd * P);
             }

@@ -98,6 +98,76 @@ void lower_inverse(int n, const std::vector<double> &L, std::vector<double> &W) 
     }
 }
 
+// A banded matrix (row r, column k) packed as fitcore::BandUnits: output rows in fours, `parts` lanes per
+// four rows.
+struct PackedBands {
+    int parts;
+    std::vector<int2> steps;
+    std::vector<int> start;
+    std::vector<float4> entry;
+};
+
+template <class At>
+PackedBands pack_bands(int rows, int cols, At at, int parts) {
+    PackedBands p;
+    p.parts = parts;
+    const int groups = (rows + 3) / 4, lanes = groups * parts, units = (lanes + 31) / 32;
+    std::vector<int> lo(groups, 0), len(groups, 0);   // per group: first column, columns per part
+    for (int g = 0; g < groups; ++g) {
+        int a = cols, b = -1;
+        for (int r = 4 * g; r < std::min(4 * g + 4, rows); ++r)
+            for (int k = 0; k < cols; ++k)
+                if (at(r, k) != 0.f) {
+                    a = std::min(a, k);
+                    b = std::max(b, k);
+                }
+        if (b >= a) {
+            lo[g] = a;
+            len[g] = (b - a + 1 + parts - 1) / parts;
+        }
+    }
+    p.start.assign((size_t)units * 32, 0);
+    for (int w = 0; w < units; ++w) {
+        int n = 0;
+        for (int l = 0; l < 32; ++l)
+            if (w * 32 + l < lanes) n = std::max(n, len[(w * 32 + l) / parts]);
+        p.steps.push_back(make_int2((int)p.entry.size(), n));
+        p.entry.resize(p.entry.size() + (size_t)n * 32, make_float4(0.f, 0.f, 0.f, 0.f));
+        float4 *e = p.entry.data() + p.steps.back().x;
+        for (int l = 0; l < 32; ++l) {
+            const int x = w * 32 + l, g = x / parts;
+            if (x >= lanes) continue;
+            const int k0 = lo[g] + (x % parts) * len[g];
+            // the lane reads n columns from its start: shifted down where they would pass the end
+            const int s = std::max(0, std::min(k0, cols - n));
+            p.start[x] = s;
+            for (int k = k0; k < std::min(k0 + len[g], cols); ++k) {
+                float v[4] = {0.f, 0.f, 0.f, 0.f};
+                for (int r = 0; r < 4; ++r)
+                    if (4 * g + r < rows) v[r] = at(4 * g + r, k);
+                e[(size_t)(k - s) * 32 + l] = make_float4(v[0], v[1], v[2], v[3]);
+            }
+        }
+    }
+    return p;
+}
+
+// Workspace sizes of a model's evaluation (everything but the prior blocks' scratch).
+void set_workspace(DevModel &h, int max_reco, int n_osc) {
+    h.max_reco = max_reco;
+    h.ws_eval_floats = fitcore::eval_ws_floats(h.N_t, h.C, max_reco, n_osc, h.remap_mode);
+    // datasets evaluated together: as many as 64 KB of workspace hold (a property of the model
+    // alone, so that the result of an evaluation does not depend on the launch)
+    h.ws_group = std::max(1, std::min(h.n_ds, (int)(64 * 1024 / (sizeof(float) * (size_t)h.ws_eval_floats))));
+}
+
+// Lanes per four reco rows in the fold: as many as keep a group's datasets on one pass of the block
+int fold_parts(const DevModel &h, int nr) {
+    int p = 1;
+    while (p < 32 && 2 * p * ((nr + 3) / 4) * h.ws_group <= fitcore::model_threads(h)) p *= 2;
+    return p;
+}
+
 struct LaunchCfg {
     int sms = 0;
     size_t smem_optin = 0;
@@ -383,60 +453,32 @@ int fit_model_create(const fit_model_desc *d, fit_model **out) {
     vector<int> det_off(d->n_det + 1, 0);
     for (int i = 0; i < d->n_det; ++i) det_off[i + 1] = det_off[i] + d->det_n_reco[i] * Nt;
     int max_reco = 0;
+    std::deque<PackedBands> det_fold, det_adj;
+    for (int i = 0; i < d->n_det; ++i) max_reco = std::max(max_reco, d->det_n_reco[i]);
+    set_workspace(h, max_reco, n_osc);
     for (int i = 0; i < d->n_det; ++i) {
         const int nr = d->det_n_reco[i];
-        max_reco = std::max(max_reco, nr);
         const double *R = d->det_response + det_off[i];
-        vector<int> rlo(nr), rlen(nr), roff(nr);
-        vector<float> rrow;
-        for (int j = 0; j < nr; ++j) {
-            int a = Nt, b = -1;
-            for (int k = 0; k < Nt; ++k) {
-                const double x = R[(size_t)j * Nt + k];
-                if (!std::isfinite(x) || x < 0.0) {
-                    delete M;
-                    return bad("response entries must be finite and >= 0");
-                }
-                if (x != 0.0) {
-                    a = std::min(a, k);
-                    b = std::max(b, k);
-                }
+        for (size_t e = 0; e < (size_t)nr * Nt; ++e)
+            if (!std::isfinite(R[e]) || R[e] < 0.0) {
+                delete M;
+                return bad("response entries must be finite and >= 0");
             }
-            if (b < a) a = b = 0;   // empty row: one zero entry
-            rlo[j] = a;
-            rlen[j] = b - a + 1;
-            roff[j] = (int)rrow.size();
-            for (int k = a; k <= b; ++k) rrow.push_back((float)R[(size_t)j * Nt + k]);
-            while (rrow.size() % 4) rrow.push_back(0.f);
-        }
-        vector<int> clo(Nt), clen(Nt);
-        int cw = 1;
-        for (int k = 0; k < Nt; ++k) {
-            int a = nr, b = -1;
-            for (int j = 0; j < nr; ++j)
-                if (R[(size_t)j * Nt + k] != 0.0) {
-                    a = std::min(a, j);
-                    b = std::max(b, j);
-                }
-            if (b < a) a = b = 0;
-            clo[k] = a;
-            clen[k] = b - a + 1;
-            cw = std::max(cw, b - a + 1);
-        }
-        vector<float> rcol((size_t)cw * Nt, 0.f);
-        for (int k = 0; k < Nt; ++k)
-            for (int b = 0; b < cw && clo[k] + b < nr; ++b)
-                rcol[(size_t)b * Nt + k] = (float)R[(size_t)(clo[k] + b) * Nt + k];
         fitcore::DevDetector &dt = h.det[i];
         dt.n_reco = nr;
-        dt.col_w = cw;
-        A.put(&dt.row_lo, rlo);
-        A.put(&dt.row_len, rlen);
-        A.put(&dt.row_off, roff);
-        A.put(&dt.rrow, rrow);
-        A.put(&dt.col_lo, clo);
-        A.put(&dt.col_len, clen);
-        A.put(&dt.rcol, rcol);
+        det_fold.push_back(pack_bands(nr, Nt, [&](int r, int k) { return (float)R[(size_t)r * Nt + k]; },
+                                      fold_parts(h, nr)));
+        det_adj.push_back(pack_bands(Nt, nr, [&](int k, int r) { return (float)R[(size_t)r * Nt + k]; }, 1));
+        for (const bool adj : {false, true}) {
+            const PackedBands &pb = adj ? det_adj.back() : det_fold.back();
+            fitcore::BandUnits &U = adj ? dt.adj : dt.fold;
+            U.n = (int)pb.steps.size();
+            U.parts = pb.parts;
+            U.outs = adj ? Nt : nr;
+            A.put(&U.steps, pb.steps);
+            A.put(&U.start, pb.start);
+            A.put(&U.entry, pb.entry);
+        }
         // dense copy for the tensor-core fold, split into a TF32-exact high part and the rest
         const int ldt = (Nt + 3) / 4 * 4;
         vector<float> rhi((size_t)nr * ldt, 0.f), rlow((size_t)nr * ldt, 0.f);
@@ -521,11 +563,15 @@ int fit_model_create(const fit_model_desc *d, fit_model **out) {
             if (sidx[k] >= 0) params.push_back(sidx[k]);
         std::sort(params.begin(), params.end());
         params.erase(std::unique(params.begin(), params.end()), params.end());
-        vector<int> ptr(params.size() + 1, 0), ks;
+        vector<int4> sp(params.size());
+        vector<int> ks;
         for (size_t q = 0; q < params.size(); ++q) {
+            const int begin = (int)ks.size();
             for (int k = 0; k < Nt; ++k)
                 if (sidx[k] == params[q]) ks.push_back(k);
-            ptr[q + 1] = (int)ks.size();
+            const int n = (int)ks.size() - begin;
+            const bool run = ks.back() - ks[begin] + 1 == n;
+            sp[q] = make_int4(params[q], run ? ks[begin] : begin, n, run ? 1 : 0);
         }
         D.n_sp = (int)params.size();
         // lanes per parameter: about four bins each
@@ -533,8 +579,7 @@ int fit_model_create(const fit_model_desc *d, fit_model **out) {
         while (D.sp_lanes < 32 && D.n_sp > 0 && Nt > 4 * D.sp_lanes * D.n_sp) D.sp_lanes *= 2;
         A.put(&D.t, t);
         A.put(&D.shape_idx, sidx);
-        A.put(&D.sp_param, params);
-        A.put(&D.sp_ptr, ptr);
+        A.put(&D.sp, sp);
         A.put(&D.sp_k, ks);
         // backgrounds of this dataset, in description order
         D.bkg_begin = (int)bkg_order.size();
@@ -745,50 +790,58 @@ int fit_model_create(const fit_model_desc *d, fit_model **out) {
             }
         }
         h.n_blocks = d->n_cov;
-        // tiles of the triangular products (tri_apply): the lower form reads the transposed
-        // copy, so that a lane per row is a coalesced load per column; the upper form the
-        // matrix itself. Tiles beyond the diagonal are left out.
+        // Tiles of the triangular products (tri_apply): rows in tiles of 128, columns in segments;
+        // the rows of a tile above (lower form) or below (upper form) all of its columns' entries
+        // are left out, so little more than the triangle is read.
         {
             vector<fitcore::TriTile> lo, up;
+            vector<float> Llo, Lup, Wlo, Wup;
             vector<int> tparam, tseg;
             int rows = 0, segs = 1;
-            constexpr int kC = fitcore::kTriCols;
             for (size_t b = 0; b < bsz.size(); ++b) {
-                const int n = bsz[b];
+                const int n = bsz[b], seg_cols = n <= 512 ? 32 : 64, nseg = (n + seg_cols - 1) / seg_cols;
+                const float *Lb = Lf.data() + moff[b], *Wb = Wf.data() + moff[b];   // [M | M^T], n x n each
                 bool contig = true;
                 for (int i = 1; i < n && contig; ++i) contig = bidx[boff[b] + i] == bidx[boff[b]] + i;
-                const int in0 = contig ? bidx[boff[b]] : -1, nseg = (n + kC - 1) / kC;
                 segs = std::max(segs, nseg);
-                for (int r0 = 0; r0 < n; r0 += 32)
-                    for (int s = 0; s < nseg; ++s) {
-                        const int last = std::min(r0 + 31, n - 1);   // last row of the tile
-                        fitcore::TriTile t;
-                        t.n = n;
-                        t.row0 = r0;
-                        t.in0 = in0;
-                        t.idx = boff[b];
-                        t.out = rows;
-                        t.seg = s;
-                        t.col0 = s * kC;                             // lower: columns <= last
-                        t.cols = std::min({kC, n - t.col0, last + 1 - t.col0});
-                        t.mat = (int)(moff[b] + (int64_t)n * n);
-                        if (t.cols > 0) lo.push_back(t);
-                        t.col0 = std::max(s * kC, r0);               // upper: columns >= r0
-                        t.cols = std::min((s + 1) * kC, n) - t.col0;
-                        t.mat = (int)moff[b];
-                        if (t.cols > 0) up.push_back(t);
-                    }
+                for (int r0 = 0; r0 < n; r0 += 128)
+                    for (int s = 0; s < nseg; ++s)
+                        for (const bool upper : {false, true}) {
+                            const int c0 = s * seg_cols, c1 = std::min(c0 + seg_cols, n);
+                            const int ra = upper ? r0 : std::max(r0, c0);
+                            const int rb = std::min({r0 + 128, n, upper ? c1 : n});
+                            if (rb <= ra) continue;
+                            fitcore::TriTile t;
+                            vector<float> &Lo = upper ? Lup : Llo, &Wo = upper ? Wup : Wlo;
+                            t.mat = (int)Lo.size();
+                            t.rows = rb - ra;
+                            t.pitch = (t.rows + 3) / 4 * 4;
+                            t.cols = c1 - c0;
+                            t.in0 = contig ? bidx[boff[b]] + c0 : -1;
+                            t.idx = boff[b] + c0;
+                            t.out = rows + ra;
+                            t.seg = s;
+                            // entry (out r, in c): M[r][c] in the lower form, M[c][r] in the upper
+                            for (int q = c0; q < c1; ++q)
+                                for (int r = ra; r < ra + t.pitch; ++r) {
+                                    const size_t e = upper ? (size_t)q * n + r : (size_t)r * n + q;
+                                    Lo.push_back(r < rb ? Lb[e] : 0.f);
+                                    Wo.push_back(r < rb ? Wb[e] : 0.f);
+                                }
+                            (upper ? up : lo).push_back(t);
+                        }
                 for (int i = 0; i < n; ++i) {
-                    const int r0 = i / 32 * 32, last = std::min(r0 + 31, n - 1);
                     tparam.push_back(bidx[boff[b] + i]);
-                    tseg.push_back((last / kC + 1) | (r0 / kC) << 8 | nseg << 16);
+                    tseg.push_back((i / seg_cols + 1) | (i / seg_cols) << 8 | nseg << 16);
                 }
                 rows += n;
             }
-            // the longest tiles first, so that no warp picks one up last
-            auto longer = [](const fitcore::TriTile &a, const fitcore::TriTile &b) { return a.cols > b.cols; };
-            std::stable_sort(lo.begin(), lo.end(), longer);
-            std::stable_sort(up.begin(), up.end(), longer);
+            // the largest tiles first, so that no warp picks one up last
+            auto larger = [](const fitcore::TriTile &a, const fitcore::TriTile &b) {
+                return a.cols * a.pitch > b.cols * b.pitch;
+            };
+            std::stable_sort(lo.begin(), lo.end(), larger);
+            std::stable_sort(up.begin(), up.end(), larger);
             h.n_tri_lo = (int)lo.size();
             h.n_tri_up = (int)up.size();
             h.tri_rows = rows;
@@ -797,6 +850,10 @@ int fit_model_create(const fit_model_desc *d, fit_model **out) {
             A.put(&h.tri_up, up);
             A.put(&h.tri_param, tparam);
             A.put(&h.tri_seg, tseg);
+            A.put(&h.L_lo, Llo);
+            A.put(&h.L_up, Lup);
+            A.put(&h.W_lo, Wlo);
+            A.put(&h.W_up, Wup);
         }
         A.put(&h.theta0, th0);
         A.put(&h.theta0_f, th0f);
@@ -831,8 +888,6 @@ int fit_model_create(const fit_model_desc *d, fit_model **out) {
             for (int64_t q = 0; q < (int64_t)n * n; ++q) M->blk_L.push_back(L64[moff[b] + q]);
         }
         A.put(&h.blk_mat_off, moff);
-        A.put(&h.blk_L, Lf);
-        A.put(&h.blk_W, Wf);
         A.put(&h.blk_L64, L64);
     }
     {
@@ -843,10 +898,6 @@ int fit_model_create(const fit_model_desc *d, fit_model **out) {
             for (int j = 0; j < h.ds[ds].n_reco; ++j) slot_ds[h.ds[ds].data_off + j] = ds;
         A.put(&h.slot_ds, slot_ds);
     }
-    h.ws_eval_floats = fitcore::eval_ws_floats(Nt, C, max_reco, n_osc);
-    // datasets evaluated together: as many as 64 KB of workspace hold (a property of the model
-    // alone, so that the result of an evaluation does not depend on the launch)
-    h.ws_group = std::max(1, std::min(h.n_ds, (int)(64 * 1024 / (sizeof(float) * (size_t)h.ws_eval_floats))));
     h.ws_floats = std::max(h.ws_group * h.ws_eval_floats, (h.tri_segs * h.tri_rows + 3) & ~3);
     h.ldt = (Nt + 3) / 4 * 4;
 
@@ -2391,7 +2442,7 @@ int fit_batch_ex(fit_model *const *models, int n_models, const fit_instance *ins
         // (multiples of 4 floats: the fit vectors start on 16-byte boundaries)
         max_need = std::max(max_need, fitcore::fit_vec_floats(h.P, o.history) + h.ws_floats);
         max_loc = std::max(max_loc, fitcore::fit_work_floats(h.P) + h.ws_floats);
-        const size_t one = (size_t)h.ws_eval_floats + 14 * (size_t)fitcore::fit_vec_pitch(h.P);
+        const size_t one = (((size_t)(4 + h.n_osc + h.C) * h.N_t + 2 * h.max_reco + 3) & ~size_t(3)) + 14 * (size_t)fitcore::fit_vec_pitch(h.P);
         ask_loc = std::max(ask_loc, 25184 + sizeof(float) * one);
         ask_all = std::max(ask_all, 25184 + sizeof(float) * (one + (size_t)fitcore::fit_hist_floats(h.P, o.history)));
     }

@@ -16,18 +16,23 @@ constexpr int kMaxWarps = 16;      // blocks of at most 512 threads
 constexpr int kMaxBkgDs = 6;       // backgrounds per dataset
 constexpr int kMaxOsc = 6;         // survival parameters (6 for the 3+1 formula, else 4)
 
+// A banded matrix packed for matrix-vector products (band_product): four consecutive outputs per lane
+// group of `parts` lanes, each lane a consecutive range of the band's inputs. Warp unit w holds
+// 32 such lanes: steps[w].y steps of 32 float4 from entry + steps[w].x; lane l of it starts at
+// input start[32 w + l]. Entries outside a lane's own range are 0 and every input read exists.
+struct BandUnits {
+    const int2 *steps;
+    const int *start;
+    const float4 *entry;
+    int n, parts, outs;
+};
+
 struct DevDetector {
     int n_reco;
-    int col_w;               // padded width of the column bands
-    const int *row_lo;       // [N_r] first true bin of row j's band
-    const int *row_len;      // [N_r] band length
-    const int *row_off;      // [N_r] offset of the row's band in rrow
-    const float *rrow;       // packed row bands
-    const int *col_lo;       // [N_t] first reco row of column k's band
-    const float *rcol;       // [col_w x N_t]: rcol[b * N_t + k] = R[col_lo[k] + b][k] (0 past the band)
+    BandUnits fold;          // outputs: reco rows in fours, inputs: true bins
+    BandUnits adj;           // outputs: true bins in fours, inputs: reco rows
     const float *rdense_hi;  // [N_r x ldt] dense response, TF32-exact high part (tensor-core fold)
     const float *rdense_lo;  // [N_r x ldt] R - rdense_hi
-    const int *col_len;      // [N_t] band length of column k
     const float *rdt_hi;     // [N_t x ldr] R^T, TF32-exact high part (tensor-core adjoint fold)
     const float *rdt_lo;     // [N_t x ldr] R^T - rdt_hi
     int ldr;                 // row stride of R^T (N_r rounded up to 4)
@@ -49,9 +54,10 @@ struct DevDataset {
     int n_sp;                // distinct shape parameters used by this dataset
     const float *t;          // [N_t] un-oscillated signal
     const int *shape_idx;    // [N_t]
-    const int *sp_param;     // [n_sp] parameter index
-    const int *sp_ptr;       // [n_sp + 1] CSR offsets into sp_k
-    const int *sp_k;         // true bins of each shape parameter
+    // Shape parameter p: parameter sp[p].x, sp[p].z true bins, consecutive from sp[p].y (sp[p].w = 1)
+    // or at sp_k + sp[p].y
+    const int4 *sp;          // [n_sp]
+    const int *sp_k;
     int lik_dup, map_dup;    // gradient totals whose parameter receives another total too: bits of
                              // (deviance, efficiency, rates) and of (a0, a1, a2, norm)
     int sp_lanes;            // lanes that share one shape parameter's sum (a power of two <= 32)
@@ -59,18 +65,12 @@ struct DevDataset {
     float kl_hi[FIT_MAX_CORES], kl_lo[FIT_MAX_CORES];  // K L_dc / pi as a float pair (half-turns)
 };
 
-// One tile of a triangular matrix-vector product: out rows row0..row0+31 of a block (clipped to it),
-// summed over `cols` <= kTriCols columns from col0.
-constexpr int kTriCols = 64;
+// One tile of a triangular matrix-vector product: out rows `out`.. (of all blocks concatenated), summed
+// over `cols` columns, the inputs in0.. (consecutive parameters) or blk_idx[idx..] (in0 < 0). The
+// tile's matrix entries are stored column after column, `pitch` (rows rounded up to 4) floats each.
 struct TriTile {
-    int mat;                 // offset of the block's matrix (rows of n floats, column-major over the
-                             // tile's lanes: element (out r, in c) at mat + c * n + r)
-    int n;                   // block size
-    int row0, col0, cols;
-    int in0;                 // first input index when the block's parameters are consecutive, else -1
-    int idx;                 // offset of the block's parameter indices (DevModel::blk_idx)
-    int out;                 // concatenated row of the block's row 0
-    int seg;                 // partial-sum slot
+    int mat, pitch, rows, cols;
+    int in0, idx, out, seg;
 };
 
 // Bin j of background q (dataset d, row of the data vector of that dataset) scaled by a shape parameter
@@ -111,16 +111,15 @@ struct DevModel {
     const int *blk_idx_off;  // [n_blocks]
     const int *blk_idx;      // concatenated parameter indices
     const int64_t *blk_mat_off;  // [n_blocks] offset of the block's m x m matrices
-    const float *blk_L;      // lower Cholesky factor of V (row-major, dense)
-    const float *blk_W;      // L^-1 (row-major, dense lower triangle)
-    const double *blk_L64;   // L in double (final theta of a fit)
+    const double *blk_L64;   // lower Cholesky factors of V, then transposed (final theta of a fit)
     const float *asimov;     // [n_data] expectation at theta0
     const int *slot_ds;      // [n_data] dataset of each data bin
     int ws_eval_floats;      // workspace of one dataset of one evaluation (a multiple of 4)
     int ws_group;            // datasets evaluated together (their workspaces are held at once)
-    // matrix-vector products with the triangular prior blocks as tiles of 32 rows x kTriCols
-    // columns (see tri_apply): tri_lo for L z / W d, tri_up for L^T g / W^T z
+    // matrix-vector products with the triangular prior blocks as packed tiles (see tri_apply):
+    // tri_lo for L z / W d, tri_up for L^T g / W^T z; the tiles' entries in L_lo, L_up, W_lo, W_up
     const TriTile *tri_lo, *tri_up;
+    const float *L_lo, *L_up, *W_lo, *W_up;
     int n_tri_lo, n_tri_up, tri_segs, tri_rows;   // tiles, column segments, rows of all blocks
     const int *tri_param;    // [tri_rows] parameter of each concatenated row
     const int *tri_seg;      // [tri_rows] its segments: lower 0..(x & 255) - 1, upper
@@ -188,17 +187,82 @@ __device__ __forceinline__ float warp_sum_split(float (&v)[N]) {
 // ------------------------------------------------------------------------------------
 // Survival probability with phase arithmetic in float pairs.
 // ------------------------------------------------------------------------------------
+// sin and cos of pi r for |r| <= 1/2 (a little more is harmless): r (pi + u P(u)) and 1 + u Q(u),
+// u = r^2, P of degree 3 and Q of degree 4 fitted for the smallest largest error (Lawson
+// iteration; sin2pi_fit.py in this directory), pi as a float pair. Within 1.3e-7 in FP32,
+// the error of sincospif's results to one unit in the last place at half its instructions
+// (the phase is already reduced, so none of them goes into reduction and quadrants).
+__device__ __forceinline__ void sincos_half(float r, float &s, float &c) {
+    const float u = r * r;
+    float t = fmaf(0.07749626f, u, -0.59821373f);
+    t = fmaf(t, u, 2.5500667f);
+    t = fmaf(t, u, -5.16771f);
+    t = fmaf(t, u, -8.742278e-8f);        // pi - (float)pi
+    s = fmaf(r, 3.14159274f, r * t);
+    float q = fmaf(-0.024417998f, u, 0.23495245f);
+    q = fmaf(q, u, -1.3352158f);
+    q = fmaf(q, u, 4.0587096f);
+    q = fmaf(q, u, -4.934802f);
+    c = fmaf(q, u, 1.f);
+}
+
 // Phase in half-turns: y = x / pi = (dm_hi + dm_lo) * (c_hi + c_lo), c = K L / (pi E), carried
 // as a float pair. The probability depends on sin^2 x and sin 2x only, so y is reduced by
 // its nearest integer, which is exact (y_hi - rint(y_hi) is representable), and sin, cos of
-// pi r, |r| <= 1/2, come from sincospif. The pair keeps r accurate to ~1e-8 even at 50 km
+// pi r, |r| <= 1/2, follow. The pair keeps r accurate to ~1e-8 even at 50 km
 // (y ~ 30), and no pi constant or multi-word reduction enters the arithmetic.
 __device__ __forceinline__ void phase_sc(float dm, float dm_lo, float c_hi, float c_lo, float &s,
                                          float &c) {
     const float yh = dm * c_hi;
-    const float yl = fmaf(dm, c_hi, -yh) + fmaf(dm, c_lo, dm_lo * c_hi);
-    const float r = (yh - rintf(yh)) + yl;
-    sincospif(r, &s, &c);
+    const float yl = fmaf(dm_lo, c_hi, fmaf(dm, c_lo, fmaf(dm, c_hi, -yh)));
+    sincos_half((yh - rintf(yh)) + yl, s, c);
+}
+
+// Packed FP32: two values in one register pair, one instruction for both.
+using f32x2 = unsigned long long;
+__device__ __forceinline__ f32x2 pack2(float a, float b) {
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 pack2(float a) { return pack2(a, a); }
+__device__ __forceinline__ float2 unpack2(f32x2 v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
+// sincos_half for two reduced phases
+__device__ __forceinline__ void sincos_half2(f32x2 r, f32x2 &s, f32x2 &c) {
+    const f32x2 u = mul2(r, r);
+    f32x2 t = fma2(pack2(0.07749626f), u, pack2(-0.59821373f));
+    t = fma2(t, u, pack2(2.5500667f));
+    t = fma2(t, u, pack2(-5.16771f));
+    t = fma2(t, u, pack2(-8.742278e-8f));
+    s = fma2(r, pack2(3.14159274f), mul2(r, t));
+    f32x2 q = fma2(pack2(-0.024417998f), u, pack2(0.23495245f));
+    q = fma2(q, u, pack2(-1.3352158f));
+    q = fma2(q, u, pack2(4.0587096f));
+    q = fma2(q, u, pack2(-4.934802f));
+    c = fma2(q, u, pack2(1.f));
+}
+
+// The reduced phase -y of phase_sc for two cores (dm, -dm, its low part; m1 = -1)
+__device__ __forceinline__ f32x2 neg_phase2(f32x2 dm, f32x2 ndm, f32x2 dm_lo, f32x2 ch, f32x2 cl, f32x2 m1) {
+    const f32x2 n = mul2(ndm, ch);
+    const f32x2 e = fma2(dm_lo, ch, fma2(dm, cl, fma2(dm, ch, n)));
+    const float2 v = unpack2(n);
+    return fma2(e, m1, fma2(pack2(rintf(v.x), rintf(v.y)), m1, n));
 }
 
 // sin^2(pi r) for |r| <= 1/2: u q(u), u = r^2, q a degree-7 polynomial fitted for the
@@ -285,52 +349,8 @@ __device__ __forceinline__ F2 f2_sqrt(F2 a) {
     return f2_norm(s, r / (2.f * s));
 }
 
-// P(L_dc, E_k) and dP/d(eta_i) for the four survival parameters.
-//  mode FIT_OSC_EQ1:     eta = (sin^2 2th13, dm2_ee, sin^2 2th12, dm2_21), Eq. 1
-//  mode FIT_OSC_VACUUM3: eta = (sin^2 th12, sin^2 th13, dm2_21, dm2_31), exact vacuum P
-// eta_lo carries the low parts of the two mass splittings; dx = pi c (dx/d dm2).
-__device__ __forceinline__ float survival_mode(int mode, const float (&eta)[4],
-                                               const float (&eta_lo)[4], const OscCoef &k,
-                                               float c_hi, float c_lo, float (&dP)[4]) {
-    const float dx = 3.14159265358979f * c_hi;
-    if (mode == FIT_OSC_EQ1) {
-        const float S13 = eta[0], S12 = eta[2];
-        const float root = sqrtf(fmaxf(1.f - S13, 1e-12f));
-        const float c2 = 0.5f * (1.f + root);
-        const float c4 = c2 * c2;
-        float se, ce, s2, cc2;
-        phase_sc(eta[1], eta_lo[1], c_hi, c_lo, se, ce);
-        phase_sc(eta[3], eta_lo[3], c_hi, c_lo, s2, cc2);
-        const float qe = se * se, q21 = s2 * s2;
-        const float P = (1.f - cterm(k, 0, qe)) - cterm(k, 1, q21);
-        const float dc4 = -c2 * 0.5f / root;
-        dP[0] = -qe - dc4 * S12 * q21;
-        dP[1] = -S13 * 2.f * se * ce * dx;
-        dP[2] = -c4 * q21;
-        dP[3] = -c4 * S12 * 2.f * s2 * cc2 * dx;
-        return P;
-    } else {
-        const float s12 = eta[0], s13 = eta[1];
-        const float c12 = 1.f - s12, c13 = 1.f - s13;
-        const float S12 = 4.f * s12 * c12, S13 = 4.f * s13 * c13;
-        float a21, b21, a31, b31;
-        phase_sc(eta[2], eta_lo[2], c_hi, c_lo, a21, b21);
-        phase_sc(eta[3], eta_lo[3], c_hi, c_lo, a31, b31);
-        const float a32 = a31 * b21 - b31 * a21;   // sin(x31 - x21)
-        const float b32 = b31 * b21 + a31 * a21;   // cos(x31 - x21)
-        const float q21 = a21 * a21, q31 = a31 * a31, q32 = a32 * a32;
-        const float d21 = 2.f * a21 * b21 * dx, d31 = 2.f * a31 * b31 * dx,
-                    d32 = 2.f * a32 * b32 * dx;
-        const float P = ((1.f - cterm(k, 0, q21)) - cterm(k, 1, q31)) - cterm(k, 2, q32);
-        dP[0] = -c13 * c13 * 4.f * (1.f - 2.f * s12) * q21 - S13 * (q32 - q31);
-        dP[1] = 2.f * c13 * S12 * q21 - 4.f * (1.f - 2.f * s13) * (c12 * q31 + s12 * q32);
-        dP[2] = -c13 * c13 * S12 * d21 + S13 * s12 * d32;
-        dP[3] = -S13 * (c12 * d31 + s12 * d32);
-        return P;
-    }
-}
-
-// The sin^2 coefficients of survival_mode from float pairs e of the exact parameter values.
+// The sin^2 coefficients of Eq. 1 and the three-flavour formula from float pairs e of the exact
+// parameter values.
 __device__ __forceinline__ OscCoef osc_coef(int mode, const F2 (&e)[4]) {
     F2 cf[3];
     if (mode == FIT_OSC_EQ1) {
@@ -354,12 +374,6 @@ __device__ __forceinline__ OscCoef osc_coef(int mode, const F2 (&e)[4]) {
         k.lo[i] = cf[i].l;
     }
     return k;
-}
-
-__device__ __forceinline__ float survival(const DevModel &m, const float (&eta)[4],
-                                          const float (&eta_lo)[4], const OscCoef &k,
-                                          float c_hi, float c_lo, float (&dP)[4]) {
-    return survival_mode(m.osc_mode, eta, eta_lo, k, c_hi, c_lo, dP);
 }
 
 // Exact 3+1 vacuum survival (FIT_OSC_STERILE4), one sterile state added to the three-flavour
@@ -433,34 +447,26 @@ __host__ __device__ __forceinline__ bool osc_is_dm(int mode, int i) {
     return mode == FIT_OSC_EQ1 ? (i == 1 || i == 3) : (i == 2 || i == 3 || i == 5);
 }
 
-// Survival of the formula with NOSC parameters: 4 (Eq. 1 or the three-flavour formula) or 6
-// (the 3+1 formula).
+// sin^2 coefficients for the formulas with 4 survival parameters (Eq. 1, three-flavour) or 6 (3+1)
 template <int NOSC>
 struct OscTraits;
 template <>
 struct OscTraits<4> {
     using Coef = OscCoefN<3>;
-    static __device__ __forceinline__ float survival(int mode, const float (&eta)[4], const float (&eta_lo)[4],
-                                                     const Coef &k, float c_hi, float c_lo, float (&dP)[4]) {
-        return survival_mode(mode, eta, eta_lo, k, c_hi, c_lo, dP);
-    }
     static __device__ __forceinline__ Coef coef(int mode, const F2 (&e)[4]) { return osc_coef(mode, e); }
 };
 template <>
 struct OscTraits<6> {
     using Coef = OscCoefN<6>;
-    static __device__ __forceinline__ float survival(int, const float (&eta)[6], const float (&eta_lo)[6],
-                                                     const Coef &k, float c_hi, float c_lo, float (&dP)[6]) {
-        return survival_sterile(eta, eta_lo, k, c_hi, c_lo, dP);
-    }
     static __device__ __forceinline__ Coef coef(int, const F2 (&e)[6]) { return osc_coef_sterile(e); }
 };
 
 // Poisson deviance 2[mu - n + n ln(n/mu)] = 2 mu h(r), r = (n - mu)/mu,
-// h(r) = (1+r) ln(1+r) - r, by its alternating series for |r| < 1/4.
-__device__ __forceinline__ float deviance(float n, float mu) {
+// h(r) = (1+r) ln(1+r) - r, by its alternating series for |r| < 1/4. diff: n - mu, which a caller
+// may hold more exactly than the rounded mu gives it.
+__device__ __forceinline__ float deviance(float n, float mu, float diff) {
     if (n == 0.f) return 2.f * mu;
-    const float r = (n - mu) / mu;
+    const float r = diff / mu;
     float h;
     if (fabsf(r) < 0.25f) {
         // h = sum_{j>=2} (-1)^j r^j / (j (j-1))
@@ -573,6 +579,36 @@ __device__ __forceinline__ void edge_bin(int e, float r, int N, int &k, float &t
     }
 }
 
+// The inverse images of the grid edges, found once per evaluation and read by the remap and its
+// adjoint (which look at five or six edges per bin): bin k and fraction t of x_e (see edge_bin),
+// k + kEdgeOff where x_e is off the grid, and r.
+constexpr int kEdgeOff = 1 << 16;
+struct EdgeTab {
+    int *k;
+    float *t, *r;
+};
+
+template <class Map>
+__device__ __forceinline__ void edge_store(const EdgeTab &T, const float *e_edge, const Map &em, int e, int N) {
+    const float r = edge_inv_r(e_edge, em, e);
+    int k;
+    float t;
+    bool in;
+    edge_bin(e, r, N, k, t, in);
+    T.k[e] = in ? k : k + kEdgeOff;
+    T.t[e] = t;
+    T.r[e] = r;
+}
+
+// v_j for target bin j
+__device__ __forceinline__ float spline_target(const float *u, const EdgeTab &T, int j, int N) {
+    const int k0 = T.k[j] & (kEdgeOff - 1), k1 = T.k[j + 1] & (kEdgeOff - 1);
+    float acc = 0.f;
+    #pragma unroll 1
+    for (int k = k0, it = 0; k < k1 && it < 64; ++k, ++it) acc += u[k];
+    return acc + (hermite_G(u, k1, T.t[j + 1], N) - hermite_G(u, k0, T.t[j], N));
+}
+
 // v_j for target bin j
 template <class Map>
 __device__ __forceinline__ float spline_target(const float *u, const float *e_edge, const Map &em, int j, int N) {
@@ -582,6 +618,7 @@ __device__ __forceinline__ float spline_target(const float *u, const float *e_ed
     edge_bin(j, edge_inv_r(e_edge, em, j), N, k0, t0, in0);
     edge_bin(j + 1, edge_inv_r(e_edge, em, j + 1), N, k1, t1, in1);
     float acc = 0.f;
+    #pragma unroll 1
     for (int k = k0, it = 0; k < k1 && it < 64; ++k, ++it) acc += u[k];
     return acc + (hermite_G(u, k1, t1, N) - hermite_G(u, k0, t0, N));
 }
@@ -590,22 +627,22 @@ __device__ __forceinline__ float spline_target(const float *u, const float *e_ed
 // weight of F(x_e) (gv outside the grid 0), dF(x_e)/du_i is 1 for i < k_e (the cumulative)
 // plus the Hermite weights of u_i in G_{k_e}; the cumulative part sums to gv_{e*-1}, e* the
 // first edge with k_e > i.
-template <class Map>
-__device__ __forceinline__ float spline_adjoint_source(const float *gv, const float *e_edge, const Map &em,
-                                                       int i, int N) {
+__device__ __forceinline__ float spline_adjoint_source(const float *gv, const EdgeTab &T, int i, int N) {
     auto kb = [&](int e, int &k, float &t) {
-        bool in;
-        edge_bin(e, edge_inv_r(e_edge, em, e), N, k, t, in);
+        k = T.k[e] & (kEdgeOff - 1);
+        t = T.t[e];
     };
     // e*: start from the inverse shift at edge i and walk to the first edge with k_e > i
-    int e = min(max(i + 1 - (int)floorf(edge_inv_r(e_edge, em, i)), 0), N + 1);
+    int e = min(max(i + 1 - (int)floorf(T.r[i]), 0), N + 1);
     int k;
     float t;
+    #pragma unroll 1
     for (int it = 0; it < 64 && e > 0; ++it) {   // step down while the edge before is past i
         kb(e - 1, k, t);
         if (k <= i) break;
         --e;
     }
+    #pragma unroll 1
     for (int it = 0; it < 64 && e <= N; ++it) {  // step up while this edge is not past i
         kb(e, k, t);
         if (k > i) break;
@@ -628,8 +665,10 @@ __device__ __forceinline__ float spline_adjoint_source(const float *gv, const fl
         g = fmaf(we, c, g);
         return true;
     };
+    #pragma unroll 1
     for (int ee = e - 1, it = 0; ee >= 0 && it < 64; --ee, ++it)
         if (!local(ee)) break;
+    #pragma unroll 1
     for (int ee = e, it = 0; ee <= N && it < 64; ++ee, ++it)
         if (!local(ee)) break;
     return g;
@@ -639,13 +678,10 @@ __device__ __forceinline__ float spline_adjoint_source(const float *gv, const fl
 // (f the spline's density per MeV, 0 off the grid); added to ep[0..2].
 template <class Map>
 __device__ __forceinline__ void spline_adjoint_edge(const float *u, const float *gv, const float *e_edge,
-                                                    const Map &em, int e, int N, float *ep) {
-    const float r = edge_inv_r(e_edge, em, e);
-    int k;
-    float t;
-    bool in;
-    edge_bin(e, r, N, k, t, in);
-    if (!in) return;
+                                                    const Map &em, const EdgeTab &T, int e, int N, float *ep) {
+    const int k = T.k[e];
+    if (k & kEdgeOff) return;
+    const float r = T.r[e], t = T.t[e];
     const float we = (e >= 1 ? gv[e - 1] : 0.f) - (e <= N - 1 ? gv[e] : 0.f);
     const float t2 = t * t;
     const float dG = fmaf(u[k], 6.f * (t - t2), fmaf(hermite_S(u, k, N), 3.f * t2 - 4.f * t + 1.f,
@@ -680,29 +716,43 @@ __device__ __forceinline__ EMap make_emap(const DevModel &m, const DevDataset &d
 // stage, and the warps that one dataset leaves over start on the next (each dataset's bins
 // begin at the warp where the previous dataset's ended).
 // ------------------------------------------------------------------------------------
-// Per-dataset workspace (floats), arrays of length N_t unless noted:
+// Per-dataset workspace (floats), arrays of N_t rounded up to 4 unless noted:
 //   u, v (-> gv), ts = t s, ptot, dp[n_osc] (dp[0] is reused for the shape gradient),
-//   pcw[C] = w_c P_c per core, f0[max_reco], gmu[max_reco]
+//   pcw[C] = w_c P_c per core, f0[max_reco], gmu[max_reco], and for the spline correction the
+//   edge table (three arrays of N_t + 1), for the overlap rule the displacements D(e_k) of the
+//   grid edges (N_t + 1, in edge.t). u is the signal, divided by the mapped width of
+//   its bin under the overlap rule (every use of it there is divided by that width).
 struct DsWs {
     float *u, *v, *ts, *ptot, *dp, *pcw, *f0, *gmu;
+    EdgeTab edge;
 };
 
-__host__ __device__ inline int eval_ws_floats(int N_t, int C, int max_reco, int n_osc) {
-    return ((4 + n_osc + C) * N_t + 2 * max_reco + 3) & ~3;
+__host__ __device__ inline int eval_ws_floats(int N_t, int C, int max_reco, int n_osc, int remap_mode) {
+    return (remap_mode == FIT_REMAP_SPLINE ? 3 : 1) * ((N_t + 4) & ~3) + (4 + n_osc + C) * ((N_t + 3) & ~3) + 2 * ((max_reco + 3) & ~3);
 }
 
 __device__ __forceinline__ DsWs carve_ds_ws(float *base, int N_t, int C, int max_reco, int n_osc) {
+    const int N4 = (N_t + 3) & ~3;
     DsWs w;
     w.u = base;
-    w.v = w.u + N_t;
-    w.ts = w.v + N_t;
-    w.ptot = w.ts + N_t;
-    w.dp = w.ptot + N_t;          // n_osc * N_t
-    w.pcw = w.dp + n_osc * N_t;   // C * N_t
-    w.f0 = w.pcw + C * N_t;       // max_reco
-    w.gmu = w.f0 + max_reco;      // max_reco
+    w.v = w.u + N4;
+    w.ts = w.v + N4;
+    w.ptot = w.ts + N4;
+    w.dp = w.ptot + N4;          // n_osc arrays (pitch N_t)
+    w.pcw = w.dp + n_osc * N4;   // C arrays (pitch N_t)
+    w.f0 = w.pcw + C * N4;       // max_reco
+    w.gmu = w.f0 + ((max_reco + 3) & ~3);
+    w.edge.t = w.gmu + ((max_reco + 3) & ~3);
+    w.edge.r = w.edge.t + ((N_t + 4) & ~3);
+    w.edge.k = reinterpret_cast<int *>(w.edge.r + ((N_t + 4) & ~3));
     return w;
 }
+
+// Two cores of a dataset: K L / pi (pair), flux share w, w p high and low part. A core that is not
+// seen, or past the last one, has all of them 0: probability 1, weight 0.
+struct alignas(16) CorePair {
+    f32x2 klh, kll, w, wp, wpl, pad;
+};
 
 // Shared state of one evaluation (one per block).
 struct EvalShared {
@@ -710,7 +760,8 @@ struct EvalShared {
     float eta[kMaxOsc], eta_lo[kMaxOsc];
     PP nrm[FIT_MAX_DATASETS], eff[FIT_MAX_DATASETS];
     EMap em[FIT_MAX_DATASETS];
-    PP power[FIT_MAX_CORES], rate[FIT_MAX_BACKGROUNDS];
+    PP rate[FIT_MAX_BACKGROUNDS];
+    CorePair core[FIT_MAX_DATASETS][(FIT_MAX_CORES + 1) / 2];   // of the group's datasets
     int dl[FIT_MAX_DATASETS];               // datasets of the current group
     int n;                                  // their number
     int bad;                                // 1: the dataset after them has an invalid energy map
@@ -781,8 +832,10 @@ static __device__ int eval_setup(const DevModel &m, EvalShared &E, const ParVecs
                 h = p >= 0 ? q.pv[p] : m.osc_val[lane];
                 l = 0.f;
             }
-            E.eta[lane] = h;
-            E.eta_lo[lane] = l;
+            // (normalised: the reduced phase must stay within a half)
+            const F2 n = f2_norm(h, l);
+            E.eta[lane] = n.h;
+            E.eta_lo[lane] = n.l;
         }
         // the sin^2 coefficients from float pairs of the exact parameter values
         F2 e[NOSC];
@@ -799,61 +852,186 @@ static __device__ int eval_setup(const DevModel &m, EvalShared &E, const ParVecs
                 E.kc.lo[i] = k.lo[i];
             }
         }
-    } else if (warp == 1) {
-        if (lane >= 16 && lane - 16 < m.C) E.power[lane - 16] = ppair(q, m.core_power_idx[lane - 16], 1.f);
+    }
+    // (every thread reads the mask itself: dataset number i of the group for core slots 16 i + c)
+#pragma unroll 1
+    for (int e = tid; e < 16 * group; e += blockDim.x) {
+        const int c = e & 15;
+        int d = first, left = e >> 4;
+        while (d < m.n_ds && !(((mask >> d) & 1u) && left-- == 0)) ++d;
+        if (d >= m.n_ds || c >= ((m.C + 1) & ~1)) continue;
+        const DevDataset &ds = m.ds[d];
+        const float w = c < m.C ? ds.w[c] : 0.f;
+        const PP p = w != 0.f ? ppair(q, m.core_power_idx[c], 1.f) : PP{0.f, 0.f};
+        const float wp = w * p.h;
+        float *k = reinterpret_cast<float *>(&E.core[e >> 4][c >> 1]) + (c & 1);
+        k[0] = w != 0.f ? ds.kl_hi[c] : 0.f;
+        k[2] = w != 0.f ? ds.kl_lo[c] : 0.f;
+        k[4] = w;
+        k[6] = wp;
+        k[8] = fmaf(w, p.l, fmaf(w, p.h, -wp));
     }
     if (warp == (int)(blockDim.x >> 5) - 1 && lane < m.n_bkg) E.rate[lane] = ppair(q, m.bkg[lane].rate_idx, 1.f);
     __syncthreads();
     return next;
 }
 
-// Stage A: u_k (and with DERIV the per-bin partials the adjoint needs). Ends with a barrier.
+// The survival sums of one true bin over the cores: pt = sum_c p_c w_c P_c, its derivatives dpt by
+// the survival parameters, and corr, the part of the sum below FP32's rounding of P (the low
+// parts of the sin^2 coefficients and of p_c w_c), which a caller adds where it still counts.
+//
+// Eq. 1 and the three-flavour formula are linear in sin^2 x_i, and their derivatives in sin^2 x_i
+// and sin 2 x_i, with coefficients that no bin or core changes. So the loop over the cores sums
+// p w sin^2 x_i and p w c sin x_i cos x_i, and the derivatives are formed once per bin: about 70
+// instructions per bin and core instead of 125 with each core's derivatives in full (the 53 km
+// model's signal stage: 60 200 cycles of 512 threads before).
+//
+// Two cores at a time in packed FP32 (f32x2): the packed instructions have no higher rate per FMA
+// here (37 against 37 T/s measured) but are half the instructions, and issue slots, not the FMA
+// units, are what this loop runs out of. The phase is taken negative (-y), which spares
+// negations: sin^2 and cos are even, the products sin cos change sign and get it back at the end.
 template <bool DERIV, int NOSC, int MODE>
+struct CoreSums {
+    static __device__ __forceinline__ void run(const EvalShared &E, int i, int C, float ih, float il, float *pcw,
+                                               int stride, float &pt, float &corr, float (&dpt)[NOSC]) {
+        constexpr int NT = MODE == FIT_OSC_EQ1 ? 2 : 3;
+        constexpr int D0 = MODE == FIT_OSC_EQ1 ? 1 : 2;   // index of the first mass splitting
+        const f32x2 one = pack2(1.f), m1 = pack2(-1.f), ih2 = pack2(ih), nih2 = pack2(-ih), il2 = pack2(il);
+        f32x2 Q[NT], H[NT], p2 = pack2(0.f), lo = p2, nC[NT];
+#pragma unroll
+        for (int j = 0; j < NT; ++j) {
+            Q[j] = H[j] = p2;
+            nC[j] = pack2(-E.kc.hi[j]);
+        }
+        const f32x2 ma = pack2(E.eta[D0]), nma = pack2(-E.eta[D0]), mal = pack2(E.eta_lo[D0]);
+        const f32x2 mb = pack2(E.eta[3]), nmb = pack2(-E.eta[3]), mbl = pack2(E.eta_lo[3]);
+#pragma unroll 1
+        for (int c = 0; c < C; c += 2) {
+            const CorePair &K = E.core[i][c >> 1];
+            const f32x2 klh = K.klh, kll = K.kll, wp = K.wp;
+            const f32x2 ch = mul2(klh, ih2), nch = mul2(klh, nih2);
+            const f32x2 cl = fma2(kll, ih2, fma2(klh, il2, fma2(klh, ih2, nch)));
+            f32x2 sa, ca, sb, cb, q[NT], h[NT];
+            sincos_half2(neg_phase2(ma, nma, mal, ch, cl, m1), sa, ca);
+            sincos_half2(neg_phase2(mb, nmb, mbl, ch, cl, m1), sb, cb);
+            q[0] = mul2(sa, sa);
+            q[1] = mul2(sb, sb);
+            if (DERIV) {
+                h[0] = mul2(sa, ca);
+                h[1] = mul2(sb, cb);
+            }
+            if constexpr (NT == 3) {   // x32 = x31 - x21
+                const f32x2 s2 = fma2(cb, mul2(sa, m1), mul2(sb, ca));
+                q[2] = mul2(s2, s2);
+                if (DERIV) h[2] = mul2(s2, fma2(sb, sa, mul2(cb, ca)));
+            }
+            f32x2 P = one;
+#pragma unroll
+            for (int j = 0; j < NT; ++j) P = fma2(nC[j], q[j], P);
+            if (DERIV) {
+                const float2 w = unpack2(mul2(K.w, P));
+                pcw[c * stride] = w.x;
+                if (c + 1 < C) pcw[(c + 1) * stride] = w.y;
+            }
+            p2 = fma2(P, wp, p2);
+            lo = fma2(P, K.wpl, lo);
+            const f32x2 wc = mul2(wp, ch);
+#pragma unroll
+            for (int j = 0; j < NT; ++j) {
+                Q[j] = fma2(wp, q[j], Q[j]);
+                if (DERIV) H[j] = fma2(wc, h[j], H[j]);
+            }
+        }
+        auto total = [](f32x2 v) {
+            const float2 t = unpack2(v);
+            return t.x + t.y;
+        };
+        {   // the two cores' halves, the rounding of their sum into the correction
+            const float2 t = unpack2(p2);
+            pt = t.x + t.y;
+            const float bb = pt - t.x;
+            corr = total(lo) + ((t.x - (pt - bb)) + (t.y - bb));
+        }
+        float Qs[NT], Hs[NT];
+#pragma unroll
+        for (int j = 0; j < NT; ++j) {
+            Qs[j] = total(Q[j]);
+            corr = fmaf(-E.kc.lo[j], Qs[j], corr);
+            if (DERIV) Hs[j] = total(H[j]);
+        }
+        if constexpr (!DERIV) return;
+        constexpr float k2pi = -6.28318531f;   // d sin^2 x / d dm2 = 2 sin x cos x dx / d dm2, dx = pi c
+        if constexpr (MODE == FIT_OSC_EQ1) {
+            const float S13 = E.eta[0], S12 = E.eta[2];
+            const float root = sqrtf(fmaxf(1.f - S13, 1e-12f)), c2 = 0.5f * (1.f + root);
+            const float dc4 = -c2 * 0.5f / root;
+            dpt[0] = -Qs[0] - dc4 * S12 * Qs[1];
+            dpt[1] = -S13 * (k2pi * Hs[0]);
+            dpt[2] = -c2 * c2 * Qs[1];
+            dpt[3] = -c2 * c2 * S12 * (k2pi * Hs[1]);
+        } else {
+            const float s12 = E.eta[0], s13 = E.eta[1], c12 = 1.f - s12, c13 = 1.f - s13;
+            const float S12 = 4.f * s12 * c12, S13 = 4.f * s13 * c13;
+            dpt[0] = -c13 * c13 * 4.f * (1.f - 2.f * s12) * Qs[0] - S13 * (Qs[2] - Qs[1]);
+            dpt[1] = 2.f * c13 * S12 * Qs[0] - 4.f * (1.f - 2.f * s13) * (c12 * Qs[1] + s12 * Qs[2]);
+            dpt[2] = k2pi * (S13 * s12 * Hs[2] - c13 * c13 * S12 * Hs[0]);
+            dpt[3] = -S13 * (k2pi * (c12 * Hs[1] + s12 * Hs[2]));
+        }
+    }
+};
+
+// The 3+1 formula: each core's probability and derivatives in full.
+template <bool DERIV>
+struct CoreSums<DERIV, 6, FIT_OSC_STERILE4> {
+    static __device__ __forceinline__ void run(const EvalShared &E, int i, int C, float ih, float il, float *pcw,
+                                               int stride, float &pt, float &corr, float (&dpt)[6]) {
+        float eta[6], eta_lo[6];
+#pragma unroll
+        for (int j = 0; j < 6; ++j) {
+            eta[j] = E.eta[j];
+            eta_lo[j] = E.eta_lo[j];
+            dpt[j] = 0.f;
+        }
+        pt = corr = 0.f;
+        for (int c = 0; c < C; ++c) {
+            const float *k = reinterpret_cast<const float *>(&E.core[i][c >> 1]) + (c & 1);
+            const float klh = k[0], kll = k[2], w = k[4], wp = k[6], wpl = k[8];
+            const float ch = klh * ih;
+            const float cl = fmaf(kll, ih, fmaf(klh, il, fmaf(klh, ih, -ch)));
+            float dP[6];
+            const float P = survival_sterile(eta, eta_lo, E.kc, ch, cl, dP);
+            if (DERIV) pcw[c * stride] = w * P;
+            pt = fmaf(P, wp, pt);
+            corr = fmaf(P, wpl, corr);
+            if (DERIV) {
+#pragma unroll
+                for (int j = 0; j < 6; ++j) dpt[j] = fmaf(wp, dP[j], dpt[j]);
+            }
+        }
+    }
+};
+
+// Stage A: u_k (and with DERIV the per-bin partials the adjoint needs), and the spline's edge table.
+// Ends with a barrier.
+template <bool DERIV, int NOSC, int MODE, bool GEN>
 static __device__ __forceinline__ void st_signal_mode(const DevModel &m, const EvalShared &E, const ParVecs &q,
                                                       float *wsb) {
-    const int N_t = m.N_t, C = m.C, nth = blockDim.x;
-    typename OscTraits<NOSC>::Coef kc;
-#pragma unroll
-    for (int i = 0; i < (int)(sizeof(kc.hi) / sizeof(float)); ++i) {
-        kc.hi[i] = E.kc.hi[i];
-        kc.lo[i] = E.kc.lo[i];
-    }
-    float eta[NOSC], eta_lo[NOSC];
-#pragma unroll
-    for (int i = 0; i < NOSC; ++i) {
-        eta[i] = E.eta[i];
-        eta_lo[i] = E.eta_lo[i];
-    }
+    const int N_t = m.N_t, nth = blockDim.x;
+    const bool spline = GEN && m.remap_mode == FIT_REMAP_SPLINE;
+    #pragma unroll 1
     for (int i = 0; i < E.n; ++i) {
         const DevDataset &ds = m.ds[E.dl[i]];
-        const DsWs ws = carve_ds_ws(wsb + (int64_t)i * m.ws_eval_floats, N_t, C, m.max_reco, m.n_osc);
+        const DsWs ws = carve_ds_ws(wsb + (int64_t)i * m.ws_eval_floats, N_t, m.C, m.max_reco, m.n_osc);
         const PP nrm = E.nrm[i];
+        const EMap em = E.em[i];
+        #pragma unroll 1
         for (int k = rot_tid(i, (N_t + 31) >> 5); k < N_t; k += nth) {
             const float ih = m.inv_e_hi[k], il = m.inv_e_lo[k];
+            const float e0 = m.e_edge[k], e1 = m.e_edge[k + 1];
             const int sp = ds.shape_idx[k];
             const float tk = ds.t[k];
-            float pt = 0.f, dpt[NOSC];
-#pragma unroll
-            for (int j = 0; j < NOSC; ++j) dpt[j] = 0.f;
-            for (int c = 0; c < C; ++c) {
-                const float w = ds.w[c];
-                if (w == 0.f) {
-                    if (DERIV) ws.pcw[c * N_t + k] = 0.f;
-                    continue;
-                }
-                const float ch = ds.kl_hi[c] * ih;
-                const float cl = fmaf(ds.kl_hi[c], ih, -ch) + ds.kl_hi[c] * il + ds.kl_lo[c] * ih;
-                float dP[NOSC];
-                const float P = OscTraits<NOSC>::survival(MODE, eta, eta_lo, kc, ch, cl, dP);
-                const PP pw = E.power[c];
-                const float wP = w * P;
-                if (DERIV) ws.pcw[c * N_t + k] = wP;
-                pt += pmul(pw, wP);
-                if (DERIV) {
-#pragma unroll
-                    for (int j = 0; j < NOSC; ++j) dpt[j] = fmaf(pw.h * w, dP[j], dpt[j]);
-                }
-            }
+            float pt, corr, dpt[NOSC];
+            CoreSums<DERIV, NOSC, MODE>::run(E, i, m.C, ih, il, ws.pcw + k, N_t, pt, corr, dpt);
             const float ts = pmul(ppair(q, sp, 1.f), tk);
             if (DERIV) {
                 ws.ts[k] = ts;
@@ -861,7 +1039,18 @@ static __device__ __forceinline__ void st_signal_mode(const DevModel &m, const E
 #pragma unroll
                 for (int j = 0; j < NOSC; ++j) ws.dp[j * N_t + k] = dpt[j];
             }
-            ws.u[k] = pmul(nrm, ts * pt);
+            // (ts pt + ts corr in one rounding: the correction is below pt's last bit)
+            const float u = pmul(nrm, fmaf(ts, pt, ts * corr));
+            if (spline) {
+                ws.u[k] = u;
+                edge_store(ws.edge, m.e_edge, em, k, N_t);
+                if (k == N_t - 1) edge_store(ws.edge, m.e_edge, em, N_t, N_t);
+            } else {
+                const float d0 = em.disp(e0), d1 = em.disp(e1);
+                ws.u[k] = u / (1.f + (d1 - d0));
+                ws.edge.t[k] = d0;
+                if (k == N_t - 1) ws.edge.t[N_t] = d1;
+            }
         }
     }
     __syncthreads();
@@ -871,34 +1060,34 @@ static __device__ __forceinline__ void st_signal_mode(const DevModel &m, const E
 template <bool DERIV, bool GEN>
 static __device__ __forceinline__ void st_signal(const DevModel &m, const EvalShared &E, const ParVecs &q, float *wsb) {
     if (GEN && m.osc_mode == FIT_OSC_STERILE4)
-        st_signal_mode<DERIV, 6, FIT_OSC_STERILE4>(m, E, q, wsb);
+        st_signal_mode<DERIV, 6, FIT_OSC_STERILE4, GEN>(m, E, q, wsb);
     else if (m.osc_mode == FIT_OSC_EQ1)
-        st_signal_mode<DERIV, 4, FIT_OSC_EQ1>(m, E, q, wsb);
+        st_signal_mode<DERIV, 4, FIT_OSC_EQ1, GEN>(m, E, q, wsb);
     else
-        st_signal_mode<DERIV, 4, FIT_OSC_VACUUM3>(m, E, q, wsb);
+        st_signal_mode<DERIV, 4, FIT_OSC_VACUUM3, GEN>(m, E, q, wsb);
 }
 
-// Corrected content of target bin t under the overlap rule. Source bin k covers [Y_k, Y_k+1] in
+// Corrected content of target bin t under the overlap rule, from the sources' contents per mapped
+// width u. Source bin k covers [Y_k, Y_k+1] in
 // grid units, Y_k = k + D(e_k); target t gathers the sources whose mapped interval overlaps
 // [t, t+1]; overlaps are computed relative to the target (k - t is an exact small integer),
 // which keeps them accurate in FP32.
-__device__ __forceinline__ float overlap_target(const float *u, const float *e_edge, const EMap &em, int t, int N_t) {
-    // first source whose mapped upper edge lies above t: start from the fixed point
-    // k ~ t - D(k) and step until the bracket is right
-    int k = t - (int)floorf(em.disp(e_edge[t]));
-    k = min(max(k, 0), N_t - 1);
-    k = t - (int)floorf(em.disp(e_edge[k]));
-    k = min(max(k - 1, 0), N_t - 1);
-    while (k > 0 && (float)(k - t) + em.disp(e_edge[k]) > 0.f) --k;
+__device__ __forceinline__ float overlap_target(const float *u, const float *D, int t, int N_t) {
+    // first source whose mapped upper edge lies above t: from k ~ t - D(t), stepping down until the
+    // bracket is right
+    int k = min(max(t - (int)floorf(D[t]) - 1, 0), N_t - 1);
+    float dlo = D[k];
+#pragma unroll 1
+    while (k > 0 && (float)(k - t) + dlo > 0.f) dlo = D[--k];
     float acc = 0.f;
-    float dlo = em.disp(e_edge[k]);
+#pragma unroll 1
     for (int it = 0; it < 64 && k < N_t; ++it, ++k) {
-        const float dhi = em.disp(e_edge[k + 1]);
+        const float dhi = D[k + 1];
         const float ylo = (float)(k - t) + dlo;      // mapped edges relative to target t
         const float yhi = (float)(k + 1 - t) + dhi;
         if (ylo >= 1.f) break;
         const float ov = fminf(yhi, 1.f) - fmaxf(ylo, 0.f);
-        if (ov > 0.f) acc = fmaf(u[k], ov / (1.f + (dhi - dlo)), acc);
+        if (ov > 0.f) acc = fmaf(u[k], ov, acc);
         dlo = dhi;
     }
     return acc;
@@ -909,62 +1098,113 @@ template <bool GEN>
 static __device__ __forceinline__ void st_remap(const DevModel &m, const EvalShared &E, float *wsb) {
     const int N_t = m.N_t, nth = blockDim.x;
     const bool spline = GEN && m.remap_mode == FIT_REMAP_SPLINE;
+    #pragma unroll 1
     for (int i = 0; i < E.n; ++i) {
         const DsWs ws = carve_ds_ws(wsb + (int64_t)i * m.ws_eval_floats, N_t, m.C, m.max_reco, m.n_osc);
         const EMap em = E.em[i];
+        #pragma unroll 1
         for (int t = rot_tid(i, (N_t + 31) >> 5); t < N_t; t += nth)
-            ws.v[t] = spline ? spline_target(ws.u, m.e_edge, em, t, N_t) : overlap_target(ws.u, m.e_edge, em, t, N_t);
+            ws.v[t] = spline ? spline_target(ws.u, ws.edge, t, N_t) : overlap_target(ws.u, ws.edge.t, t, N_t);
     }
     __syncthreads();
 }
 
-// Stage C: fold into reco bins, f0 = R v (before the efficiency), banded rows. Each warp takes
-// four rows at a time and two strides of each, so eight independent load/FMA chains per lane
-// are in flight. Ends with a barrier.
-static __device__ __forceinline__ void st_fold(const DevModel &m, const EvalShared &E, float *wsb) {
-    const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    for (int i = 0; i < E.n; ++i) {
-        const DevDataset &ds = m.ds[E.dl[i]];
-        const DevDetector &dt = m.det[ds.det];
-        const DsWs ws = carve_ds_ws(wsb + (int64_t)i * m.ws_eval_floats, m.N_t, m.C, m.max_reco, m.n_osc);
-        const int nr = ds.n_reco;
-        for (int j0 = rot_tid(i, nr) >> 5; j0 < nr; j0 += 4 * nw) {
-            int lo[4], len[4];
-            const float *rr[4];
-            int lmax = 0;
+// out[4 g + e] (+ lo) = sum of a banded row times x, for warp units w0, w0 + nw, ... of U. One 16-byte
+// load of the matrix and one x serve four products, eight loads in flight: the response comes
+// from L2 (0.9 MB for the 53 km model's two detectors), and what counts besides bytes in flight
+// is instructions: a warp per row with its tree and addresses took 50 000 of the 358 000 warp
+// instructions of an evaluation there, this 9 000. The sum over the lanes of an output
+// group keeps its rounding errors (two-sums; into lo when it is not null).
+__device__ __forceinline__ void band_product(const BandUnits &U, const float *x, int w0, int nw, PP scale, float *out,
+                                             float *lo) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll 1
+    for (int w = w0; w < U.n; w += nw) {
+        const int2 st = U.steps[w];
+        const float *xs = x + U.start[w * 32 + lane];
+        const float4 *r = U.entry + st.x + lane;
+        float a[4] = {0.f, 0.f, 0.f, 0.f}, b[4] = {0.f, 0.f, 0.f, 0.f};
+        int k = 0;
+#pragma unroll 1
+        for (; k + 8 <= st.y; k += 8, r += 256, xs += 8) {
+            float4 q[8];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int j = j0 + u * nw;
-                const bool on = j < nr;
-                lo[u] = on ? dt.row_lo[j] : 0;
-                len[u] = on ? dt.row_len[j] : 0;
-                rr[u] = dt.rrow + (on ? dt.row_off[j] : 0);
-                lmax = max(lmax, len[u]);
+            for (int u = 0; u < 8; ++u) q[u] = r[32 * u];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const float v = xs[u];
+                float (&t)[4] = (u & 1) ? b : a;
+                t[0] = fmaf(q[u].x, v, t[0]);
+                t[1] = fmaf(q[u].y, v, t[1]);
+                t[2] = fmaf(q[u].z, v, t[2]);
+                t[3] = fmaf(q[u].w, v, t[3]);
             }
-            float s[4][2] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
-            for (int b = lane; b < lmax; b += 64) {
+        }
+#pragma unroll 1
+        for (; k < st.y; ++k, r += 32, ++xs) {
+            const float4 q = *r;
+            const float v = *xs;
+            a[0] = fmaf(q.x, v, a[0]);
+            a[1] = fmaf(q.y, v, a[1]);
+            a[2] = fmaf(q.z, v, a[2]);
+            a[3] = fmaf(q.w, v, a[3]);
+        }
+        float h[4], l[4];
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    if (b < len[u]) s[u][0] = fmaf(rr[u][b], ws.v[lo[u] + b], s[u][0]);
-                    if (b + 32 < len[u]) s[u][1] = fmaf(rr[u][b + 32], ws.v[lo[u] + b + 32], s[u][1]);
+        for (int e = 0; e < 4; ++e) {
+            h[e] = a[e] + b[e];
+            const float bb = h[e] - a[e];
+            l[e] = (a[e] - (h[e] - bb)) + (b[e] - bb);
+        }
+#pragma unroll 1
+        for (int o = U.parts >> 1; o > 0; o >>= 1) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const float g = __shfl_xor_sync(0xffffffffu, h[e], o), gl = __shfl_xor_sync(0xffffffffu, l[e], o);
+                const float t = h[e] + g, bb = t - h[e];
+                l[e] = (l[e] + gl) + ((h[e] - (t - bb)) + (g - bb));
+                h[e] = t;
+            }
+        }
+        const int x0 = w * 32 + lane;
+        if ((x0 & (U.parts - 1)) == 0) {
+            const int g = 4 * (x0 / U.parts);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                if (g + e >= U.outs) break;
+                if (lo) {
+                    out[g + e] = h[e];
+                    lo[g + e] = l[e];
+                } else {
+                    out[g + e] = pmul(scale, h[e]);
                 }
             }
-            float t[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) t[u] = s[u][0] + s[u][1];
-            const float tot = warp_sum_split<4>(t);
-            const int j = j0 + (lane >> 3) * nw;
-            if ((lane & 7) == 0 && j < nr) ws.f0[j] = tot;
         }
+    }
+}
+
+// Stage C: fold into reco bins, f0 = R v (before the efficiency), banded rows. The sums are float
+// pairs (low parts in gmu until st_lik): a bin's dD/dmu = 2 (mu - n) / mu is the difference of
+// near equals, so the last bits of mu are what the gradient near a minimum is made of. Ends with
+// a barrier.
+static __device__ __forceinline__ void st_fold(const DevModel &m, const EvalShared &E, float *wsb) {
+    const int nw = blockDim.x >> 5;
+#pragma unroll 1
+    for (int i = 0; i < E.n; ++i) {
+        const BandUnits &U = m.det[m.ds[E.dl[i]].det].fold;
+        const DsWs ws = carve_ds_ws(wsb + (int64_t)i * m.ws_eval_floats, m.N_t, m.C, m.max_reco, m.n_osc);
+        band_product(U, ws.v, rot_tid(i, U.n) >> 5, nw, PP{1.f, 0.f}, ws.f0, ws.gmu);
     }
     __syncthreads();
 }
 
-// Expected counts of one bin: efficiency x fold + backgrounds; tm / sh receive the templates and
-// 1 + delta of the dataset's backgrounds (the loads of all of them in flight together).
+// Expected counts of one bin as sig + rest: sig the efficiency x fold, rest what its rounding left out
+// and the backgrounds, so that a caller can form mu - n = (sig - n) + rest without rounding at the
+// size of mu (fold pair f0 + f1). tm / sh receive the templates and 1 + delta of the dataset's
+// backgrounds (the loads of all of them in flight together).
 __device__ __forceinline__ float bin_mu(const DevModel &m, const EvalShared &E, int i, const DevDataset &ds,
-                                        const ParVecs &q, float f0, int j, int nb, float (&tm)[kMaxBkgDs],
-                                        float (&sh)[kMaxBkgDs]) {
+                                        const ParVecs &q, float f0, float f1, int j, int nb, float (&tm)[kMaxBkgDs],
+                                        float (&sh)[kMaxBkgDs], float &rest) {
     int si[kMaxBkgDs];
 #pragma unroll
     for (int b = 0; b < kMaxBkgDs; ++b) {
@@ -972,27 +1212,35 @@ __device__ __forceinline__ float bin_mu(const DevModel &m, const EvalShared &E, 
         tm[b] = b < nb ? bk.tmpl[j] : 0.f;
         si[b] = b < nb ? bk.shape_idx[j] : -1;
     }
-    float mu = pmul(E.eff[i], f0);
+    const PP eff = E.eff[i];
+    const float sig = f0 * eff.h;
+    const float low = fmaf(f1, eff.h, fmaf(f0, eff.l, fmaf(f0, eff.h, -sig)));
+    float bg = 0.f;
 #pragma unroll
     for (int b = 0; b < kMaxBkgDs; ++b) {
         if (b >= nb) break;
         const float del = si[b] >= 0 ? q.pv[si[b]] : 0.f;
         sh[b] = 1.f + del;
-        mu += pmul(E.rate[ds.bkg_begin + b], fmaf(tm[b], del, tm[b]));
+        bg += pmul(E.rate[ds.bkg_begin + b], fmaf(tm[b], del, tm[b]));
     }
-    return mu;
+    rest = bg + low;
+    return sig;
 }
 
 // Expected counts of the group's datasets into mu (the whole data vector). Ends with a barrier.
 static __device__ __forceinline__ void st_mu(const DevModel &m, const EvalShared &E, const ParVecs &q, float *wsb,
                                              float *mu) {
     const int nth = blockDim.x;
+    #pragma unroll 1
     for (int i = 0; i < E.n; ++i) {
         const DevDataset &ds = m.ds[E.dl[i]];
         const DsWs ws = carve_ds_ws(wsb + (int64_t)i * m.ws_eval_floats, m.N_t, m.C, m.max_reco, m.n_osc);
+        #pragma unroll 1
         for (int j = rot_tid(i, (ds.n_reco + 31) >> 5); j < ds.n_reco; j += nth) {
             float tm[kMaxBkgDs], sh[kMaxBkgDs];
-            mu[ds.data_off + j] = bin_mu(m, E, i, ds, q, ws.f0[j], j, ds.bkg_end - ds.bkg_begin, tm, sh);
+            float rest;
+            const float sig = bin_mu(m, E, i, ds, q, ws.f0[j], ws.gmu[j], j, ds.bkg_end - ds.bkg_begin, tm, sh, rest);
+            mu[ds.data_off + j] = sig + rest;
         }
     }
     __syncthreads();
@@ -1005,6 +1253,7 @@ template <bool GRAD>
 static __device__ __forceinline__ void st_lik(const DevModel &m, EvalShared &E, const ParVecs &q, const float *data,
                                               float *wsb) {
     const int nth = blockDim.x, lane = threadIdx.x & 31;
+    #pragma unroll 1
     for (int i = 0; i < E.n; ++i) {
         const DevDataset &ds = m.ds[E.dl[i]];
         const DsWs ws = carve_ds_ws(wsb + (int64_t)i * m.ws_eval_floats, m.N_t, m.C, m.max_reco, m.n_osc);
@@ -1014,16 +1263,18 @@ static __device__ __forceinline__ void st_lik(const DevModel &m, EvalShared &E, 
         float part[8];   // deviance, d/d eff, d/d rate_b
 #pragma unroll
         for (int b = 0; b < 8; ++b) part[b] = 0.f;
+        #pragma unroll 1
         for (int j = t0; j < nr; j += nth) {
             const float n = data[ds.data_off + j], f0 = ws.f0[j];
-            float tm[kMaxBkgDs], sh[kMaxBkgDs];
-            const float mu = bin_mu(m, E, i, ds, q, f0, j, nb, tm, sh);
+            float tm[kMaxBkgDs], sh[kMaxBkgDs], rest;
+            const float sig = bin_mu(m, E, i, ds, q, f0, ws.gmu[j], j, nb, tm, sh, rest);
+            const float mu = sig + rest, diff = (sig - n) + rest;   // mu - n
             if (!(mu > 0.f)) {
                 atomicOr(&E.status, kStMuNonpos);
                 continue;
             }
-            part[0] += deviance(n, mu);
-            const float g = 2.f * (mu - n) / mu;
+            part[0] += deviance(n, mu, -diff);
+            const float g = 2.f * diff / mu;
             ws.gmu[j] = g;
             if (GRAD) {
                 part[1] = fmaf(g, f0, part[1]);
@@ -1048,6 +1299,7 @@ static __device__ __forceinline__ void st_lik(const DevModel &m, EvalShared &E, 
 // on as many warps as they need.
 __device__ __forceinline__ double quad_total(const float *p, int stride, int n, int sub) {
     double s = 0.0;
+    #pragma unroll 1
     for (int w = sub; w < n; w += 4) s += (double)p[w * stride];
     s += __shfl_xor_sync(0xffffffffu, s, 1);
     s += __shfl_xor_sync(0xffffffffu, s, 2);
@@ -1060,6 +1312,7 @@ __device__ __forceinline__ double quad_total(const float *p, int stride, int n, 
 template <bool GRAD>
 static __device__ __forceinline__ void lik_finish(const DevModel &m, EvalShared &E, float *grad) {
     const int nw = blockDim.x >> 5, sub = threadIdx.x & 3;
+    #pragma unroll 1
     for (int v0 = 0; v0 < 8 * E.n; v0 += blockDim.x >> 2) {
         const int v = v0 + (int)(threadIdx.x >> 2), i = v >> 3, q = v & 7;
         if ((v & ~7) >= 8 * E.n) break;   // uniform over the warp
@@ -1083,11 +1336,14 @@ static __device__ __forceinline__ void lik_finish(const DevModel &m, EvalShared 
 // in E.dup, in order.
 static __device__ __forceinline__ void lik_dups(const DevModel &m, EvalShared &E, float *grad) {
     double nll = E.nll;
+    #pragma unroll 1
     for (int i = 0; i < E.n; ++i) nll += E.nll_ds[i];
     E.nll = nll;
     if (grad == nullptr) return;
+    #pragma unroll 1
     for (int i = 0; i < E.n; ++i) {
         const DevDataset &ds = m.ds[E.dl[i]];
+        #pragma unroll 1
         for (int left = ds.lik_dup; left; left &= left - 1) {
             const int q = __ffs(left) - 1;
             const int p = q == 1 ? ds.eff_idx : m.bkg[ds.bkg_begin + q - 2].rate_idx;
@@ -1099,10 +1355,13 @@ static __device__ __forceinline__ void lik_dups(const DevModel &m, EvalShared &E
 // Background-shape gradient: a thread per shape parameter sums its (background, bin) pairs of
 // the group's datasets in a fixed order (several datasets may share a shape).
 static __device__ __forceinline__ void st_bkg_shape(const DevModel &m, const EvalShared &E, float *wsb, float *grad) {
+    #pragma unroll 1
     for (int p = threadIdx.x; p < m.n_bs; p += blockDim.x) {
         float s = 0.f;
+        #pragma unroll 1
         for (int r = m.bs_ptr[p]; r < m.bs_ptr[p + 1]; ++r) {
             const BkgShapeRef ref = m.bs_ref[r];
+            #pragma unroll 1
             for (int i = 0; i < E.n; ++i) {
                 if (E.dl[i] != ref.d) continue;
                 const DsWs ws = carve_ds_ws(wsb + (int64_t)i * m.ws_eval_floats, m.N_t, m.C, m.max_reco, m.n_osc);
@@ -1113,33 +1372,15 @@ static __device__ __forceinline__ void st_bkg_shape(const DevModel &m, const Eva
     }
 }
 
-// Stage D: adjoint of the fold, v <- gv = eff R^T gmu (column bands). rcol is exactly 0 past each
-// column's band, so the loop runs the widest band of the warp's 32 adjacent columns (nearly
-// their own widths: the resolution changes slowly with energy) with the row index clamped (no
-// early exit) and four partial sums. No barrier.
+// Stage D: adjoint of the fold, v <- gv = eff R^T gmu. No barrier.
 static __device__ __forceinline__ void st_adjoint_fold(const DevModel &m, const EvalShared &E, float *wsb) {
-    const int N_t = m.N_t, nth = blockDim.x;
+    const int nw = blockDim.x >> 5;
+#pragma unroll 1
     for (int i = 0; i < E.n; ++i) {
-        const DevDataset &ds = m.ds[E.dl[i]];
-        const DevDetector &dt = m.det[ds.det];
-        const DsWs ws = carve_ds_ws(wsb + (int64_t)i * m.ws_eval_floats, N_t, m.C, m.max_reco, m.n_osc);
-        const int jmax = ds.n_reco - 1;
-        const PP eff = E.eff[i];
-        float *gv = ws.v;   // v is dead after the fold
-        for (int k = rot_tid(i, (N_t + 31) >> 5); k < N_t; k += nth) {
-            const int lo = dt.col_lo[k];
-            const int cw = __reduce_max_sync(__activemask(), dt.col_len[k]);
-            const float *rc = dt.rcol + k;
-            float s[4] = {0.f, 0.f, 0.f, 0.f};
-            int b = 0;
-            for (; b + 7 < cw; b += 8) {   // eight loads in flight
-#pragma unroll
-                for (int u = 0; u < 8; ++u)
-                    s[u & 3] = fmaf(rc[(int64_t)(b + u) * N_t], ws.gmu[min(lo + b + u, jmax)], s[u & 3]);
-            }
-            for (; b < cw; ++b) s[0] = fmaf(rc[(int64_t)b * N_t], ws.gmu[min(lo + b, jmax)], s[0]);
-            gv[k] = pmul(eff, (s[0] + s[1]) + (s[2] + s[3]));
-        }
+        const BandUnits &U = m.det[m.ds[E.dl[i]].det].adj;
+        const DsWs ws = carve_ds_ws(wsb + (int64_t)i * m.ws_eval_floats, m.N_t, m.C, m.max_reco, m.n_osc);
+        // (v is dead after the fold)
+        band_product(U, ws.gmu, rot_tid(i, U.n) >> 5, nw, E.eff[i], ws.v, nullptr);
     }
 }
 
@@ -1156,6 +1397,7 @@ static __device__ __forceinline__ void st_adjoint_rest_n(const DevModel &m, Eval
     for (int j = 0; j < NOSC; ++j) eo[j] = 0.f;
 #pragma unroll
     for (int c = 0; c < NC; ++c) ec[c] = 0.f;
+    #pragma unroll 1
     for (int i = 0; i < E.n; ++i) {
         const DevDataset &ds = m.ds[E.dl[i]];
         const DsWs ws = carve_ds_ws(wsb + (int64_t)i * m.ws_eval_floats, N_t, C, m.max_reco, m.n_osc);
@@ -1163,28 +1405,31 @@ static __device__ __forceinline__ void st_adjoint_rest_n(const DevModel &m, Eval
         const PP nrm = E.nrm[i];
         const float *gv = ws.v;
         float ep[4] = {0.f, 0.f, 0.f, 0.f};   // d/da0, d/da1, d/da2, d/d norm
+        #pragma unroll 1
         for (int k = rot_tid(i, (N_t + 31) >> 5); k < N_t; k += nth) {
             float gu = 0.f;
             if (spline) {
-                gu = spline_adjoint_source(gv, m.e_edge, em, k, N_t);
-                spline_adjoint_edge(ws.u, gv, m.e_edge, em, k, N_t, ep);
-                if (k == N_t - 1) spline_adjoint_edge(ws.u, gv, m.e_edge, em, N_t, N_t, ep);
+                gu = spline_adjoint_source(gv, ws.edge, k, N_t);
+                spline_adjoint_edge(ws.u, gv, m.e_edge, em, ws.edge, k, N_t, ep);
+                if (k == N_t - 1) spline_adjoint_edge(ws.u, gv, m.e_edge, em, ws.edge, N_t, N_t, ep);
             } else {
                 // per source k: gu = sum_t F_kt gv_t; A0 = (gu - gv(floor Y_k)) / w,
                 // A1 = (gv(floor Y_k+1) - gu) / w
                 const float e0 = m.e_edge[k], e1 = m.e_edge[k + 1];
-                const float d0 = em.disp(e0), d1 = em.disp(e1);
+                const float d0 = ws.edge.t[k], d1 = ws.edge.t[k + 1];
                 const float w = 1.f + (d1 - d0), iw = 1.f / w;
                 const int f0i = (int)floorf(d0), f1i = (int)floorf(d1);
                 const int t0 = k + f0i, t1 = k + 1 + f1i;
+                #pragma unroll 1
                 for (int t = max(t0, 0); t <= min(t1, N_t - 1); ++t) {
                     const float ylo = (float)(k - t) + d0, yhi = (float)(k + 1 - t) + d1;
                     const float ov = fminf(yhi, 1.f) - fmaxf(ylo, 0.f);
-                    if (ov > 0.f) gu = fmaf(ov * iw, gv[t], gu);
+                    if (ov > 0.f) gu = fmaf(ov, gv[t], gu);
                 }
+                gu *= iw;
                 const float g0 = (t0 >= 0 && t0 < N_t) ? gv[t0] : 0.f;
                 const float g1 = (t1 >= 0 && t1 < N_t) ? gv[t1] : 0.f;
-                const float uk = ws.u[k] * iw;
+                const float uk = ws.u[k];   // (already per mapped width)
                 const float A0 = uk * (gu - g0), A1 = uk * (g1 - gu);
                 ep[0] += (A0 + A1) * em.inv_de;
                 ep[1] += (A0 * e0 + A1 * e1) * em.inv_de;
@@ -1230,6 +1475,7 @@ static __device__ __forceinline__ void st_adjoint_finish(const DevModel &m, Eval
         // totals: four per dataset, then the survival parameters and powers; four lanes each,
         // from the last warp down (the shapes below start at the first)
         const int nmap = 4 * E.n, nv = nmap + NOSC + m.C, sub = tid & 3;
+        #pragma unroll 1
         for (int v0 = 0; v0 < nv; v0 += nth >> 2) {
             const int v = v0 + ((nth - 1 - tid) >> 2);
             if (v0 + (((nth - 1 - (tid | 31))) >> 2) >= nv) break;   // uniform over the warp
@@ -1252,6 +1498,7 @@ static __device__ __forceinline__ void st_adjoint_finish(const DevModel &m, Eval
     if (m.any_map_dup) {
         __syncthreads();
         if (tid == 0) {
+            #pragma unroll 1
             for (int v = 0; v < 4 * E.n + NOSC + m.C; ++v) {
                 const bool map = v < 4 * E.n;
                 const int q = map ? (v & 3) : v - 4 * E.n;
@@ -1262,18 +1509,25 @@ static __device__ __forceinline__ void st_adjoint_finish(const DevModel &m, Eval
         }
     }
     if (m.shared_roles) __syncthreads();
+    #pragma unroll 1
     for (int i = 0; i < E.n; ++i) {
         const DevDataset &ds = m.ds[E.dl[i]];
         const float *gs = carve_ds_ws(wsb + (int64_t)i * m.ws_eval_floats, m.N_t, m.C, m.max_reco, m.n_osc).dp;
         const int L = ds.sp_lanes, per = nth / L;   // lanes per parameter, parameters per pass
         const int work = ds.n_sp * L;
+        #pragma unroll 1
         for (int q0 = rot_tid(i, (work + 31) >> 5); q0 < ((work + 31) & ~31); q0 += per * L) {
             const int p = q0 / L, sub = q0 & (L - 1);
+            const int4 sp = p < ds.n_sp ? ds.sp[p] : make_int4(0, 0, 0, 1);
             float s = 0.f;
-            if (p < ds.n_sp)
-                for (int r = ds.sp_ptr[p] + sub; r < ds.sp_ptr[p + 1]; r += L) s += gs[ds.sp_k[r]];
+            if (sp.w)
+                #pragma unroll 1
+                for (int r = sub; r < sp.z; r += L) s += gs[sp.y + r];
+            else
+                #pragma unroll 1
+                for (int r = sub; r < sp.z; r += L) s += gs[ds.sp_k[sp.y + r]];
             for (int o = L >> 1; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-            if (p < ds.n_sp && sub == 0) grad[ds.sp_param[p]] += s;
+            if (p < ds.n_sp && sub == 0) grad[sp.x] += s;
         }
         if (m.shared_roles) __syncthreads();
     }
@@ -1304,10 +1558,10 @@ static __device__ __forceinline__ int eval_setup_any(const DevModel &m, EvalShar
     return eval_setup<4>(m, E, q, mask, first, group);
 }
 
-// The Poisson -2lnL of the datasets in `mask` and (grad != nullptr) its theta gradient added to
+// The Poisson -2lnL of the datasets in `mask` and (GRAD) its theta gradient added to
 // grad. wsb: ws_group dataset workspaces. Returns the -2lnL on every thread; E.status (cleared
 // here) holds kSt* bits on failure. Starts and ends with a barrier.
-template <bool GEN>
+template <bool GEN, bool GRAD>
 static __device__ double eval_datasets(const DevModel &m, EvalShared &E, const ParVecs &q, uint32_t mask,
                                        const float *data, float *wsb, float *grad) {
     __syncthreads();
@@ -1315,19 +1569,14 @@ static __device__ double eval_datasets(const DevModel &m, EvalShared &E, const P
         E.status = 0;
         E.nll = 0.0;
     }
+    #pragma unroll 1
     for (int first = 0; first < m.n_ds;) {
         first = eval_setup_any<GEN>(m, E, q, mask, first, m.ws_group);
         if (E.n > 0) {
-            if (grad != nullptr)
-                st_signal<true, GEN>(m, E, q, wsb);
-            else
-                st_signal<false, GEN>(m, E, q, wsb);
+            st_signal<GRAD, GEN>(m, E, q, wsb);
             st_remap<GEN>(m, E, wsb);
             st_fold(m, E, wsb);
-            if (grad != nullptr)
-                st_lik<true>(m, E, q, data, wsb);
-            else
-                st_lik<false>(m, E, q, data, wsb);
+            st_lik<GRAD>(m, E, q, data, wsb);
         }
         if (E.status || E.bad) {   // block-uniform after the barriers
             __syncthreads();
@@ -1336,7 +1585,7 @@ static __device__ double eval_datasets(const DevModel &m, EvalShared &E, const P
             return INFINITY;
         }
         if (E.n == 0) continue;
-        if (grad != nullptr) {
+        if (GRAD) {
             lik_finish<true>(m, E, grad);
             if (m.shared_roles) __syncthreads();
             st_bkg_shape(m, E, wsb, grad);
@@ -1361,6 +1610,7 @@ template <bool GEN>
 static __device__ void expected_datasets(const DevModel &m, EvalShared &E, const ParVecs &q, float *wsb, float *mu) {
     __syncthreads();
     if (threadIdx.x == 0) E.status = 0;
+    #pragma unroll 1
     for (int first = 0; first < m.n_ds;) {
         first = eval_setup_any<GEN>(m, E, q, 0xffffffffu, first, m.ws_group);
         if (E.n > 0) {
@@ -1381,35 +1631,59 @@ static __device__ void expected_datasets(const DevModel &m, EvalShared &E, const
 
 // ------------------------------------------------------------------------------------
 // Triangular matrix-vector products of the prior blocks: out_r = sum_c M(r, c) x_c over the rows
-// of all blocks together, as tiles of 32 rows x kTriCols columns (a warp per tile, a lane per
-// row: every column is one coalesced load and one broadcast of x, sixteen in flight). A tile
-// leaves its partial sum at part[seg * tri_rows + row]; after a barrier tri_sum adds a row's
-// segments in order. x: by parameter index.
-static __device__ __forceinline__ void tri_apply(const DevModel &m, const TriTile *tiles, int n_tiles, const float *M,
+// of all blocks together, as tiles of up to 128 rows x 32 (64 for blocks of more than 512)
+// columns, a warp per tile and four rows per lane: a column of a tile is one coalesced 16-byte
+// load per lane and one broadcast of x, eight in flight (the factors come from L2: 0.7 MB per
+// evaluation for the 400 x 400 block's two products). A tile leaves its partial sums at
+// part[seg * tri_rows + row]; after a barrier tri_sum adds a row's segments in order. With
+// 4-byte loads of 32-row tiles each product of that block took 13 500 cycles with 512 threads.
+// x: by parameter index.
+static __device__ __noinline__ void tri_apply(const DevModel &m, const TriTile *tiles, int n_tiles, const float *M,
                                                  const float *x, float *part) {
     const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    for (int t = threadIdx.x >> 5; t < n_tiles; t += nw) {
-        const TriTile T = tiles[t];
-        const int r = min(T.row0 + lane, T.n - 1), cols = T.cols;
-        const float *col = M + T.mat + (int64_t)T.col0 * T.n + r;
-        float s[4] = {0.f, 0.f, 0.f, 0.f};
+        int t = threadIdx.x >> 5;
+    if (t >= n_tiles) return;
+    TriTile T = tiles[t];
+#pragma unroll 1
+    while (true) {
+        const TriTile next = tiles[min(t + nw, n_tiles - 1)];   // its latency behind this tile's
+        const int p4 = T.pitch >> 2;
+        const float4 *col = reinterpret_cast<const float4 *>(M + T.mat) + min(lane, p4 - 1);
+        const float *xb = x + T.in0;
+        const int *idx = m.blk_idx + T.idx;
+        const bool seq = T.in0 >= 0;
+        float4 s[2] = {make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f)};
+        #pragma unroll 1
         int c = 0;
-        if (T.in0 >= 0) {
-            const float *xb = x + T.in0 + T.col0;
-            for (; c + 15 < cols; c += 16) {
+        auto add = [](float4 &a, const float4 &r, float v) {
+            a.x = fmaf(r.x, v, a.x);
+            a.y = fmaf(r.y, v, a.y);
+            a.z = fmaf(r.z, v, a.z);
+            a.w = fmaf(r.w, v, a.w);
+        };
+#pragma unroll 1
+        for (; c + 8 <= T.cols; c += 8, col += 8 * p4) {
+            float4 r[8];
 #pragma unroll
-                for (int u = 0; u < 16; ++u) s[u & 3] = fmaf(col[(int64_t)(c + u) * T.n], xb[c + u], s[u & 3]);
-            }
-            for (; c < cols; ++c) s[0] = fmaf(col[(int64_t)c * T.n], xb[c], s[0]);
-        } else {
-            const int *idx = m.blk_idx + T.idx + T.col0;
-            for (; c + 7 < cols; c += 8) {
+            for (int u = 0; u < 8; ++u) r[u] = col[u * p4];
+            if (seq) {
 #pragma unroll
-                for (int u = 0; u < 8; ++u) s[u & 3] = fmaf(col[(int64_t)(c + u) * T.n], x[idx[c + u]], s[u & 3]);
+                for (int u = 0; u < 8; ++u) add(s[u & 1], r[u], xb[c + u]);
+            } else {
+#pragma unroll
+                for (int u = 0; u < 8; ++u) add(s[u & 1], r[u], x[idx[c + u]]);
             }
-            for (; c < cols; ++c) s[0] = fmaf(col[(int64_t)c * T.n], x[idx[c]], s[0]);
         }
-        if (T.row0 + lane < T.n) part[T.seg * m.tri_rows + T.out + T.row0 + lane] = (s[0] + s[1]) + (s[2] + s[3]);
+#pragma unroll 1
+        for (; c < T.cols; ++c, col += p4) add(s[0], *col, seq ? xb[c] : x[idx[c]]);
+        float *o = part + T.seg * m.tri_rows + T.out + 4 * lane;
+        const float e[4] = {s[0].x + s[1].x, s[0].y + s[1].y, s[0].z + s[1].z, s[0].w + s[1].w};
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (4 * lane + u < T.rows) o[u] = e[u];
+        t += nw;
+        if (t >= n_tiles) break;
+        T = next;
     }
 }
 
@@ -1417,6 +1691,7 @@ __device__ __forceinline__ float tri_sum(const DevModel &m, const float *part, i
     const int x = m.tri_seg[row];
     const int s0 = upper ? (x >> 8) & 255 : 0, s1 = upper ? x >> 16 : x & 255;
     float t = part[s0 * m.tri_rows + row];
+    #pragma unroll 1
     for (int q = s0 + 1; q < s1; ++q) t += part[q * m.tri_rows + row];
     return t;
 }

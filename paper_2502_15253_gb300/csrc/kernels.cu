@@ -14,6 +14,7 @@ __device__ double prior_theta(const DevModel &m, const float *pd, float *grad, f
     const int tid = threadIdx.x, nth = blockDim.x;
     __syncthreads();
     float acc = 0.f;
+    #pragma unroll 1
     for (int i = tid; i < m.P; i += nth) {
         const float pi = m.prior_inv[i];
         if (pi > 0.f) {
@@ -23,8 +24,9 @@ __device__ double prior_theta(const DevModel &m, const float *pd, float *grad, f
         }
     }
     if (m.tri_rows > 0) {
-        tri_apply(m, m.tri_lo, m.n_tri_lo, m.blk_W, pd, part);
+        tri_apply(m, m.tri_lo, m.n_tri_lo, m.W_lo, pd, part);
         __syncthreads();
+        #pragma unroll 1
         for (int r = tid; r < m.tri_rows; r += nth) {
             const float z = tri_sum(m, part, r, false);
             zs[m.tri_param[r]] = z;
@@ -32,8 +34,9 @@ __device__ double prior_theta(const DevModel &m, const float *pd, float *grad, f
         }
         __syncthreads();
         if (grad) {
-            tri_apply(m, m.tri_up, m.n_tri_up, m.blk_W, zs, part);
+            tri_apply(m, m.tri_up, m.n_tri_up, m.W_up, zs, part);
             __syncthreads();
+            #pragma unroll 1
             for (int r = tid; r < m.tri_rows; r += nth) grad[m.tri_param[r]] += 2.f * tri_sum(m, part, r, true);
         }
     }
@@ -67,6 +70,7 @@ __global__ void __launch_bounds__(T, MINB) eval_kernel(EvalArgs A) {
 
     for (int b = blockIdx.x; b < A.B; b += gridDim.x) {
         const double *th = A.theta + (int64_t)b * P;
+        #pragma unroll 1
         for (int i = threadIdx.x; i < P; i += blockDim.x) {
             const double t = th[i];
             const float h = (float)t, d = (float)(t - m.theta0[i]);
@@ -80,7 +84,9 @@ __global__ void __launch_bounds__(T, MINB) eval_kernel(EvalArgs A) {
             expected_datasets<GEN>(m, S.E, q, ws, A.mu + (int64_t)b * m.n_data);
         } else {
             const float *dat = A.data ? A.data + (int64_t)b * m.n_data : m.asimov;
-            nll = eval_datasets<GEN>(m, S.E, q, A.masks ? A.masks[b] : 0xffffffffu, dat, ws, want_grad ? grad : nullptr);
+            const uint32_t mask = A.masks ? A.masks[b] : 0xffffffffu;
+            nll = want_grad ? eval_datasets<GEN, true>(m, S.E, q, mask, dat, ws, grad)
+                            : eval_datasets<GEN, false>(m, S.E, q, mask, dat, ws, nullptr);
         }
         const int st = S.E.status;
         if (A.mu == nullptr && st == 0) nll += prior_theta(m, pd, want_grad ? grad : nullptr, zs, ws, S.red);
@@ -92,6 +98,7 @@ __global__ void __launch_bounds__(T, MINB) eval_kernel(EvalArgs A) {
         }
         __syncthreads();
         if (want_grad)
+            #pragma unroll 1
             for (int i = threadIdx.x; i < P; i += blockDim.x) A.grad[(int64_t)b * P + i] = st ? NAN : grad[i];
         __syncthreads();
     }
@@ -195,6 +202,7 @@ __global__ void __launch_bounds__(128) ls_init_kernel(LsArgs A) {
 __device__ __forceinline__ ParVecs ls_params_in(const LsArgs &A, int g, int P, float *pv) {
     const FitVecs V = ls_vecs(A, g, P);
     float *pd = pv + fit_vec_pitch(P), *pl = pd + fit_vec_pitch(P);
+    #pragma unroll 1
     for (int i = threadIdx.x; i < P; i += blockDim.x) {
         pv[i] = V.pv[i];
         pd[i] = V.pd[i];
@@ -368,7 +376,10 @@ __device__ __forceinline__ void ls_tc_lik_body(LsArgs A) {
         const int nr = m.ds[d].n_reco;
         const float *fr = A.fbuf + ((int64_t)d * A.n + a) * A.ldf;
         const ParVecs q = ls_params_in(A, g, P, pv);
-        for (int j = threadIdx.x; j < nr; j += blockDim.x) ws.f0[j] = fr[j];
+        for (int j = threadIdx.x; j < nr; j += blockDim.x) {
+            ws.f0[j] = fr[j];
+            ws.gmu[j] = 0.f;   // (the fold's low part: none here)
+        }
         if (threadIdx.x == 0) {
             S.E.status = 0;
             S.E.nll = 0.0;
@@ -454,6 +465,7 @@ __global__ void __launch_bounds__(128) ls_step_kernel(LsArgs A) {
         copy_state(&S.st, A.state + g);
         // theta gradient = sum of the dataset slices in a fixed order; the slices are cleared
         float *gs = A.gsl + (int64_t)g * nd * P;
+        #pragma unroll 1
         for (int i = threadIdx.x; i < P; i += blockDim.x) {
             float t = 0.f;
             for (int d = 0; d < nd; ++d) {

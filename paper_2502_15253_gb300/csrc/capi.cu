@@ -469,6 +469,17 @@ int fit_model_create(const fit_model_desc *d, fit_model **out) {
         det_fold.push_back(pack_bands(nr, Nt, [&](int r, int k) { return (float)R[(size_t)r * Nt + k]; },
                                       fold_parts(h, nr)));
         det_adj.push_back(pack_bands(Nt, nr, [&](int k, int r) { return (float)R[(size_t)r * Nt + k]; }, 1));
+        vector<int2> row_band(nr);
+        for (int j = 0; j < nr; ++j) {
+            int a = Nt, b = -1;
+            for (int k = 0; k < Nt; ++k)
+                if (R[(size_t)j * Nt + k] != 0.0) {
+                    a = std::min(a, k);
+                    b = k;
+                }
+            row_band[j] = b >= a ? make_int2(a, b - a + 1) : make_int2(0, 1);
+        }
+        A.put(&dt.row_band, row_band);
         for (const bool adj : {false, true}) {
             const PackedBands &pb = adj ? det_adj.back() : det_fold.back();
             fitcore::BandUnits &U = adj ? dt.adj : dt.fold;
@@ -1258,6 +1269,26 @@ struct WsRefresh {
     int n_rows = 0;                    // T_n
 };
 
+// fitcore::expected_rows on host buffers
+int expected_rows_host(fit_model *M, int R, const double *theta, float *mu, int *status, cudaStream_t s) {
+    const size_t P = M->n_params, D = M->n_data;
+    Staged th, m, st;
+    bool hm = false, hs = false;
+    int rc = stage_in(theta, sizeof(double) * P * R, s, th);
+    if (!rc) rc = stage_out(mu, sizeof(float) * D * R, s, m, hm);
+    if (!rc) rc = stage_out(status, sizeof(int) * R, s, st, hs);
+    if (!rc)
+        rc = fitcore::expected_rows(M->host, M->dev, R, (const double *)th.dev, (float *)m.dev, (int *)st.dev, s);
+    if (!rc && (cudaMemcpyAsync(mu, m.dev, sizeof(float) * D * R, cudaMemcpyDeviceToHost, s) ||
+                cudaMemcpyAsync(status, st.dev, sizeof(int) * R, cudaMemcpyDeviceToHost, s)))
+        rc = fail(FIT_ERR_CUDA, "expected rows: copy back");
+    release(th, s);
+    release(m, s);
+    release(st, s);
+    if (!rc && cudaStreamSynchronize(s) != cudaSuccess) rc = fail(FIT_ERR_CUDA, "expected rows: synchronise");
+    return rc;
+}
+
 int linear_mle_rows(fit_model *M, const fit_warmstart_geom &G, cudaStream_t s, std::vector<float> &K1,
                     std::vector<float> &K2, std::vector<float> &zf, int &n_var, WsRefresh *ref = nullptr) {
     const int P = M->n_params, D = M->n_data, nt = G.n_targets;
@@ -1271,7 +1302,7 @@ int linear_mle_rows(fit_model *M, const fit_warmstart_geom &G, cudaStream_t s, s
     }
     std::vector<float> mu((size_t)R * D);
     std::vector<int> st(R, 0);
-    int rc = fit_model_expected(M, R, th.data(), mu.data(), st.data(), s);
+    int rc = expected_rows_host(M, R, th.data(), mu.data(), st.data(), s);
     if (rc) return rc;
     for (int q = 0; q < R; ++q)
         if (st[q] != 0) return fail(FIT_ERR_INVALID_CONFIG, "warm start: expectation near the nominal point failed");
@@ -2007,7 +2038,7 @@ bool fisher_U(fit_model *M, cudaStream_t s) {
     }
     std::vector<float> mu((size_t)R * D);
     std::vector<int> st(R, 0);
-    if (fit_model_expected(M, R, th.data(), mu.data(), st.data(), s) != FIT_OK) return false;
+    if (expected_rows_host(M, R, th.data(), mu.data(), st.data(), s) != FIT_OK) return false;
     for (int q = 0; q < R; ++q)
         if (st[q] != 0) return false;
     std::vector<double> U((size_t)P * D, 0.0);
@@ -2095,7 +2126,7 @@ int lin_base(fit_model *M, cudaStream_t s) {
     const int D = M->n_data;
     std::vector<float> mu(D);
     std::vector<int> st(1, 0);
-    int rc = fit_model_expected(M, 1, M->theta0.data(), mu.data(), st.data(), s);
+    int rc = expected_rows_host(M, 1, M->theta0.data(), mu.data(), st.data(), s);
     if (rc) return rc;
     if (st[0] != 0) return fail(FIT_ERR_INVALID_CONFIG, "linearised fit: expectation at theta0 failed");
     if (!fisher_U(M, s)) return fail(FIT_ERR_INVALID_CONFIG, "linearised fit: expectation near theta0 failed");

@@ -31,6 +31,7 @@ struct DevDetector {
     int n_reco;
     BandUnits fold;          // outputs: reco rows in fours, inputs: true bins
     BandUnits adj;           // outputs: true bins in fours, inputs: reco rows
+    const int2 *row_band;    // [N_r] first true bin and length of each row's band
     const float *rdense_hi;  // [N_r x ldt] dense response, TF32-exact high part (tensor-core fold)
     const float *rdense_lo;  // [N_r x ldt] R - rdense_hi
     const float *rdt_hi;     // [N_t x ldr] R^T, TF32-exact high part (tensor-core adjoint fold)

@@ -129,6 +129,9 @@ int linear_start_apply(int B, int P, int D, const double *theta0_dev, const floa
                        const float *const *K, int n_var, const int *sel_dev, double *theta_out, cudaStream_t s);
 int expected_tc(const DevModel &h, const DevModel *dev, int B, const double *theta, float *mu, int *status,
                 int precision, cudaStream_t s);
+// jacobian.cu: expectations in a fixed order of operations, for central differences
+int expected_rows(const DevModel &h, const DevModel *dev, int B, const double *theta, float *mu, int *status,
+                  cudaStream_t s);
 int poisson_sample(int64_t n, const float *mu, uint64_t seed, uint64_t offset, float *out, cudaStream_t s);
 int features(int B, int n_data, const float *data, const float *nbar, const uint32_t *masks, const int *slot_ds,
              const int *status, int n_in, int slot0, int onehot, float *x, cudaStream_t s);

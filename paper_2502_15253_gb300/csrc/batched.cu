@@ -27,200 +27,132 @@ __device__ __forceinline__ float tf32_round(float x) {
     return __uint_as_float(b);
 }
 
-// One block per (instance b, dataset d): survival (FP32 float-pair phases and the fitted
-// sin^2(pi r) polynomial, as the event kernel) x reweights on the true grid, energy
-// correction gathered per target bin, written as V_hi / V_lo rows of length ldt. Blocks of
-// dataset 0 also store the instance's parameter pairs for the epilogue.
-__global__ void __launch_bounds__(256) signal_v_kernel(const DevModel *__restrict__ gm, int B,
-                                                       const double *__restrict__ theta, float *__restrict__ vhi,
-                                                       float *__restrict__ vlo, float *__restrict__ pv_out,
-                                                       float *__restrict__ pd_out, int *__restrict__ status) {
+// One (instance b, dataset d) at a time per block (grid.y = datasets, the instances strided over
+// grid.x): survival x reweights on the true grid (the evaluation's sums over core pairs, without
+// derivatives), energy correction gathered per target bin, written as V_hi / V_lo rows of length
+// ldt. Blocks of dataset 0 also store the instance's parameter pairs for the epilogue.
+// Bound by instruction issue in the survival sums (20 000 bin-cores per instance and dataset on
+// the 53 km model); a block keeps its copy of the model's header for all its instances. 4096
+// instances of that model took 700 us with a block per (instance, dataset), FP64 coefficients
+// by one thread and the phase count of the formula tested per bin.
+struct SignalSmem {
+    DevModel m;
+    EvalShared E;
+};
+inline size_t signal_smem_bytes(const DevModel &h) {
+    const int edge = (h.N_t + 4) & ~3;
+    return sizeof(SignalSmem) + sizeof(float) * (3 * (size_t)fit_vec_pitch(h.P) + ((h.N_t + 3) & ~3) +
+                                                 (h.remap_mode == FIT_REMAP_SPLINE ? 3 : 1) * edge);
+}
+
+template <int NOSC, int MODE>
+__global__ void __launch_bounds__(256, 3) signal_v_kernel(const DevModel *__restrict__ gm, int B,
+                                                          const double *__restrict__ theta, float *__restrict__ vhi,
+                                                          float *__restrict__ vlo, float *__restrict__ pv_out,
+                                                          float *__restrict__ pl_out, int *__restrict__ status) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    DevModel &m = *reinterpret_cast<DevModel *>(smem_raw);
+    SignalSmem &S = *reinterpret_cast<SignalSmem *>(smem_raw);
     {
         const int n = (int)(sizeof(DevModel) / sizeof(int));
         const int *src = reinterpret_cast<const int *>(gm);
-        int *dst = reinterpret_cast<int *>(smem_raw);
+        int *dst = reinterpret_cast<int *>(&S.m);
         for (int i = threadIdx.x; i < n; i += blockDim.x) dst[i] = src[i];
     }
     __syncthreads();
-    float *pv = reinterpret_cast<float *>(smem_raw + sizeof(DevModel));
-    float *pd = pv + m.P;
-    float *u = pd + m.P;
-    __shared__ OscCoefN<6> kco;
-    const int b = blockIdx.x, d = blockIdx.y, tid = threadIdx.x, nth = blockDim.x;
+    const DevModel &m = S.m;
+    const int d = blockIdx.y, tid = threadIdx.x, nth = blockDim.x, N_t = m.N_t;
+    const int Pp = fit_vec_pitch(m.P), edge = (N_t + 4) & ~3;
+    float *pv = reinterpret_cast<float *>(smem_raw + sizeof(SignalSmem)), *pd = pv + Pp, *pl = pd + Pp;
+    float *u = pl + Pp;
+    EdgeTab T;   // (overlap rule: T.t holds the displacements of the grid edges)
+    T.t = u + ((N_t + 3) & ~3);
+    T.r = T.t + edge;
+    T.k = reinterpret_cast<int *>(T.r + edge);
+    const ParVecs q{pv, pd, pl};
     const DevDataset &ds = m.ds[d];
-    const int N_t = m.N_t;
-    const double *th = theta + (int64_t)b * m.P;
-    for (int i = tid; i < m.P; i += nth) {
-        const double t = th[i];
-        pv[i] = (float)t;
-        pd[i] = (float)(t - m.theta0[i]);
-        if (d == 0) {
-            pv_out[(int64_t)b * m.P + i] = pv[i];
-            pd_out[(int64_t)b * m.P + i] = pd[i];
-        }
-    }
-    float eta[kMaxOsc], eta_lo[kMaxOsc];
-#pragma unroll
-    for (int i = 0; i < kMaxOsc; ++i) {
-        const int p = i < m.n_osc ? m.osc_idx[i] : -1;
-        if (osc_is_dm(m.osc_mode, i)) {
-            eta[i] = p >= 0 ? m.theta0_f[p] : m.osc_val[i];
-            eta_lo[i] = p >= 0 ? m.theta0_lo[p] + (float)(th[p] - m.theta0[p]) : m.osc_val_lo[i];
-        } else {
-            eta[i] = p >= 0 ? (float)th[p] : m.osc_val[i];
-            eta_lo[i] = 0.f;
-        }
-    }
-    if (tid == 0) {
-        double e[kMaxOsc];
-        for (int i = 0; i < kMaxOsc; ++i)
-            e[i] = i >= m.n_osc ? 0.0 : (m.osc_idx[i] >= 0 ? th[m.osc_idx[i]] : m.osc_val_d[i]);
-        double c[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-        if (m.osc_mode == FIT_OSC_EQ1) {
-            const double c2 = 0.5 * (1.0 + sqrt(fmax(1.0 - e[0], 0.0)));
-            c[0] = e[0];
-            c[1] = c2 * c2 * e[2];
-        } else {
-            const double S12 = 4.0 * e[0] * (1.0 - e[0]), S13 = 4.0 * e[1] * (1.0 - e[1]);
-            double C4 = 1.0;   // cos^4 th14 (3+1 formula; 1 without a sterile state)
-            if (m.osc_mode == FIT_OSC_STERILE4) {
-                const double c14 = 0.5 * (1.0 + sqrt(fmax(1.0 - e[4], 0.0)));
-                C4 = c14 * c14;
-                c[3] = e[4] * (1.0 - e[1]) * (1.0 - e[0]);
-                c[4] = e[4] * (1.0 - e[1]) * e[0];
-                c[5] = e[4] * e[1];
-            }
-            c[0] = C4 * (1.0 - e[1]) * (1.0 - e[1]) * S12;
-            c[1] = C4 * S13 * (1.0 - e[0]);
-            c[2] = C4 * S13 * e[0];
-        }
-        for (int i = 0; i < 6; ++i) {
-            kco.hi[i] = (float)c[i];
-            kco.lo[i] = (float)(c[i] - (double)kco.hi[i]);
-        }
-    }
-    __syncthreads();
-    const OscCoefN<6> kc6 = kco;
-    // the phases of the sin^2 terms in the order of the coefficients: Eq. 1: x_ee, x_21;
-    // three-flavour: x_21, x_31, x_32; 3+1: and x_41, x_42, x_43 (mass splittings as float pairs)
-    float pdm[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, pdl[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    int nph;
-    {
-        // normalised pairs: sin2_phase needs the low part to stay below an ulp of the high one
-        // (the parameter offset sits in eta_lo here), so that the reduced phase is within 1/2
-        auto pr = [&](int i) { return f2_norm(eta[i], eta_lo[i]); };
-        auto sub = [](F2 a, F2 b) { return f2_add(a, F2{-b.h, -b.l}); };
-        F2 d[6];
-        if (m.osc_mode == FIT_OSC_EQ1) {
-            nph = 2;
-            d[0] = pr(1);
-            d[1] = pr(3);
-        } else {
-            nph = 3;
-            d[0] = pr(2);
-            d[1] = pr(3);
-            d[2] = sub(pr(3), pr(2));
-            if (m.osc_mode == FIT_OSC_STERILE4) {
-                nph = 6;
-                d[3] = pr(5);
-                d[4] = sub(pr(5), pr(2));
-                d[5] = sub(pr(5), pr(3));
+    const bool spline = m.remap_mode == FIT_REMAP_SPLINE;
+#pragma unroll 1
+    for (int b = blockIdx.x; b < B; b += gridDim.x) {
+        const double *th = theta + (int64_t)b * m.P;
+        for (int i = tid; i < m.P; i += nth) {
+            const double t = th[i];
+            const float h = (float)t, del = (float)(t - m.theta0[i]);
+            pv[i] = h;
+            pd[i] = del;
+            pl[i] = presid(m, h, del, i);
+            if (d == 0) {
+                pv_out[(int64_t)b * m.P + i] = h;
+                pl_out[(int64_t)b * m.P + i] = pl[i];
             }
         }
-        for (int i = 0; i < nph; ++i) {
-            pdm[i] = d[i].h;
-            pdl[i] = d[i].l;
+        eval_setup<NOSC>(m, S.E, q, 1u << d, 0, 1);
+        float *vh = vhi + ((int64_t)d * B + b) * m.ldt, *vl = vlo + ((int64_t)d * B + b) * m.ldt;
+        if (S.E.bad) {   // (block-uniform) the energy map is not increasing on the grid
+            if (tid == 0) atomicExch(&status[b], FIT_STATUS_ESCALE_NONMONOTONE);
+            for (int k = tid; k < m.ldt; k += nth) vh[k] = vl[k] = 0.f;
+            continue;
         }
-    }
-    const PP nrm = ppair(m, pv, pd, ds.norm_idx, 1.f);
-    const EMap em = make_emap(m, ds, pv, pd);
-    {
-        const float s0 = em.slope(m.e_edge[0]), s1 = em.slope(m.e_edge[N_t]);
-        if (!(s0 > 0.25f && s0 < 4.f && s1 > 0.25f && s1 < 4.f)) {
-            if (tid == 0) atomicOr(&status[b], kStEscale);
-            for (int k = tid; k < m.ldt; k += nth) {
-                vhi[((int64_t)d * B + b) * m.ldt + k] = 0.f;
-                vlo[((int64_t)d * B + b) * m.ldt + k] = 0.f;
-            }
-            return;
-        }
-    }
-    for (int k = tid; k < N_t; k += nth) {
-        const float ih = m.inv_e_hi[k], il = m.inv_e_lo[k];
-        float pt = 0.f;
-        for (int c = 0; c < m.C; ++c) {
-            const float w = ds.w[c];
-            if (w == 0.f) continue;
-            const float ch = ds.kl_hi[c] * ih;
-            const float cl = fmaf(ds.kl_hi[c], ih, -ch) + ds.kl_hi[c] * il + ds.kl_lo[c] * ih;
-            // P = 1 - sum_i C_i sin^2(x_i) with the fitted sin^2(pi r) polynomial (no
-            // derivatives are needed here)
-            float P = 1.f;
-#pragma unroll
-            for (int i = 0; i < 6; ++i)
-                if (i < nph) P -= cterm(kc6, i, sin2_phase(pdm[i], pdl[i], ch, cl));
-            pt += pmul(ppair(m, pv, pd, m.core_power_idx[c], 1.f), w * P);
-        }
-        const float ts = pmul(ppair(m, pv, pd, ds.shape_idx[k], 1.f), ds.t[k]);
-        u[k] = pmul(nrm, ts * pt);
-    }
-    __syncthreads();
-    for (int t = tid; t < m.ldt; t += nth) {
-        float acc = 0.f;
-        if (t < N_t && m.remap_mode == FIT_REMAP_SPLINE) {
-            acc = spline_target(u, m.e_edge, em, t, N_t);
-        } else if (t < N_t) {
-            int k = t - (int)floorf(em.disp(m.e_edge[t]));
-            k = min(max(k, 0), N_t - 1);
-            k = t - (int)floorf(em.disp(m.e_edge[k]));
-            k = min(max(k - 1, 0), N_t - 1);
-            while (k > 0 && (float)(k - t) + em.disp(m.e_edge[k]) > 0.f) --k;
-            float dlo = em.disp(m.e_edge[k]);
-            for (int it = 0; it < 64 && k < N_t; ++it, ++k) {
-                const float dhi = em.disp(m.e_edge[k + 1]);
-                const float ylo = (float)(k - t) + dlo, yhi = (float)(k + 1 - t) + dhi;
-                if (ylo >= 1.f) break;
-                const float ov = fminf(yhi, 1.f) - fmaxf(ylo, 0.f);
-                if (ov > 0.f) acc = fmaf(u[k], ov / (1.f + (dhi - dlo)), acc);
-                dlo = dhi;
+        const PP nrm = S.E.nrm[0];
+        const EMap em = S.E.em[0];
+#pragma unroll 1
+        for (int k = tid; k < N_t; k += nth) {
+            const float ih = m.inv_e_hi[k], il = m.inv_e_lo[k], e0 = m.e_edge[k], e1 = m.e_edge[k + 1];
+            const int sp = ds.shape_idx[k];
+            const float tk = ds.t[k];
+            float pt, corr, dpt[NOSC];
+            CoreSums<false, NOSC, MODE>::run(S.E, 0, m.C, ih, il, nullptr, 0, pt, corr, dpt);
+            const float ts = pmul(ppair(q, sp, 1.f), tk);
+            const float x = pmul(nrm, fmaf(ts, pt, ts * corr));
+            if (spline) {
+                u[k] = x;
+                edge_store(T, m.e_edge, em, k, N_t);
+                if (k == N_t - 1) edge_store(T, m.e_edge, em, N_t, N_t);
+            } else {
+                const float d0 = em.disp(e0), d1 = em.disp(e1);
+                u[k] = x / (1.f + (d1 - d0));
+                T.t[k] = d0;
+                if (k == N_t - 1) T.t[N_t] = d1;
             }
         }
-        const float hi = tf32_round(acc);
-        vhi[((int64_t)d * B + b) * m.ldt + t] = hi;
-        vlo[((int64_t)d * B + b) * m.ldt + t] = acc - hi;
+        __syncthreads();
+#pragma unroll 1
+        for (int t = tid; t < m.ldt; t += nth) {
+            float acc = 0.f;
+            if (t < N_t) acc = spline ? spline_target(u, T, t, N_t) : overlap_target(u, T.t, t, N_t);
+            const float hi = tf32_round(acc);
+            vh[t] = hi;
+            vl[t] = acc - hi;
+        }
     }
 }
 
-// mu[b][off_d + j] = eps_d F_d[b][j] + sum_b r B (1 + delta); status bits become FIT_STATUS_*
-__global__ void mu_epilogue_kernel(const DevModel *__restrict__ gm, int B, const float *__restrict__ F,
-                                   int ldf, const float *__restrict__ pv_all, const float *__restrict__ pd_all,
-                                   float *__restrict__ mu, int *__restrict__ status) {
+// mu[b][off_d + j] = eps_d F_d[b][j] + sum_b r B (1 + delta), NaN where the instance has a status; a
+// block per instance at a time
+__global__ void __launch_bounds__(128) mu_epilogue_kernel(const DevModel *__restrict__ gm, int B,
+                                                          const float *__restrict__ F, int ldf,
+                                                          const float *__restrict__ pv_all,
+                                                          const float *__restrict__ pl_all, float *__restrict__ mu,
+                                                          const int *__restrict__ status) {
     const DevModel &m = *gm;
-    const int64_t total = (int64_t)B * m.n_data;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-        const int b = (int)(e / m.n_data), q = (int)(e % m.n_data);
-        int d = 0;
-        while (d + 1 < m.n_ds && m.ds[d + 1].data_off <= q) ++d;
-        const int j = q - m.ds[d].data_off;
-        const DevDataset &ds = m.ds[d];
-        const float *pv = pv_all + (int64_t)b * m.P, *pd = pd_all + (int64_t)b * m.P;
-        const float f = F[((int64_t)d * B + b) * ldf + j];
-        float v = pmul(ppair(m, pv, pd, ds.eff_idx, 1.f), f);
-        for (int k = ds.bkg_begin; k < ds.bkg_end; ++k) {
-            const DevBkg &bk = m.bkg[k];
-            const float tm = bk.tmpl[j];
-            const float shaped = bk.shape_idx[j] >= 0 ? fmaf(tm, pv[bk.shape_idx[j]], tm) : tm;
-            v += pmul(ppair(m, pv, pd, bk.rate_idx, 1.f), shaped);
+    const int P = m.P, n_data = m.n_data, n_ds = m.n_ds;
+    for (int b = blockIdx.x; b < B; b += gridDim.x) {
+        const ParVecs q{pv_all + (int64_t)b * P, nullptr, pl_all + (int64_t)b * P};
+        const bool bad = status[b] != 0;
+        for (int d = 0; d < n_ds; ++d) {
+            const DevDataset &ds = m.ds[d];
+            const PP eff = ppair(q, ds.eff_idx, 1.f);
+            for (int j = threadIdx.x; j < ds.n_reco; j += blockDim.x) {
+                float v = pmul(eff, F[((int64_t)d * B + b) * ldf + j]);
+                for (int k = ds.bkg_begin; k < ds.bkg_end; ++k) {
+                    const DevBkg &bk = m.bkg[k];
+                    const float tm = bk.tmpl[j];
+                    const float shaped = bk.shape_idx[j] >= 0 ? fmaf(tm, q.pv[bk.shape_idx[j]], tm) : tm;
+                    v += pmul(ppair(q, bk.rate_idx, 1.f), shaped);
+                }
+                mu[(int64_t)b * n_data + ds.data_off + j] = bad ? NAN : v;
+            }
         }
-        mu[e] = status[b] ? NAN : v;
     }
-}
-
-__global__ void status_finish_kernel(int B, int *status) {
-    for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < B; b += gridDim.x * blockDim.x)
-        status[b] = (status[b] & kStEscale) ? FIT_STATUS_ESCALE_NONMONOTONE : 0;
 }
 
 }  // namespace
@@ -232,24 +164,37 @@ int expected_tc(const DevModel &h, const DevModel *dev, int B, const double *the
     int ldf = 0;
     for (int d = 0; d < nds; ++d) ldf = std::max(ldf, h.ds[d].n_reco);
     ldf = (ldf + 3) / 4 * 4;
-    float *vhi = nullptr, *vlo = nullptr, *F = nullptr, *pv = nullptr, *pd = nullptr;
+    float *vhi = nullptr, *vlo = nullptr, *F = nullptr, *pv = nullptr, *pl = nullptr;
     auto cleanup = [&]() {
-        for (float *p : {vhi, vlo, F, pv, pd})
+        for (float *p : {vhi, vlo, F, pv, pl})
             if (p) cudaFreeAsync(p, s);
     };
     if (cudaMallocAsync(&vhi, sizeof(float) * (size_t)nds * B * ldt, s) ||
         cudaMallocAsync(&vlo, sizeof(float) * (size_t)nds * B * ldt, s) ||
         cudaMallocAsync(&F, sizeof(float) * (size_t)nds * B * ldf, s) ||
         cudaMallocAsync(&pv, sizeof(float) * (size_t)B * h.P, s) ||
-        cudaMallocAsync(&pd, sizeof(float) * (size_t)B * h.P, s)) {
+        cudaMallocAsync(&pl, sizeof(float) * (size_t)B * h.P, s)) {
         cudaGetLastError();
         cleanup();
         return fitcore_fail(FIT_ERR_OOM, "fit_model_expected_tc: workspace");
     }
     cudaMemsetAsync(status, 0, sizeof(int) * B, s);
-    const size_t smem = sizeof(DevModel) + sizeof(float) * (2 * (size_t)h.P + h.N_t);
-    cudaFuncSetAttribute(signal_v_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    signal_v_kernel<<<dim3(B, nds), 256, smem, s>>>(dev, B, theta, vhi, vlo, pv, pd, status);
+    const size_t smem = signal_smem_bytes(h);
+    const void *fn = h.osc_mode == FIT_OSC_EQ1       ? (const void *)signal_v_kernel<4, FIT_OSC_EQ1>
+                     : h.osc_mode == FIT_OSC_VACUUM3 ? (const void *)signal_v_kernel<4, FIT_OSC_VACUUM3>
+                                                     : (const void *)signal_v_kernel<6, FIT_OSC_STERILE4>;
+    int dev_id = 0, sms = 0, per_sm = 0;
+    cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (cudaGetDevice(&dev_id) || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev_id) ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, 256, smem) || per_sm < 1) {
+        cudaGetLastError();
+        cleanup();
+        return fitcore_fail(FIT_ERR_CUDA, "fit_model_expected_tc: launch shape");
+    }
+    // one wave of resident blocks over (instance, dataset)
+    const int gx = std::max(1, std::min(B, (per_sm * sms + nds - 1) / nds));
+    void *args[] = {(void *)&dev, &B, &theta, &vhi, &vlo, &pv, &pl, &status};
+    cudaLaunchKernel(fn, dim3(gx, nds), dim3(256), args, smem, s);
     fitcore_count_launch();
     int rc = FIT_OK;
     for (int d = 0; d < nds && rc == FIT_OK; ++d) {
@@ -259,18 +204,11 @@ int expected_tc(const DevModel &h, const DevModel *dev, int B, const double *the
         o.C = F + (size_t)d * B * ldf;
         o.ldc = ldf;
         const float *Vh = vhi + (size_t)d * B * ldt, *Vl = vlo + (size_t)d * B * ldt;
-        rc = tc_gemm(true, B, dt.n_reco, h.N_t, Vh, ldt, dt.rdense_hi, ldt, o, s, nullptr);
-        if (rc == FIT_OK && precision == 1) {
-            o.epi = EPI_F32_ADD;
-            rc = tc_gemm(true, B, dt.n_reco, h.N_t, Vh, ldt, dt.rdense_lo, ldt, o, s, nullptr);
-            if (rc == FIT_OK) rc = tc_gemm(true, B, dt.n_reco, h.N_t, Vl, ldt, dt.rdense_hi, ldt, o, s, nullptr);
-        }
+        rc = precision == 1 ? tc_gemm_split(B, dt.n_reco, h.N_t, Vh, Vl, ldt, dt.rdense_hi, dt.rdense_lo, ldt, o, s)
+                            : tc_gemm(true, B, dt.n_reco, h.N_t, Vh, ldt, dt.rdense_hi, ldt, o, s, nullptr);
     }
     if (rc == FIT_OK) {
-        mu_epilogue_kernel<<<std::min<int64_t>(((int64_t)B * h.n_data + 255) / 256, 4096), 256, 0, s>>>(
-            dev, B, F, ldf, pv, pd, mu, status);
-        status_finish_kernel<<<(B + 255) / 256, 256, 0, s>>>(B, status);
-        fitcore_count_launch();
+        mu_epilogue_kernel<<<std::min(B, 152 * 16), 128, 0, s>>>(dev, B, F, ldf, pv, pl, mu, status);
         fitcore_count_launch();
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) rc = fitcore_fail(FIT_ERR_CUDA, std::string("fit_model_expected_tc: ") + cudaGetErrorString(e));

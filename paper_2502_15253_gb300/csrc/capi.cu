@@ -1881,15 +1881,8 @@ int fit_batch_lockstep(fit_model *const *models, int n_models, const fit_instanc
                     go.C = A.fbuf + (size_t)d * n * A.ldf;
                     go.ldc = A.ldf;
                     go.epi = fitcore::EPI_F32;
-                    rc = fitcore::tc_gemm(true, active, dt.n_reco, h.N_t, A.vhi + vo, h.ldt, dt.rdense_hi, h.ldt, go, s,
-                                          nullptr);
-                    go.epi = fitcore::EPI_F32_ADD;
-                    if (!rc)
-                        rc = fitcore::tc_gemm(true, active, dt.n_reco, h.N_t, A.vhi + vo, h.ldt, dt.rdense_lo, h.ldt,
-                                              go, s, nullptr);
-                    if (!rc)
-                        rc = fitcore::tc_gemm(true, active, dt.n_reco, h.N_t, A.vlo + vo, h.ldt, dt.rdense_hi, h.ldt,
-                                              go, s, nullptr);
+                    rc = fitcore::tc_gemm_split(active, dt.n_reco, h.N_t, A.vhi + vo, A.vlo + vo, h.ldt, dt.rdense_hi,
+                                                dt.rdense_lo, h.ldt, go, s);
                 }
                 if (rc) break;
                 cudaLaunchKernel(kl, dim3(std::max(1, std::min(active * nd, cap_l))), dim3(128), largs, esm, s);
@@ -1901,15 +1894,8 @@ int fit_batch_lockstep(fit_model *const *models, int n_models, const fit_instanc
                     go.C = A.gvbuf + (size_t)d * n * h.ldt;
                     go.ldc = h.ldt;
                     go.epi = fitcore::EPI_F32;
-                    rc = fitcore::tc_gemm(true, active, h.N_t, dt.n_reco, A.ghi + go_, A.ldr, dt.rdt_hi, dt.ldr, go, s,
-                                          nullptr);
-                    go.epi = fitcore::EPI_F32_ADD;
-                    if (!rc)
-                        rc = fitcore::tc_gemm(true, active, h.N_t, dt.n_reco, A.ghi + go_, A.ldr, dt.rdt_lo, dt.ldr, go,
-                                              s, nullptr);
-                    if (!rc)
-                        rc = fitcore::tc_gemm(true, active, h.N_t, dt.n_reco, A.glo + go_, A.ldr, dt.rdt_hi, dt.ldr, go,
-                                              s, nullptr);
+                    rc = fitcore::tc_gemm_split(active, h.N_t, dt.n_reco, A.ghi + go_, A.glo + go_, A.ldr, dt.rdt_hi,
+                                                dt.rdt_lo, dt.ldr, go, s);
                 }
                 if (rc) break;
             }

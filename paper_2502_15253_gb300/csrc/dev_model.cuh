@@ -237,6 +237,11 @@ __device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
     return r;
 }
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
 __device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
     f32x2 r;
     asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
@@ -500,13 +505,6 @@ struct PP {
     float h, l;
 };
 
-__device__ __forceinline__ PP ppair(const DevModel &m, const float *pv, const float *pd, int p,
-                                    float dflt) {
-    if (p < 0) return PP{dflt, 0.f};
-    const float h = pv[p];
-    return PP{h, ((m.theta0_f[p] - h) + pd[p]) + m.theta0_lo[p]};
-}
-
 // the residual l of parameter p, for a vector of them
 __device__ __forceinline__ float presid(const DevModel &m, float h, float delta, int p) {
     return ((m.theta0_f[p] - h) + delta) + m.theta0_lo[p];
@@ -605,23 +603,9 @@ __device__ __forceinline__ void edge_store(const EdgeTab &T, const float *e_edge
 __device__ __forceinline__ float spline_target(const float *u, const EdgeTab &T, int j, int N) {
     const int k0 = T.k[j] & (kEdgeOff - 1), k1 = T.k[j + 1] & (kEdgeOff - 1);
     float acc = 0.f;
-    #pragma unroll 1
+#pragma unroll 1
     for (int k = k0, it = 0; k < k1 && it < 64; ++k, ++it) acc += u[k];
     return acc + (hermite_G(u, k1, T.t[j + 1], N) - hermite_G(u, k0, T.t[j], N));
-}
-
-// v_j for target bin j
-template <class Map>
-__device__ __forceinline__ float spline_target(const float *u, const float *e_edge, const Map &em, int j, int N) {
-    int k0, k1;
-    float t0, t1;
-    bool in0, in1;
-    edge_bin(j, edge_inv_r(e_edge, em, j), N, k0, t0, in0);
-    edge_bin(j + 1, edge_inv_r(e_edge, em, j + 1), N, k1, t1, in1);
-    float acc = 0.f;
-    #pragma unroll 1
-    for (int k = k0, it = 0; k < k1 && it < 64; ++k, ++it) acc += u[k];
-    return acc + (hermite_G(u, k1, t1, N) - hermite_G(u, k0, t0, N));
 }
 
 // Adjoint of the spline remap for source bin i: d(-2lnL)/du_i. With w_e = gv_{e-1} - gv_e the
@@ -637,13 +621,13 @@ __device__ __forceinline__ float spline_adjoint_source(const float *gv, const Ed
     int e = min(max(i + 1 - (int)floorf(T.r[i]), 0), N + 1);
     int k;
     float t;
-    #pragma unroll 1
+#pragma unroll 1
     for (int it = 0; it < 64 && e > 0; ++it) {   // step down while the edge before is past i
         kb(e - 1, k, t);
         if (k <= i) break;
         --e;
     }
-    #pragma unroll 1
+#pragma unroll 1
     for (int it = 0; it < 64 && e <= N; ++it) {  // step up while this edge is not past i
         kb(e, k, t);
         if (k > i) break;
@@ -666,10 +650,10 @@ __device__ __forceinline__ float spline_adjoint_source(const float *gv, const Ed
         g = fmaf(we, c, g);
         return true;
     };
-    #pragma unroll 1
+#pragma unroll 1
     for (int ee = e - 1, it = 0; ee >= 0 && it < 64; --ee, ++it)
         if (!local(ee)) break;
-    #pragma unroll 1
+#pragma unroll 1
     for (int ee = e, it = 0; ee <= N && it < 64; ++ee, ++it)
         if (!local(ee)) break;
     return g;
@@ -1019,13 +1003,13 @@ static __device__ __forceinline__ void st_signal_mode(const DevModel &m, const E
                                                       float *wsb) {
     const int N_t = m.N_t, nth = blockDim.x;
     const bool spline = GEN && m.remap_mode == FIT_REMAP_SPLINE;
-    #pragma unroll 1
+#pragma unroll 1
     for (int i = 0; i < E.n; ++i) {
         const DevDataset &ds = m.ds[E.dl[i]];
         const DsWs ws = carve_ds_ws(wsb + (int64_t)i * m.ws_eval_floats, N_t, m.C, m.max_reco, m.n_osc);
         const PP nrm = E.nrm[i];
         const EMap em = E.em[i];
-        #pragma unroll 1
+#pragma unroll 1
         for (int k = rot_tid(i, (N_t + 31) >> 5); k < N_t; k += nth) {
             const float ih = m.inv_e_hi[k], il = m.inv_e_lo[k];
             const float e0 = m.e_edge[k], e1 = m.e_edge[k + 1];
@@ -1099,11 +1083,11 @@ template <bool GEN>
 static __device__ __forceinline__ void st_remap(const DevModel &m, const EvalShared &E, float *wsb) {
     const int N_t = m.N_t, nth = blockDim.x;
     const bool spline = GEN && m.remap_mode == FIT_REMAP_SPLINE;
-    #pragma unroll 1
+#pragma unroll 1
     for (int i = 0; i < E.n; ++i) {
         const DsWs ws = carve_ds_ws(wsb + (int64_t)i * m.ws_eval_floats, N_t, m.C, m.max_reco, m.n_osc);
         const EMap em = E.em[i];
-        #pragma unroll 1
+#pragma unroll 1
         for (int t = rot_tid(i, (N_t + 31) >> 5); t < N_t; t += nth)
             ws.v[t] = spline ? spline_target(ws.u, ws.edge, t, N_t) : overlap_target(ws.u, ws.edge.t, t, N_t);
     }
@@ -1232,11 +1216,11 @@ __device__ __forceinline__ float bin_mu(const DevModel &m, const EvalShared &E, 
 static __device__ __forceinline__ void st_mu(const DevModel &m, const EvalShared &E, const ParVecs &q, float *wsb,
                                              float *mu) {
     const int nth = blockDim.x;
-    #pragma unroll 1
+#pragma unroll 1
     for (int i = 0; i < E.n; ++i) {
         const DevDataset &ds = m.ds[E.dl[i]];
         const DsWs ws = carve_ds_ws(wsb + (int64_t)i * m.ws_eval_floats, m.N_t, m.C, m.max_reco, m.n_osc);
-        #pragma unroll 1
+#pragma unroll 1
         for (int j = rot_tid(i, (ds.n_reco + 31) >> 5); j < ds.n_reco; j += nth) {
             float tm[kMaxBkgDs], sh[kMaxBkgDs];
             float rest;
@@ -1254,7 +1238,7 @@ template <bool GRAD>
 static __device__ __forceinline__ void st_lik(const DevModel &m, EvalShared &E, const ParVecs &q, const float *data,
                                               float *wsb) {
     const int nth = blockDim.x, lane = threadIdx.x & 31;
-    #pragma unroll 1
+#pragma unroll 1
     for (int i = 0; i < E.n; ++i) {
         const DevDataset &ds = m.ds[E.dl[i]];
         const DsWs ws = carve_ds_ws(wsb + (int64_t)i * m.ws_eval_floats, m.N_t, m.C, m.max_reco, m.n_osc);
@@ -1264,7 +1248,7 @@ static __device__ __forceinline__ void st_lik(const DevModel &m, EvalShared &E, 
         float part[8];   // deviance, d/d eff, d/d rate_b
 #pragma unroll
         for (int b = 0; b < 8; ++b) part[b] = 0.f;
-        #pragma unroll 1
+#pragma unroll 1
         for (int j = t0; j < nr; j += nth) {
             const float n = data[ds.data_off + j], f0 = ws.f0[j];
             float tm[kMaxBkgDs], sh[kMaxBkgDs], rest;
@@ -1300,7 +1284,7 @@ static __device__ __forceinline__ void st_lik(const DevModel &m, EvalShared &E, 
 // on as many warps as they need.
 __device__ __forceinline__ double quad_total(const float *p, int stride, int n, int sub) {
     double s = 0.0;
-    #pragma unroll 1
+#pragma unroll 1
     for (int w = sub; w < n; w += 4) s += (double)p[w * stride];
     s += __shfl_xor_sync(0xffffffffu, s, 1);
     s += __shfl_xor_sync(0xffffffffu, s, 2);
@@ -1313,7 +1297,7 @@ __device__ __forceinline__ double quad_total(const float *p, int stride, int n, 
 template <bool GRAD>
 static __device__ __forceinline__ void lik_finish(const DevModel &m, EvalShared &E, float *grad) {
     const int nw = blockDim.x >> 5, sub = threadIdx.x & 3;
-    #pragma unroll 1
+#pragma unroll 1
     for (int v0 = 0; v0 < 8 * E.n; v0 += blockDim.x >> 2) {
         const int v = v0 + (int)(threadIdx.x >> 2), i = v >> 3, q = v & 7;
         if ((v & ~7) >= 8 * E.n) break;   // uniform over the warp
@@ -1337,14 +1321,14 @@ static __device__ __forceinline__ void lik_finish(const DevModel &m, EvalShared 
 // in E.dup, in order.
 static __device__ __forceinline__ void lik_dups(const DevModel &m, EvalShared &E, float *grad) {
     double nll = E.nll;
-    #pragma unroll 1
+#pragma unroll 1
     for (int i = 0; i < E.n; ++i) nll += E.nll_ds[i];
     E.nll = nll;
     if (grad == nullptr) return;
-    #pragma unroll 1
+#pragma unroll 1
     for (int i = 0; i < E.n; ++i) {
         const DevDataset &ds = m.ds[E.dl[i]];
-        #pragma unroll 1
+#pragma unroll 1
         for (int left = ds.lik_dup; left; left &= left - 1) {
             const int q = __ffs(left) - 1;
             const int p = q == 1 ? ds.eff_idx : m.bkg[ds.bkg_begin + q - 2].rate_idx;
@@ -1356,13 +1340,13 @@ static __device__ __forceinline__ void lik_dups(const DevModel &m, EvalShared &E
 // Background-shape gradient: a thread per shape parameter sums its (background, bin) pairs of
 // the group's datasets in a fixed order (several datasets may share a shape).
 static __device__ __forceinline__ void st_bkg_shape(const DevModel &m, const EvalShared &E, float *wsb, float *grad) {
-    #pragma unroll 1
+#pragma unroll 1
     for (int p = threadIdx.x; p < m.n_bs; p += blockDim.x) {
         float s = 0.f;
-        #pragma unroll 1
+#pragma unroll 1
         for (int r = m.bs_ptr[p]; r < m.bs_ptr[p + 1]; ++r) {
             const BkgShapeRef ref = m.bs_ref[r];
-            #pragma unroll 1
+#pragma unroll 1
             for (int i = 0; i < E.n; ++i) {
                 if (E.dl[i] != ref.d) continue;
                 const DsWs ws = carve_ds_ws(wsb + (int64_t)i * m.ws_eval_floats, m.N_t, m.C, m.max_reco, m.n_osc);
@@ -1398,7 +1382,7 @@ static __device__ __forceinline__ void st_adjoint_rest_n(const DevModel &m, Eval
     for (int j = 0; j < NOSC; ++j) eo[j] = 0.f;
 #pragma unroll
     for (int c = 0; c < NC; ++c) ec[c] = 0.f;
-    #pragma unroll 1
+#pragma unroll 1
     for (int i = 0; i < E.n; ++i) {
         const DevDataset &ds = m.ds[E.dl[i]];
         const DsWs ws = carve_ds_ws(wsb + (int64_t)i * m.ws_eval_floats, N_t, C, m.max_reco, m.n_osc);
@@ -1406,7 +1390,7 @@ static __device__ __forceinline__ void st_adjoint_rest_n(const DevModel &m, Eval
         const PP nrm = E.nrm[i];
         const float *gv = ws.v;
         float ep[4] = {0.f, 0.f, 0.f, 0.f};   // d/da0, d/da1, d/da2, d/d norm
-        #pragma unroll 1
+#pragma unroll 1
         for (int k = rot_tid(i, (N_t + 31) >> 5); k < N_t; k += nth) {
             float gu = 0.f;
             if (spline) {
@@ -1421,7 +1405,7 @@ static __device__ __forceinline__ void st_adjoint_rest_n(const DevModel &m, Eval
                 const float w = 1.f + (d1 - d0), iw = 1.f / w;
                 const int f0i = (int)floorf(d0), f1i = (int)floorf(d1);
                 const int t0 = k + f0i, t1 = k + 1 + f1i;
-                #pragma unroll 1
+#pragma unroll 1
                 for (int t = max(t0, 0); t <= min(t1, N_t - 1); ++t) {
                     const float ylo = (float)(k - t) + d0, yhi = (float)(k + 1 - t) + d1;
                     const float ov = fminf(yhi, 1.f) - fmaxf(ylo, 0.f);
@@ -1476,7 +1460,7 @@ static __device__ __forceinline__ void st_adjoint_finish(const DevModel &m, Eval
         // totals: four per dataset, then the survival parameters and powers; four lanes each,
         // from the last warp down (the shapes below start at the first)
         const int nmap = 4 * E.n, nv = nmap + NOSC + m.C, sub = tid & 3;
-        #pragma unroll 1
+#pragma unroll 1
         for (int v0 = 0; v0 < nv; v0 += nth >> 2) {
             const int v = v0 + ((nth - 1 - tid) >> 2);
             if (v0 + (((nth - 1 - (tid | 31))) >> 2) >= nv) break;   // uniform over the warp
@@ -1499,7 +1483,7 @@ static __device__ __forceinline__ void st_adjoint_finish(const DevModel &m, Eval
     if (m.any_map_dup) {
         __syncthreads();
         if (tid == 0) {
-            #pragma unroll 1
+#pragma unroll 1
             for (int v = 0; v < 4 * E.n + NOSC + m.C; ++v) {
                 const bool map = v < 4 * E.n;
                 const int q = map ? (v & 3) : v - 4 * E.n;
@@ -1510,22 +1494,22 @@ static __device__ __forceinline__ void st_adjoint_finish(const DevModel &m, Eval
         }
     }
     if (m.shared_roles) __syncthreads();
-    #pragma unroll 1
+#pragma unroll 1
     for (int i = 0; i < E.n; ++i) {
         const DevDataset &ds = m.ds[E.dl[i]];
         const float *gs = carve_ds_ws(wsb + (int64_t)i * m.ws_eval_floats, m.N_t, m.C, m.max_reco, m.n_osc).dp;
         const int L = ds.sp_lanes, per = nth / L;   // lanes per parameter, parameters per pass
         const int work = ds.n_sp * L;
-        #pragma unroll 1
+#pragma unroll 1
         for (int q0 = rot_tid(i, (work + 31) >> 5); q0 < ((work + 31) & ~31); q0 += per * L) {
             const int p = q0 / L, sub = q0 & (L - 1);
             const int4 sp = p < ds.n_sp ? ds.sp[p] : make_int4(0, 0, 0, 1);
             float s = 0.f;
             if (sp.w)
-                #pragma unroll 1
+#pragma unroll 1
                 for (int r = sub; r < sp.z; r += L) s += gs[sp.y + r];
             else
-                #pragma unroll 1
+#pragma unroll 1
                 for (int r = sub; r < sp.z; r += L) s += gs[ds.sp_k[sp.y + r]];
             for (int o = L >> 1; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
             if (p < ds.n_sp && sub == 0) grad[sp.x] += s;
@@ -1570,7 +1554,7 @@ static __device__ double eval_datasets(const DevModel &m, EvalShared &E, const P
         E.status = 0;
         E.nll = 0.0;
     }
-    #pragma unroll 1
+#pragma unroll 1
     for (int first = 0; first < m.n_ds;) {
         first = eval_setup_any<GEN>(m, E, q, mask, first, m.ws_group);
         if (E.n > 0) {
@@ -1611,7 +1595,7 @@ template <bool GEN>
 static __device__ void expected_datasets(const DevModel &m, EvalShared &E, const ParVecs &q, float *wsb, float *mu) {
     __syncthreads();
     if (threadIdx.x == 0) E.status = 0;
-    #pragma unroll 1
+#pragma unroll 1
     for (int first = 0; first < m.n_ds;) {
         first = eval_setup_any<GEN>(m, E, q, 0xffffffffu, first, m.ws_group);
         if (E.n > 0) {
@@ -1654,7 +1638,6 @@ static __device__ __noinline__ void tri_apply(const DevModel &m, const TriTile *
         const int *idx = m.blk_idx + T.idx;
         const bool seq = T.in0 >= 0;
         float4 s[2] = {make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f)};
-        #pragma unroll 1
         int c = 0;
         auto add = [](float4 &a, const float4 &r, float v) {
             a.x = fmaf(r.x, v, a.x);
@@ -1692,7 +1675,7 @@ __device__ __forceinline__ float tri_sum(const DevModel &m, const float *part, i
     const int x = m.tri_seg[row];
     const int s0 = upper ? (x >> 8) & 255 : 0, s1 = upper ? x >> 16 : x & 255;
     float t = part[s0 * m.tri_rows + row];
-    #pragma unroll 1
+#pragma unroll 1
     for (int q = s0 + 1; q < s1; ++q) t += part[q * m.tri_rows + row];
     return t;
 }

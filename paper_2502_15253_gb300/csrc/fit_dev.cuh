@@ -14,8 +14,7 @@ __device__ __forceinline__ void copy_model(DevModel *dst, const DevModel *src) {
     const int *s = reinterpret_cast<const int *>(src);
     int *d = reinterpret_cast<int *>(dst);
 #pragma unroll 4
-    #pragma unroll 1
-    #pragma unroll 1
+#pragma unroll 1
     for (int i = threadIdx.x; i < n; i += blockDim.x) d[i] = s[i];
     __syncthreads();
 }
@@ -112,8 +111,7 @@ __device__ __forceinline__ FitVecs carve_fit_vecs(float *base, float *hbase, int
 // block-wide dot product of two P-vectors (double result on every thread)
 __device__ __forceinline__ double bdot(const float *a, const float *b, int n, double *red) {
     float acc = 0.f;
-    #pragma unroll 1
-    #pragma unroll 1
+#pragma unroll 1
     for (int i = threadIdx.x; i < n; i += blockDim.x) acc = fmaf(a[i], b[i], acc);
     return block_sum(acc, red);
 }
@@ -128,11 +126,11 @@ static __device__ __noinline__ void fused_dots(const float *Sv, const float *Yv,
     const int pitch = fit_vec_pitch(P), n4 = P >> 2, tail = (P & ~3) + lane;
     const int live = __popc(occ);
     const float *yn = ynew ? ynew : g;
-    #pragma unroll 1
+#pragma unroll 1
     for (int w = warp; w <= live; w += nw) {
         if (w == live) {   // g.g
             float acc = 0.f;
-            #pragma unroll 1
+#pragma unroll 1
             for (int k = lane; k < n4; k += 32) {
                 const float4 x = reinterpret_cast<const float4 *>(g)[k];
                 acc = fmaf(x.x, x.x, fmaf(x.y, x.y, fmaf(x.z, x.z, fmaf(x.w, x.w, acc))));
@@ -144,12 +142,12 @@ static __device__ __noinline__ void fused_dots(const float *Sv, const float *Yv,
             continue;
         }
         unsigned left = occ;   // the w-th occupied slot
-        #pragma unroll 1
+#pragma unroll 1
         for (int i = 0; i < w; ++i) left &= left - 1;
         const int j = __ffs(left) - 1;
         const float *s = Sv + (int64_t)j * pitch, *y = Yv + (int64_t)j * pitch;
         float acc[4] = {0.f, 0.f, 0.f, 0.f};
-        #pragma unroll 1
+#pragma unroll 1
         for (int k = lane; k < n4; k += 32) {
             const float4 a = reinterpret_cast<const float4 *>(s)[k], b = reinterpret_cast<const float4 *>(y)[k];
             const float4 u = reinterpret_cast<const float4 *>(yn)[k], v = reinterpret_cast<const float4 *>(g)[k];
@@ -246,7 +244,7 @@ static __device__ double lbfgs_scalars(FitSmem &S, int hist_max, bool pending) {
     const double rho = live ? st.rho[sl] : 0.0;
     // alpha_k = rho_k (s_k.g - sum_{l > k} alpha_l s_k.y_l), newest first; u_k = sum_l alpha_l y_k.y_l
     double a = rho * sg, alpha = 0.0, u = 0.0;
-    #pragma unroll 1
+#pragma unroll 1
     for (int l = hn - 1; l >= 0; --l) {
         const int sll = slot_of(l);
         const double rs = lane < l ? rho * st.SY[sl][sll] : 0.0, yy = live ? st.YY[sl][sll] : 0.0;
@@ -257,7 +255,7 @@ static __device__ double lbfgs_scalars(FitSmem &S, int hist_max, bool pending) {
     }
     // beta_k = rho_k (gam (y_k.g - u_k) + sum_{l < k} (alpha_l - beta_l) s_l.y_k), oldest first
     double b = rho * (gam * (yg - u)), beta = 0.0;
-    #pragma unroll 1
+#pragma unroll 1
     for (int l = 0; l < hn; ++l) {
         const double rs = live && lane > l ? rho * st.SY[slot_of(l)][sl] : 0.0;
         const double al = __shfl_sync(0xffffffffu, alpha, l), bl = __shfl_sync(0xffffffffu, b, l);
@@ -296,7 +294,7 @@ static __device__ __noinline__ void theta_of_z(const DevModel &m, const float *z
         V.pv[i] = h;
         V.pl[i] = presid(m, h, d, i);
     };
-    #pragma unroll 1
+#pragma unroll 1
     for (int i = tid; i < m.P; i += nth) {
         const float s = m.zscale[i];
         if (s > 0.f) put(i, s * z[i]);
@@ -304,7 +302,7 @@ static __device__ __noinline__ void theta_of_z(const DevModel &m, const float *z
     if (m.tri_rows > 0) {
         tri_apply(m, m.tri_lo, m.n_tri_lo, m.L_lo, z, part);
         __syncthreads();
-        #pragma unroll 1
+#pragma unroll 1
         for (int r = tid; r < m.tri_rows; r += nth) put(m.tri_param[r], tri_sum(m, part, r, false));
     }
     __syncthreads();
@@ -317,7 +315,7 @@ static __device__ double eval_z_prior(const DevModel &m, const float *z, const f
                                double *red) {
     const int tid = threadIdx.x, nth = blockDim.x;
     float acc = 0.f;
-    #pragma unroll 1
+#pragma unroll 1
     for (int i = tid; i < m.P; i += nth) {
         const float s = m.zscale[i];
         if (s > 0.f) {
@@ -329,7 +327,7 @@ static __device__ double eval_z_prior(const DevModel &m, const float *z, const f
     if (m.tri_rows > 0) {
         tri_apply(m, m.tri_up, m.n_tri_up, m.L_up, gth, part);
         __syncthreads();
-        #pragma unroll 1
+#pragma unroll 1
         for (int r = tid; r < m.tri_rows; r += nth) {
             const int p = m.tri_param[r];
             const float zj = z[p];
@@ -345,7 +343,7 @@ static __device__ double eval_z_prior(const DevModel &m, const float *z, const f
 // blocks can be held (their z coordinate is the parameter itself, scaled).
 __device__ __forceinline__ void hold_fixed(const uint8_t *fixed, float *gz, int P) {
     if (fixed == nullptr) return;
-    #pragma unroll 1
+#pragma unroll 1
     for (int i = threadIdx.x; i < P; i += blockDim.x)
         if (fixed[i]) gz[i] = 0.f;
 }
@@ -364,7 +362,7 @@ static __device__ __noinline__ void pre_apply(const DevModel &m, const float *co
     const int nfull = P >> 2;
     const float4 *x4 = reinterpret_cast<const float4 *>(x);
     // four rows per warp and pass, so that their loads are in flight together
-    #pragma unroll 1
+#pragma unroll 1
     for (int k0 = warp; k0 < r; k0 += 4 * nw) {
         const float4 *q4[4];
 #pragma unroll
@@ -397,11 +395,11 @@ static __device__ __noinline__ void pre_apply(const DevModel &m, const float *co
         if ((lane & 7) == 0 && k < r) u[k] = __ldg(coef + k) * t;
     }
     __syncthreads();
-    #pragma unroll 1
+#pragma unroll 1
     for (int i = threadIdx.x; i < P; i += blockDim.x) {
         float acc = x[i];
         if (!(fixed && fixed[i])) {
-            #pragma unroll 1
+#pragma unroll 1
             for (int k0 = 0; k0 < r; k0 += 16) {   // sixteen rows' loads in flight
                 float q[16];
 #pragma unroll
@@ -421,7 +419,7 @@ template <bool GEN>
 static __device__ double eval_z(const DevModel &m, const float *z, float *gz, FitVecs &V, float *ws,
                          const float *data, uint32_t mask, FitSmem &S, const uint8_t *fixed) {
     theta_of_z(m, z, V, ws);
-    #pragma unroll 1
+#pragma unroll 1
     for (int i = threadIdx.x; i < m.P; i += blockDim.x) V.gth[i] = 0.f;
     const double nll = eval_datasets<GEN, true>(m, S.E, ParVecs{V.pv, V.pd, V.pl}, mask, data, ws, V.gth);
     if (S.E.status) return INFINITY;
@@ -689,21 +687,21 @@ static __device__ bool fit_decide(FitSmem &S, FitVecs &V, int P, double fa, cons
     __syncthreads();
     const FitStep q = S.step;
     if (q.init) {
-        #pragma unroll 1
+#pragma unroll 1
         for (int i = tid; i < P; i += nth) {
             V.z[i] = V.zt[i];
             V.g[i] = V.gt[i];
         }
     }
     if (q.save_cr) {
-        #pragma unroll 1
+#pragma unroll 1
         for (int i = tid; i < P; i += nth) {
             V.zcr[i] = V.zt[i];
             V.gcr[i] = V.gt[i];
         }
     }
     if (q.save_lo) {
-        #pragma unroll 1
+#pragma unroll 1
         for (int i = tid; i < P; i += nth) {
             V.zlo[i] = V.zt[i];
             V.glo[i] = V.gt[i];
@@ -713,7 +711,7 @@ static __device__ bool fit_decide(FitSmem &S, FitVecs &V, int P, double fa, cons
         const float *zs = q.src == 1 ? V.zt : q.src == 2 ? V.zcr : V.zlo;
         const float *gs = q.src == 1 ? V.gt : q.src == 2 ? V.gcr : V.glo;
         const int64_t c = (int64_t)S.st.head * fit_vec_pitch(P);
-        #pragma unroll 1
+#pragma unroll 1
         for (int i = tid; i < P; i += nth) {
             const float zn = zs[i], gn = gs[i];
             V.S[c + i] = zn - V.z[i];
@@ -723,7 +721,7 @@ static __device__ bool fit_decide(FitSmem &S, FitVecs &V, int P, double fa, cons
         }
     }
     if (q.next == kNextTrial) {   // the next point along the same direction
-        #pragma unroll 1
+#pragma unroll 1
         for (int i = tid; i < P; i += nth) V.zt[i] = fmaf(q.alpha, V.d[i], V.z[i]);
         __syncthreads();
         return true;
@@ -748,11 +746,11 @@ static __device__ bool fit_decide(FitSmem &S, FitVecs &V, int P, double fa, cons
         // loads in flight per thread
         const float cg = S.cg, af = S.step.alpha;
         const int n = S.n_dir, Pp = fit_vec_pitch(P);
-        #pragma unroll 1
+#pragma unroll 1
         for (int i = tid; i < P; i += nth) {
             float h = cg * V.g[i];
             int k = 0;
-            #pragma unroll 1
+#pragma unroll 1
             for (; k + 7 < n; k += 8) {
                 float s[8], y[8];
 #pragma unroll
@@ -764,7 +762,7 @@ static __device__ bool fit_decide(FitSmem &S, FitVecs &V, int P, double fa, cons
 #pragma unroll
                 for (int u = 0; u < 8; ++u) h = fmaf(S.cy[k + u], y[u], fmaf(S.cs[k + u], s[u], h));
             }
-            #pragma unroll 1
+#pragma unroll 1
             for (; k < n; ++k) {
                 const int64_t o = (int64_t)S.slot[k] * Pp + i;
                 h = fmaf(S.cy[k], V.Y[o], fmaf(S.cs[k], V.S[o], h));
@@ -796,7 +794,7 @@ __device__ __forceinline__ void init_state(FitState &st) {
 // pd is scratch, part as in theta_of_z. Ends with a barrier.
 static __device__ void start_z(const DevModel &m, const double *st, float *z, float *pd, float *part) {
     const int tid = threadIdx.x, P = m.P, nth = blockDim.x;
-    #pragma unroll 1
+#pragma unroll 1
     for (int i = tid; i < P; i += nth) {
         const float dd = st ? (float)(st[i] - m.theta0[i]) : 0.f;
         pd[i] = dd;
@@ -807,7 +805,7 @@ static __device__ void start_z(const DevModel &m, const double *st, float *z, fl
     if (m.tri_rows > 0) {
         tri_apply(m, m.tri_lo, m.n_tri_lo, m.W_lo, pd, part);
         __syncthreads();
-        #pragma unroll 1
+#pragma unroll 1
         for (int r = tid; r < m.tri_rows; r += nth) z[m.tri_param[r]] = tri_sum(m, part, r, false);
     }
     __syncthreads();
@@ -819,7 +817,7 @@ static __device__ void start_z(const DevModel &m, const double *st, float *z, fl
 static __device__ void write_result(const DevModel &m, const FitState &st, const float *z, double *best,
                              fit_result *out, const double *start, const uint8_t *fixed) {
     const int tid = threadIdx.x;
-    #pragma unroll 1
+#pragma unroll 1
     for (int i = tid; i < m.P; i += blockDim.x) {
         const float s = m.zscale[i];
         if (fixed && fixed[i]) best[i] = start ? start[i] : m.theta0[i];
@@ -831,16 +829,16 @@ static __device__ void write_result(const DevModel &m, const FitState &st, const
         // a thread per row over L^T (coalesced), four partial sums so that the products of one
         // row do not wait for one another
         const double *Lt = m.blk_L64 + m.blk_mat_off[b] + (int64_t)n * n;
-        #pragma unroll 1
+#pragma unroll 1
         for (int i = tid; i < n; i += blockDim.x) {
             double s[4] = {0.0, 0.0, 0.0, 0.0};
             int j = 0;
-            #pragma unroll 1
+#pragma unroll 1
             for (; j + 3 <= i; j += 4) {
 #pragma unroll
                 for (int u = 0; u < 4; ++u) s[u] = fma(Lt[(int64_t)(j + u) * n + i], (double)z[idx[j + u]], s[u]);
             }
-            #pragma unroll 1
+#pragma unroll 1
             for (; j <= i; ++j) s[0] = fma(Lt[(int64_t)j * n + i], (double)z[idx[j]], s[0]);
             best[idx[i]] = m.theta0[idx[i]] + ((s[0] + s[1]) + (s[2] + s[3]));
         }
@@ -892,7 +890,7 @@ __global__ void __launch_bounds__(T, MINB) fit_kernel(FitArgs A) {
             if (tid == 0) {
                 const uint32_t mk = in.mask & ((1u << S.m.n_ds) - 1u);
                 const PreEntry *e = A.pre_tab + (int64_t)in.model * A.pre_per_model;
-                #pragma unroll 1
+#pragma unroll 1
                 for (int k = 0; k < A.pre_per_model; ++k)
                     if (e[k].Q && e[k].mask == mk) {
                         S.m.pre_Q = e[k].Q;
@@ -920,7 +918,7 @@ __global__ void __launch_bounds__(T, MINB) fit_kernel(FitArgs A) {
         if (tid == 0) init_state(S.st);
         __syncthreads();
         if (global_ns() > F.deadline) {
-            #pragma unroll 1
+#pragma unroll 1
             for (int i = tid; i < P; i += blockDim.x) V.z[i] = 0.f;
             if (tid == 0) S.st.status = FIT_STATUS_TIMEOUT;
             __syncthreads();

@@ -37,6 +37,12 @@ struct GemmOut {
     bool deterministic = false;
 };
 
+// C = (Ah + Al)(Bh + Bl)^T without Al Bl^T (FP32 operands as a TF32-exact part and the rest: the split
+// product that keeps FP32 accuracy), one launch: the three products Ah Bl^T, Al Bh^T and Ah Bh^T
+// accumulate in tensor memory one after another. Epilogue EPI_F32 only.
+int tc_gemm_split(int M, int N, int K, const float *Ah, const float *Al, int lda, const float *Bh, const float *Bl,
+                  int ldb, const GemmOut &out, cudaStream_t stream);
+
 // Returns 0, or a negative FIT_ERR_* code (message through the library's error string).
 // A: M x K, lda elements per row; B: N x K, ldb per row; element type bf16 (tf32 = false) or
 // float (tf32 = true). Rows of A and B must start 16-byte aligned. err: device int that the

@@ -14,7 +14,7 @@ __device__ double prior_theta(const DevModel &m, const float *pd, float *grad, f
     const int tid = threadIdx.x, nth = blockDim.x;
     __syncthreads();
     float acc = 0.f;
-    #pragma unroll 1
+#pragma unroll 1
     for (int i = tid; i < m.P; i += nth) {
         const float pi = m.prior_inv[i];
         if (pi > 0.f) {
@@ -26,7 +26,7 @@ __device__ double prior_theta(const DevModel &m, const float *pd, float *grad, f
     if (m.tri_rows > 0) {
         tri_apply(m, m.tri_lo, m.n_tri_lo, m.W_lo, pd, part);
         __syncthreads();
-        #pragma unroll 1
+#pragma unroll 1
         for (int r = tid; r < m.tri_rows; r += nth) {
             const float z = tri_sum(m, part, r, false);
             zs[m.tri_param[r]] = z;
@@ -36,7 +36,7 @@ __device__ double prior_theta(const DevModel &m, const float *pd, float *grad, f
         if (grad) {
             tri_apply(m, m.tri_up, m.n_tri_up, m.W_up, zs, part);
             __syncthreads();
-            #pragma unroll 1
+#pragma unroll 1
             for (int r = tid; r < m.tri_rows; r += nth) grad[m.tri_param[r]] += 2.f * tri_sum(m, part, r, true);
         }
     }
@@ -70,7 +70,7 @@ __global__ void __launch_bounds__(T, MINB) eval_kernel(EvalArgs A) {
 
     for (int b = blockIdx.x; b < A.B; b += gridDim.x) {
         const double *th = A.theta + (int64_t)b * P;
-        #pragma unroll 1
+#pragma unroll 1
         for (int i = threadIdx.x; i < P; i += blockDim.x) {
             const double t = th[i];
             const float h = (float)t, d = (float)(t - m.theta0[i]);
@@ -98,7 +98,7 @@ __global__ void __launch_bounds__(T, MINB) eval_kernel(EvalArgs A) {
         }
         __syncthreads();
         if (want_grad)
-            #pragma unroll 1
+#pragma unroll 1
             for (int i = threadIdx.x; i < P; i += blockDim.x) A.grad[(int64_t)b * P + i] = st ? NAN : grad[i];
         __syncthreads();
     }
@@ -202,7 +202,7 @@ __global__ void __launch_bounds__(128) ls_init_kernel(LsArgs A) {
 __device__ __forceinline__ ParVecs ls_params_in(const LsArgs &A, int g, int P, float *pv) {
     const FitVecs V = ls_vecs(A, g, P);
     float *pd = pv + fit_vec_pitch(P), *pl = pd + fit_vec_pitch(P);
-    #pragma unroll 1
+#pragma unroll 1
     for (int i = threadIdx.x; i < P; i += blockDim.x) {
         pv[i] = V.pv[i];
         pd[i] = V.pd[i];
@@ -465,7 +465,7 @@ __global__ void __launch_bounds__(128) ls_step_kernel(LsArgs A) {
         copy_state(&S.st, A.state + g);
         // theta gradient = sum of the dataset slices in a fixed order; the slices are cleared
         float *gs = A.gsl + (int64_t)g * nd * P;
-        #pragma unroll 1
+#pragma unroll 1
         for (int i = threadIdx.x; i < P; i += blockDim.x) {
             float t = 0.f;
             for (int d = 0; d < nd; ++d) {

@@ -1164,8 +1164,7 @@ int fit_warmstart_predict(fit_mlp *mlp, const fit_model *model, int B, const flo
         rc = fail(FIT_ERR_CUDA, "fit_warmstart_predict: upload");
     if (!rc) rc = fit_mlp_forward(mlp, B, x, out, stream);
     if (!rc)
-        rc = fitcore::starts(B, model->n_params, model->host.theta0, n_targets, idx, scl, out, n_out, theta_out,
-                             theta_out, s);
+        rc = fitcore::starts(B, model->n_params, n_targets, idx, scl, out, n_out, theta_out, s);
     for (void *p : {(void *)out, (void *)idx, (void *)scl})
         if (p) cudaFreeAsync(p, s);
     if (!rc && cudaStreamSynchronize(s) != cudaSuccess) rc = fail(FIT_ERR_CUDA, "fit_warmstart_predict: sync");

@@ -156,8 +156,8 @@ int mle_targets(int B, int P, int D, const double *theta, const double *theta0, 
 int lin_residual_targets(int B, int D, int n_t, const float *Kt, const float *mu0, const float *cnt, int n_var,
                          const uint32_t *choices, const uint32_t *masks, int n_out, const int *status, float *y,
                          cudaStream_t s);
-int starts(int B, int P, const double *theta0, int n_t, const int *idx, const double *scale, const float *out,
-           int n_out, const double *base, double *theta, cudaStream_t s);
+int starts(int B, int P, int n_t, const int *idx, const double *scale, const float *out, int n_out, double *theta,
+           cudaStream_t s);
 size_t fit_smem_bytes(int floats);
 // Fit vectors are spaced by P rounded up to 4 floats, so that every vector starts on a
 // 16-byte boundary and the history can be read as float4.

@@ -169,11 +169,11 @@ int expected_tc(const DevModel &h, const DevModel *dev, int B, const double *the
         for (float *p : {vhi, vlo, F, pv, pl})
             if (p) cudaFreeAsync(p, s);
     };
-    if (cudaMallocAsync(&vhi, sizeof(float) * (size_t)nds * B * ldt, s) ||
-        cudaMallocAsync(&vlo, sizeof(float) * (size_t)nds * B * ldt, s) ||
-        cudaMallocAsync(&F, sizeof(float) * (size_t)nds * B * ldf, s) ||
-        cudaMallocAsync(&pv, sizeof(float) * (size_t)B * h.P, s) ||
-        cudaMallocAsync(&pl, sizeof(float) * (size_t)B * h.P, s)) {
+    if (fitcore::pool_alloc(&vhi, sizeof(float) * (size_t)nds * B * ldt, s) ||
+        fitcore::pool_alloc(&vlo, sizeof(float) * (size_t)nds * B * ldt, s) ||
+        fitcore::pool_alloc(&F, sizeof(float) * (size_t)nds * B * ldf, s) ||
+        fitcore::pool_alloc(&pv, sizeof(float) * (size_t)B * h.P, s) ||
+        fitcore::pool_alloc(&pl, sizeof(float) * (size_t)B * h.P, s)) {
         cudaGetLastError();
         cleanup();
         return fitcore_fail(FIT_ERR_OOM, "fit_model_expected_tc: workspace");

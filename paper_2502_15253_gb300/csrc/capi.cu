@@ -18,6 +18,53 @@ int mlp_dims(const fit_mlp *m, int *n_in, int *n_out);
 using fitcore::DevModel;
 
 namespace {
+std::mutex g_pool_mutex;
+std::vector<cudaMemPool_t> g_pools;   // by device, made with its first object; nullptr: none
+int g_pool_users = 0;
+}  // namespace
+
+namespace fitcore {
+
+cudaError_t pool_alloc_bytes(void **p, size_t bytes, cudaStream_t s) {
+    int dev = 0;
+    const cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    cudaMemPool_t pool = nullptr;
+    {
+        std::lock_guard<std::mutex> lock(g_pool_mutex);
+        if (dev < (int)g_pools.size()) pool = g_pools[dev];
+    }
+    return pool ? cudaMallocFromPoolAsync(p, bytes, pool, s) : cudaMallocAsync(p, bytes, s);
+}
+
+void pool_user(int change) {
+    std::lock_guard<std::mutex> lock(g_pool_mutex);
+    g_pool_users += change;
+    int dev = 0;
+    if (change > 0 && cudaGetDevice(&dev) == cudaSuccess) {
+        if ((int)g_pools.size() <= dev) g_pools.resize(dev + 1, nullptr);
+        if (g_pools[dev]) return;
+        cudaMemPoolProps props = {};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = dev;
+        uint64_t keep = kPoolKeep;
+        cudaMemPool_t made = nullptr;
+        if (cudaMemPoolCreate(&made, &props) != cudaSuccess) {
+            cudaGetLastError();   // no pool: the default one serves
+            return;
+        }
+        if (cudaMemPoolSetAttribute(made, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) cudaGetLastError();
+        g_pools[dev] = made;
+    }
+    if (g_pool_users > 0) return;
+    for (cudaMemPool_t pool : g_pools)
+        if (pool && cudaMemPoolTrimTo(pool, 0) != cudaSuccess) cudaGetLastError();
+}
+
+}  // namespace fitcore
+
+namespace {
 
 thread_local std::string g_err;
 thread_local int64_t g_launches = 0;
@@ -198,7 +245,7 @@ int stage_in(const void *src, size_t bytes, cudaStream_t s, Staged &out) {
         out.dev = const_cast<void *>(src);
         return FIT_OK;
     }
-    FIT_CUDA(cudaMallocAsync(&out.dev, bytes, s));
+    FIT_CUDA(fitcore::pool_alloc(&out.dev, bytes, s));
     out.owned = true;
     FIT_CUDA(cudaMemcpyAsync(out.dev, src, bytes, cudaMemcpyHostToDevice, s));
     return FIT_OK;
@@ -215,7 +262,7 @@ int stage_out(void *dst, size_t bytes, cudaStream_t s, Staged &out, bool &host) 
         return FIT_OK;
     }
     host = true;
-    FIT_CUDA(cudaMallocAsync(&out.dev, bytes, s));
+    FIT_CUDA(fitcore::pool_alloc(&out.dev, bytes, s));
     out.owned = true;
     return FIT_OK;
 }
@@ -259,6 +306,7 @@ struct fit_model {
     std::vector<std::string> names;   // parameter names (models created from a configuration)
     std::vector<double> sigma;        // prior width per parameter (block members: sqrt(V_ii))
     int device = -1;                  // the CUDA device holding the model's memory
+    bool counted = false;             // created in full (fitcore::pool_user)
 };
 
 // error / launch-count hooks for the other translation units of the library
@@ -345,6 +393,7 @@ void fit_model_destroy(fit_model *model) {
     for (auto &le : model->lin)
         if (le.K) cudaFree(le.K);
     if (model->lin_mu0) cudaFree(model->lin_mu0);
+    if (model->counted) fitcore::pool_user(-1);
     delete model;
 }
 
@@ -957,6 +1006,8 @@ int fit_model_create(const fit_model_desc *d, fit_model **out) {
             return rc;
         }
     }
+    M->counted = true;
+    fitcore::pool_user(1);
     *out = M;
     return FIT_OK;
 }
@@ -979,7 +1030,7 @@ static int launch_eval(fit_model *model, int B, const double *theta_d, const flo
     if (per_sm < 1) return fail(FIT_ERR_INVALID_CONFIG, "fit_model_eval: model too large for one block");
     const int grid = std::max(1, std::min(B, per_sm * cfg.sms));
     float *ws = nullptr;
-    if (!in_smem) FIT_CUDA(cudaMallocAsync(&ws, sizeof(float) * (size_t)grid * h.ws_floats, s));
+    if (!in_smem) FIT_CUDA(fitcore::pool_alloc(&ws, sizeof(float) * (size_t)grid * h.ws_floats, s));
     fitcore::EvalArgs a{model->dev, B, theta_d, data_d, masks_d, nll_d, grad_d, mu_d, st_d, ws, in_smem ? 1 : 0};
     void *args[] = {&a};
     const cudaError_t e = cudaLaunchKernel(L.func, dim3(grid), dim3(L.threads), args, smem, s);
@@ -1086,7 +1137,7 @@ int fit_model_expected_tc(fit_model *model, int B, const double *theta, float *m
         if (status_out) {
             rc = stage_out(status_out, sizeof(int) * B, s, st, hst);
         } else {
-            if (cudaMallocAsync(&st.dev, sizeof(int) * B, s)) rc = fail(FIT_ERR_OOM, "fit_model_expected_tc: status");
+            if (fitcore::pool_alloc(&st.dev, sizeof(int) * B, s)) rc = fail(FIT_ERR_OOM, "fit_model_expected_tc: status");
             st.owned = true;
         }
     }
@@ -1156,8 +1207,8 @@ int fit_warmstart_predict(fit_mlp *mlp, const fit_model *model, int B, const flo
     float *out = nullptr;
     int *idx = nullptr;
     double *scl = nullptr;
-    if (!rc && (cudaMallocAsync(&out, sizeof(float) * (size_t)B * n_out, s) ||
-                cudaMallocAsync(&idx, sizeof(int) * n_targets, s) || cudaMallocAsync(&scl, sizeof(double) * n_targets, s)))
+    if (!rc && (fitcore::pool_alloc(&out, sizeof(float) * (size_t)B * n_out, s) ||
+                fitcore::pool_alloc(&idx, sizeof(int) * n_targets, s) || fitcore::pool_alloc(&scl, sizeof(double) * n_targets, s)))
         rc = fail(FIT_ERR_OOM, "fit_warmstart_predict: workspace");
     if (!rc && (cudaMemcpyAsync(idx, target_idx, sizeof(int) * n_targets, cudaMemcpyHostToDevice, s) ||
                 cudaMemcpyAsync(scl, target_scale, sizeof(double) * n_targets, cudaMemcpyHostToDevice, s)))
@@ -1196,11 +1247,11 @@ struct GeomDev {
 };
 
 int upload_geom(const fit_warmstart_geom &g, GeomDev &d, cudaStream_t s) {
-    if (cudaMallocAsync(&d.tidx, sizeof(int) * FIT_WS_MAX_TARGETS, s) ||
-        cudaMallocAsync(&d.uidx, sizeof(int) * FIT_WS_MAX_TARGETS, s) ||
-        cudaMallocAsync(&d.tscale, sizeof(double) * FIT_WS_MAX_TARGETS, s) ||
-        cudaMallocAsync(&d.uhalf, sizeof(double) * FIT_WS_MAX_TARGETS, s) ||
-        cudaMallocAsync(&d.choices, sizeof(uint32_t) * FIT_WS_MAX_MASKS, s))
+    if (fitcore::pool_alloc(&d.tidx, sizeof(int) * FIT_WS_MAX_TARGETS, s) ||
+        fitcore::pool_alloc(&d.uidx, sizeof(int) * FIT_WS_MAX_TARGETS, s) ||
+        fitcore::pool_alloc(&d.tscale, sizeof(double) * FIT_WS_MAX_TARGETS, s) ||
+        fitcore::pool_alloc(&d.uhalf, sizeof(double) * FIT_WS_MAX_TARGETS, s) ||
+        fitcore::pool_alloc(&d.choices, sizeof(uint32_t) * FIT_WS_MAX_MASKS, s))
         return fail(FIT_ERR_OOM, "warm start: geometry tables");
     if (cudaMemcpyAsync(d.tidx, g.target_idx, sizeof(int) * FIT_WS_MAX_TARGETS, cudaMemcpyHostToDevice, s) ||
         cudaMemcpyAsync(d.uidx, g.uniform_idx, sizeof(int) * FIT_WS_MAX_TARGETS, cudaMemcpyHostToDevice, s) ||
@@ -1492,13 +1543,13 @@ int fit_warmstart_train(fit_mlp *mlp, fit_model *const *models, const fit_warmst
     int *status = nullptr;
     GeomDev gd[16];
     int rc = FIT_OK;
-    if (cudaMallocAsync(&theta, sizeof(double) * (size_t)batch * max_p, s) ||
-        cudaMallocAsync(&mu, sizeof(float) * (size_t)batch * max_d, s) ||
-        cudaMallocAsync(&cnt, sizeof(float) * (size_t)batch * max_d, s) ||
-        cudaMallocAsync(&y, sizeof(float) * (size_t)batch * n_out, s) ||
-        cudaMallocAsync(&masks, sizeof(uint32_t) * (size_t)batch, s) ||
-        cudaMallocAsync(&status, sizeof(int) * (size_t)batch, s) ||
-        cudaMallocAsync(&loss, sizeof(double) * (size_t)n_steps, s))
+    if (fitcore::pool_alloc(&theta, sizeof(double) * (size_t)batch * max_p, s) ||
+        fitcore::pool_alloc(&mu, sizeof(float) * (size_t)batch * max_d, s) ||
+        fitcore::pool_alloc(&cnt, sizeof(float) * (size_t)batch * max_d, s) ||
+        fitcore::pool_alloc(&y, sizeof(float) * (size_t)batch * n_out, s) ||
+        fitcore::pool_alloc(&masks, sizeof(uint32_t) * (size_t)batch, s) ||
+        fitcore::pool_alloc(&status, sizeof(int) * (size_t)batch, s) ||
+        fitcore::pool_alloc(&loss, sizeof(double) * (size_t)n_steps, s))
         rc = fail(FIT_ERR_OOM, "fit_warmstart_train: workspace");
     for (int g = 0; g < n_geoms && !rc; ++g) rc = upload_geom(geoms[g], gd[g], s);
     // linearised maximum-likelihood rows per geometry (targets = where a fit of the sample ends,
@@ -1513,7 +1564,7 @@ int fit_warmstart_train(fit_mlp *mlp, fit_model *const *models, const fit_warmst
     float *mup = nullptr;
     int *stp = nullptr;
     int max_k = 0;
-    if (!rc && cudaMallocAsync(&zbuf, sizeof(float) * (size_t)batch * max_p, s) != cudaSuccess)
+    if (!rc && fitcore::pool_alloc(&zbuf, sizeof(float) * (size_t)batch * max_p, s) != cudaSuccess)
         rc = fail(FIT_ERR_OOM, "fit_warmstart_train: workspace");
     for (int g = 0; g < n_geoms && !rc; ++g) {
         std::vector<float> K1, K2, zf;
@@ -1527,9 +1578,9 @@ int fit_warmstart_train(fit_mlp *mlp, fit_model *const *models, const fit_warmst
             ints.insert(ints.end(), R.o_param.begin(), R.o_param.end());
             ints.insert(ints.end(), R.n_param.begin(), R.n_param.end());
             ints.insert(ints.end(), R.tkind.begin(), R.tkind.end());
-            if (cudaMallocAsync(&rbuf[g], sizeof(float) * R.buf.size(), s) != cudaSuccess ||
-                cudaMallocAsync(&rlam[g], sizeof(float) * R.lam_o.size(), s) != cudaSuccess ||
-                cudaMallocAsync(&rint[g], sizeof(int) * ints.size(), s) != cudaSuccess) {
+            if (fitcore::pool_alloc(&rbuf[g], sizeof(float) * R.buf.size(), s) != cudaSuccess ||
+                fitcore::pool_alloc(&rlam[g], sizeof(float) * R.lam_o.size(), s) != cudaSuccess ||
+                fitcore::pool_alloc(&rint[g], sizeof(int) * ints.size(), s) != cudaSuccess) {
                 rc = fail(FIT_ERR_OOM, "fit_warmstart_train: workspace");
                 break;
             }
@@ -1542,7 +1593,7 @@ int fit_warmstart_train(fit_mlp *mlp, fit_model *const *models, const fit_warmst
             }
         }
         const size_t n = K1.size() + K2.size() + zf.size();
-        if (cudaMallocAsync(&krows[g], sizeof(float) * n, s) != cudaSuccess) {
+        if (fitcore::pool_alloc(&krows[g], sizeof(float) * n, s) != cudaSuccess) {
             rc = fail(FIT_ERR_OOM, "fit_warmstart_train: workspace");
             break;
         }
@@ -1573,7 +1624,7 @@ int fit_warmstart_train(fit_mlp *mlp, fit_model *const *models, const fit_warmst
                 }
                 (void)P;
             }
-            if (!rc && (cudaMallocAsync(&ktl[g], sizeof(float) * kt.size(), s) != cudaSuccess ||
+            if (!rc && (fitcore::pool_alloc(&ktl[g], sizeof(float) * kt.size(), s) != cudaSuccess ||
                         cudaMemcpyAsync(ktl[g], kt.data(), sizeof(float) * kt.size(), cudaMemcpyHostToDevice, s) !=
                             cudaSuccess ||
                         cudaStreamSynchronize(s) != cudaSuccess))
@@ -1581,9 +1632,9 @@ int fit_warmstart_train(fit_mlp *mlp, fit_model *const *models, const fit_warmst
         }
     }
     if (!rc && max_k > 0 &&
-        (cudaMallocAsync(&thp, sizeof(double) * (size_t)batch * 2 * max_k * max_p, s) != cudaSuccess ||
-         cudaMallocAsync(&mup, sizeof(float) * (size_t)batch * 2 * max_k * max_d, s) != cudaSuccess ||
-         cudaMallocAsync(&stp, sizeof(int) * (size_t)batch * 2 * max_k, s) != cudaSuccess))
+        (fitcore::pool_alloc(&thp, sizeof(double) * (size_t)batch * 2 * max_k * max_p, s) != cudaSuccess ||
+         fitcore::pool_alloc(&mup, sizeof(float) * (size_t)batch * 2 * max_k * max_d, s) != cudaSuccess ||
+         fitcore::pool_alloc(&stp, sizeof(int) * (size_t)batch * 2 * max_k, s) != cudaSuccess))
         rc = fail(FIT_ERR_OOM, "fit_warmstart_train: workspace");
     float *x = rc ? nullptr : fitcore::mlp_input_buffer(mlp, batch);
     if (!rc && !x) rc = fail(FIT_ERR_OOM, "fit_warmstart_train: input buffer");
@@ -1799,7 +1850,7 @@ int fit_batch_lockstep(fit_model *const *models, int n_models, const fit_instanc
         std::vector<void *> bufs;
         auto al = [&](void **p, size_t bytes) {
             if (rc) return;
-            if (cudaMallocAsync(p, std::max<size_t>(bytes, 16), s) != cudaSuccess) {
+            if (fitcore::pool_alloc(p, std::max<size_t>(bytes, 16), s) != cudaSuccess) {
                 cudaGetLastError();
                 rc = fail(FIT_ERR_OOM, "fit_batch: lockstep buffers");
                 return;
@@ -2357,7 +2408,7 @@ int fit_linear_start(fit_model *model, int B, const float *data, const uint32_t 
         K[v] = le->K;
     }
     int *sel_d = nullptr;
-    if (cudaMallocAsync(&sel_d, sizeof(int) * (size_t)B, s) != cudaSuccess ||
+    if (fitcore::pool_alloc(&sel_d, sizeof(int) * (size_t)B, s) != cudaSuccess ||
         cudaMemcpyAsync(sel_d, sel.data(), sizeof(int) * (size_t)B, cudaMemcpyHostToDevice, s) != cudaSuccess) {
         cudaGetLastError();
         if (sel_d) cudaFreeAsync(sel_d, s);
@@ -2600,12 +2651,12 @@ int fit_batch_ex(fit_model *const *models, int n_models, const fit_instance *ins
     if (!rc) rc = stage_out(best, sizeof(double) * par_len, s, dbe, hbe);
     if (!rc) rc = stage_out(results, sizeof(fit_result) * n_inst, s, dre, hre);
     if (!rc && !in_smem) {
-        if (cudaMallocAsync(&dws.dev, sizeof(float) * (size_t)grid * max_need, s))
+        if (fitcore::pool_alloc(&dws.dev, sizeof(float) * (size_t)grid * max_need, s))
             rc = fail(FIT_ERR_OOM, "fit_batch: workspace");
         dws.owned = true;
     }
     if (!rc) {
-        if (cudaMallocAsync(&dq.dev, sizeof(int), s) || (!o.use_graph && cudaMemsetAsync(dq.dev, 0, sizeof(int), s)))
+        if (fitcore::pool_alloc(&dq.dev, sizeof(int), s) || (!o.use_graph && cudaMemsetAsync(dq.dev, 0, sizeof(int), s)))
             rc = fail(FIT_ERR_CUDA, "fit_batch: queue");
         dq.owned = true;
     }

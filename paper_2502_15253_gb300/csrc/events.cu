@@ -30,6 +30,7 @@ void fitcore_count_launch();
 
 struct fit_mc {
     int mode = 0, n_cores = 0, n_bins = 0;
+    bool counted = false;              // created in full (fitcore::pool_user)
     int64_t n_events = 0, n_pad = 0;   // n_pad: events rounded up to whole staging blocks
     float *energy = nullptr, *weight = nullptr;
     uint8_t *core = nullptr;
@@ -417,6 +418,8 @@ int fit_mc_create(int osc_mode, int n_cores, const double *core_L, int64_t n_eve
         fit_mc_destroy(m);
         return fitcore_fail(FIT_ERR_CUDA, "fit_mc_create: upload");
     }
+    m->counted = true;
+    fitcore::pool_user(1);
     *out = m;
     return FIT_OK;
 }
@@ -425,6 +428,7 @@ void fit_mc_destroy(fit_mc *m) {
     if (!m) return;
     for (void *p : {(void *)m->energy, (void *)m->weight, (void *)m->core, (void *)m->bin, (void *)m->err})
         if (p) cudaFree(p);
+    if (m->counted) fitcore::pool_user(-1);
     delete m;
 }
 
@@ -450,10 +454,10 @@ int fit_mc_spectrum(fit_mc *m, int B, const double *params, double *out, void *s
     double *pd = nullptr, *od = nullptr;
     int rc = FIT_OK;
     const size_t np = m->mode == FIT_OSC_STERILE4 ? 6 : 4;   // survival parameters per set
-    if (!p_dev && (cudaMallocAsync(&pd, sizeof(double) * np * B, s) ||
+    if (!p_dev && (fitcore::pool_alloc(&pd, sizeof(double) * np * B, s) ||
                    cudaMemcpyAsync(pd, params, sizeof(double) * np * B, cudaMemcpyHostToDevice, s)))
         rc = fitcore_fail(FIT_ERR_CUDA, "fit_mc_spectrum: parameters");
-    if (!rc && !o_dev && cudaMallocAsync(&od, sizeof(double) * (size_t)B * m->n_bins, s))
+    if (!rc && !o_dev && fitcore::pool_alloc(&od, sizeof(double) * (size_t)B * m->n_bins, s))
         rc = fitcore_fail(FIT_ERR_OOM, "fit_mc_spectrum: output");
     double *outd = o_dev ? out : od;
     if (!rc && cudaMemsetAsync(outd, 0, sizeof(double) * (size_t)B * m->n_bins, s))

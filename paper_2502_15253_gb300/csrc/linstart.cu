@@ -10,6 +10,7 @@
 
 #include "../../include/fitcore.h"
 #include "gemm_tc.cuh"
+#include "kernels.cuh"
 
 int fitcore_fail(int code, const std::string &msg);
 void fitcore_count_launch();
@@ -59,8 +60,8 @@ int linear_start_apply(int B, int P, int D, const double *theta0_dev, const floa
                        const float *const *K, int n_var, const int *sel_dev, double *theta_out, cudaStream_t s) {
     const int Dp = (D + 3) & ~3, Pp = (P + 3) & ~3;
     float *R = nullptr, *delta = nullptr;
-    if (cudaMallocAsync(&R, sizeof(float) * 2 * (size_t)B * Dp, s) != cudaSuccess ||
-        cudaMallocAsync(&delta, sizeof(float) * (size_t)n_var * B * Pp, s) != cudaSuccess) {
+    if (fitcore::pool_alloc(&R, sizeof(float) * 2 * (size_t)B * Dp, s) != cudaSuccess ||
+        fitcore::pool_alloc(&delta, sizeof(float) * (size_t)n_var * B * Pp, s) != cudaSuccess) {
         cudaGetLastError();
         if (R) cudaFreeAsync(R, s);
         return fitcore_fail(FIT_ERR_OOM, "fit_linear_start: workspace");

@@ -259,6 +259,7 @@ struct fit_mlp {
     int ld[kMaxLayers + 1] = {0};   // padded row lengths (multiples of 8)
     uint64_t seed = 0;
     int step = 0;
+    bool counted = false;           // created in full (fitcore::pool_user)
     // parameters (device)
     float *w[kMaxLayers] = {nullptr}, *b[kMaxLayers] = {nullptr};
     float *mw[kMaxLayers] = {nullptr}, *vw[kMaxLayers] = {nullptr}, *mb[kMaxLayers] = {nullptr}, *vb[kMaxLayers] = {nullptr};
@@ -424,6 +425,8 @@ int fit_mlp_create(int n_in, int n_hidden, int n_hidden_layers, int n_out, uint6
         fit_mlp_destroy(m);
         return rc;
     }
+    m->counted = true;
+    fitcore::pool_user(1);
     *out = m;
     return FIT_OK;
 }
@@ -440,6 +443,7 @@ void fit_mlp_destroy(fit_mlp *m) {
     }
     for (void *p : {(void *)m->out, (void *)m->x32})
         if (p) cudaFree(p);
+    if (m->counted) fitcore::pool_user(-1);
     delete m;
 }
 

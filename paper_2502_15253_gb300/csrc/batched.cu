@@ -45,8 +45,17 @@ inline size_t signal_smem_bytes(const DevModel &h) {
                                                  (h.remap_mode == FIT_REMAP_SPLINE ? 3 : 1) * edge);
 }
 
+// Four blocks of 256 fit the registers (62 a thread): with 32 instead of 24 warps per SM 4096
+// instances of the 53 km model (2000 bins) took 549 us instead of 567. On short rows the set-up
+// and its barriers weigh more than the sums, and more, smaller blocks hide them: 128 threads
+// against 256 for 4000 instances took 44 against 50 us with 200 bins, 171 against 208 with 400, 111
+// against 120 with 600, but 245 against 239 with 997 and 557 against 549 with 2000 (four even
+// quarters per block: 160 or 224 threads lose 6 % there).
+constexpr int kSignalThreads = 256;
+inline int signal_threads(int n_t) { return n_t <= 640 ? 128 : kSignalThreads; }
+
 template <int NOSC, int MODE>
-__global__ void __launch_bounds__(256, 3) signal_v_kernel(const DevModel *__restrict__ gm, int B,
+__global__ void __launch_bounds__(kSignalThreads, 4) signal_v_kernel(const DevModel *__restrict__ gm, int B,
                                                           const double *__restrict__ theta, float *__restrict__ vhi,
                                                           float *__restrict__ vlo, float *__restrict__ pv_out,
                                                           float *__restrict__ pl_out, int *__restrict__ status) {
@@ -183,10 +192,11 @@ int expected_tc(const DevModel &h, const DevModel *dev, int B, const double *the
     const void *fn = h.osc_mode == FIT_OSC_EQ1       ? (const void *)signal_v_kernel<4, FIT_OSC_EQ1>
                      : h.osc_mode == FIT_OSC_VACUUM3 ? (const void *)signal_v_kernel<4, FIT_OSC_VACUUM3>
                                                      : (const void *)signal_v_kernel<6, FIT_OSC_STERILE4>;
+    const int threads = signal_threads(h.N_t);
     int dev_id = 0, sms = 0, per_sm = 0;
     cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (cudaGetDevice(&dev_id) || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev_id) ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, 256, smem) || per_sm < 1) {
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem) || per_sm < 1) {
         cudaGetLastError();
         cleanup();
         return fitcore_fail(FIT_ERR_CUDA, "fit_model_expected_tc: launch shape");
@@ -194,7 +204,7 @@ int expected_tc(const DevModel &h, const DevModel *dev, int B, const double *the
     // one wave of resident blocks over (instance, dataset)
     const int gx = std::max(1, std::min(B, (per_sm * sms + nds - 1) / nds));
     void *args[] = {(void *)&dev, &B, &theta, &vhi, &vlo, &pv, &pl, &status};
-    cudaLaunchKernel(fn, dim3(gx, nds), dim3(256), args, smem, s);
+    cudaLaunchKernel(fn, dim3(gx, nds), dim3(threads), args, smem, s);
     fitcore_count_launch();
     int rc = FIT_OK;
     for (int d = 0; d < nds && rc == FIT_OK; ++d) {

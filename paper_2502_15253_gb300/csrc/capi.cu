@@ -2532,8 +2532,11 @@ int fit_batch_ex(fit_model *const *models, int n_models, const fit_instance *ins
         // vectors and the evaluation workspace in shared memory (the history in L2) when two
         // blocks, or one, then fit an SM; blocks of 128 threads keep everything in L2 for five
         // fits per SM. Measured (ms, 128 x 5 / 256 x 2 / 512 x 1 per SM): 1000 fits of the 53 km
-        // model 23.8 / 15.3 / 15.4 and a scan of 42 of its fits 11.1 / 5.8 / 4.0; 2500
-        // three-dataset fits 14.0 / 10.9 / 15.4; 2500 single-detector fits 2.9 / 3.4 / 4.8.
+        // model 14.0 / 11.5 / 10.8 and a scan of 42 of its fits 6.5 / 3.9 / 2.6; 300 three-dataset
+        // fits 7.0 / 4.2 / -, 2500 with the spline 7.1 / 8.5 / 12.0; 2500 single-detector fits 2.2 / 2.5
+        // / 4.1. Many waves of fits run faster in blocks of 128 (8192: 62.5 against 75.3 and 43.5
+        // against 50.0 under this rule), which fit_batch_autotune finds; the number of fits is not
+        // looked at, so that a fit does not depend on the batch around it.
         for (int i = 0; i < n_models; ++i) o.threads = std::max(o.threads, fitcore::model_threads(models[i]->host));
         if (o.threads > 128) o.placement = smem_for(2) * (512 / o.threads) > cfg.smem_optin ? 3 : 2;
     }

@@ -185,9 +185,10 @@ __host__ __device__ inline int fit_work_floats(int P) { return 15 * fit_vec_pitc
 // Threads per block for a model: one wide block per vector or fit leaves the fewest dependent
 // steps, but each thread then holds fewer bins and every barrier spans more warps, so the block
 // grows with the true bins evaluated together. Measured (us, batched -2lnL with gradient, 128 /
-// 256 / 512 threads): 200 bins x 4096 vectors 116 / 182 / 338; 1200 bins x 4096 550 / 504 / 720;
-// 2000 bins x 2048 3636 / 2124 / 1407. A property of the model alone: the result of a vector or
-// a fit does not depend on the batch around it.
+// 256 / 512 threads): 200 bins x 4096 vectors 105 / 175 / 322; 1200 bins x 4096 462 / 464 / 628
+// (where few vectors or fits run, 256 threads win: capi.cu); 2000 bins x 2048 1929 / 1227 / 941. A
+// property of the model alone: the result of a vector or a fit does not depend on the batch
+// around it.
 inline int model_threads(const DevModel &h) {
     const int bins = h.N_t * h.ws_group;
     return bins <= 512 ? 128 : bins <= 1600 ? 256 : 512;

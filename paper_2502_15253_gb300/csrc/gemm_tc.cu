@@ -41,15 +41,17 @@ __device__ int g_gemm_err;
 // z >= 0, absolute error <= 1.5e-7 (the level of FP32 rounding of erf itself). For x < 0 Phi
 // is formed directly as erfc(|x| / sqrt 2) / 2, so the left tail has no cancellation. The GELU
 // of the network is x Phi(x) ("exact erf" form), its derivative Phi(x) + x phi(x); both share
-// the one exponential.
+// the one exponential. The last products and the difference are rounded one by one (no
+// contraction): fused, 1 - h moves by an ulp, which the bf16 roundings of the back-propagated
+// error carry into 1e-4 of the first layers' gradients, from one build to the next.
 __device__ __forceinline__ void phi_pair(float x, float &cdf, float &e) {
     const float z = fabsf(x) * 0.70710678118654752f;
     const float t = __fdividef(1.f, fmaf(0.3275911f, z, 1.f));
     const float q = t * fmaf(t, fmaf(t, fmaf(t, fmaf(t, 1.061405429f, -1.453152027f), 1.421413741f), -0.284496736f),
                              0.254829592f);
     e = __expf(-0.5f * x * x);
-    const float h = 0.5f * q * e;   // erfc(z) / 2
-    cdf = x < 0.f ? h : 1.f - h;
+    const float h = __fmul_rn(__fmul_rn(0.5f, q), e);   // erfc(z) / 2
+    cdf = x < 0.f ? h : __fsub_rn(1.f, h);
 }
 
 __device__ __forceinline__ float gelu(float x) {
@@ -251,9 +253,9 @@ __device__ __forceinline__ void stage_aux(EpiStage &st, const float4 (&q)[4]) {
 }
 
 // Epilogue of one 32-row x 16-column chunk: rows row0 + [0, nrow), columns n + [0, nv); v holds
-// this thread's row (row0 + lane) of the accumulator.
-__device__ __forceinline__ void epi_chunk(const GemmOut &out, EpiStage &st, bool split, int row0, int n, int nrow,
-                                          int nv, float (&v)[16]) {
+// this thread's row (row0 + lane) of the accumulator. C: out.C, or this K share's own product.
+__device__ __forceinline__ void epi_chunk(const GemmOut &out, float *C, EpiStage &st, bool split, int row0, int n,
+                                          int nrow, int nv, float (&v)[16]) {
     const int lane = threadIdx.x & 31;
     const bool vc = out.vec & 1, vy = out.vec & 2, vt = out.vec & 8;
     switch (out.epi) {
@@ -264,7 +266,7 @@ __device__ __forceinline__ void epi_chunk(const GemmOut &out, EpiStage &st, bool
 #pragma unroll
             for (int j = 0; j < 4; ++j) st.c[cidx(lane, j)] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
             __syncwarp();
-            flush_c(st, out.C, out.ldc, row0, n, nrow, nv, vc, split, out.epi == EPI_F32_ADD);
+            flush_c(st, C, out.ldc, row0, n, nrow, nv, vc, split, out.epi == EPI_F32_ADD);
             break;
         }
         case EPI_BIAS_GELU: {
@@ -276,7 +278,7 @@ __device__ __forceinline__ void epi_chunk(const GemmOut &out, EpiStage &st, bool
             for (int j = 0; j < 4; ++j) st.c[cidx(lane, j)] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
             stage_bf16(st, w, out.Yt != nullptr);
             __syncwarp();
-            flush_c(st, out.C, out.ldc, row0, n, nrow, nv, vc, false, false);
+            flush_c(st, C, out.ldc, row0, n, nrow, nv, vc, false, false);
             flush_y(st, out.Y, out.ldy, row0, n, nrow, nv, vy);
             if (out.Yt) flush_yt(st, out.Yt, out.ldyt, row0, n, nrow, nv, vt);
             break;
@@ -332,7 +334,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     constexpr int kPasses = SPLIT ? 3 : 1;
     const int kel = TF32 ? 32 : 64;
     const int ktiles = (K + kel - 1) / kel;
-    const bool split = pl.splits > 1;
+    const bool split = pl.splits > 1 && out.share_stride == 0;
     const uint32_t tcols = 2u * (uint32_t)pl.acc_cols;
 
     if (warp == 2) umma::tmem_alloc(tmem_slot, tcols);
@@ -458,6 +460,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 break;
             }
             umma::tc_fence_after();
+            float *C = out.C + (kt0 / pl.kt_per) * out.share_stride;
             const uint32_t tbase = tmem + (uint32_t)(a * pl.acc_cols) + ((uint32_t)(quad * 32) << 16);
             for (int c = sub * 16; c < n_tile; c += 64) {
                 const int nv = chunk_nv(c);
@@ -470,7 +473,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                         const int nv2 = chunk_nv(c + 64);
                         if (nv2 > 0) load_aux(out, row0, n0 + c + 64, nrow, nv2, qa);
                     }
-                    epi_chunk(out, st, split, row0, n0 + c, nrow, nv, v);
+                    epi_chunk(out, C, st, split, row0, n0 + c, nrow, nv, v);
                 }
             }
             umma::tc_fence_before();
@@ -581,6 +584,8 @@ static int launch_gemm(bool tf32, int M, int N, int K, const void *A, const void
               ((out.aux && !((uintptr_t)out.aux & 15) && out.ldaux % 4 == 0) ? 4 : 0) |
               ((out.Yt && !((uintptr_t)out.Yt & 15) && out.ldyt % 8 == 0) ? 8 : 0) |
               ((out.bias && !((uintptr_t)out.bias & 15)) ? 16 : 0);
+    if (out.share_stride % 4 || (out.share_stride && out.epi != EPI_F32))
+        return fitcore_fail(FIT_ERR_INVALID_ARG, "tensor-core GEMM: stride of the K shares");
     const Plan pl = make_plan(tf32, M, N, K, out.epi, out.deterministic);
     CUtensorMap ta, tb;
     if ((rc = make_map(&ta, tf32, A, M, K, lda, kTileM))) return rc;
@@ -623,7 +628,7 @@ static int launch_gemm(bool tf32, int M, int N, int K, const void *A, const void
             cur = (int)smem;
         }
     }
-    if (pl.splits > 1 && out.epi == EPI_F32) {
+    if (pl.splits > 1 && out.epi == EPI_F32 && out.share_stride == 0) {
         // C = 0 first: rows of ldc floats (the row tails beyond N are left as they were)
         cudaError_t e = (out.ldc == N) ? cudaMemsetAsync(out.C, 0, sizeof(float) * (size_t)M * N, stream)
                                        : cudaMemset2DAsync(out.C, sizeof(float) * (size_t)out.ldc, 0,
@@ -642,6 +647,14 @@ static int launch_gemm(bool tf32, int M, int N, int K, const void *A, const void
     if (e != cudaSuccess)
         return fitcore_fail(FIT_ERR_CUDA, std::string("tensor-core GEMM launch: ") + cudaGetErrorString(e));
     return FIT_OK;
+}
+
+int tc_gemm_shares(bool tf32, int M, int N, int K) { return make_plan(tf32, M, N, K, EPI_F32, false).splits; }
+
+// make_plan splits K for up to an SM per share of every tile, shares of four K slices or more
+int tc_gemm_max_shares(bool tf32, int M, int N, int k_max) {
+    const int kel = tf32 ? 32 : 64, tiles = ((M + kTileM - 1) / kTileM) * ((N + 255) / 256);
+    return std::max(1, std::min(kNumSMs / tiles, (k_max + kel - 1) / kel / 4));
 }
 
 int tc_gemm(bool tf32, int M, int N, int K, const void *A, int lda, const void *B, int ldb, const GemmOut &out,

@@ -35,7 +35,16 @@ struct GemmOut {
     // never split K over CTAs (the split adds partial tiles with atomics, so its FP32 sums
     // depend on their order): results identical from call to call
     bool deterministic = false;
+    // EPI_F32: not 0 = the shares of a K split are stored apart instead, share z's product at
+    // C + z * share_stride (floats, a multiple of 4); the caller adds tc_gemm_shares of them in
+    // the order it likes, so that its sums do not depend on the order in which CTAs finish
+    int64_t share_stride = 0;
 };
+
+// K shares of tc_gemm's plan for an EPI_F32 product of these sizes, and the most that any K up to
+// k_max takes.
+int tc_gemm_shares(bool tf32, int M, int N, int K);
+int tc_gemm_max_shares(bool tf32, int M, int N, int k_max);
 
 // C = (Ah + Al)(Bh + Bl)^T without Al Bl^T (FP32 operands as a TF32-exact part and the rest: the split
 // product that keeps FP32 accuracy), one launch: the three products Ah Bl^T, Al Bh^T and Ah Bh^T

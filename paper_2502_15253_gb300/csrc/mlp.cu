@@ -25,6 +25,13 @@ constexpr int kMaxLayers = 8;
 
 inline int pad8(int x) { return (x + 7) / 8 * 8; }
 
+// Samples per block of the kernels that sum over the batch. A step's gradients and loss are the same
+// bits on every run: each such block and each K share of a weight gradient leaves its own partial
+// sum, and the AdamW kernel, which reads every gradient once, adds them in order. With atomics the
+// first step's gradients differed by 1e-7 from run to run, and the steps after it, through AdamW and
+// the bf16 roundings, by up to 1.5e-3 (438 -> 3 x 512 -> 12, batch 4096).
+constexpr int kColRows = 256;
+
 __global__ void prep_input_kernel(int B, int n_in, int ld, const float *__restrict__ x, __nv_bfloat16 *__restrict__ a0) {
     const int64_t total = (int64_t)B * ld;
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
@@ -35,51 +42,50 @@ __global__ void prep_input_kernel(int B, int n_in, int ld, const float *__restri
 
 // d loss / d out for the mean squared error over B x n_out (n_out <= 256): a thread per sample
 // writes its row of dout (ld per row, zero padding) and its column of the transpose doutT (ldt
-// per feature row, coalesced over the samples); the output layer's bias gradient db (cleared
-// by the caller) gets the column sums of the bf16 values, and the loss (double) is
-// accumulated; one atomic per block and column / per block.
-__global__ void __launch_bounds__(256) mse_kernel(int B, int n_out, int ld, const float *__restrict__ out,
-                                                  const float *__restrict__ tgt, __nv_bfloat16 *__restrict__ dout,
-                                                  int ldt, __nv_bfloat16 *__restrict__ doutT, float *__restrict__ db,
-                                                  double *__restrict__ loss) {
-    __shared__ double part[8];
-    __shared__ float col[256];
-    for (int o = threadIdx.x; o < n_out; o += blockDim.x) col[o] = 0.f;
-    __syncthreads();
+// per feature row, coalesced over the samples). Block k's sums go to bpart[k][o] (columns of
+// the bf16 values: its part of the output layer's bias gradient) and lpart[k] (the loss).
+__global__ void __launch_bounds__(kColRows) mse_kernel(int B, int n_out, int ld, const float *__restrict__ out,
+                                                       const float *__restrict__ tgt, __nv_bfloat16 *__restrict__ dout,
+                                                       int ldt, __nv_bfloat16 *__restrict__ doutT,
+                                                       float *__restrict__ bpart, double *__restrict__ lpart) {
+    constexpr int kWarps = kColRows / 32;
+    __shared__ double part[kWarps];
+    __shared__ float col[kWarps][256];
     const float scale = 2.f / (float)((int64_t)B * n_out);
     double acc = 0.0;
-    // the loop bound is uniform over the block, so every lane takes part in the shuffles
-    for (int b0 = blockIdx.x * blockDim.x; b0 < B; b0 += gridDim.x * blockDim.x) {
-        const int b = b0 + threadIdx.x;
-        const bool valid = b < B;
-        for (int o = 0; o < ld; ++o) {
-            float q = 0.f;   // the bf16-rounded gradient (0 past B and in the padding)
-            if (valid) {
-                float g = 0.f;
-                if (o < n_out) {
-                    const float r = out[(int64_t)b * n_out + o] - tgt[(int64_t)b * n_out + o];
-                    acc += (double)r * r;
-                    g = scale * r;
-                    doutT[(int64_t)o * ldt + b] = __float2bfloat16(g);
-                }
-                const __nv_bfloat16 h = __float2bfloat16(g);
-                dout[(int64_t)b * ld + o] = h;
-                q = __bfloat162float(h);
+    const int b = blockIdx.x * kColRows + threadIdx.x;
+    const bool valid = b < B;
+    for (int o = 0; o < ld; ++o) {
+        float q = 0.f;   // the bf16-rounded gradient (0 past B and in the padding)
+        if (valid) {
+            float g = 0.f;
+            if (o < n_out) {
+                const float r = out[(int64_t)b * n_out + o] - tgt[(int64_t)b * n_out + o];
+                acc += (double)r * r;
+                g = scale * r;
+                doutT[(int64_t)o * ldt + b] = __float2bfloat16(g);
             }
-            if (o < n_out) {   // column sum: a shuffle tree, one shared atomic per warp
-                for (int k = 16; k > 0; k >>= 1) q += __shfl_xor_sync(0xffffffffu, q, k);
-                if ((threadIdx.x & 31) == 0) atomicAdd(&col[o], q);
-            }
+            const __nv_bfloat16 h = __float2bfloat16(g);
+            dout[(int64_t)b * ld + o] = h;
+            q = __bfloat162float(h);
+        }
+        if (o < n_out) {   // column sum: a shuffle tree, then the warps in order
+            for (int k = 16; k > 0; k >>= 1) q += __shfl_xor_sync(0xffffffffu, q, k);
+            if ((threadIdx.x & 31) == 0) col[threadIdx.x >> 5][o] = q;
         }
     }
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
     if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = acc;
     __syncthreads();
-    for (int o = threadIdx.x; o < n_out; o += blockDim.x) atomicAdd(db + o, col[o]);
+    for (int o = threadIdx.x; o < n_out; o += kColRows) {
+        float t = col[0][o];
+        for (int w = 1; w < kWarps; ++w) t += col[w][o];
+        bpart[(int64_t)blockIdx.x * n_out + o] = t;
+    }
     if (threadIdx.x == 0) {
         double t = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += part[w];
-        atomicAdd(loss, t / (double)((int64_t)B * n_out));
+        for (int w = 0; w < kWarps; ++w) t += part[w];
+        lpart[blockIdx.x] = t / (double)((int64_t)B * n_out);
     }
 }
 
@@ -103,11 +109,10 @@ __global__ void prep_input_t_kernel(int B, int n_in, int ld, const float *__rest
     }
 }
 
-// db[o] += sum_b d[b][o] (db cleared by the caller): block (32, 8) covers 64 columns (a column
-// pair per thread, read as bf16x2 along the row, so a warp reads 128 contiguous bytes) and
-// kColRows rows; partial sums meet in shared memory and go out with one atomic per column.
-constexpr int kColRows = 256;
-__global__ void colsum_kernel(int B, int n, int ld, const __nv_bfloat16 *__restrict__ d, float *__restrict__ db) {
+// bpart[k][o] = sum of d[b][o] over the kColRows rows of row block k = blockIdx.y: block (32, 8)
+// covers 64 columns (a column pair per thread, read as bf16x2 along the row, so a warp reads 128
+// contiguous bytes); partial sums meet in shared memory.
+__global__ void colsum_kernel(int B, int n, int ld, const __nv_bfloat16 *__restrict__ d, float *__restrict__ bpart) {
     __shared__ float2 part[8][33];
     const int cp = blockIdx.x * 32 + threadIdx.x;   // column pair
     const int c = 2 * cp;
@@ -128,8 +133,9 @@ __global__ void colsum_kernel(int B, int n, int ld, const __nv_bfloat16 *__restr
             t.x += part[y][threadIdx.x].x;
             t.y += part[y][threadIdx.x].y;
         }
-        atomicAdd(&db[c], t.x);
-        if (c + 1 < n) atomicAdd(&db[c + 1], t.y);
+        float *q = bpart + (int64_t)blockIdx.y * n + c;
+        q[0] = t.x;
+        if (c + 1 < n) q[1] = t.y;
     }
 }
 
@@ -146,21 +152,28 @@ __device__ __forceinline__ void adamw_one(const AdamW &h, float *p, float gr, fl
 }
 
 // Per-layer arguments of the fused AdamW launch: the [out x in] weights (W bf16 copy with rows
-// of ldw, W^T with rows of ldwt) and the bias.
+// of ldw, W^T with rows of ldwt) and the bias. The weight gradient comes as `shares` (> 1) products
+// of a K share each, `pitch` floats apart, or whole in g (1); the bias gradient as row sums.
 struct AdamLayer {
     int out, in, ldw, ldwt, tiles_i, wtiles;   // wtiles = ceil(out/32) ceil(in/32) weight tiles
+    int shares;
+    int64_t pitch;
+    const float *part, *bpart;
     float *w, *g, *mw, *vw, *b, *gb, *mb, *vb;
     __nv_bfloat16 *wbf, *wt;
 };
 struct AdamAll {
-    int n;
+    int n, rows;                 // rows: row blocks of the batch (kColRows samples each)
+    const double *lpart;         // [rows] parts of the loss
+    double *loss;
     int first[kMaxLayers + 1];   // first block of each layer: its weight tiles, then its bias blocks
     AdamLayer L[kMaxLayers];
 };
 
 // AdamW on every layer in one launch. A block (32 x 8 threads) updates a 32 x 32 weight tile
 // (rows of W along the lanes) and rewrites both bf16 copies, the transposed one through a
-// shared-memory tile so that its writes are coalesced too; the bias blocks update 256 biases.
+// shared-memory tile so that its writes are coalesced too; the bias blocks update 256 biases, the
+// last layer's also adds up the loss.
 __global__ void __launch_bounds__(256) adamw_all_kernel(AdamW h, AdamAll A) {
     __shared__ __nv_bfloat16 tile[32][34];
     int t = blockIdx.x, l = 0;
@@ -174,7 +187,16 @@ __global__ void __launch_bounds__(256) adamw_all_kernel(AdamW h, AdamAll A) {
             __nv_bfloat16 q = __float2bfloat16(0.f);
             if (o < L.out && i < L.in) {
                 const int64_t e = (int64_t)o * L.in + i;
-                adamw_one(h, L.w + e, L.g[e], L.mw + e, L.vw + e, true);
+                float g;
+                if (L.shares > 1) {
+                    g = L.part[e];
+#pragma unroll 4
+                    for (int z = 1; z < L.shares; ++z) g += L.part[z * L.pitch + e];
+                    L.g[e] = g;
+                } else {
+                    g = L.g[e];
+                }
+                adamw_one(h, L.w + e, g, L.mw + e, L.vw + e, true);
                 q = __float2bfloat16(L.w[e]);
                 L.wbf[(int64_t)o * L.ldw + i] = q;
             }
@@ -187,7 +209,19 @@ __global__ void __launch_bounds__(256) adamw_all_kernel(AdamW h, AdamAll A) {
         }
     } else {
         const int k = (t - L.wtiles) * 256 + threadIdx.y * 32 + threadIdx.x;
-        if (k < L.out) adamw_one(h, L.b + k, L.gb[k], L.mb + k, L.vb + k, false);
+        if (k < L.out) {
+            float g = L.bpart[k];
+#pragma unroll 8
+            for (int r = 1; r < A.rows; ++r) g += L.bpart[(int64_t)r * L.out + k];
+            L.gb[k] = g;
+            adamw_one(h, L.b + k, g, L.mb + k, L.vb + k, false);
+        }
+        if (l + 1 == A.n && threadIdx.y == 7) {   // (the last layer has one bias block: n_out <= 256)
+            double s = 0.0;
+            for (int r = threadIdx.x; r < A.rows; r += 32) s += A.lpart[r];
+            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if (threadIdx.x == 0) *A.loss = s;
+        }
     }
 }
 
@@ -276,6 +310,12 @@ struct fit_mlp {
     __nv_bfloat16 *actT[kMaxLayers] = {nullptr};
     __nv_bfloat16 *dpreT[kMaxLayers] = {nullptr};
     double *loss = nullptr;
+    // partial sums of a training step (kColRows): the loss, the bias gradients and, for layers whose
+    // weight gradient is a product split over K, its shares (wpitch floats each)
+    double *lpart = nullptr;
+    float *bpart[kMaxLayers] = {nullptr}, *wpart[kMaxLayers] = {nullptr};
+    int64_t wpitch[kMaxLayers] = {0};
+    void *parts = nullptr;          // the allocation that holds them
     std::vector<void *> owned;
 };
 
@@ -314,8 +354,11 @@ int ensure_batch(fit_mlp *m, int B) {
         m->actT[l] = nullptr;
         m->dpreT[l] = nullptr;
     }
-    for (void *p : {(void *)m->out, (void *)m->x32})
-        if (p) cudaFree(p);
+    for (void **p : {(void **)&m->out, (void **)&m->x32, &m->parts}) {
+        if (*p) cudaFree(*p);
+        *p = nullptr;
+    }
+    m->cap = 0;
     int rc = FIT_OK;
     const int L = m->n_layers, Bp = pad8(B);
     auto al = [&](void **p, size_t bytes) {
@@ -334,7 +377,36 @@ int ensure_batch(fit_mlp *m, int B) {
     al((void **)&m->x32, sizeof(float) * (size_t)B * m->dims[0]);
     for (int l = 0; l < L; ++l) al((void **)&m->actT[l], sizeof(__nv_bfloat16) * (size_t)m->dims[l] * Bp);
     for (int l = 0; l < L; ++l) al((void **)&m->dpreT[l], sizeof(__nv_bfloat16) * (size_t)m->dims[l + 1] * Bp);
-    if (rc == FIT_OK) m->cap = B;
+    // partial sums: every one is written before it is read, in any step of up to B samples
+    size_t bytes = 0;
+    auto take = [&](size_t n) {
+        const size_t at = bytes;
+        bytes += (n + 255) / 256 * 256;
+        return at;
+    };
+    size_t at_b[kMaxLayers], at_w[kMaxLayers];
+    const int rows = (B + kColRows - 1) / kColRows;
+    const size_t at_l = take(sizeof(double) * rows);
+    for (int l = 0; l < L; ++l) {
+        const int o = m->dims[l + 1], in = m->dims[l];
+        m->wpitch[l] = ((int64_t)o * in + 3) & ~int64_t(3);
+        at_b[l] = take(sizeof(float) * (size_t)rows * o);
+        const int shares = fitcore::tc_gemm_max_shares(false, o, in, B);
+        at_w[l] = shares > 1 ? take(sizeof(float) * (size_t)shares * m->wpitch[l]) : 0;
+    }
+    if (!rc && cudaMalloc(&m->parts, bytes) != cudaSuccess) {
+        cudaGetLastError();
+        m->parts = nullptr;
+        rc = fitcore_fail(FIT_ERR_OOM, "fit_mlp: batch buffers");
+    }
+    if (rc) return rc;
+    char *base = static_cast<char *>(m->parts);
+    m->lpart = reinterpret_cast<double *>(base + at_l);
+    for (int l = 0; l < L; ++l) {
+        m->bpart[l] = reinterpret_cast<float *>(base + at_b[l]);
+        m->wpart[l] = reinterpret_cast<float *>(base + at_w[l]);
+    }
+    m->cap = B;
     return rc;
 }
 
@@ -441,7 +513,7 @@ void fit_mlp_destroy(fit_mlp *m) {
         if (m->actT[l]) cudaFree(m->actT[l]);
         if (m->dpreT[l]) cudaFree(m->dpreT[l]);
     }
-    for (void *p : {(void *)m->out, (void *)m->x32})
+    for (void *p : {(void *)m->out, (void *)m->x32, m->parts})
         if (p) cudaFree(p);
     if (m->counted) fitcore::pool_user(-1);
     delete m;
@@ -474,28 +546,29 @@ int fit_mlp_train_step(fit_mlp *m, int B, const float *x, const float *target, f
     const int L = m->n_layers, Bp = pad8(B);
     prep_input_t_kernel<<<dim3((m->ld[0] + 31) / 32, (B + 31) / 32), dim3(32, 8), 0, s>>>(
         B, m->dims[0], m->ld[0], x, m->act[0], Bp, m->actT[0]);
-    cudaMemsetAsync(m->loss, 0, sizeof(double), s);
     fitcore_count_launch();
     if ((rc = forward(m, B, s, true))) return rc;
     // bias gradients (column sums of the bf16 backward signals): the output layer's from the
-    // MSE kernel, the hidden layers' from colsum_kernel
-    for (int l = 0; l < L; ++l) cudaMemsetAsync(m->gb[l], 0, sizeof(float) * m->dims[l + 1], s);
-    mse_kernel<<<(B + 255) / 256, 256, 0, s>>>(
-        B, m->dims[L], m->ld[L], m->out, target, m->dpre[L - 1], Bp, m->dpreT[L - 1], m->gb[L - 1], m->loss);
+    // MSE kernel, the hidden layers' from colsum_kernel, both per row block
+    const int rows = (B + kColRows - 1) / kColRows;
+    mse_kernel<<<rows, kColRows, 0, s>>>(B, m->dims[L], m->ld[L], m->out, target, m->dpre[L - 1], Bp, m->dpreT[L - 1],
+                                         m->bpart[L - 1], m->lpart);
     fitcore_count_launch();
+    int shares[kMaxLayers];
     for (int l = L - 1; l >= 0; --l) {
         const int o = m->dims[l + 1], in = m->dims[l];
         if (l < L - 1) {   // bias gradient of a hidden layer (the output layer's: mse_kernel)
-            colsum_kernel<<<dim3((o + 63) / 64, (B + kColRows - 1) / kColRows), dim3(32, 8), 0, s>>>(
-                B, o, m->ld[l + 1], m->dpre[l], m->gb[l]);
+            colsum_kernel<<<dim3((o + 63) / 64, rows), dim3(32, 8), 0, s>>>(B, o, m->ld[l + 1], m->dpre[l], m->bpart[l]);
             fitcore_count_launch();
         }
         // dW = dpre^T act: both operands K-major over the batch, as the producing kernels
         // wrote them (dpreT, actT)
         fitcore::GemmOut gw;
         gw.epi = fitcore::EPI_F32;
-        gw.C = m->gw[l];
+        shares[l] = fitcore::tc_gemm_shares(false, o, in, B);
+        gw.C = shares[l] > 1 ? m->wpart[l] : m->gw[l];
         gw.ldc = in;
+        gw.share_stride = shares[l] > 1 ? m->wpitch[l] : 0;
         if ((rc = fitcore::tc_gemm(false, o, in, B, m->dpreT[l], Bp, m->actT[l], Bp, gw, s, nullptr))) return rc;
         if (l > 0) {
             // d pre_{l-1} = (d pre_l W_l) * gelu'(pre_{l-1})
@@ -522,6 +595,9 @@ int fit_mlp_train_step(fit_mlp *m, int B, const float *x, const float *target, f
     h.c2 = (float)(1.0 / (1.0 - std::pow(0.999, m->step)));
     AdamAll A;
     A.n = L;
+    A.rows = rows;
+    A.lpart = m->lpart;
+    A.loss = m->loss;
     int nblk = 0;
     for (int l = 0; l < L; ++l) {
         AdamLayer &q = A.L[l];
@@ -531,6 +607,10 @@ int fit_mlp_train_step(fit_mlp *m, int B, const float *x, const float *target, f
         q.ldwt = m->ld[l + 1];
         q.tiles_i = (q.in + 31) / 32;
         q.wtiles = ((q.out + 31) / 32) * q.tiles_i;
+        q.shares = shares[l];
+        q.pitch = m->wpitch[l];
+        q.part = m->wpart[l];
+        q.bpart = m->bpart[l];
         q.w = m->w[l];
         q.g = m->gw[l];
         q.mw = m->mw[l];

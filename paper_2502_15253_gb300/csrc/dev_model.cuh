@@ -1053,20 +1053,22 @@ static __device__ __forceinline__ void st_signal(const DevModel &m, const EvalSh
 }
 
 // Corrected content of target bin t under the overlap rule, from the sources' contents per mapped
-// width u. Source bin k covers [Y_k, Y_k+1] in
+// width u and the map's slope at mid grid. Source bin k covers [Y_k, Y_k+1] in
 // grid units, Y_k = k + D(e_k); target t gathers the sources whose mapped interval overlaps
 // [t, t+1]; overlaps are computed relative to the target (k - t is an exact small integer),
 // which keeps them accurate in FP32.
-__device__ __forceinline__ float overlap_target(const float *u, const float *D, int t, int N_t) {
-    // first source whose mapped upper edge lies above t: from k ~ t - D(t), stepping down until the
-    // bracket is right
-    int k = min(max(t - (int)floorf(D[t]) - 1, 0), N_t - 1);
+__device__ __forceinline__ float overlap_target(const float *u, const float *D, float inv_slope, int t, int N_t) {
+    // first source whose mapped upper edge lies above t: from k ~ t - D(t) / slope (exact for a linear
+    // map), stepping down until the bracket is right; the sum steps up over what lies below t.
+    // Neither is capped: the map is increasing, so both end, and at scales a few percent off 1
+    // neither takes more than a step.
+    int k = min(max(t - (int)floorf(D[t] * inv_slope) - 1, 0), N_t - 1);
     float dlo = D[k];
 #pragma unroll 1
     while (k > 0 && (float)(k - t) + dlo > 0.f) dlo = D[--k];
     float acc = 0.f;
 #pragma unroll 1
-    for (int it = 0; it < 64 && k < N_t; ++it, ++k) {
+    for (; k < N_t; ++k) {
         const float dhi = D[k + 1];
         const float ylo = (float)(k - t) + dlo;      // mapped edges relative to target t
         const float yhi = (float)(k + 1 - t) + dhi;
@@ -1086,10 +1088,10 @@ static __device__ __forceinline__ void st_remap(const DevModel &m, const EvalSha
 #pragma unroll 1
     for (int i = 0; i < E.n; ++i) {
         const DsWs ws = carve_ds_ws(wsb + (int64_t)i * m.ws_eval_floats, N_t, m.C, m.max_reco, m.n_osc);
-        const EMap em = E.em[i];
+        const float is = 1.f / E.em[i].slope(0.5f * (m.e_first + m.e_last));
 #pragma unroll 1
         for (int t = rot_tid(i, (N_t + 31) >> 5); t < N_t; t += nth)
-            ws.v[t] = spline ? spline_target(ws.u, ws.edge, t, N_t) : overlap_target(ws.u, ws.edge.t, t, N_t);
+            ws.v[t] = spline ? spline_target(ws.u, ws.edge, t, N_t) : overlap_target(ws.u, ws.edge.t, is, t, N_t);
     }
     __syncthreads();
 }

@@ -190,9 +190,10 @@ __device__ void expected_dataset(const DevModel &m, int d, const float *pv, cons
         k = t - (int)floorf(em.disp(m.e_edge[k]));
         k = min(max(k - 1, 0), N_t - 1);
         while (k > 0 && (float)(k - t) + em.disp(m.e_edge[k]) > 0.f) --k;
+        while (k + 1 < N_t && (float)(k + 1 - t) + em.disp(m.e_edge[k + 1]) <= 0.f) ++k;
         float acc = 0.f;
         float dlo = em.disp(m.e_edge[k]);
-        for (int it = 0; it < 64 && k < N_t; ++it, ++k) {
+        for (; k < N_t; ++k) {
             const float dhi = em.disp(m.e_edge[k + 1]);
             const float ylo = (float)(k - t) + dlo;
             const float yhi = (float)(k + 1 - t) + dhi;

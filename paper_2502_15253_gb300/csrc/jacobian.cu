@@ -262,7 +262,9 @@ __global__ void __launch_bounds__(256) expected_rows_kernel(const DevModel *__re
             else
                 expected_dataset<4>(m, d, pv, pd, u, v, f0, &S.status, mu + (int64_t)b * m.n_data);
             __syncthreads();
-            if (S.status) break;
+            const int bad = S.status;
+            __syncthreads();   // every warp has read it before the next dataset can set it
+            if (bad) break;
         }
         if (threadIdx.x == 0) status[b] = S.status ? FIT_STATUS_ESCALE_NONMONOTONE : 0;
         __syncthreads();

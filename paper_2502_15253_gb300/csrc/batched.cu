@@ -15,6 +15,7 @@
 
 int fitcore_fail(int code, const std::string &msg);
 void fitcore_count_launch();
+int fitcore_raise_eval_smem(const void *func, size_t bytes);   // capi.cu
 
 namespace fitcore {
 
@@ -195,7 +196,12 @@ int expected_tc(const DevModel &h, const DevModel *dev, int B, const double *the
                                                      : (const void *)signal_v_kernel<6, FIT_OSC_STERILE4>;
     const int threads = signal_threads(h.N_t);
     int dev_id = 0, sms = 0, per_sm = 0;
-    cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // (raised only: the attribute is shared with other threads' calls for larger models)
+    if (fitcore_raise_eval_smem(fn, smem) != FIT_OK) {
+        cudaGetLastError();
+        cleanup();
+        return FIT_ERR_CUDA;
+    }
     if (cudaGetDevice(&dev_id) || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev_id) ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem) || per_sm < 1) {
         cudaGetLastError();

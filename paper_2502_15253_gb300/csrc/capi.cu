@@ -321,8 +321,8 @@ int fitcore_model_device(fit_model *model, const DevModel **dev, const DevModel 
     return FIT_OK;
 }
 
-// The largest dynamic shared memory each build of eval_kernel has been allowed on each device. The
-// attribute is shared by every thread of the process, so the evaluation paths only ever raise it
+// The largest dynamic shared memory each evaluation and expectation kernel has been allowed on each
+// device. The attribute is shared by every thread of the process, so these paths only ever raise it
 // (under this lock): a smaller request never lowers a limit another thread's launch relies on.
 namespace {
 std::mutex g_eval_smem_mutex;

@@ -15,6 +15,7 @@
 
 int fitcore_fail(int code, const std::string &msg);
 void fitcore_count_launch();
+int fitcore_raise_eval_smem(const void *func, size_t bytes);   // capi.cu
 
 namespace fitcore {
 
@@ -277,9 +278,10 @@ __global__ void __launch_bounds__(256) expected_rows_kernel(const DevModel *__re
 int expected_rows(const DevModel &h, const DevModel *dev, int B, const double *theta, float *mu, int *status,
                   cudaStream_t s) {
     const size_t smem = ((sizeof(RowSmem) + 15) & ~size_t(15)) + sizeof(float) * (2 * (size_t)h.P + 2 * h.N_t + h.max_reco);
-    if (cudaFuncSetAttribute(expected_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
+    // (raised only: the attribute is shared with other threads' calls for larger models)
+    if (fitcore_raise_eval_smem(reinterpret_cast<const void *>(&expected_rows_kernel), smem) != FIT_OK) {
         cudaGetLastError();
-        return fitcore_fail(FIT_ERR_CUDA, "expected rows: shared memory");
+        return FIT_ERR_CUDA;
     }
     expected_rows_kernel<<<std::min(B, 152 * 4), 256, smem, s>>>(dev, B, theta, mu, status);
     fitcore_count_launch();

@@ -874,7 +874,7 @@ __global__ void __launch_bounds__(T, MINB) fit_kernel(FitArgs A) {
     F.restarts = A.restarts;
     F.edm_tol = A.edm_tol;
     F.f_noise_rel = A.f_noise_rel;
-    F.deadline = global_ns() + A.budget_ns;   // per-block clock budget
+    F.deadline = global_ns() + A.budget_ns;   // per-block clock budget (the first thread's counts)
     const int tid = threadIdx.x;
 
     while (true) {
@@ -915,9 +915,13 @@ __global__ void __launch_bounds__(T, MINB) fit_kernel(FitArgs A) {
         float *ws = base + fit_work_floats(P);
         const float *data = A.data + in.data_off;
         constexpr bool pre = PRE;
-        if (tid == 0) init_state(S.st);
+        // (one thread reads the clock: the branches hold barriers, so the block must agree)
+        if (tid == 0) {
+            init_state(S.st);
+            S.step.next = global_ns() > F.deadline ? kNextDone : kNextDirection;
+        }
         __syncthreads();
-        if (global_ns() > F.deadline) {
+        if (S.step.next == kNextDone) {
 #pragma unroll 1
             for (int i = tid; i < P; i += blockDim.x) V.z[i] = 0.f;
             if (tid == 0) S.st.status = FIT_STATUS_TIMEOUT;

@@ -230,14 +230,16 @@ typedef struct fit_batch_opts {
                              on one warp, a lane per pair)                                   */
     double f_noise_rel;   /* relative noise allowance of -2lnL in the line search (1e-6)     */
     int threads;          /* threads per block, multiple of 32 in [64, 128]; 0 = chosen by the
-                             library from the models' sizes (128, 256 or 512) when blocks_per_sm
-                             and placement are 0 too, else 128                              */
+                             library from each model's size (128, 256 or 512; models of several
+                             sizes are fitted by launches side by side, each fit as it would be
+                             alone) when blocks_per_sm and placement are 0 too, else 128     */
     int blocks_per_sm;    /* resident blocks per SM (an upper bound): 5 or more selects the
                              96-register build of the kernel, 1-4 the 128-register one;
                              0 = automatic                                                  */
     int use_graph;        /* 1 = launch through a cached CUDA graph (work-queue memset and
                              kernel nodes, parameters updated in place for each call)        */
-    double time_budget_s; /* per-launch clock budget (0 = 60 s); exceeded -> FIT_STATUS_TIMEOUT */
+    double time_budget_s; /* clock budget of the fits, from their launch on (0 = 60 s); exceeded ->
+                             FIT_STATUS_TIMEOUT                                              */
     int restarts;         /* history restarts after the first EDM convergence, 0..8 (default 0):
                              each rebuilds the L-BFGS pairs for at least `history` iterations,
                              which firms up the EDM estimate in flat directions             */

@@ -2363,6 +2363,136 @@ bool pre_for_mask(fit_model *M, uint32_t mask, fitcore::PreEntry &e) {
 
 }  // namespace
 
+namespace {
+
+// the general build of the kernels: the 3+1 formula or the spline correction
+bool general_model(const DevModel &h) { return h.remap_mode == FIT_REMAP_SPLINE || h.n_osc == 6; }
+
+// A launch of the persistent fit kernel: the models whose instances it fits and its shape.
+struct FitLaunch {
+    std::vector<int> models;
+    int n = 0, threads = 128, grid = 0, placement = 0;
+    bool general = false, precond = false;
+    int max_need = 0, max_loc = 0;   // floats per block: all vectors and workspace; without the history
+    const void *kern = nullptr;
+
+    size_t smem_for(int pl) const { return fitcore::fit_smem_bytes(pl == 1 ? max_need : pl == 2 ? max_loc : 0); }
+};
+
+// Workspace placement and kernel variant (resident blocks per SM the registers allow).
+int fit_launch_shape(fit_model *const *models, const fit_batch_opts &o, bool auto_shape, const LaunchCfg &cfg,
+                     FitLaunch &L) {
+    // what a requested placement is judged by: 14 working vectors, the history, one dataset's
+    // workspace and 25184 bytes of block state within 112 KB
+    size_t ask_all = 0, ask_loc = 0;
+    for (int mi : L.models) {
+        const DevModel &h = models[mi]->host;
+        L.general = L.general || general_model(h);
+        // (multiples of 4 floats: the fit vectors start on 16-byte boundaries)
+        L.max_need = std::max(L.max_need, fitcore::fit_vec_floats(h.P, o.history) + h.ws_floats);
+        L.max_loc = std::max(L.max_loc, fitcore::fit_work_floats(h.P) + h.ws_floats);
+        const size_t one = (((size_t)(4 + h.n_osc + h.C) * h.N_t + 2 * h.max_reco + 3) & ~size_t(3)) + 14 * (size_t)fitcore::fit_vec_pitch(h.P);
+        ask_loc = std::max(ask_loc, 25184 + sizeof(float) * one);
+        ask_all = std::max(ask_all, 25184 + sizeof(float) * (one + (size_t)fitcore::fit_hist_floats(h.P, o.history)));
+    }
+    // Shared memory holds what fits in ~1/2 of an SM's share; the automatic choice takes the
+    // combination with the most resident fits per SM (ties: more in shared memory).
+    size_t kSmemCap = 112 * 1024;
+    L.placement = o.placement;
+    if (auto_shape && L.threads > 128) {
+        // Threads by the model (model_threads). Blocks of 256 and 512 threads keep the
+        // vectors and the evaluation workspace in shared memory (the history in L2) when two
+        // blocks, or one, then fit an SM; blocks of 128 threads keep everything in L2 for five
+        // fits per SM. Measured (ms, 128 x 5 / 256 x 2 / 512 x 1 per SM): 1000 fits of the 53 km
+        // model 14.0 / 11.5 / 10.8 and a scan of 42 of its fits 6.5 / 3.9 / 2.6; 300 three-dataset
+        // fits 7.0 / 4.2 / -, 2500 with the spline 7.1 / 8.5 / 12.0; 2500 single-detector fits 2.2 / 2.5
+        // / 4.1. Many waves of fits run faster in blocks of 128 (8192: 62.5 against 75.3 and 43.5
+        // against 50.0 under this rule), which fit_batch_autotune finds; the number of fits is not
+        // looked at, so that a fit does not depend on the batch around it.
+        L.placement = L.smem_for(2) * (512 / L.threads) > cfg.smem_optin ? 3 : 2;
+    }
+    auto kernel_for = [&](int variant) { return fitcore::fit_kernel_func(L.threads, variant, L.general, L.precond); };
+    auto blocks_for = [&](int pl, int variant) -> int {
+        const size_t sm = L.smem_for(pl);
+        if (sm > std::min(kSmemCap, cfg.smem_optin)) return 0;
+        auto k = kernel_for(variant);
+        if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess) {
+            cudaGetLastError();
+            return 0;
+        }
+        int n = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, L.threads, sm) != cudaSuccess) {
+            cudaGetLastError();
+            return 0;
+        }
+        return n;
+    };
+    int variant = o.blocks_per_sm >= 5 ? 5 : 4;
+    if (L.placement == 0) {
+        int best_n = -1;
+        for (int pl : {1, 2, 3}) {
+            const int v = o.blocks_per_sm > 0 ? variant : (pl == 3 ? 5 : 4);
+            const int n = blocks_for(pl, v);
+            if (n > best_n) {
+                best_n = n;
+                L.placement = pl;
+                variant = v;
+            }
+        }
+    } else {
+        if (o.blocks_per_sm == 0) variant = L.placement == 3 ? 5 : 4;
+        const size_t ask = L.placement == 1 ? ask_all : L.placement == 2 ? ask_loc : 0;
+        if (!auto_shape && ask > 112 * 1024)
+            return fail(FIT_ERR_INVALID_CONFIG, "fit_batch: the requested workspace placement does not fit an SM");
+        kSmemCap = cfg.smem_optin;
+    }
+    if (blocks_for(L.placement, variant) < 1)
+        return fail(FIT_ERR_INVALID_CONFIG, "fit_batch: the requested workspace placement does not fit an SM");
+    L.kern = kernel_for(variant);
+    return FIT_OK;
+}
+
+// The grid: the resident blocks, at most one per instance.
+int fit_launch_grid(const fit_batch_opts &o, const LaunchCfg &cfg, FitLaunch &L) {
+    const size_t smem = L.smem_for(L.placement);
+    FIT_CUDA(cudaFuncSetAttribute(L.kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)std::min(smem, cfg.smem_optin)));
+    int per_sm = 0;
+    FIT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, L.kern, L.threads, smem));
+    if (per_sm < 1) return fail(FIT_ERR_INVALID_CONFIG, "fit_batch: launch configuration does not fit an SM");
+    if (o.blocks_per_sm > 0) per_sm = std::min(per_sm, o.blocks_per_sm);
+    L.grid = std::max(1, std::min(L.n, per_sm * cfg.sms));
+    return FIT_OK;
+}
+
+// Streams for the launches of a call past the first, one set per device, made on first use (guarded by
+// g_ws_mutex, as their use is: fit_batch joins them to the caller's stream before it lets go).
+struct SideStreams {
+    std::vector<cudaStream_t> streams;
+    std::vector<cudaEvent_t> done;   // one per stream
+    cudaEvent_t ready = nullptr;
+};
+
+int side_streams(int n, SideStreams *&out) {
+    static std::vector<SideStreams> all;
+    int dev = 0;
+    FIT_CUDA(cudaGetDevice(&dev));
+    if ((int)all.size() <= dev) all.resize(dev + 1);
+    SideStreams &S = all[dev];
+    if (!S.ready) FIT_CUDA(cudaEventCreateWithFlags(&S.ready, cudaEventDisableTiming));
+    while ((int)S.done.size() < n) {
+        cudaStream_t st;
+        cudaEvent_t ev;
+        FIT_CUDA(cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking));
+        S.streams.push_back(st);
+        FIT_CUDA(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
+        S.done.push_back(ev);
+    }
+    out = &S;
+    return FIT_OK;
+}
+
+}  // namespace
+
 extern "C" {
 
 int fit_linear_start(fit_model *model, int B, const float *data, const uint32_t *masks, double *theta_out,
@@ -2464,7 +2594,6 @@ int fit_batch_ex(fit_model *const *models, int n_models, const fit_instance *ins
     cudaStream_t s = (cudaStream_t)stream;
     // extents of the flat data / parameter arrays
     int64_t data_len = 0, par_len = 0;
-    int max_need = 0;
     for (int i = 0; i < n_inst; ++i) {
         const fit_instance &q = inst[i];
         if (q.model < 0 || q.model >= n_models || !models[q.model] || q.data_off < 0 || q.param_off < 0)
@@ -2498,48 +2627,11 @@ int fit_batch_ex(fit_model *const *models, int n_models, const fit_instance *ins
                                   data_len, par_len, pre, o.engine == 2);
     }
     if (o.engine != 0) return fail(FIT_ERR_INVALID_ARG, "fit_batch: engine must be 0, 1 or 2");
-    int max_loc = 0;   // working vectors + evaluation workspace, without the history
-    // what a requested placement is judged by: 14 working vectors, the history, one dataset's
-    // workspace and 25184 bytes of block state within 112 KB
-    size_t ask_all = 0, ask_loc = 0;
-    bool general = false;   // the general build when any model uses the 3+1 formula or the spline
-    for (int mi = 0; mi < n_models; ++mi) {
-        const DevModel &h = models[mi]->host;
-        general = general || h.remap_mode == FIT_REMAP_SPLINE || h.n_osc == 6;
-        // (multiples of 4 floats: the fit vectors start on 16-byte boundaries)
-        max_need = std::max(max_need, fitcore::fit_vec_floats(h.P, o.history) + h.ws_floats);
-        max_loc = std::max(max_loc, fitcore::fit_work_floats(h.P) + h.ws_floats);
-        const size_t one = (((size_t)(4 + h.n_osc + h.C) * h.N_t + 2 * h.max_reco + 3) & ~size_t(3)) + 14 * (size_t)fitcore::fit_vec_pitch(h.P);
-        ask_loc = std::max(ask_loc, 25184 + sizeof(float) * one);
-        ask_all = std::max(ask_all, 25184 + sizeof(float) * (one + (size_t)fitcore::fit_hist_floats(h.P, o.history)));
-    }
     if (o.placement < 0 || o.placement > 3) return fail(FIT_ERR_INVALID_ARG, "fit_batch: placement must be 0..3");
     LaunchCfg cfg;
     int rc = device_cfg(cfg);
     if (rc) return rc;
     std::lock_guard<std::mutex> lock(g_ws_mutex);
-    // Workspace placement and kernel variant (resident blocks per SM the registers allow).
-    // Shared memory holds what fits in ~1/2 of an SM's share; the automatic choice takes the
-    // combination with the most resident fits per SM (ties: more in shared memory).
-    size_t kSmemCap = 112 * 1024;
-    auto smem_for = [&](int pl) -> size_t {
-        if (pl == 1) return fitcore::fit_smem_bytes(max_need);
-        if (pl == 2) return fitcore::fit_smem_bytes(max_loc);
-        return fitcore::fit_smem_bytes(0);
-    };
-    if (auto_shape) {
-        // Threads by the largest model (model_threads). Blocks of 256 and 512 threads keep the
-        // vectors and the evaluation workspace in shared memory (the history in L2) when two
-        // blocks, or one, then fit an SM; blocks of 128 threads keep everything in L2 for five
-        // fits per SM. Measured (ms, 128 x 5 / 256 x 2 / 512 x 1 per SM): 1000 fits of the 53 km
-        // model 14.0 / 11.5 / 10.8 and a scan of 42 of its fits 6.5 / 3.9 / 2.6; 300 three-dataset
-        // fits 7.0 / 4.2 / -, 2500 with the spline 7.1 / 8.5 / 12.0; 2500 single-detector fits 2.2 / 2.5
-        // / 4.1. Many waves of fits run faster in blocks of 128 (8192: 62.5 against 75.3 and 43.5
-        // against 50.0 under this rule), which fit_batch_autotune finds; the number of fits is not
-        // looked at, so that a fit does not depend on the batch around it.
-        for (int i = 0; i < n_models; ++i) o.threads = std::max(o.threads, fitcore::model_threads(models[i]->host));
-        if (o.threads > 128) o.placement = smem_for(2) * (512 / o.threads) > cfg.smem_optin ? 3 : 2;
-    }
     // the preconditioned build when asked for and every model has its preconditioner
     bool precond = o.precondition != 0;
     std::vector<fitcore::PreEntry> pre_tab;   // [n_models x pre_k]: dataset-subset preconditioners
@@ -2550,77 +2642,77 @@ int fit_batch_ex(fit_model *const *models, int n_models, const fit_instance *ins
             build_preconditioner(models[i], s);
             precond = precond && models[i]->pre_state == 1;
         }
-        if (precond) {
-            // the distinct dataset subsets each model's instances fit (up to 8 per model; an
-            // instance whose subset has no entry uses the all-datasets preconditioner)
-            constexpr int kMaxSubsets = 8;
-            std::vector<std::vector<uint32_t>> subsets(n_models);
-            for (int i = 0; i < n_inst; ++i) {
-                const fit_model *mm = models[inst[i].model];
-                const uint32_t all = (1u << mm->host.n_ds) - 1u, mk = inst[i].mask & all;
-                auto &v = subsets[inst[i].model];
-                if (mk != all && (int)v.size() < kMaxSubsets && std::find(v.begin(), v.end(), mk) == v.end())
-                    v.push_back(mk);
-            }
-            for (auto &v : subsets) pre_k = std::max(pre_k, (int)v.size());
-            if (pre_k > 0) {
-                pre_tab.assign((size_t)n_models * pre_k, fitcore::PreEntry{});
-                for (int mi = 0; mi < n_models; ++mi)
-                    for (size_t q = 0; q < subsets[mi].size(); ++q) {
-                        fitcore::PreEntry e{};
-                        if (pre_for_mask(models[mi], subsets[mi][q], e)) pre_tab[(size_t)mi * pre_k + q] = e;
-                    }
-            }
+        // the distinct dataset subsets each model's instances fit (up to 8 per model; an
+        // instance whose subset has no entry uses the all-datasets preconditioner)
+        constexpr int kMaxSubsets = 8;
+        std::vector<std::vector<uint32_t>> subsets(n_models);
+        for (int i = 0; i < n_inst; ++i) {
+            const fit_model *mm = models[inst[i].model];
+            const uint32_t all = (1u << mm->host.n_ds) - 1u, mk = inst[i].mask & all;
+            auto &v = subsets[inst[i].model];
+            if (mm->pre_state == 1 && mk != all && (int)v.size() < kMaxSubsets &&
+                std::find(v.begin(), v.end(), mk) == v.end())
+                v.push_back(mk);
+        }
+        for (auto &v : subsets) pre_k = std::max(pre_k, (int)v.size());
+        if (pre_k > 0) {
+            pre_tab.assign((size_t)n_models * pre_k, fitcore::PreEntry{});
+            for (int mi = 0; mi < n_models; ++mi)
+                for (size_t q = 0; q < subsets[mi].size(); ++q) {
+                    fitcore::PreEntry e{};
+                    if (pre_for_mask(models[mi], subsets[mi][q], e)) pre_tab[(size_t)mi * pre_k + q] = e;
+                }
         }
     }
-    auto kernel_for = [&](int variant) { return fitcore::fit_kernel_func(o.threads, variant, general, precond); };
-    auto blocks_for = [&](int pl, int variant) -> int {
-        const size_t sm = smem_for(pl);
-        if (sm > std::min(kSmemCap, cfg.smem_optin)) return 0;
-        auto k = kernel_for(variant);
-        if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess) {
-            cudaGetLastError();
-            return 0;
-        }
-        int n = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, o.threads, sm) != cudaSuccess) {
-            cudaGetLastError();
-            return 0;
-        }
-        return n;
-    };
-    int placement = o.placement, variant = o.blocks_per_sm >= 5 ? 5 : 4;
-    if (placement == 0) {
-        int best_n = -1;
-        for (int pl : {1, 2, 3}) {
-            const int v = o.blocks_per_sm > 0 ? variant : (pl == 3 ? 5 : 4);
-            const int n = blocks_for(pl, v);
-            if (n > best_n) {
-                best_n = n;
-                placement = pl;
-                variant = v;
-            }
-        }
+    // One launch over all instances where the caller gives any part of its shape; else one per shape
+    // that the models select, so that a fit's kernel and bits are those of its own model whatever is
+    // fitted beside it. (With the largest model's shape for the whole call 2500 single-detector
+    // fits took 9.7 instead of 6.0 ms beside a 53 km model that no instance used, 5461 three-dataset and
+    // 2731 53 km fits 72.1 instead of 57.5; 60 and 30 of them, which leave SMs idle, 2.9, not 3.8.)
+    std::vector<FitLaunch> launches;
+    if (!auto_shape) {
+        FitLaunch L;
+        L.threads = o.threads;
+        L.precond = precond;
+        for (int i = 0; i < n_models; ++i) L.models.push_back(i);
+        if ((rc = fit_launch_shape(models, o, false, cfg, L))) return rc;
+        launches.push_back(L);
     } else {
-        if (o.blocks_per_sm == 0) variant = placement == 3 ? 5 : 4;
-        const size_t ask = placement == 1 ? ask_all : placement == 2 ? ask_loc : 0;
-        if (!auto_shape && ask > 112 * 1024)
-            return fail(FIT_ERR_INVALID_CONFIG, "fit_batch: the requested workspace placement does not fit an SM");
-        kSmemCap = cfg.smem_optin;
+        std::vector<char> used(n_models, 0);
+        for (int i = 0; i < n_inst; ++i) used[inst[i].model] = 1;
+        for (int i = 0; i < n_models; ++i) {
+            if (!used[i]) continue;
+            FitLaunch L;
+            L.threads = fitcore::model_threads(models[i]->host);
+            L.precond = o.precondition != 0 && models[i]->pre_state == 1;
+            L.models.push_back(i);
+            if ((rc = fit_launch_shape(models, o, true, cfg, L))) return rc;
+            FitLaunch *with = nullptr;
+            for (FitLaunch &q : launches)
+                if (q.kern == L.kern && q.threads == L.threads && q.placement == L.placement) with = &q;
+            if (with) {
+                with->models.push_back(i);
+                with->max_need = std::max(with->max_need, L.max_need);
+                with->max_loc = std::max(with->max_loc, L.max_loc);
+            } else {
+                launches.push_back(L);
+            }
+        }
+        // the largest blocks, which hold the longest fits, first
+        std::stable_sort(launches.begin(), launches.end(),
+                         [](const FitLaunch &x, const FitLaunch &y) { return x.threads > y.threads; });
     }
-    if (blocks_for(placement, variant) < 1)
-        return fail(FIT_ERR_INVALID_CONFIG, "fit_batch: the requested workspace placement does not fit an SM");
-    const bool in_smem = placement == 1;
-    const size_t smem = smem_for(placement);
-    auto kern = kernel_for(variant);
-    FIT_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)std::min(smem, cfg.smem_optin)));
-    int per_sm = 0;
-    FIT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, o.threads, smem));
-    if (per_sm < 1) return fail(FIT_ERR_INVALID_CONFIG, "fit_batch: launch configuration does not fit an SM");
-    if (o.blocks_per_sm > 0) per_sm = std::min(per_sm, o.blocks_per_sm);
-    const int grid = std::max(1, std::min(n_inst, per_sm * cfg.sms));
+    std::vector<int> launch_of(n_models, 0);
+    for (size_t q = 0; q < launches.size(); ++q)
+        for (int mi : launches[q].models) launch_of[mi] = (int)q;
+    for (int i = 0; i < n_inst; ++i) launches[launch_of[inst[i].model]].n++;
+    for (FitLaunch &L : launches)
+        if ((rc = fit_launch_grid(o, cfg, L))) return rc;
+    SideStreams *side = nullptr;
+    if (launches.size() > 1 && (rc = side_streams((int)launches.size() - 1, side))) return rc;
 
-    Staged dm, di, dd, dst, dfx, dbe, dre, dws, dq, dord;
+    Staged dm, di, dd, dst, dfx, dbe, dre, dq, dord;
+    std::vector<Staged> dws(launches.size());
     bool hbe = false, hre = false;
     std::vector<DevModel> hm(n_models);
     for (int i = 0; i < n_models; ++i) hm[i] = models[i]->host;
@@ -2639,13 +2731,17 @@ int fit_batch_ex(fit_model *const *models, int n_models, const fit_instance *ins
             cost[i] = (double)nd * h.N_t * (h.C + 4) + h.P;
             order[i] = i;
         }
-        std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return cost[a] > cost[b]; });
+        std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
+            const int la = launch_of[inst[a].model], lb = launch_of[inst[b].model];
+            return la != lb ? la < lb : cost[a] > cost[b];   // launch after launch
+        });
+        reordered = launches.size() > 1;
         for (int i = 0; i < n_inst && !reordered; ++i) reordered = order[i] != i;
     }
     Staged dpre;
     rc = stage_in(hm.data(), sizeof(DevModel) * n_models, s, dm);
     if (!rc && reordered) rc = stage_in(order.data(), sizeof(int) * n_inst, s, dord);
-    if (!rc && precond && pre_k > 0)
+    if (!rc && pre_k > 0)
         rc = stage_in(pre_tab.data(), sizeof(fitcore::PreEntry) * pre_tab.size(), s, dpre);
     if (!rc) rc = stage_in(inst, sizeof(fit_instance) * n_inst, s, di);
     if (!rc) rc = stage_in(data, sizeof(float) * data_len, s, dd);
@@ -2653,21 +2749,38 @@ int fit_batch_ex(fit_model *const *models, int n_models, const fit_instance *ins
     if (!rc && fixed) rc = stage_in(fixed, (size_t)par_len, s, dfx);
     if (!rc) rc = stage_out(best, sizeof(double) * par_len, s, dbe, hbe);
     if (!rc) rc = stage_out(results, sizeof(fit_result) * n_inst, s, dre, hre);
-    if (!rc && !in_smem) {
-        if (fitcore::pool_alloc(&dws.dev, sizeof(float) * (size_t)grid * max_need, s))
+    for (size_t q = 0; q < launches.size() && !rc; ++q) {
+        if (launches[q].placement == 1) continue;
+        if (fitcore::pool_alloc(&dws[q].dev, sizeof(float) * (size_t)launches[q].grid * launches[q].max_need, s))
             rc = fail(FIT_ERR_OOM, "fit_batch: workspace");
-        dws.owned = true;
+        dws[q].owned = true;
     }
+    // the work queues, 8 bytes apart, then (several launches) the time that the first block started at
+    const size_t q_bytes = 8 * (launches.size() + 1);
     if (!rc) {
-        if (fitcore::pool_alloc(&dq.dev, sizeof(int), s) || (!o.use_graph && cudaMemsetAsync(dq.dev, 0, sizeof(int), s)))
+        if (fitcore::pool_alloc(&dq.dev, q_bytes, s) ||
+            ((!o.use_graph || side) && cudaMemsetAsync(dq.dev, 0, q_bytes, s)))
             rc = fail(FIT_ERR_CUDA, "fit_batch: queue");
         dq.owned = true;
     }
-    if (!rc) {
+    if (!rc && side && cudaEventRecord(side->ready, s) != cudaSuccess) rc = fail(FIT_ERR_CUDA, "fit_batch: fork");
+    size_t forked = 0;
+    for (size_t q = 0, first = 0; q < launches.size() && !rc; first += launches[q++].n) {
+        const FitLaunch &L = launches[q];
+        // the launches run side by side: the first on the caller's stream, the others on streams that wait for
+        // the staging here and are waited for below
+        cudaStream_t ls = s;
+        if (q > 0) {
+            ls = side->streams[q - 1];
+            if (cudaStreamWaitEvent(ls, side->ready, 0) != cudaSuccess) {
+                rc = fail(FIT_ERR_CUDA, "fit_batch: fork");
+                break;
+            }
+        }
         fitcore::FitArgs a;
         a.models = (const DevModel *)dm.dev;
         a.inst = (const fit_instance *)di.dev;
-        a.n_inst = n_inst;
+        a.n_inst = L.n;
         a.hist = o.history;
         a.max_iter = o.max_iter;
         a.max_ls = 8;
@@ -2679,25 +2792,40 @@ int fit_batch_ex(fit_model *const *models, int n_models, const fit_instance *ins
         a.fixed = fixed ? (const uint8_t *)dfx.dev : nullptr;
         a.best = (double *)dbe.dev;
         a.results = (fit_result *)dre.dev;
-        a.queue = (int *)dq.dev;
-        a.ws_global = (float *)dws.dev;
-        a.ws_stride = max_need;
-        a.smem_floats = placement == 1 ? max_need : placement == 2 ? max_loc : 0;
-        a.hist_global = placement == 1 ? 0 : 1;
+        a.queue = (int *)((char *)dq.dev + 8 * q);
+        a.ws_global = (float *)dws[q].dev;
+        a.ws_stride = L.max_need;
+        a.smem_floats = L.placement == 1 ? L.max_need : L.placement == 2 ? L.max_loc : 0;
+        a.hist_global = L.placement == 1 ? 0 : 1;
         a.budget_ns = (uint64_t)(o.time_budget_s * 1e9);
-        a.precond = precond ? 1 : 0;
-        a.order = reordered ? (const int *)dord.dev : nullptr;
-        a.pre_tab = (precond && pre_k > 0) ? (const fitcore::PreEntry *)dpre.dev : nullptr;
+        a.began = side ? (unsigned long long *)((char *)dq.dev + 8 * launches.size()) : nullptr;
+        a.precond = L.precond ? 1 : 0;
+        a.order = reordered ? (const int *)dord.dev + first : nullptr;
+        a.pre_tab = (L.precond && pre_k > 0) ? (const fitcore::PreEntry *)dpre.dev : nullptr;
         a.pre_per_model = pre_k;
+        const size_t smem = L.smem_for(L.placement);
         if (o.use_graph) {
-            rc = graph_launch(kern, grid, o.threads, smem, a, (int *)dq.dev, s);
+            rc = graph_launch(L.kern, L.grid, L.threads, smem, a, a.queue, ls);
         } else {
             void *args[] = {&a};
-            cudaError_t e = cudaLaunchKernel(kern, dim3(grid), dim3(o.threads), args, smem, s);
-            if (e != cudaSuccess) rc = fail(FIT_ERR_CUDA, std::string("fit_kernel launch: ") + cudaGetErrorString(e));
+            cudaError_t e = cudaLaunchKernel(L.kern, dim3(L.grid), dim3(L.threads), args, smem, ls);
+            if (e != cudaSuccess) {
+                cudaGetLastError();
+                rc = fail(FIT_ERR_CUDA, std::string("fit_kernel launch: ") + cudaGetErrorString(e));
+            }
         }
         g_launches++;
+        if (q > 0) {
+            if (cudaEventRecord(side->done[q - 1], ls) == cudaSuccess) {
+                forked = q;
+            } else {
+                cudaStreamSynchronize(ls);
+                rc = fail(FIT_ERR_CUDA, "fit_batch: join");
+            }
+        }
     }
+    for (size_t q = 0; q < forked; ++q)   // also after an error: nothing below may overtake a launch
+        if (cudaStreamWaitEvent(s, side->done[q], 0) != cudaSuccess && !rc) rc = fail(FIT_ERR_CUDA, "fit_batch: join");
     if (!rc && hbe) {
         // copy back only the parameter ranges the instances own (merged intervals), so that
         // other entries of a host `best` array keep their values
@@ -2723,7 +2851,8 @@ int fit_batch_ex(fit_model *const *models, int n_models, const fit_instance *ins
     }
     if (!rc && hre && cudaMemcpyAsync(results, dre.dev, sizeof(fit_result) * n_inst, cudaMemcpyDeviceToHost, s))
         rc = fail(FIT_ERR_CUDA, "fit_batch: copy back");
-    for (Staged *b : {&dm, &di, &dd, &dst, &dfx, &dbe, &dre, &dws, &dq, &dord, &dpre}) release(*b, s);
+    for (Staged *b : {&dm, &di, &dd, &dst, &dfx, &dbe, &dre, &dq, &dord, &dpre}) release(*b, s);
+    for (Staged &b : dws) release(b, s);
     // the staged model table and instance table are host vectors: finish before they go away
     if (!rc && cudaStreamSynchronize(s) != cudaSuccess) rc = fail(FIT_ERR_CUDA, "fit_batch: synchronise");
     return rc;

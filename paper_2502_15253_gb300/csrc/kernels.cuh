@@ -47,6 +47,8 @@ struct FitArgs {
     int hist_global;             // 1: the L-BFGS history lives in the global slice
     const uint8_t *fixed;        // device, indexed like start/best, or nullptr: held parameters
     uint64_t budget_ns;
+    unsigned long long *began;   // device word, zero at launch, or nullptr: several launches of one call
+                                 // share the clock budget, from their first block's start
     int precond;                 // 1: fit in the models' preconditioned coordinates (if built)
     const int *order;            // device [n_inst] or nullptr: the instance taken at each queue
                                  // position (costliest first, so no long fit starts last)

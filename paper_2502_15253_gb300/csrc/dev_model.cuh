@@ -273,7 +273,7 @@ __device__ __forceinline__ f32x2 neg_phase2(f32x2 dm, f32x2 ndm, f32x2 dm_lo, f3
 
 // sin^2(pi r) for |r| <= 1/2: u q(u), u = r^2, q a degree-7 polynomial fitted for the
 // smallest largest absolute error (Lawson iteration; sin2pi_fit.py in this directory). Its
-// FP32 evaluation is within 1.8e-7 of sin^2.
+// FP32 evaluation is within 1.8e-7 of sin^2. (This form states the constants for one phase.)
 __device__ __forceinline__ float sin2pi(float r) {
     const float u = r * r;
     float q = -0.122019291f;
@@ -287,13 +287,17 @@ __device__ __forceinline__ float sin2pi(float r) {
     return u * q;
 }
 
-// sin^2 of the phase pi (dm + dm_lo)(c_hi + c_lo): the half-turn count reduced by its nearest
-// integer as in the binned evaluation. Both pairs normalised (|low| <= ulp(high) / 2), so the
-// reduced phase stays within 1/2 (the polynomial's range) up to rounding.
-__device__ __forceinline__ float sin2_phase(float dm, float dm_lo, float c_hi, float c_lo) {
-    const float yh = dm * c_hi;
-    const float yl = fmaf(dm, c_hi, -yh) + fmaf(dm, c_lo, dm_lo * c_hi);
-    return sin2pi((yh - rintf(yh)) + yl);
+// The same for two phases: what the event kernel evaluates.
+__device__ __forceinline__ f32x2 sin2pi2(f32x2 r) {
+    const f32x2 u = mul2(r, r);
+    f32x2 q = fma2(pack2(-0.122019291f), u, pack2(0.848584056f));
+    q = fma2(q, u, pack2(-3.94964409f));
+    q = fma2(q, u, pack2(13.2128229f));
+    q = fma2(q, u, pack2(-30.1222954f));
+    q = fma2(q, u, pack2(42.7284088f));
+    q = fma2(q, u, pack2(-32.469696f));
+    q = fma2(q, u, pack2(9.86960411f));
+    return mul2(u, q);
 }
 
 // Coefficients of the sin^2 terms of P, formed once per evaluation in double from the exact

@@ -123,8 +123,8 @@ __device__ McSet make_set(int mode, const double *p) {
     return s;
 }
 
-// P(L, E) of a lane's kV events for one set, in pairs: 1 - sum_i C_i sin^2(x_i), the arithmetic of
-// sin2_phase in packed FP32 (the phase negative, which sin^2 does not see). From two or three
+// P(L, E) of a lane's kV events for one set, in pairs: 1 - sum_i C_i sin^2(x_i), the phases
+// reduced as float pairs (negative, which sin^2 does not see), all in packed FP32. From two or three
 // sets per pass on the kernel is bound by instruction issue, and a packed instruction does two
 // events' work in one slot; the phases are the outer loop, so that a set's operands are read
 // once per lane. 24 sets of 1.5M three-flavour events: 122 us with scalar instructions, 110 us.
@@ -139,15 +139,7 @@ __device__ __forceinline__ void survival_run(const McSet &S, const f32x2 (&c_hi)
 #pragma unroll
         for (int v = 0; v < kV / 2; ++v) {
             const f32x2 r = neg_phase2(p.dm, p.ndm, p.dm_lo, c_hi[v], c_lo[v], pack2(-1.f));
-            const f32x2 u = mul2(r, r);   // sin2pi (even)
-            f32x2 q = fma2(pack2(-0.122019291f), u, pack2(0.848584056f));
-            q = fma2(q, u, pack2(-3.94964409f));
-            q = fma2(q, u, pack2(13.2128229f));
-            q = fma2(q, u, pack2(-30.1222954f));
-            q = fma2(q, u, pack2(42.7284088f));
-            q = fma2(q, u, pack2(-32.469696f));
-            q = fma2(q, u, pack2(9.86960411f));
-            P[v] = fma2(p.nC, mul2(u, q), P[v]);
+            P[v] = fma2(p.nC, sin2pi2(r), P[v]);
         }
     }
 }

@@ -481,7 +481,6 @@ int fit_model_create(const fit_model_desc *d, fit_model **out) {
         h.osc_idx[i] = i < n_osc ? d->osc_idx[i] : -1;
         h.osc_val[i] = (float)v;
         h.osc_val_lo[i] = (float)(v - (double)h.osc_val[i]);
-        h.osc_val_d[i] = v;
     }
     for (int c = 0; c < C; ++c) h.core_power_idx[c] = d->core_power_idx[c];
     {

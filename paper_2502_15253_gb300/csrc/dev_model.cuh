@@ -91,7 +91,6 @@ struct DevModel {
     int osc_idx[kMaxOsc];
     float osc_val[kMaxOsc];
     float osc_val_lo[kMaxOsc];   // low parts of the constant survival parameters
-    double osc_val_d[kMaxOsc];   // the constant survival parameters in double
     float osc_th_f[kMaxOsc], osc_th_lo[kMaxOsc];   // theta0 of the fitted ones as a float pair
     int osc_dup;             // as DevDataset::map_dup: bits of the survival parameters, then the powers
     int any_map_dup;         // 1: osc_dup or some dataset's map_dup is not 0
@@ -497,9 +496,6 @@ __device__ __forceinline__ float deviance(float n, float mu, float diff) {
 struct ParVecs {
     const float *pv, *pd, *pl;
 };
-__device__ __forceinline__ float pval(const float *pv, int idx, float dflt) {
-    return idx >= 0 ? pv[idx] : dflt;
-}
 
 // A parameter as the float pair h + l: h = its float value, l = the exact rounding residual
 // (theta0_f - h) + delta + theta0_lo. Products x * theta are then formed as fma(x, l, x h),

@@ -13,7 +13,6 @@ __device__ __forceinline__ void copy_model(DevModel *dst, const DevModel *src) {
     const int n = (int)(sizeof(DevModel) / sizeof(int));
     const int *s = reinterpret_cast<const int *>(src);
     int *d = reinterpret_cast<int *>(dst);
-#pragma unroll 4
 #pragma unroll 1
     for (int i = threadIdx.x; i < n; i += blockDim.x) d[i] = s[i];
     __syncthreads();

@@ -175,9 +175,10 @@ __device__ __forceinline__ void reset_history(FitState &st) {
     st.gamma = 1.0;
 }
 
-// num / den in double from the FP32 reciprocal, two Newton steps and one correction of the quotient
-// by its residual (within an ulp): the library's double division takes 1467 cycles here, this
-// about 450. Operands outside FP32's normal range take the division.
+// num / den in double: the FP32 reciprocal, two Newton-Raphson steps for 1 / den and one correction of
+// the quotient by its residual (within an ulp: tests/test_quick_division.py). The library's double
+// division takes 1467 cycles here, this about 450. Operands outside FP32's normal range take the
+// division.
 static __device__ __noinline__ double quick_div(double num, double den) {
     const float d = (float)den;
     if (!(fabsf(d) > 1e-30f && fabsf(d) < 1e30f)) return num / den;

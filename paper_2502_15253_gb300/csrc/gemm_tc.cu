@@ -253,8 +253,8 @@ __device__ __forceinline__ void stage_aux(EpiStage &st, const float4 (&q)[4]) {
 }
 
 // Epilogue of one 32-row x 16-column chunk: rows row0 + [0, nrow), columns n + [0, nv); v holds
-// this thread's row (row0 + lane) of the accumulator. C: out.C, or this K share's own product.
-__device__ __forceinline__ void epi_chunk(const GemmOut &out, float *C, EpiStage &st, bool split, int row0, int n,
+// this thread's row (row0 + lane) of the accumulator. share: the K share, if they are stored apart.
+__device__ __forceinline__ void epi_chunk(const GemmOut &out, int share, EpiStage &st, bool split, int row0, int n,
                                           int nrow, int nv, float (&v)[16]) {
     const int lane = threadIdx.x & 31;
     const bool vc = out.vec & 1, vy = out.vec & 2, vt = out.vec & 8;
@@ -266,7 +266,7 @@ __device__ __forceinline__ void epi_chunk(const GemmOut &out, float *C, EpiStage
 #pragma unroll
             for (int j = 0; j < 4; ++j) st.c[cidx(lane, j)] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
             __syncwarp();
-            flush_c(st, C, out.ldc, row0, n, nrow, nv, vc, split, out.epi == EPI_F32_ADD);
+            flush_c(st, out.C + share * out.share_stride, out.ldc, row0, n, nrow, nv, vc, split, out.epi == EPI_F32_ADD);
             break;
         }
         case EPI_BIAS_GELU: {
@@ -278,7 +278,7 @@ __device__ __forceinline__ void epi_chunk(const GemmOut &out, float *C, EpiStage
             for (int j = 0; j < 4; ++j) st.c[cidx(lane, j)] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
             stage_bf16(st, w, out.Yt != nullptr);
             __syncwarp();
-            flush_c(st, C, out.ldc, row0, n, nrow, nv, vc, false, false);
+            flush_c(st, out.C, out.ldc, row0, n, nrow, nv, vc, false, false);
             flush_y(st, out.Y, out.ldy, row0, n, nrow, nv, vy);
             if (out.Yt) flush_yt(st, out.Yt, out.ldyt, row0, n, nrow, nv, vt);
             break;
@@ -460,7 +460,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 break;
             }
             umma::tc_fence_after();
-            float *C = out.C + (kt0 / pl.kt_per) * out.share_stride;
+            const int share = u / (pl.ntn * pl.mt);
             const uint32_t tbase = tmem + (uint32_t)(a * pl.acc_cols) + ((uint32_t)(quad * 32) << 16);
             for (int c = sub * 16; c < n_tile; c += 64) {
                 const int nv = chunk_nv(c);
@@ -473,7 +473,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                         const int nv2 = chunk_nv(c + 64);
                         if (nv2 > 0) load_aux(out, row0, n0 + c + 64, nrow, nv2, qa);
                     }
-                    epi_chunk(out, C, st, split, row0, n0 + c, nrow, nv, v);
+                    epi_chunk(out, share, st, split, row0, n0 + c, nrow, nv, v);
                 }
             }
             umma::tc_fence_before();

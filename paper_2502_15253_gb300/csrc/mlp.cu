@@ -29,7 +29,9 @@ inline int pad8(int x) { return (x + 7) / 8 * 8; }
 // bits on every run: each such block and each K share of a weight gradient leaves its own partial
 // sum, and the AdamW kernel, which reads every gradient once, adds them in order. With atomics the
 // first step's gradients differed by 1e-7 from run to run, and the steps after it, through AdamW and
-// the bf16 roundings, by up to 1.5e-3 (438 -> 3 x 512 -> 12, batch 4096).
+// the bf16 roundings, by up to 1.5e-3 (438 -> 3 x 512 -> 12, batch 4096). A step took 163 us at batch
+// 512, 205 at 4096 and 357 at 16384 with atomics and their clears; it takes 144, 195 and 362 (the
+// largest batch has 57 MB of shares to store and read).
 constexpr int kColRows = 256;
 
 __global__ void prep_input_kernel(int B, int n_in, int ld, const float *__restrict__ x, __nv_bfloat16 *__restrict__ a0) {
@@ -182,21 +184,33 @@ __global__ void __launch_bounds__(256) adamw_all_kernel(AdamW h, AdamAll A) {
     t -= A.first[l];
     if (t < L.wtiles) {
         const int o0 = (t / L.tiles_i) * 32, i0 = (t % L.tiles_i) * 32;
-        for (int r = threadIdx.y; r < 32; r += blockDim.y) {
-            const int o = o0 + r, i = i0 + threadIdx.x;
+        // the gradients of this thread's four weights: the K shares added in order, sixteen loads in
+        // flight (the shares come from L2; past the ends the last row or share is read again)
+        const int i = i0 + threadIdx.x, shares = L.shares, last = L.out - 1;
+        const int64_t in = L.in, pitch = shares > 1 ? L.pitch : 0;
+        const float *src = (shares > 1 ? L.part : L.g) + min(i, L.in - 1);
+        float g[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 1
+        for (int z0 = 0; z0 < shares; z0 += 4) {
+            float q[4][4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    q[j][k] = __ldcg(src + min(z0 + j, shares - 1) * pitch + min(o0 + (int)threadIdx.y + 8 * k, last) * in);
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+#pragma unroll
+                for (int k = 0; k < 4; ++k) g[k] += z0 + j < shares ? q[j][k] : 0.f;
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int r = threadIdx.y + 8 * k, o = o0 + r;
             __nv_bfloat16 q = __float2bfloat16(0.f);
             if (o < L.out && i < L.in) {
                 const int64_t e = (int64_t)o * L.in + i;
-                float g;
-                if (L.shares > 1) {
-                    g = L.part[e];
-#pragma unroll 4
-                    for (int z = 1; z < L.shares; ++z) g += L.part[z * L.pitch + e];
-                    L.g[e] = g;
-                } else {
-                    g = L.g[e];
-                }
-                adamw_one(h, L.w + e, g, L.mw + e, L.vw + e, true);
+                if (L.shares > 1) L.g[e] = g[k];
+                adamw_one(h, L.w + e, g[k], L.mw + e, L.vw + e, true);
                 q = __float2bfloat16(L.w[e]);
                 L.wbf[(int64_t)o * L.ldw + i] = q;
             }

@@ -253,9 +253,9 @@ __device__ __forceinline__ void stage_aux(EpiStage &st, const float4 (&q)[4]) {
 }
 
 // Epilogue of one 32-row x 16-column chunk: rows row0 + [0, nrow), columns n + [0, nv); v holds
-// this thread's row (row0 + lane) of the accumulator. share: the K share, if they are stored apart.
-__device__ __forceinline__ void epi_chunk(const GemmOut &out, int share, EpiStage &st, bool split, int row0, int n,
-                                          int nrow, int nv, float (&v)[16]) {
+// this thread's row (row0 + lane) of the accumulator.
+__device__ __forceinline__ void epi_chunk(const GemmOut &out, EpiStage &st, bool split, int row0, int n, int nrow,
+                                          int nv, float (&v)[16]) {
     const int lane = threadIdx.x & 31;
     const bool vc = out.vec & 1, vy = out.vec & 2, vt = out.vec & 8;
     switch (out.epi) {
@@ -266,7 +266,7 @@ __device__ __forceinline__ void epi_chunk(const GemmOut &out, int share, EpiStag
 #pragma unroll
             for (int j = 0; j < 4; ++j) st.c[cidx(lane, j)] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
             __syncwarp();
-            flush_c(st, out.C + share * out.share_stride, out.ldc, row0, n, nrow, nv, vc, split, out.epi == EPI_F32_ADD);
+            flush_c(st, out.C, out.ldc, row0, n, nrow, nv, vc, split, out.epi == EPI_F32_ADD);
             break;
         }
         case EPI_BIAS_GELU: {
@@ -313,7 +313,9 @@ struct SplitMaps<true> {
 // SPLIT: three passes over K into one accumulator, A B2^T, A2 B^T and last A B^T: the tensor core's
 // accumulation cuts off below the last bit of the running sum, so the small products go first
 // (last, they doubled the product's error, 1.1e-6 to 2.2e-6 of the expectation).
-template <bool TF32, bool SPLIT>
+// APART: the shares of a K split go to rows of their own (GemmOut::shares_apart); a build of its own,
+// because the fused epilogues use all 96 registers and one more value spills (GELU form +5 %).
+template <bool TF32, bool SPLIT, bool APART>
 __global__ void __launch_bounds__(kThreads, 1)
     tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, int M, int N,
                    int K, Plan pl, GemmOut out, int *err, const __grid_constant__ SplitMaps<SPLIT> second) {
@@ -334,7 +336,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     constexpr int kPasses = SPLIT ? 3 : 1;
     const int kel = TF32 ? 32 : 64;
     const int ktiles = (K + kel - 1) / kel;
-    const bool split = pl.splits > 1 && out.share_stride == 0;
+    const bool split = pl.splits > 1 && !APART;
     const uint32_t tcols = 2u * (uint32_t)pl.acc_cols;
 
     if (warp == 2) umma::tmem_alloc(tmem_slot, tcols);
@@ -451,7 +453,9 @@ __global__ void __launch_bounds__(kThreads, 1)
             int m0, n0, kt0, kn;
             unit(u, m0, n0, kt0, kn);
             const int a = lt & 1;
-            const int row0 = m0 + quad * 32, nrow = min(32, M - row0);
+            int row0 = m0 + quad * 32;
+            const int nrow = min(32, M - row0);
+            if constexpr (APART) row0 += u / (pl.ntn * pl.mt) * M;   // this share's rows of C
             auto chunk_nv = [&](int c) { return c < n_tile ? min(min(16, n_tile - c), N - (n0 + c)) : 0; };
             if (dgelu && nrow > 0 && chunk_nv(sub * 16) > 0)   // travels while the products accumulate
                 load_aux(out, row0, n0 + sub * 16, nrow, chunk_nv(sub * 16), qa);
@@ -460,7 +464,6 @@ __global__ void __launch_bounds__(kThreads, 1)
                 break;
             }
             umma::tc_fence_after();
-            const int share = u / (pl.ntn * pl.mt);
             const uint32_t tbase = tmem + (uint32_t)(a * pl.acc_cols) + ((uint32_t)(quad * 32) << 16);
             for (int c = sub * 16; c < n_tile; c += 64) {
                 const int nv = chunk_nv(c);
@@ -473,7 +476,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                         const int nv2 = chunk_nv(c + 64);
                         if (nv2 > 0) load_aux(out, row0, n0 + c + 64, nrow, nv2, qa);
                     }
-                    epi_chunk(out, share, st, split, row0, n0 + c, nrow, nv, v);
+                    epi_chunk(out, st, split, row0, n0 + c, nrow, nv, v);
                 }
             }
             umma::tc_fence_before();
@@ -584,8 +587,8 @@ static int launch_gemm(bool tf32, int M, int N, int K, const void *A, const void
               ((out.aux && !((uintptr_t)out.aux & 15) && out.ldaux % 4 == 0) ? 4 : 0) |
               ((out.Yt && !((uintptr_t)out.Yt & 15) && out.ldyt % 8 == 0) ? 8 : 0) |
               ((out.bias && !((uintptr_t)out.bias & 15)) ? 16 : 0);
-    if (out.share_stride % 4 || (out.share_stride && out.epi != EPI_F32))
-        return fitcore_fail(FIT_ERR_INVALID_ARG, "tensor-core GEMM: stride of the K shares");
+    if (out.shares_apart && (out.epi != EPI_F32 || tf32))
+        return fitcore_fail(FIT_ERR_INVALID_ARG, "tensor-core GEMM: K shares of this form");
     const Plan pl = make_plan(tf32, M, N, K, out.epi, out.deterministic);
     CUtensorMap ta, tb;
     if ((rc = make_map(&ta, tf32, A, M, K, lda, kTileM))) return rc;
@@ -612,12 +615,15 @@ static int launch_gemm(bool tf32, int M, int N, int K, const void *A, const void
     }
     const size_t smem = 1024 + (size_t)pl.stages * (kTileM + pl.n_tile) * kRowBytes + kEpiWarps * sizeof(EpiStage) +
                         (2 * pl.stages + 5) * 8 + 16;
-    const int which = A2 ? 2 : tf32 ? 1 : 0;
-    const void *kern = A2 ? (const void *)tc_gemm_kernel<true, true>
-                       : tf32 ? (const void *)tc_gemm_kernel<true, false> : (const void *)tc_gemm_kernel<false, false>;
+    const bool apart = out.shares_apart;
+    const int which = A2 ? 2 : apart ? 3 : tf32 ? 1 : 0;
+    const void *kern = A2      ? (const void *)tc_gemm_kernel<true, true, false>
+                       : apart ? (const void *)tc_gemm_kernel<false, false, true>
+                       : tf32  ? (const void *)tc_gemm_kernel<true, false, false>
+                               : (const void *)tc_gemm_kernel<false, false, false>;
     {
         static std::mutex attr_mutex;
-        static int attr_set[3] = {0, 0, 0};
+        static int attr_set[4] = {0, 0, 0, 0};
         std::lock_guard<std::mutex> lock(attr_mutex);
         int &cur = attr_set[which];
         if ((int)smem > cur) {   // only ever raised
@@ -628,7 +634,7 @@ static int launch_gemm(bool tf32, int M, int N, int K, const void *A, const void
             cur = (int)smem;
         }
     }
-    if (pl.splits > 1 && out.epi == EPI_F32 && out.share_stride == 0) {
+    if (pl.splits > 1 && out.epi == EPI_F32 && !out.shares_apart) {
         // C = 0 first: rows of ldc floats (the row tails beyond N are left as they were)
         cudaError_t e = (out.ldc == N) ? cudaMemsetAsync(out.C, 0, sizeof(float) * (size_t)M * N, stream)
                                        : cudaMemset2DAsync(out.C, sizeof(float) * (size_t)out.ldc, 0,
@@ -637,11 +643,13 @@ static int launch_gemm(bool tf32, int M, int N, int K, const void *A, const void
     }
     const int grid = std::min(pl.units, kNumSMs);
     if (A2)
-        tc_gemm_kernel<true, true><<<grid, kThreads, smem, stream>>>(ta, tb, M, N, K, pl, out, err_dev, second);
+        tc_gemm_kernel<true, true, false><<<grid, kThreads, smem, stream>>>(ta, tb, M, N, K, pl, out, err_dev, second);
+    else if (apart)
+        tc_gemm_kernel<false, false, true><<<grid, kThreads, smem, stream>>>(ta, tb, M, N, K, pl, out, err_dev, {});
     else if (tf32)
-        tc_gemm_kernel<true, false><<<grid, kThreads, smem, stream>>>(ta, tb, M, N, K, pl, out, err_dev, {});
+        tc_gemm_kernel<true, false, false><<<grid, kThreads, smem, stream>>>(ta, tb, M, N, K, pl, out, err_dev, {});
     else
-        tc_gemm_kernel<false, false><<<grid, kThreads, smem, stream>>>(ta, tb, M, N, K, pl, out, err_dev, {});
+        tc_gemm_kernel<false, false, false><<<grid, kThreads, smem, stream>>>(ta, tb, M, N, K, pl, out, err_dev, {});
     fitcore_count_launch();
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess)

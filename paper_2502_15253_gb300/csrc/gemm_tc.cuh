@@ -35,10 +35,10 @@ struct GemmOut {
     // never split K over CTAs (the split adds partial tiles with atomics, so its FP32 sums
     // depend on their order): results identical from call to call
     bool deterministic = false;
-    // EPI_F32: not 0 = the shares of a K split are stored apart instead, share z's product at
-    // C + z * share_stride (floats, a multiple of 4); the caller adds tc_gemm_shares of them in
-    // the order it likes, so that its sums do not depend on the order in which CTAs finish
-    int64_t share_stride = 0;
+    // EPI_F32, bf16: the shares of a K split are stored apart instead, share z's product in rows z M on of
+    // C; the caller adds tc_gemm_shares of them in the order it likes, so that its sums do not
+    // depend on the order in which CTAs finish
+    bool shares_apart = false;
 };
 
 // K shares of tc_gemm's plan for an EPI_F32 product of these sizes, and the most that any K up to

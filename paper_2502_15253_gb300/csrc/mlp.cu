@@ -29,9 +29,8 @@ inline int pad8(int x) { return (x + 7) / 8 * 8; }
 // bits on every run: each such block and each K share of a weight gradient leaves its own partial
 // sum, and the AdamW kernel, which reads every gradient once, adds them in order. With atomics the
 // first step's gradients differed by 1e-7 from run to run, and the steps after it, through AdamW and
-// the bf16 roundings, by up to 1.5e-3 (438 -> 3 x 512 -> 12, batch 4096). A step took 163 us at batch
-// 512, 205 at 4096 and 357 at 16384 with atomics and their clears; it takes 144, 195 and 362 (the
-// largest batch has 57 MB of shares to store and read).
+// the bf16 roundings, by up to 1.5e-3 (438 -> 3 x 512 -> 12, batch 4096). A step took 167 us at batch
+// 512, 206 at 4096 and 360 at 16384 with atomics and their clears; it takes 148, 195 and 354.
 constexpr int kColRows = 256;
 
 __global__ void prep_input_kernel(int B, int n_in, int ld, const float *__restrict__ x, __nv_bfloat16 *__restrict__ a0) {
@@ -155,11 +154,10 @@ __device__ __forceinline__ void adamw_one(const AdamW &h, float *p, float gr, fl
 
 // Per-layer arguments of the fused AdamW launch: the [out x in] weights (W bf16 copy with rows
 // of ldw, W^T with rows of ldwt) and the bias. The weight gradient comes as `shares` (> 1) products
-// of a K share each, `pitch` floats apart, or whole in g (1); the bias gradient as row sums.
+// of a K share each, one after another, or whole in g (1); the bias gradient as row sums.
 struct AdamLayer {
     int out, in, ldw, ldwt, tiles_i, wtiles;   // wtiles = ceil(out/32) ceil(in/32) weight tiles
     int shares;
-    int64_t pitch;
     const float *part, *bpart;
     float *w, *g, *mw, *vw, *b, *gb, *mb, *vb;
     __nv_bfloat16 *wbf, *wt;
@@ -187,7 +185,7 @@ __global__ void __launch_bounds__(256) adamw_all_kernel(AdamW h, AdamAll A) {
         // the gradients of this thread's four weights: the K shares added in order, sixteen loads in
         // flight (the shares come from L2; past the ends the last row or share is read again)
         const int i = i0 + threadIdx.x, shares = L.shares, last = L.out - 1;
-        const int64_t in = L.in, pitch = shares > 1 ? L.pitch : 0;
+        const int64_t in = L.in, pitch = in * L.out;
         const float *src = (shares > 1 ? L.part : L.g) + min(i, L.in - 1);
         float g[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll 1
@@ -325,10 +323,9 @@ struct fit_mlp {
     __nv_bfloat16 *dpreT[kMaxLayers] = {nullptr};
     double *loss = nullptr;
     // partial sums of a training step (kColRows): the loss, the bias gradients and, for layers whose
-    // weight gradient is a product split over K, its shares (wpitch floats each)
+    // weight gradient is a product split over K, its shares one after another
     double *lpart = nullptr;
     float *bpart[kMaxLayers] = {nullptr}, *wpart[kMaxLayers] = {nullptr};
-    int64_t wpitch[kMaxLayers] = {0};
     void *parts = nullptr;          // the allocation that holds them
     std::vector<void *> owned;
 };
@@ -403,10 +400,9 @@ int ensure_batch(fit_mlp *m, int B) {
     const size_t at_l = take(sizeof(double) * rows);
     for (int l = 0; l < L; ++l) {
         const int o = m->dims[l + 1], in = m->dims[l];
-        m->wpitch[l] = ((int64_t)o * in + 3) & ~int64_t(3);
         at_b[l] = take(sizeof(float) * (size_t)rows * o);
         const int shares = fitcore::tc_gemm_max_shares(false, o, in, B);
-        at_w[l] = shares > 1 ? take(sizeof(float) * (size_t)shares * m->wpitch[l]) : 0;
+        at_w[l] = shares > 1 ? take(sizeof(float) * (size_t)shares * o * in) : 0;
     }
     if (!rc && cudaMalloc(&m->parts, bytes) != cudaSuccess) {
         cudaGetLastError();
@@ -582,7 +578,7 @@ int fit_mlp_train_step(fit_mlp *m, int B, const float *x, const float *target, f
         shares[l] = fitcore::tc_gemm_shares(false, o, in, B);
         gw.C = shares[l] > 1 ? m->wpart[l] : m->gw[l];
         gw.ldc = in;
-        gw.share_stride = shares[l] > 1 ? m->wpitch[l] : 0;
+        gw.shares_apart = shares[l] > 1;
         if ((rc = fitcore::tc_gemm(false, o, in, B, m->dpreT[l], Bp, m->actT[l], Bp, gw, s, nullptr))) return rc;
         if (l > 0) {
             // d pre_{l-1} = (d pre_l W_l) * gelu'(pre_{l-1})
@@ -622,7 +618,6 @@ int fit_mlp_train_step(fit_mlp *m, int B, const float *x, const float *target, f
         q.tiles_i = (q.in + 31) / 32;
         q.wtiles = ((q.out + 31) / 32) * q.tiles_i;
         q.shares = shares[l];
-        q.pitch = m->wpitch[l];
         q.part = m->wpart[l];
         q.bpart = m->bpart[l];
         q.w = m->w[l];

@@ -104,7 +104,6 @@ __global__ void __launch_bounds__(kSignalThreads, 4) signal_v_kernel(const DevMo
         }
         const PP nrm = S.E.nrm[0];
         const EMap em = S.E.em[0];
-        const float is = 1.f / em.slope(0.5f * (m.e_first + m.e_last));
 #pragma unroll 1
         for (int k = tid; k < N_t; k += nth) {
             const float ih = m.inv_e_hi[k], il = m.inv_e_lo[k], e0 = m.e_edge[k], e1 = m.e_edge[k + 1];
@@ -129,7 +128,7 @@ __global__ void __launch_bounds__(kSignalThreads, 4) signal_v_kernel(const DevMo
 #pragma unroll 1
         for (int t = tid; t < m.ldt; t += nth) {
             float acc = 0.f;
-            if (t < N_t) acc = spline ? spline_target(u, T, t, N_t) : overlap_target(u, T.t, is, t, N_t);
+            if (t < N_t) acc = spline ? spline_target(u, T, t, N_t) : overlap_target(u, T.t, em.inv_slope, t, N_t);
             const float hi = tf32_round(acc);
             vh[t] = hi;
             vl[t] = acc - hi;

@@ -522,7 +522,7 @@ constexpr int kStEscale = 2;
 
 // Energy map of dataset d in grid units: displacement D(e) = (a0 + (a1-1) e + a2 e^2) / de.
 struct EMap {
-    float a0, a1m1, a2, inv_de, e_lo, de;
+    float a0, a1m1, a2, inv_de, inv_slope, de;   // inv_slope: 1 / slope at mid grid, nearly (a first guess)
     __device__ __forceinline__ float disp(float e) const {
         return fmaf(fmaf(a2, e, a1m1), e, a0) * inv_de;
     }
@@ -685,7 +685,7 @@ __device__ __forceinline__ EMap make_emap(const DevModel &m, const DevDataset &d
     em.a1m1 = ds.esc_idx[1] >= 0 ? ds.a1_off + pd[ds.esc_idx[1]] : 0.f;
     em.a2 = ds.esc_idx[2] >= 0 ? pv[ds.esc_idx[2]] : 0.f;
     em.inv_de = m.inv_de;
-    em.e_lo = m.e_lo;
+    em.inv_slope = __fdividef(1.f, em.slope(0.5f * (m.e_first + m.e_last)));
     em.de = m.de;
     return em;
 }
@@ -1088,7 +1088,7 @@ static __device__ __forceinline__ void st_remap(const DevModel &m, const EvalSha
 #pragma unroll 1
     for (int i = 0; i < E.n; ++i) {
         const DsWs ws = carve_ds_ws(wsb + (int64_t)i * m.ws_eval_floats, N_t, m.C, m.max_reco, m.n_osc);
-        const float is = 1.f / E.em[i].slope(0.5f * (m.e_first + m.e_last));
+        const float is = E.em[i].inv_slope;
 #pragma unroll 1
         for (int t = rot_tid(i, (N_t + 31) >> 5); t < N_t; t += nth)
             ws.v[t] = spline ? spline_target(ws.u, ws.edge, t, N_t) : overlap_target(ws.u, ws.edge.t, is, t, N_t);

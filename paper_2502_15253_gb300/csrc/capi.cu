@@ -2754,7 +2754,7 @@ int fit_batch_ex(fit_model *const *models, int n_models, const fit_instance *ins
             rc = fail(FIT_ERR_OOM, "fit_batch: workspace");
         dws[q].owned = true;
     }
-    // the work queues, 8 bytes apart, then (several launches) the time that the first block started at
+    // the work queues, 8 bytes apart, then (several launches) the clock that their budget counts from
     const size_t q_bytes = 8 * (launches.size() + 1);
     if (!rc) {
         if (fitcore::pool_alloc(&dq.dev, q_bytes, s) ||
@@ -2762,7 +2762,13 @@ int fit_batch_ex(fit_model *const *models, int n_models, const fit_instance *ins
             rc = fail(FIT_ERR_CUDA, "fit_batch: queue");
         dq.owned = true;
     }
-    if (!rc && side && cudaEventRecord(side->ready, s) != cudaSuccess) rc = fail(FIT_ERR_CUDA, "fit_batch: fork");
+    uint64_t *began = side ? (uint64_t *)((char *)dq.dev + 8 * launches.size()) : nullptr;
+    if (!rc && side) {
+        fitcore::clock_kernel<<<1, 1, 0, s>>>(began);
+        g_launches++;
+        if (cudaGetLastError() != cudaSuccess || cudaEventRecord(side->ready, s) != cudaSuccess)
+            rc = fail(FIT_ERR_CUDA, "fit_batch: fork");
+    }
     size_t forked = 0;
     for (size_t q = 0, first = 0; q < launches.size() && !rc; first += launches[q++].n) {
         const FitLaunch &L = launches[q];
@@ -2797,7 +2803,7 @@ int fit_batch_ex(fit_model *const *models, int n_models, const fit_instance *ins
         a.smem_floats = L.placement == 1 ? L.max_need : L.placement == 2 ? L.max_loc : 0;
         a.hist_global = L.placement == 1 ? 0 : 1;
         a.budget_ns = (uint64_t)(o.time_budget_s * 1e9);
-        a.began = side ? (unsigned long long *)((char *)dq.dev + 8 * launches.size()) : nullptr;
+        a.began = began;
         a.precond = L.precond ? 1 : 0;
         a.order = reordered ? (const int *)dord.dev + first : nullptr;
         a.pre_tab = (L.precond && pre_k > 0) ? (const fitcore::PreEntry *)dpre.dev : nullptr;

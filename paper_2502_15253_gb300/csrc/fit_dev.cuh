@@ -874,12 +874,8 @@ __global__ void __launch_bounds__(T, MINB) fit_kernel(FitArgs A) {
     F.restarts = A.restarts;
     F.edm_tol = A.edm_tol;
     F.f_noise_rel = A.f_noise_rel;
-    F.deadline = global_ns() + A.budget_ns;   // per-block clock budget (the first thread's counts)
+    F.deadline = (A.began ? *A.began : global_ns()) + A.budget_ns;   // (the first thread's counts)
     const int tid = threadIdx.x;
-    if (A.began && tid == 0) {
-        const unsigned long long now = global_ns(), first = atomicCAS(A.began, 0ull, now);
-        F.deadline = (first ? first : now) + A.budget_ns;
-    }
 
     while (true) {
         if (tid == 0) S.inst = atomicAdd(A.queue, 1);

@@ -47,8 +47,8 @@ struct FitArgs {
     int hist_global;             // 1: the L-BFGS history lives in the global slice
     const uint8_t *fixed;        // device, indexed like start/best, or nullptr: held parameters
     uint64_t budget_ns;
-    unsigned long long *began;   // device word, zero at launch, or nullptr: several launches of one call
-                                 // share the clock budget, from their first block's start
+    const uint64_t *began;       // device word: the clock that the budget counts from (clock_kernel), for
+                                 // several launches of one call; nullptr: each block's start
     int precond;                 // 1: fit in the models' preconditioned coordinates (if built)
     const int *order;            // device [n_inst] or nullptr: the instance taken at each queue
                                  // position (costliest first, so no long fit starts last)
@@ -129,6 +129,8 @@ __global__ void ls_step_kernel(LsArgs A);
 size_t ls_state_bytes();
 size_t ls_step_smem_bytes(const DevModel &hm);
 size_t ls_eval_smem_bytes(int P, int ws_floats);
+
+__global__ void clock_kernel(uint64_t *t);   // *t = the device's clock
 
 // the persistent fit kernel (host entry address): blocks of up to 128 threads compiled for 4 or 5
 // resident blocks per SM (variant), of 256 threads (2 per SM) or of 512 (1 per SM)

@@ -2381,8 +2381,12 @@ struct FitLaunch {
 // Workspace placement and kernel variant (resident blocks per SM the registers allow).
 int fit_launch_shape(fit_model *const *models, const fit_batch_opts &o, bool auto_shape, const LaunchCfg &cfg,
                      FitLaunch &L) {
-    // what a requested placement is judged by: 14 working vectors, the history, one dataset's
-    // workspace and 25184 bytes of block state within 112 KB
+    // What a caller's placement is judged by, apart from what the kernel needs now (which is checked below
+    // against the device's limit): the interface accepts a placement if 14 working vectors, the
+    // history where it is asked for, one dataset's workspace and kAskState bytes of block state
+    // stay within kAskCap, two such blocks per SM. The kernel has since grown (15 vectors, the
+    // workspaces of several datasets); the line stays where callers know it.
+    constexpr size_t kAskState = 25184, kAskCap = 112 * 1024;
     size_t ask_all = 0, ask_loc = 0;
     for (int mi : L.models) {
         const DevModel &h = models[mi]->host;
@@ -2391,8 +2395,8 @@ int fit_launch_shape(fit_model *const *models, const fit_batch_opts &o, bool aut
         L.max_need = std::max(L.max_need, fitcore::fit_vec_floats(h.P, o.history) + h.ws_floats);
         L.max_loc = std::max(L.max_loc, fitcore::fit_work_floats(h.P) + h.ws_floats);
         const size_t one = (((size_t)(4 + h.n_osc + h.C) * h.N_t + 2 * h.max_reco + 3) & ~size_t(3)) + 14 * (size_t)fitcore::fit_vec_pitch(h.P);
-        ask_loc = std::max(ask_loc, 25184 + sizeof(float) * one);
-        ask_all = std::max(ask_all, 25184 + sizeof(float) * (one + (size_t)fitcore::fit_hist_floats(h.P, o.history)));
+        ask_loc = std::max(ask_loc, kAskState + sizeof(float) * one);
+        ask_all = std::max(ask_all, kAskState + sizeof(float) * (one + (size_t)fitcore::fit_hist_floats(h.P, o.history)));
     }
     // Shared memory holds what fits in ~1/2 of an SM's share; the automatic choice takes the
     // combination with the most resident fits per SM (ties: more in shared memory).
@@ -2406,8 +2410,9 @@ int fit_launch_shape(fit_model *const *models, const fit_batch_opts &o, bool aut
         // model 14.0 / 11.5 / 10.8 and a scan of 42 of its fits 6.5 / 3.9 / 2.6; 300 three-dataset
         // fits 7.0 / 4.2 / -, 2500 with the spline 7.1 / 8.5 / 12.0; 2500 single-detector fits 2.2 / 2.5
         // / 4.1. Many waves of fits run faster in blocks of 128 (8192: 62.5 against 75.3 and 43.5
-        // against 50.0 under this rule), which fit_batch_autotune finds; the number of fits is not
-        // looked at, so that a fit does not depend on the batch around it.
+        // against 50.0 under this rule), which fit_batch_autotune finds (it does not try this rule's
+        // shapes); the number of fits is not looked at, so that a fit does not depend on the batch
+        // around it.
         L.placement = L.smem_for(2) * (512 / L.threads) > cfg.smem_optin ? 3 : 2;
     }
     auto kernel_for = [&](int variant) { return fitcore::fit_kernel_func(L.threads, variant, L.general, L.precond); };
@@ -2441,7 +2446,7 @@ int fit_launch_shape(fit_model *const *models, const fit_batch_opts &o, bool aut
     } else {
         if (o.blocks_per_sm == 0) variant = L.placement == 3 ? 5 : 4;
         const size_t ask = L.placement == 1 ? ask_all : L.placement == 2 ? ask_loc : 0;
-        if (!auto_shape && ask > 112 * 1024)
+        if (!auto_shape && ask > kAskCap)
             return fail(FIT_ERR_INVALID_CONFIG, "fit_batch: the requested workspace placement does not fit an SM");
         kSmemCap = cfg.smem_optin;
     }

@@ -190,9 +190,12 @@ __host__ __device__ inline int fit_work_floats(int P) { return 15 * fit_vec_pitc
 // steps, but each thread then holds fewer bins and every barrier spans more warps, so the block
 // grows with the true bins evaluated together. Measured (us, batched -2lnL with gradient, 128 /
 // 256 / 512 threads): 200 bins x 4096 vectors 105 / 175 / 322; 1200 bins x 4096 462 / 464 / 628
-// (where few vectors or fits run, 256 threads win: capi.cu); 2000 bins x 2048 1929 / 1227 / 941. A
-// property of the model alone: the result of a vector or a fit does not depend on the batch
-// around it.
+// (where few vectors or fits run, 256 threads win: capi.cu); 2000 bins and ten cores x 2048 1929 / 1227 /
+// 941. Between and past the lines, x 4096: 450 bins 223 / 309 / 510, 600 bins 207 / 275 / 463 (one
+// vector 31 / 25 / 27), 1000 bins 340 / 386 / 591, 1500 bins 663 / 506 / 703, 1800 bins and four cores
+// 766 / 569 / 794 (one vector 54 / 40 / 33), 3000 bins and ten cores 1752 / 1344 / 1642 (one vector
+// 117 / 76 / 58). A property of the model alone: the result of a vector or a fit does not depend
+// on the batch around it.
 inline int model_threads(const DevModel &h) {
     const int bins = h.N_t * h.ws_group;
     return bins <= 512 ? 128 : bins <= 1600 ? 256 : 512;
